@@ -200,3 +200,39 @@ def test_exposure_registration_matches_oracle(gs, ctx):
     with pytest.raises(gs.GsError):
         gs.gs_register(ctx, g, g, [], [(cam, dev(t_rgb), dev(t_dep))], 2,
                        gs.default_options(exposure=1, tracking_loss=1))
+
+
+@pytest.mark.parametrize("w,h", [(1, 1), (7, 1), (64, 1), (8193, 1), (128, 64), (317, 241), (1031, 509)])
+@pytest.mark.parametrize("kind", ["spread", "ties", "few", "none"])
+def test_track_median_sizes(gs, ctx, w, h, kind):
+    # pixel counts around a cluster's split of a keyframe (8 slices of
+    # 1024-pixel rounds), two keyframes of different sizes in one call; the
+    # median and the inliers are exact (an order statistic of FP32 values)
+    rng = np.random.default_rng(w * 1000 + h)
+    sizes = [(w, h), (97, 33)]
+    cams = np.stack([synth.camera(50.0, 50.0, x / 2, y / 2, x, y, np.eye(3, 4)) for x, y in sizes])
+    dep, tgt = [], []
+    for x, y in sizes:
+        n = x * y
+        d = (rng.uniform(0.5, 4.0, n) * 10.0 ** rng.integers(-6, 3, n)).astype(np.float32)
+        t = rng.uniform(0.5, 4.0, n).astype(np.float32)
+        if kind == "ties":
+            d, t = np.round(d, 1).astype(np.float32), np.ones(n, np.float32)
+        if kind == "few":
+            t[rng.random(n) < 0.9] = 0.0
+        if kind == "none":
+            t[:] = 0.0
+        dep.append(d)
+        tgt.append(t)
+    n = sum(len(d) for d in dep)
+    rgb, tf = rng.uniform(0, 1, 3 * n), rng.uniform(0, 1, n)
+    _, _, _, inl, med = gs.gs_track_loss(ctx, cams, dev(rgb), dev(np.concatenate(dep)), dev(tf),
+                                         dev(rng.uniform(0, 1, 3 * n)), dev(np.concatenate(tgt)))
+    inl, med, o = inl.cpu().numpy(), med.cpu().numpy(), 0
+    for k, (d, t) in enumerate(zip(dep, tgt)):
+        e = np.abs(d - t)
+        v = np.sort(e[t > 0])
+        want = v[(len(v) - 1) // 2] if len(v) else np.float32(0)
+        assert med[k] == want
+        np.testing.assert_array_equal(inl[o:o + len(d)].astype(bool), (t > 0) & (e <= np.float32(50.0) * want))
+        o += len(d)
