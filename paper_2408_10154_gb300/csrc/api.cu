@@ -21,10 +21,9 @@
 namespace {
 
 enum Slot {
-    S_VPS, S_GROUPS, S_TILEVP, S_POSE32, S_REC, S_AUX, S_COUNTS, S_PARTIALS, S_NDUPS, S_K0, S_V0, S_V1,
-    S_HIST, S_HISTP, S_RANGES, S_FLAGS, S_TF, S_LAST, S_CODE, S_TLOSS, S_TTWIST, S_POSE64, S_ADAM, S_PIVOT,
+    S_VPS, S_GROUPS, S_TILEVP, S_POSE32, S_REC, S_AUX, S_COUNTS, S_PARTIALS, S_NDUPS, S_K0, S_V0, S_RANGES, S_FLAGS, S_TF, S_LAST, S_CODE, S_TLOSS, S_TTWIST, S_POSE64, S_ADAM, S_PIVOT,
     S_CCAM, S_CENT, S_LOSS, S_SETVP, S_REV, S_PFIRST, S_PCOUNT, S_TOUT, S_CONF, S_EST, S_GRAD, S_DUPG,
-    S_PAIRS, S_RK0, S_RK1, S_RP0, S_RP1, S_RRANGES, S_TERR, S_TCOL, S_TW,
+    S_PAIRS, S_RSLOT, S_RSLOTN, S_TERR, S_TCOL, S_TW,
     S_TMED, S_TNV, S_TVPS, S_EXPO, S_EXPO32, S_TEXPO, S_OPT, S_ONN1, S_ONN2, S_OD2, S_OT, S_OCNT, S_MAPS, S_OS, S_ORDER, S_ORDC, S_SK, S_SV, S_SN, S_OBOX, S_GCELL, S_GSTART, S_GCUR, S_GPART, S_GPTS, S_GIDX, S_GLIST, S_GNL, S_GCELL2, S_GSTART2, S_GCUR2, S_GPART2, S_GPTS2, S_GIDX2, S_GLIST2, S_GNL2, S_SEGZ, S_SEGCUR, S_SEGBIG, S_SEGLIST, S_PROBE, S_QUEUE, S_COUNT
 };
 
@@ -389,10 +388,6 @@ gs_status_t alloc_sort(gs_ctx *ctx, uint64_t want, Pipe &p)
     const uint32_t cap = (uint32_t)std::max<uint64_t>(want, 1024);
     GS_TRY(wsT(ctx, S_K0, cap, &p.tkeys[0]));
     GS_TRY(wsT(ctx, S_V0, cap, &p.vals[0]));
-    GS_TRY(wsT(ctx, S_V1, cap, &p.vals[1]));
-    const size_t hn = gsl::sort_hist_entries((uint32_t)std::max<uint64_t>(cap, p.n_records));
-    GS_TRY(wsT(ctx, S_HIST, hn, &p.hist));
-    GS_TRY(wsT(ctx, S_HISTP, gsl::scan_partials(hn), &p.histp));
     p.cap = cap;
     return GS_OK;
 }
@@ -971,18 +966,17 @@ gs_status_t backward_core(gs_ctx *ctx, const Plan &P, const DevPlan &D, Pipe &p,
         ++gsl::g_launches;
     }
     r.c_cam = ccam;
-    if (full)
-        GS_TRY(wsT(ctx, S_DUPG, 10 * (size_t)p.cap, &r.dup_grads));
+    uint32_t *slots = nullptr;
+    if (full) {
+        uint32_t *total = nullptr;
+        GS_TRY(wsT(ctx, S_DUPG, 12 * (size_t)p.cap, &r.dup_grads));
+        GS_TRY(wsT(ctx, S_RSLOT, (size_t)std::max<uint64_t>(P.n_records, 1), &slots));
+        GS_TRY(wsT(ctx, S_RSLOTN, 1, &total));
+        gsl::rec_slots(p.counts, (uint32_t)P.n_records, total, slots, s);
+        r.rec_slot = slots;
+    }
     gsl::backward(r, false, full, s);
     if (full) {
-        // group the duplicates by record, then chain per Gaussian
-        uint32_t *rk[2] = {nullptr, nullptr}, *rp[2] = {nullptr, nullptr};
-        uint2 *rr = nullptr;
-        GS_TRY(wsT(ctx, S_RK0, p.cap, &rk[0]));
-        GS_TRY(wsT(ctx, S_RK1, p.cap, &rk[1]));
-        GS_TRY(wsT(ctx, S_RP0, p.cap, &rp[0]));
-        GS_TRY(wsT(ctx, S_RP1, p.cap, &rp[1]));
-        GS_TRY(wsT(ctx, S_RRANGES, (size_t)std::max<uint64_t>(P.n_records, 1), &rr));
         gsl::ParamArgs pa{};
         pa.vps = D.vps;
         pa.n_vps = nv;
@@ -991,6 +985,8 @@ gs_status_t backward_core(gs_ctx *ctx, const Plan &P, const DevPlan &D, Pipe &p,
         pa.aux = p.aux;
         pa.pose32 = poses;
         pa.dup_grads = r.dup_grads;
+        pa.counts = p.counts;
+        pa.rec_slot = slots;
         pa.quats = (const float4 *)g->quats;
         pa.scales = (const float4 *)g->log_scales;
         pa.logits = g->opacity_logits;
@@ -999,8 +995,7 @@ gs_status_t backward_core(gs_ctx *ctx, const Plan &P, const DevPlan &D, Pipe &p,
         pa.g_quats = grads->quats;
         pa.g_logits = grads->opacity_logits;
         pa.g_rgb = grads->rgb;
-        gsl::param_grads(pa, p.vals[cur], p.ndups, p.cap, rk, rp, tile_bits(P.n_records), p.hist, p.histp, rr,
-                         (uint32_t)P.n_records, s);
+        gsl::param_grads(pa, s);
     }
     gsl::PoseArgs a{};
     a.vps = D.vps;
@@ -1262,11 +1257,6 @@ gs_status_t gs_render_backward_saved(gs_ctx_t *ctx, const gs_saved_t *saved, con
     p.cap = saved->cap;
     p.n_records = std::max<uint64_t>(P.n_records, 1);
     const bool full = wants_params(grads);
-    if (full) {
-        const size_t hn = gsl::sort_hist_entries((uint32_t)std::max<uint64_t>(p.cap, p.n_records));
-        GS_TRY(wsT(ctx, S_HIST, hn, &p.hist));
-        GS_TRY(wsT(ctx, S_HISTP, gsl::scan_partials(hn), &p.histp));
-    }
     return backward_core(ctx, P, saved->D, p, 0, &saved->g, saved->pose32, &saved->opt, saved->t_final,
                          saved->last, d_rgb, d_depth, d_alpha, pivots, pose_grad, grads, full, s);
 }
@@ -2485,8 +2475,8 @@ double srv_now(const gs_server *srv)
 // Scratch of a request in a plan, from its measured tile duplicates nd:
 // per record 100 B (record 48, auxiliary 32, count 4, list entry 16); per
 // list entry of capacity (headroom x nd; a plan's 64 Ki spare entries come
-// out of the arena's slack) 12.5 B (depth bits, two value buffers,
-// histogram share); per pixel 9 B (final transmittance,
+// out of the arena's slack) 12.5 B (depth bits, value, and 4.5 B to
+// spare); per pixel 9 B (final transmittance,
 // last contributor, loss sign code), 12 B more for tracking masks; per tile
 // 92 B (range, keyframe, loss, twist, counters, cursors, order); per
 // keyframe problem its FP64 optimiser state.

@@ -1058,26 +1058,6 @@ __global__ void __launch_bounds__(1024) k_seg_sort_big(const gsl::BinArgs a)
     }
 }
 
-// stable LSD radix sort of (key, value) over `bits` low key bits, 8 per pass;
-// returns the buffer index holding the result
-template <typename K>
-int radix_sort(K *keys[2], uint32_t *vals[2], const uint32_t *n_dev, uint32_t cap, int bits, uint32_t *hist,
-               uint32_t *hist_partials, cudaStream_t s)
-{
-    const uint32_t sb = div_up(cap ? cap : 1, kSortTile);
-    const size_t hn = (size_t)256 * sb;
-    int cur = 0;
-    for (int shift = 0; shift < bits; shift += 8) {
-        k_rs_hist<K><<<sb, kSortThreads, 0, s>>>(keys[cur], n_dev, cap, shift, hist, sb);
-        gsl::scan_excl(hist, hist, hn, hist_partials, nullptr, s);
-        k_rs_scatter<K><<<sb, kSortThreads, 0, s>>>(keys[cur], vals[cur], n_dev, cap, shift, hist, sb, keys[cur ^ 1],
-                                                    vals[cur ^ 1]);
-        gsl::g_launches += 2;
-        cur ^= 1;
-    }
-    return cur;
-}
-
 }  // namespace
 
 namespace gsl {
@@ -1151,12 +1131,6 @@ int onesweep_u32(uint32_t *keys[2], uint32_t *vals[2], const uint32_t *n_dev, ui
         cur ^= 1;
     }
     return cur;
-}
-
-int sort_u32(uint32_t *keys[2], uint32_t *vals[2], const uint32_t *n_dev, uint32_t cap, int bits, uint32_t *hist,
-             uint32_t *hist_partials, cudaStream_t s)
-{
-    return radix_sort<uint32_t>(keys, vals, n_dev, cap, bits, hist, hist_partials, s);
 }
 
 size_t seg_zero_bytes(int n_vps, uint64_t n_diff)

@@ -343,7 +343,11 @@ struct RasterArgs {
     int count_contrib;               // count the pairs that pass the alpha test (forward variant)
     float2 *tile_twist;       // [tiles][6] camera-frame twist as FP32 (hi, lo) pairs (value hi + lo)
     const double *c_cam;      // [vp][3] pivot in camera frame
-    float *dup_grads;         // [dups][10] screen-space partials (full mode)
+    // full mode: screen-space partials of each (tile, record) pair, 12
+    // floats (10 used) per slot; the record's tiles own consecutive slots
+    // from rec_slot[record], row-major in its tile rectangle
+    float *dup_grads;
+    const uint32_t *rec_slot;
     // tracking-loss keyframes (loss_kind 1): the forward writes the FP32
     // depth error (+inf without input depth) and the colour L1 per pixel;
     // the backward scales the loss signs by the per-pixel mask weight
@@ -494,11 +498,6 @@ void loss(const gsk::VpDesc *vps, int n_vps, uint32_t n_tiles, const uint32_t *t
 void transform(const float4 *means, const float4 *quats, int64_t n, const double *T, float4 *out_means,
                float4 *out_quats, cudaStream_t s);
 
-// stable LSD radix sort of 32-bit keys with 32-bit values over `bits` low
-// bits (device-side count); returns the buffer index of the result
-int sort_u32(uint32_t *keys[2], uint32_t *vals[2], const uint32_t *n_dev, uint32_t cap, int bits, uint32_t *hist,
-             uint32_t *hist_partials, cudaStream_t s);
-
 // adjoint to every Gaussian parameter of one submap seen by n_vps cameras
 struct ParamArgs {
     const gsk::VpDesc *vps;
@@ -506,16 +505,15 @@ struct ParamArgs {
     int n;                    // Gaussians
     const float4 *rec, *aux;  // records of the forward
     const float *pose32;      // [vp][12]
-    const float *dup_grads;   // [dups][10] screen gradients, tile-sorted order
-    const uint32_t *rpos;     // dup positions grouped by record (filled by param_grads)
-    const uint2 *rec_ranges;  // [records] (filled by param_grads)
+    const float *dup_grads;   // [dups][12] screen gradients (see RasterArgs)
+    const int32_t *counts;    // [records] tiles touched
+    const uint32_t *rec_slot; // [records] first slot
     const float4 *quats, *scales;
     const float *logits;
     float *g_means, *g_scales, *g_quats, *g_logits, *g_rgb;  // outputs (any may be null)
 };
-void param_grads(const ParamArgs &a, const uint32_t *sorted_recs, const uint32_t *n_dups, uint32_t cap,
-                 uint32_t *rkeys[2], uint32_t *rpos[2], int rec_bits, uint32_t *hist, uint32_t *hist_partials,
-                 uint2 *rec_ranges, uint32_t n_records, cudaStream_t s);
-
+// first slots of the records from their tile counts; total: device scratch word
+void rec_slots(const int32_t *counts, uint32_t n_records, uint32_t *total, uint32_t *first, cudaStream_t s);
+void param_grads(const ParamArgs &a, cudaStream_t s);
 
 }  // namespace gsl

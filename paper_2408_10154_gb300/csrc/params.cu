@@ -1,61 +1,154 @@
 // params.cu -- the adjoint to every Gaussian parameter (the optional output
-// of gs_render_backward): per-duplicate screen gradients are grouped by
-// record (a radix sort of the duplicates by record index), then one thread
-// per Gaussian sums its records over the cameras in camera order and
-// chains the result through the projection, the rigid transform
-// (Eq. 8/9) and the scale / rotation / opacity parameterisation.  Fixed
-// summation order, no atomics.
+// of gs_render_backward): the adjoint kernel leaves each (tile, record)
+// pair's screen gradients in the record's own slots, and one thread per
+// Gaussian chains its records' sums, over the cameras in camera order,
+// through the projection, the rigid transform (Eq. 8/9) and the scale /
+// rotation / opacity parameterisation.  Fixed summation order, no atomics
+// on the gradients.
 #include "gs_internal.cuh"
 
 namespace {
 
 using namespace gsk;
 
-__global__ void k_iota_copy(const uint32_t *src, const uint32_t *n_dev, uint32_t cap, uint32_t *keys,
-                            uint32_t *pos)
+// First slot of every record's (tile, record) gradients: the record of tile
+// rectangle [x0, x1) x [y0, y1) owns (x1 - x0)(y1 - y0) consecutive slots,
+// one per tile in row-major order, so that the adjoint's tile CTA knows its
+// slot from the record alone and nothing has to be sorted by record.  A
+// block's records are consecutive; where the block's slots start follows
+// the order in which the blocks ask (no result depends on it).
+__global__ void __launch_bounds__(kScanThreads) k_rec_slots(const int32_t *counts, uint32_t n, uint32_t *total,
+                                                           uint32_t *first)
 {
-    const uint32_t n = min(*n_dev, cap);
-    const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) {
-        keys[i] = src[i];
-        pos[i] = i;
+    __shared__ uint32_t s_warp[kScanThreads / 32 + 1];
+    __shared__ uint32_t s_base;
+    constexpr int K = kScanTile / kScanThreads;
+    const uint32_t base = blockIdx.x * kScanTile + threadIdx.x * K;
+    uint32_t c[K], sum = 0;
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+        c[k] = base + k < n ? (uint32_t)counts[base + k] : 0u;
+        sum += c[k];
+    }
+    uint32_t tot;
+    uint32_t ex = block_excl_scan<kScanThreads>(sum, s_warp, tot);
+    if (threadIdx.x == 0)
+        s_base = tot ? atomicAdd(total, tot) : 0u;
+    __syncthreads();
+    ex += s_base;
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+        if (c[k])
+            first[base + k] = ex;
+        ex += c[k];
     }
 }
 
-// ranges of equal keys in a sorted key array (key = record index)
-__global__ void k_key_ranges(const uint32_t *keys, const uint32_t *n_dev, uint32_t cap, uint2 *ranges)
-{
-    const uint32_t n = min(*n_dev, cap);
-    const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n)
-        return;
-    const uint32_t k = keys[i];
-    if (i == 0 || keys[i - 1] != k)
-        ranges[k].x = i;
-    if (i == n - 1 || keys[i + 1] != k)
-        ranges[k].y = i + 1;
-}
+constexpr int kParamThreads = 128, kParamWarps = kParamThreads / 32;
+// a record of more slots is staged through shared memory
+constexpr uint32_t kShortSlots = 32;
+constexpr int kStage = 64;  // slots staged at a time (two per lane)
 
-__global__ void __launch_bounds__(128) k_param_grads(const gsl::ParamArgs a)
+// One thread per Gaussian chains its records' gradients.  The sum over a
+// record's tiles before that runs in tile order (an FP32 sum of a splat
+// over thousands of tiles cancels by 1e4, so another order shows at 1e-4 of
+// the gradient), one lane per component: a short record by loads straight
+// from its slots, several in flight, three records per warp; a long one by
+// a whole warp that stages 64 slots in shared memory while the next 64 are
+// loading.  Most visible records cover a handful of tiles, a few near the
+// camera all of a frame's 3,225: one thread summing its own records, each
+// slot's load waiting for the last, took 646 us on the 300k-Gaussian,
+// 4 x 1200x680 step (ncu), 33 MB or 5 us of HBM traffic, and grouping the
+// slots by record took 14 launches of radix sort.  That step: 1.86 -> 1.21 ms.
+__global__ void __launch_bounds__(kParamThreads) k_param_grads(const gsl::ParamArgs a)
 {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= a.n)
-        return;
+    __shared__ float s_G[kParamThreads][10];
+    __shared__ __align__(16) float s_stage[kParamWarps][kStage * 12];
+    __shared__ uint8_t s_long[kParamThreads];
+    __shared__ int s_n_long;
+    static_assert(kParamThreads <= 256, "s_long holds thread indices in a byte");
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int i0 = blockIdx.x * kParamThreads, i = i0 + threadIdx.x;
+    const int comp = lane % 10, sub = lane / 10;  // lanes 30 and 31 sum nothing
     // object-frame accumulators over cameras
     float gmu[3] = {0, 0, 0}, GS[3][3] = {{0, 0, 0}, {0, 0, 0}, {0, 0, 0}}, dop = 0.0f, drgb[3] = {0, 0, 0};
     for (int c = 0; c < a.n_vps; ++c) {
         const VpDesc &d = a.vps[c];
         const uint32_t r = d.rec_base + (uint32_t)i;
-        const uint2 seg = a.rec_ranges[r];
-        if (seg.y <= seg.x)
-            continue;
-        float G[10] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0};
-        for (uint32_t p = seg.x; p < seg.y; ++p) {
-            const float *src = a.dup_grads + (size_t)a.rpos[p] * 10;
+        const uint32_t cnt = i < a.n ? (uint32_t)a.counts[r] : 0u;
+        const uint32_t off = cnt ? a.rec_slot[r] : 0u;
+        if (threadIdx.x == 0)
+            s_n_long = 0;
+        __syncthreads();
+        if (cnt > kShortSlots)
+            s_long[atomicAdd(&s_n_long, 1)] = (uint8_t)threadIdx.x;
+        unsigned m = __ballot_sync(0xffffffffu, cnt > 0 && cnt <= kShortSlots);
+        while (m) {
+            int src = -1;
 #pragma unroll
-            for (int k = 0; k < 10; ++k)
-                G[k] += src[k];
+            for (int o = 0; o < 3; ++o) {
+                const int f = __ffs(m) - 1;
+                m &= m - 1;
+                if (sub == o)
+                    src = f;
+            }
+            const uint32_t n = __shfl_sync(0xffffffffu, cnt, src & 31), b = __shfl_sync(0xffffffffu, off, src & 31);
+            if (src >= 0) {
+                const float *p = a.dup_grads + 12 * (size_t)b + comp;
+                float G = 0.0f;
+#pragma unroll 8
+                for (uint32_t k = 0; k < n; ++k)
+                    G += p[12 * k];
+                s_G[32 * warp + src][comp] = G;
+            }
         }
+        __syncthreads();
+        // the block's long records, dealt to its warps
+        const int n_long = s_n_long;
+        for (int l = warp; l < n_long; l += kParamWarps) {
+            const int src = s_long[l];
+            const uint32_t rl = d.rec_base + (uint32_t)(i0 + src);
+            const uint32_t n = (uint32_t)a.counts[rl];
+            const float4 *p = reinterpret_cast<const float4 *>(a.dup_grads) + 3 * (size_t)a.rec_slot[rl];
+            float4 *st = reinterpret_cast<float4 *>(s_stage[warp]);
+            // batch b: float4s [192 b, 192 b + 192) of the record's 3 n
+            float4 v[6];
+            const uint32_t n4 = 3 * n;
+#pragma unroll
+            for (int u = 0; u < 6; ++u)
+                if (32u * u + lane < n4)
+                    v[u] = p[32 * u + lane];
+            float G = 0.0f;
+            for (uint32_t b = 0; b < n; b += kStage) {
+#pragma unroll
+                for (int u = 0; u < 6; ++u)
+                    st[32 * u + lane] = v[u];
+                __syncwarp();
+#pragma unroll
+                for (int u = 0; u < 6; ++u) {
+                    const uint32_t q = 3 * (b + kStage) + 32 * u + lane;
+                    if (q < n4)
+                        v[u] = p[q];
+                }
+                const int cntb = (int)min((uint32_t)kStage, n - b);
+                if (lane < 10) {
+#pragma unroll 8
+                    for (int k = 0; k < cntb; ++k)
+                        G += s_stage[warp][12 * k + lane];
+                }
+                __syncwarp();
+            }
+            if (lane < 10)
+                s_G[src][lane] = G;
+        }
+        if (n_long > 0)
+            __syncthreads();
+        if (cnt == 0)
+            continue;
+        float G[10];
+#pragma unroll
+        for (int k = 0; k < 10; ++k)
+            G[k] = s_G[threadIdx.x][k];
         const float4 q1 = a.rec[3 * (size_t)r + 1];
         const float4 x0 = a.aux[2 * (size_t)r], x1 = a.aux[2 * (size_t)r + 1];
         const float fx = d.fx, fy = d.fy;
@@ -105,6 +198,8 @@ __global__ void __launch_bounds__(128) k_param_grads(const gsl::ParamArgs a)
         drgb[1] += G[8];
         drgb[2] += G[9];
     }
+    if (i >= a.n)
+        return;
     // Sigma = R(q) S^2 R(q)^T with S = diag(e^s); o = sigmoid(logit)
     const float4 q = a.quats[i], sc = a.scales[i];
     const float n2 = q.x * q.x + q.y * q.y + q.z * q.z + q.w * q.w;
@@ -161,21 +256,21 @@ inline uint32_t div_up(size_t a, size_t b) { return (uint32_t)((a + b - 1) / b);
 
 namespace gsl {
 
-void param_grads(const ParamArgs &a, const uint32_t *sorted_recs, const uint32_t *n_dups, uint32_t cap,
-                 uint32_t *rkeys[2], uint32_t *rpos[2], int rec_bits, uint32_t *hist, uint32_t *hist_partials,
-                 uint2 *rec_ranges, uint32_t n_records, cudaStream_t s)
+void rec_slots(const int32_t *counts, uint32_t n_records, uint32_t *total, uint32_t *first, cudaStream_t s)
 {
-    k_iota_copy<<<div_up(cap ? cap : 1, 256), 256, 0, s>>>(sorted_recs, n_dups, cap, rkeys[0], rpos[0]);
+    cudaMemsetAsync(total, 0, sizeof(uint32_t), s);
+    if (n_records == 0)
+        return;
+    k_rec_slots<<<div_up(n_records, kScanTile), kScanThreads, 0, s>>>(counts, n_records, total, first);
     ++g_launches;
-    const int c = sort_u32(rkeys, rpos, n_dups, cap, rec_bits, hist, hist_partials, s);
-    cudaMemsetAsync(rec_ranges, 0, sizeof(uint2) * (size_t)(n_records ? n_records : 1), s);
-    k_key_ranges<<<div_up(cap ? cap : 1, 256), 256, 0, s>>>(rkeys[c], n_dups, cap, rec_ranges);
-    ParamArgs b = a;
-    b.rpos = rpos[c];
-    b.rec_ranges = rec_ranges;
-    if (a.n > 0)
-        k_param_grads<<<div_up((size_t)a.n, 128), 128, 0, s>>>(b);
-    g_launches += 2;
+}
+
+void param_grads(const ParamArgs &a, cudaStream_t s)
+{
+    if (a.n <= 0)
+        return;
+    k_param_grads<<<div_up((size_t)a.n, kParamThreads), kParamThreads, 0, s>>>(a);
+    ++g_launches;
 }
 
 }  // namespace gsl

@@ -938,6 +938,15 @@ __device__ __forceinline__ bool pix_adj_x2(PixAdj2 &P, int jj, const RecX2 &R, f
 
 static_assert(kBwd2Chunk <= kBwd2Threads && kBwd2Chunk % 32 == 0, "one thread stages one record");
 
+// Slot of tile (tx, ty) among the record's (full mode; rx, ry: the record's
+// tile rectangle words).
+__device__ __forceinline__ uint32_t tile_slot(const gsl::RasterArgs &a, uint32_t r, float rx, float ry, int tx, int ty)
+{
+    const uint32_t x = __float_as_uint(rx), y = __float_as_uint(ry);
+    const uint32_t x0 = x & 0xffffu, x1 = x >> 16, y0 = y & 0xffffu;
+    return a.rec_slot[r] + ((uint32_t)ty - y0) * (x1 - x0) + ((uint32_t)tx - x0);
+}
+
 // One tile of the adjoint (all kBwd2Threads threads of the CTA take part).
 template <bool REG, bool FULL>
 __device__ __forceinline__ void bwd_tile(const gsl::RasterArgs &a, const uint32_t t)
@@ -969,14 +978,18 @@ __device__ __forceinline__ void bwd_tile(const gsl::RasterArgs &a, const uint32_
     const bool cull = a.alpha_min > 0.0f;
     const uint2 rg = a.ranges[t];
     // staging of one record of a chunk (thread i, chunk position i)
+    uint32_t slot = 0;  // full mode: where the staged record's gradients of this tile go
     auto stage = [&](uint32_t r) {
         const float4 *R = a.rec + 3 * (size_t)r;
         s0[threadIdx.x] = R[0];
-        float4 q1 = stage_cutoff(R[1], a);
+        const float4 r1 = R[1], r2 = R[2];
+        float4 q1 = stage_cutoff(r1, a);
         if (PK)
             q1.y = -q1.y;
         s1[threadIdx.x] = q1;
-        s2[threadIdx.x] = R[2];
+        s2[threadIdx.x] = r2;
+        if (FULL)
+            slot = tile_slot(a, r, r1.w, r2.w, tx, ty);
         if (a.tile_twist) {
             // the camera-frame mean and covariance, staged with the record
             // (not read after the walk) so that these loads overlap
@@ -1131,14 +1144,24 @@ __device__ __forceinline__ void bwd_tile(const gsl::RasterArgs &a, const uint32_
                 G[k] = -s;  // the packed walk sums the negated gradient
                 any |= s != 0.0f;
             }
-            if (FULL) {
-                float *dst = a.dup_grads + (size_t)(rg.x + lo + threadIdx.x) * 10;
-#pragma unroll
-                for (int k = 0; k < NG; ++k)
-                    dst[k] = G[k];
+            if constexpr (FULL) {
+                float4 *dst = reinterpret_cast<float4 *>(a.dup_grads) + 3 * (size_t)slot;
+                dst[0] = make_float4(G[0], G[1], G[2], G[3]);
+                dst[1] = make_float4(G[4], G[5], G[6], G[7]);
+                *reinterpret_cast<float2 *>(dst + 2) = make_float2(G[8], G[9]);
             }
             if (any && a.tile_twist)
                 chain_twist(G, s1[threadIdx.x], s_x0[threadIdx.x], s_x1[threadIdx.x], d.fx, d.fy, cc, tw);
+        }
+    }
+    if constexpr (FULL) {
+        // the list past the tile's last contributor adds nothing
+        for (int k = maxl + (int)threadIdx.x; k < n_list; k += kBwd2Threads) {
+            const uint32_t r = a.vals[rg.x + k];
+            const float4 *R = a.rec + 3 * (size_t)r;
+            float4 *dst = reinterpret_cast<float4 *>(a.dup_grads) + 3 * (size_t)tile_slot(a, r, R[1].w, R[2].w, tx, ty);
+            dst[0] = dst[1] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+            *reinterpret_cast<float2 *>(dst + 2) = make_float2(0.0f, 0.0f);
         }
     }
     if (!a.tile_twist)

@@ -123,3 +123,45 @@ def test_saved_forward_equals_render_and_backward(env, n, W, H, f, views):
         for k in gr1:
             assert torch.equal(gr1[k], gr2[k]), k
     sv.close()
+
+
+def test_parameter_adjoint_list_lengths(env):
+    # records over 1 to 3,225 tiles of a 1200x680 frame, both sides of the
+    # length where the sum over a record's tiles changes hands (32) and of
+    # its staging (64), two cameras, Gaussian counts around a block of 128
+    rng = np.random.default_rng(77)
+    for n in (1, 127, 129):
+        gd = synth.gaussians_box(n, rng, center=(0.0, 0.0, 2.5), half=1.2, ls_mean=-2.5, ls_std=0.1)
+        gd["log_scales4"][:, :3] = rng.uniform(-5.5, 0.6, (n, 1)) + rng.normal(0.0, 0.2, (n, 3))
+        gd["logits"][:] = rng.normal(-3.0, 0.5, n)
+        cams = np.stack([synth.camera(600.0, 600.0, 600.0, 340.0, 1200, 680, np.eye(3, 4)),
+                         synth.camera(300.0, 300.0, 150.0, 90.0, 301, 181, np.eye(3, 4))])
+        poses = np.stack([synth.random_rigid(rng, 3.0, 0.03) for _ in cams])
+        check(env, gd, cams, poses, n)
+
+
+def test_parameter_adjoint_ignores_earlier_calls(env):
+    # list entries behind a tile's last contributor hold no gradient of an
+    # earlier call on the context: near-opaque layers hide many of them
+    gs, _, ctx = env
+    rng = np.random.default_rng(78)
+    g1 = synth.gaussians_box(4000, rng, half=0.8, ls_mean=-2.5)
+    g2 = synth.gaussians_box(3000, rng, half=0.8, ls_mean=-2.3)
+    g2["logits"][:] = 7.0
+    cams = synth.circle_cameras(2, 0.25, (0.0, 0.0, 2.5), 320, 240, 250.0)
+    P = dev(np.stack([np.eye(3, 4).reshape(12)] * 2))
+
+    def grads(c, gd, scale):
+        g = gs.Gaussians.from_numpy(gd)
+        out = gs.gs_render(c, g, P, cams)
+        cr, cd = torch.full_like(out["rgb"], scale), torch.full_like(out["depth"], scale)
+        return gs.gs_render_backward(c, g, P, cams, out["t_final"], out["last"], cr, cd, params=True)[1]
+
+    fresh = gs.Context(0)
+    want = grads(fresh, g2, 1.0)
+    for _ in range(2):
+        grads(ctx, g1, 1e6)
+        got = grads(ctx, g2, 1.0)
+        for k in want:
+            assert torch.equal(got[k], want[k]), k
+    fresh.close()
