@@ -1529,8 +1529,14 @@ gs_status_t gs_transform(gs_ctx_t *ctx, const gs_gaussians_t *g, const double *T
     if (!T_host || (g->n > 0 && (!out_means || !out_quats || !aligned16(out_means) || !aligned16(out_quats))))
         return fail(ctx, GS_ERR_INVALID_ARG, "gs_transform: bad arguments");
     DeviceGuard dg(ctx->device);
-    gsl::transform((const float4 *)g->means, (const float4 *)g->quats, g->n, T_host, (float4 *)out_means,
-                   (float4 *)out_quats, (cudaStream_t)stream);
+    gsl::MapDesc m{};
+    m.means = (const float4 *)g->means;
+    m.quats = (const float4 *)g->quats;
+    m.out_means = (float4 *)out_means;
+    m.out_quats = (float4 *)out_quats;
+    m.n = g->n;
+    m.r = gsl::make_rigid(T_host);
+    gsl::transform(m, (cudaStream_t)stream);
     GS_CUDA(cudaGetLastError());
     return GS_OK;
 }
@@ -1605,9 +1611,9 @@ gs_status_t gs_transform_batch(gs_ctx_t *ctx, const gs_gaussians_t *maps, int n_
         m.out_quats = (float4 *)out_quats[k];
         m.n = maps[k].n;
         m.blk_base = blocks;
-        std::memcpy(m.T, T_host + 12 * k, sizeof m.T);
+        m.r = gsl::make_rigid(T_host + 12 * k);
         md.push_back(m);
-        blocks += (unsigned)((m.n + 255) / 256);
+        blocks += gsl::transform_blocks(m.n);
     }
     if (md.empty())
         return GS_OK;

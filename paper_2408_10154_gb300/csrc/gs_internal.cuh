@@ -135,6 +135,45 @@ __device__ __forceinline__ void two_sum_add(float &hi, float &lo, float bhi, flo
     lo = lo + blo + e;
 }
 
+// Packed pairs: add/sub/mul/fma.rn.f32x2 round each of the two lanes exactly
+// as the scalar .rn operation does, and issue once for both.
+typedef unsigned long long f32x2;
+__device__ __forceinline__ f32x2 x2(float lo, float hi)
+{
+    f32x2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+    return r;
+}
+__device__ __forceinline__ void x2_split(f32x2 v, float &lo, float &hi)
+{
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+}
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b)
+{
+    f32x2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ f32x2 sub2(f32x2 a, f32x2 b)
+{
+    f32x2 r;
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b)
+{
+    f32x2 r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c)
+{
+    f32x2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+__device__ __forceinline__ f32x2 bc2(float v) { return x2(v, v); }
+
 // M = V o T (3x4 row-major) in FP32
 __device__ __forceinline__ void compose_ct(const float *V, const float *T, float *M)
 {
@@ -392,15 +431,23 @@ void track_loss(const TrackArgs &a, cudaStream_t s);
 // err / col of rendered images (standalone gs_track_loss)
 void track_prep(const TrackArgs &a, const float *rgb, const float *depth, float *err, float *col, cudaStream_t s);
 
-// One submap of a batched rigid update (map adjustment after pose-graph
-// optimisation, Eq. 8/9): blocks [blk_base, blk_base + ceil(n / 256)).
+// A rigid map T = [R | t] and R's quaternion (w >= 0 in the first branch; the
+// largest pivot else), each also split into FP32 high and low parts.
+struct Rigid {
+    double T[12];
+    float Th[12], Tl[12], qh[4], ql[4];
+};
+// One submap of a rigid update (map adjustment after pose-graph
+// optimisation, Eq. 8/9): blocks [blk_base, blk_base + transform_blocks(n)).
 struct MapDesc {
     const float4 *means, *quats;
     float4 *out_means, *out_quats;
     int64_t n;
     unsigned blk_base;
-    double T[12];
+    Rigid r;
 };
+Rigid make_rigid(const double *T);
+unsigned transform_blocks(int64_t n);
 void transform_batch(const MapDesc *maps, int n_maps, unsigned blocks, cudaStream_t s);
 
 // Overlap ratio of two submaps (loop filter): moved means of P, exact
@@ -495,8 +542,7 @@ void pose_step_raw(int n, double *pose, double *state, const double *grad, const
                    float lr_rot, float lr_trans, float b1, float b2, float eps, float lr_final, cudaStream_t s);
 void loss(const gsk::VpDesc *vps, int n_vps, uint32_t n_tiles, const uint32_t *tile_vp, const float *rgb,
           const float *depth, double *loss, float *d_rgb, float *d_depth, float *tile_loss, cudaStream_t s);
-void transform(const float4 *means, const float4 *quats, int64_t n, const double *T, float4 *out_means,
-               float4 *out_quats, cudaStream_t s);
+void transform(const MapDesc &m, cudaStream_t s);
 
 // adjoint to every Gaussian parameter of one submap seen by n_vps cameras
 struct ParamArgs {

@@ -5,6 +5,8 @@
 // pose update about the moving submap's centroid (Sec. 3.2; learning rates
 // Supp. B), the standalone L1 loss, the Eq. 7 fusion and the Eq. 8/9 rigid
 // transform of a submap.  Latency-bound tiny kernels, FP64 state.
+#include <cmath>
+
 #include "gs_internal.cuh"
 
 namespace {
@@ -465,16 +467,10 @@ __global__ void __launch_bounds__(256) k_loss_tiles(const VpDesc *vps, const uin
 }
 
 // ---------------------------------------------------------------- Eq. 8/9
-struct Rigid {
-    double T[12];
-};
-
-// mu <- R mu + t and q <- q_R (x) q of one Gaussian (FP64 arithmetic)
-__device__ __forceinline__ void rigid_apply(const double *T, const float4 m, const float4 q, float4 &om, float4 &oq)
+// quaternion of R (largest-pivot branch), w >= 0
+__host__ __device__ __forceinline__ void rigid_quat(const double *T, double &qw, double &qx, double &qy, double &qz)
 {
-    // quaternion of R (largest-pivot branch), w >= 0
     const double tr = T[0] + T[5] + T[10];
-    double qw, qx, qy, qz;
     if (tr > 0) {
         const double s = sqrt(tr + 1.0) * 2;
         qw = 0.25 * s; qx = (T[9] - T[6]) / s; qy = (T[2] - T[8]) / s; qz = (T[4] - T[1]) / s;
@@ -488,49 +484,145 @@ __device__ __forceinline__ void rigid_apply(const double *T, const float4 m, con
         const double s = sqrt(1.0 + T[10] - T[0] - T[5]) * 2;
         qw = (T[4] - T[1]) / s; qx = (T[2] + T[8]) / s; qy = (T[6] + T[9]) / s; qz = 0.25 * s;
     }
-    float4 r;
-    r.x = (float)(T[0] * m.x + T[1] * m.y + T[2] * m.z + T[3]);
-    r.y = (float)(T[4] * m.x + T[5] * m.y + T[6] * m.z + T[7]);
-    r.z = (float)(T[8] * m.x + T[9] * m.y + T[10] * m.z + T[11]);
-    r.w = 0.0f;
-    // q_R (x) q
-    float4 p;
-    p.x = (float)(qw * q.x - qx * q.y - qy * q.z - qz * q.w);
-    p.y = (float)(qw * q.y + qx * q.x + qy * q.w - qz * q.z);
-    p.z = (float)(qw * q.z - qx * q.w + qy * q.x + qz * q.y);
-    p.w = (float)(qw * q.w + qx * q.z - qy * q.y + qz * q.x);
-    om = r;
-    oq = p;
 }
 
-__global__ void k_transform(const float4 *means, const float4 *quats, int64_t n, const Rigid rt, float4 *om,
-                            float4 *oq)
+// mu <- R mu + t and q <- q_R (x) q of one Gaussian in FP64, each result
+// rounded once to FP32
+__device__ __noinline__ void rigid_apply64(const double *T, const float4 m, const float4 q, float4 &om, float4 &oq)
 {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n)
-        return;
-    float4 a, b;
-    rigid_apply(rt.T, means[i], quats[i], a, b);
-    om[i] = a;
-    oq[i] = b;
+    double qw, qx, qy, qz;
+    rigid_quat(T, qw, qx, qy, qz);
+    om.x = (float)(T[0] * m.x + T[1] * m.y + T[2] * m.z + T[3]);
+    om.y = (float)(T[4] * m.x + T[5] * m.y + T[6] * m.z + T[7]);
+    om.z = (float)(T[8] * m.x + T[9] * m.y + T[10] * m.z + T[11]);
+    om.w = 0.0f;
+    oq.x = (float)(qw * q.x - qx * q.y - qy * q.z - qz * q.w);
+    oq.y = (float)(qw * q.y + qx * q.x + qy * q.w - qz * q.z);
+    oq.z = (float)(qw * q.z - qx * q.w + qy * q.x + qz * q.y);
+    oq.w = (float)(qw * q.w + qx * q.z - qy * q.y + qz * q.x);
+}
+
+// s + e = a + b exactly (Knuth), both lanes
+__device__ __forceinline__ f32x2 two_sum2(f32x2 a, f32x2 b, f32x2 &e)
+{
+    const f32x2 s = add2(a, b), bb = sub2(s, a);
+    e = add2(sub2(a, sub2(s, bb)), sub2(b, bb));
+    return s;
+}
+
+__device__ __forceinline__ f32x2 abs2(f32x2 v) { return v & 0x7fffffff7fffffffull; }
+
+// c0 m0 + c1 m1 + c2 m2 + c3 m3 of two Gaussians (the lanes), c = ch + cl:
+// products by fma, sums by TwoSum, their errors in L.  The value S + L is
+// within 33 u^2 of the terms' magnitudes `mag` (u = 2^-24; the split of c,
+// the products' and the sums' second-order roundings) plus underflows of
+// 2^-149, so where S + L - e and S + L + e round alike with e = 2^-42 mag
+// and mag >= 2^-100, that is the nearest FP32 value, and `sure` (per lane)
+// stays set; so it does where every product is 0.
+__device__ __forceinline__ f32x2 dot4_x2(const float *ch, const float *cl, const f32x2 (&m)[4], bool &sure0, bool &sure1)
+{
+    f32x2 S = 0, L = 0, mag = 0;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const f32x2 c = bc2(ch[k]), p = mul2(c, m[k]);
+        const f32x2 e = fma2(bc2(cl[k]), m[k], fma2(c, m[k], p ^ 0x8000000080000000ull));
+        if (k == 0) {
+            S = p;
+            L = e;
+            mag = abs2(p);
+        } else {
+            f32x2 r;
+            S = two_sum2(S, p, r);
+            L = add2(L, add2(e, r));
+            mag = add2(mag, abs2(p));
+        }
+    }
+    const f32x2 err = mul2(mag, bc2(2.2737368e-13f));  // 2^-42
+    const f32x2 hi = add2(S, add2(L, err)), lo = add2(S, sub2(L, err));
+    float h0, h1, l0, l1, g0, g1;
+    x2_split(hi, h0, h1);
+    x2_split(lo, l0, l1);
+    x2_split(mag, g0, g1);
+    constexpr float kTiny = 7.8886091e-31f;                  // 2^-100
+    sure0 = sure0 && h0 == l0 && (g0 >= kTiny || g0 == 0.0f);  // (a NaN is not equal to itself)
+    sure1 = sure1 && h1 == l1 && (g1 >= kTiny || g1 == 0.0f);
+    return hi;
+}
+
+constexpr int kRigidThreads = 128, kRigidPairs = 2;  // two Gaussians per pair
+constexpr int kRigidPerBlock = kRigidThreads * 2 * kRigidPairs;
+
+// Eq. 8/9 of kRigidPerBlock Gaussians per block.  64 B of traffic per
+// Gaussian against 25 FP64 operations in the plain form, which this part's
+// FP64 pipe (two lanes per SM and clock) runs at a fifth of HBM's rate: with
+// R's quaternion found per Gaussian as well, 4.4 M Gaussians took 661 us
+// (ncu).  So the sums are taken in FP32 pairs (dot4_x2), packed two
+// Gaussians at a time, and the few whose rounding that leaves open (about
+// one in 10^4) in FP64: every result is FP64's rounded to FP32.  A call on 24
+// maps of 4.4 M Gaussians in all: 665 -> 189 us, most of that the host's.
+__device__ __forceinline__ void rigid_block(const gsl::MapDesc &m, unsigned blk)
+{
+    const int64_t base = (int64_t)blk * kRigidPerBlock + threadIdx.x;
+    float4 a[2 * kRigidPairs], q[2 * kRigidPairs];
+#pragma unroll
+    for (int u = 0; u < 2 * kRigidPairs; ++u) {
+        const int64_t i = base + u * kRigidThreads;
+        const bool in = i < m.n;
+        a[u] = in ? m.means[i] : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        q[u] = in ? m.quats[i] : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    }
+    const float *qh = m.r.qh, *ql = m.r.ql;
+    // rows of the quaternion product q_R (x) q
+    const float ch[4][4] = {{qh[0], -qh[1], -qh[2], -qh[3]},
+                            {qh[1], qh[0], -qh[3], qh[2]},
+                            {qh[2], qh[3], qh[0], -qh[1]},
+                            {qh[3], -qh[2], qh[1], qh[0]}};
+    const float cl[4][4] = {{ql[0], -ql[1], -ql[2], -ql[3]},
+                            {ql[1], ql[0], -ql[3], ql[2]},
+                            {ql[2], ql[3], ql[0], -ql[1]},
+                            {ql[3], -ql[2], ql[1], ql[0]}};
+#pragma unroll
+    for (int u = 0; u < kRigidPairs; ++u) {
+        const float4 a0 = a[2 * u], a1 = a[2 * u + 1], q0 = q[2 * u], q1 = q[2 * u + 1];
+        const f32x2 am[4] = {x2(a0.x, a1.x), x2(a0.y, a1.y), x2(a0.z, a1.z), bc2(1.0f)};
+        const f32x2 qm[4] = {x2(q0.x, q1.x), x2(q0.y, q1.y), x2(q0.z, q1.z), x2(q0.w, q1.w)};
+        bool sure[2] = {true, true};
+        float rm[3][2], rq[4][2];
+#pragma unroll
+        for (int k = 0; k < 3; ++k)
+            x2_split(dot4_x2(m.r.Th + 4 * k, m.r.Tl + 4 * k, am, sure[0], sure[1]), rm[k][0], rm[k][1]);
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+            x2_split(dot4_x2(ch[k], cl[k], qm, sure[0], sure[1]), rq[k][0], rq[k][1]);
+#pragma unroll
+        for (int v = 0; v < 2; ++v) {
+            const int64_t i = base + (2 * u + v) * kRigidThreads;
+            if (i >= m.n)
+                continue;
+            float4 om = make_float4(rm[0][v], rm[1][v], rm[2][v], 0.0f);
+            float4 oq = make_float4(rq[0][v], rq[1][v], rq[2][v], rq[3][v]);
+            if (!sure[v])
+                rigid_apply64(m.r.T, a[2 * u + v], q[2 * u + v], om, oq);
+            m.out_means[i] = om;
+            m.out_quats[i] = oq;
+        }
+    }
+}
+
+__global__ void __launch_bounds__(kRigidThreads) k_transform(const __grid_constant__ gsl::MapDesc m)
+{
+    rigid_block(m, blockIdx.x);
 }
 
 // many submaps, each with its own T: blocks [blk_base, next blk_base) of map k
-__global__ void k_transform_batch(const gsl::MapDesc *maps, int n_maps)
+__global__ void __launch_bounds__(kRigidThreads) k_transform_batch(const gsl::MapDesc *maps, int n_maps)
 {
     int lo = 0, hi = n_maps - 1;
     while (lo < hi) {
         const int mid = (lo + hi + 1) >> 1;
         if (maps[mid].blk_base <= blockIdx.x) lo = mid; else hi = mid - 1;
     }
-    const gsl::MapDesc &m = maps[lo];
-    const int64_t i = (int64_t)(blockIdx.x - m.blk_base) * blockDim.x + threadIdx.x;
-    if (i >= m.n)
-        return;
-    float4 a, b;
-    rigid_apply(m.T, m.means[i], m.quats[i], a, b);
-    m.out_means[i] = a;
-    m.out_quats[i] = b;
+    rigid_block(maps[lo], blockIdx.x - maps[lo].blk_base);
 }
 
 }  // namespace
@@ -615,15 +707,40 @@ void loss_reduce(const VpDesc *vps, int n_vps, const float *tile_loss, double *l
     ++g_launches;
 }
 
-void transform(const float4 *means, const float4 *quats, int64_t n, const double *T, float4 *out_means,
-               float4 *out_quats, cudaStream_t s)
+Rigid make_rigid(const double *T)
 {
-    if (n <= 0)
-        return;
     Rigid r;
-    for (int k = 0; k < 12; ++k)
+    double q[4];
+    rigid_quat(T, q[0], q[1], q[2], q[3]);
+    for (int k = 0; k < 12; ++k) {
         r.T[k] = T[k];
-    k_transform<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(means, quats, n, r, out_means, out_quats);
+        r.Th[k] = (float)T[k];
+        r.Tl[k] = (float)(T[k] - (double)r.Th[k]);
+    }
+    for (int k = 0; k < 4; ++k) {
+        r.qh[k] = (float)q[k];
+        r.ql[k] = (float)(q[k] - (double)r.qh[k]);
+    }
+    // a coefficient whose low part would underflow sends every Gaussian to
+    // FP64 (NaN sums are never sure)
+    auto splits = [](double c) { return c == 0.0 || fabs(c) >= 7.8886090522101181e-31; };
+    bool ok = true;
+    for (int k = 0; k < 12; ++k)
+        ok = ok && splits(T[k]);
+    for (int k = 0; k < 4; ++k)
+        ok = ok && splits(q[k]);
+    if (!ok)
+        r.Th[0] = NAN;
+    return r;
+}
+
+unsigned transform_blocks(int64_t n) { return (unsigned)((n + kRigidPerBlock - 1) / kRigidPerBlock); }
+
+void transform(const MapDesc &m, cudaStream_t s)
+{
+    if (m.n <= 0)
+        return;
+    k_transform<<<transform_blocks(m.n), kRigidThreads, 0, s>>>(m);
     ++g_launches;
 }
 
@@ -631,7 +748,7 @@ void transform_batch(const MapDesc *maps, int n_maps, unsigned blocks, cudaStrea
 {
     if (n_maps <= 0 || blocks == 0)
         return;
-    k_transform_batch<<<blocks, 256, 0, s>>>(maps, n_maps);
+    k_transform_batch<<<blocks, kRigidThreads, 0, s>>>(maps, n_maps);
     ++g_launches;
 }
 

@@ -112,48 +112,10 @@ __device__ __forceinline__ bool conic_safe(float ca, float cb, float cc)
 }
 
 // ---------------------------------------------------------------------------
-// Packed pixel pairs.  In the registration forward and adjoint a thread
-// walks two pixels (same column, rows r and r + 4) with one f32x2 operation
-// per step: add/sub/mul/fma.rn.f32x2 round each of the two lanes exactly as
-// the scalar .rn operation does, and issue once for both.
+// Packed pixel pairs.  In the forward and the adjoint a thread walks two
+// pixels (same column, rows r and r + 4) with one f32x2 operation per step:
+// {lo, hi} = {pixel 0, pixel 1}.
 // ---------------------------------------------------------------------------
-typedef unsigned long long f32x2;  // {lo, hi} = {pixel 0, pixel 1}
-__device__ __forceinline__ f32x2 x2(float lo, float hi)
-{
-    f32x2 r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
-    return r;
-}
-__device__ __forceinline__ void x2_split(f32x2 v, float &lo, float &hi)
-{
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
-}
-__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b)
-{
-    f32x2 r;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-__device__ __forceinline__ f32x2 sub2(f32x2 a, f32x2 b)
-{
-    f32x2 r;
-    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b)
-{
-    f32x2 r;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c)
-{
-    f32x2 r;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-    return r;
-}
-__device__ __forceinline__ f32x2 bc2(float v) { return x2(v, v); }
-
 // A record's values, each broadcast to both lanes ({v, v} pairs), for the
 // packed walks: {u, v}, {ca, cb}, {cc, o} (-o in the adjoint), {z, r}, {g, b}.
 // Built from the staged float4s as they are loaded (staging the pairs

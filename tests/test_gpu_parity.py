@@ -689,6 +689,62 @@ def test_transform_batch_equals_single_transforms(gs, ctx):
             np.testing.assert_allclose(o.means4.cpu().numpy(), ref.means4, atol=2e-6)
 
 
+@pytest.mark.parametrize("kind", ["room", "planar", "turned", "special", "tiny", "far"])
+@pytest.mark.parametrize("n", [1, 511, 513, 40000])
+def test_transform_is_fp64_rounded_once(gs, ctx, kind, n):
+    # every result is the FP64 sum rounded to FP32, also where FP32 pairs
+    # cannot decide the rounding, with zeros, infinities, NaN, values whose
+    # products underflow or overflow, and the four branches of R's quaternion
+    rng = np.random.default_rng(n)
+    m = np.concatenate([rng.uniform(-3, 3, (n, 3)), np.zeros((n, 1))], 1).astype(np.float32)
+    q = rng.standard_normal((n, 4)).astype(np.float32)
+    T = synth.random_rigid(rng, 12.0, 0.3)
+    if kind == "planar":
+        m[:, 2], T = 0.0, np.concatenate([synth.axis_angle_matrix((0, 0, 1), 0.3), [[0.5], [0.25], [0.0]]], 1)
+    elif kind == "turned":
+        T = np.concatenate([synth.axis_angle_matrix(rng.choice([(1, 0, 0), (0, 1, 0), (0, 0, 1)]), math.pi - 1e-3),
+                            rng.uniform(-1, 1, (3, 1))], 1)
+    elif kind == "special":
+        m[rng.random(n) < 0.3, 0] = np.inf
+        m[rng.random(n) < 0.3, 1] = np.nan
+        m[rng.random(n) < 0.3, 2] = 3e38
+        q[rng.random(n) < 0.3, 3] = -np.inf
+    elif kind == "tiny":
+        m *= np.float32(1e-36)
+        q[:, 1] *= np.float32(1e-40)
+        T[:, 3] = 0.0
+    elif kind == "far":
+        m *= np.float32(1e6)
+        T[:, 3] = -(T[:, :3] @ m[0, :3].astype(np.float64))
+        T[0, 1] = 1e-33
+    gd = dict(means4=m, log_scales4=np.zeros_like(m), quats4=q, logits=np.zeros(n, np.float32), rgb4=np.zeros_like(m))
+    out = gs.gs_transform(ctx, gs.Gaussians.from_numpy(gd), T)
+    with np.errstate(all="ignore"):
+        # (FP64 sums by fused multiply-adds, as the kernel's: the first point
+        # of "far" cancels to FP64's own rounding)
+        fma = lambda u, v, w: (np.longdouble(u) * v.astype(np.longdouble) + w).astype(np.float64)
+        x, y = m.astype(np.float64), q.astype(np.float64)
+        want = [fma(T[k, 2], x[:, 2], fma(T[k, 0], x[:, 0], T[k, 1] * x[:, 1])) + T[k, 3] for k in range(3)]
+        want = np.stack(want + [np.zeros(n)], 1).astype(np.float32)
+        R = T[:, :3]
+        tr = np.trace(R)
+        k = int(np.argmax([tr if tr > 0 else -9.0, *np.diag(R)])) if tr <= 0 else 0
+        if k == 0:
+            s = np.sqrt(tr + 1.0) * 2
+            w, a, b, c = 0.25 * s, (R[2, 1] - R[1, 2]) / s, (R[0, 2] - R[2, 0]) / s, (R[1, 0] - R[0, 1]) / s
+        else:
+            i, j, l = k - 1, k % 3, (k + 1) % 3
+            s = np.sqrt(1.0 + R[i, i] - R[j, j] - R[l, l]) * 2
+            v = [0.0] * 3
+            v[i], v[j], v[l] = 0.25 * s, (R[j, i] + R[i, j]) / s, (R[l, i] + R[i, l]) / s
+            w, (a, b, c) = (R[l, j] - R[j, l]) / s, v
+        y0, y1, y2, y3 = y.T
+        wq = np.stack([w * y0 - a * y1 - b * y2 - c * y3, w * y1 + a * y0 + b * y3 - c * y2,
+                       w * y2 - a * y3 + b * y0 + c * y1, w * y3 + a * y2 - b * y1 + c * y0], 1).astype(np.float32)
+    np.testing.assert_array_equal(out.means4.cpu().numpy(), want)
+    np.testing.assert_array_equal(out.quats4.cpu().numpy(), wq)
+
+
 def test_tile_schedules_give_identical_registrations(gs, ctx):
     # two full-size room keyframes (3225 tiles each): natural tile order,
     # longest lists first, either of them through the persistent kernels'
