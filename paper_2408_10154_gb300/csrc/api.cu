@@ -22,7 +22,7 @@ namespace {
 
 enum Slot {
     S_VPS, S_GROUPS, S_TILEVP, S_POSE32, S_REC, S_AUX, S_COUNTS, S_PARTIALS, S_NDUPS, S_K0, S_V0, S_RANGES, S_FLAGS, S_TF, S_LAST, S_CODE, S_TLOSS, S_TTWIST, S_POSE64, S_ADAM, S_PIVOT,
-    S_CCAM, S_CENT, S_LOSS, S_SETVP, S_REV, S_PFIRST, S_PCOUNT, S_TOUT, S_CONF, S_EST, S_GRAD, S_DUPG,
+    S_CCAM, S_CENT, S_CENTP, S_LOSS, S_SETVP, S_REV, S_PFIRST, S_PCOUNT, S_TOUT, S_CONF, S_EST, S_GRAD, S_DUPG,
     S_PAIRS, S_RSLOT, S_RSLOTN, S_TERR, S_TCOL, S_TW,
     S_TMED, S_TNV, S_TVPS, S_EXPO, S_EXPO32, S_TEXPO, S_OPT, S_ONN1, S_ONN2, S_OD2, S_OT, S_OCNT, S_MAPS, S_OS, S_ORDER, S_ORDC, S_SK, S_SV, S_SN, S_OBOX, S_GCELL, S_GSTART, S_GCUR, S_GPART, S_GPTS, S_GIDX, S_GLIST, S_GNL, S_GCELL2, S_GSTART2, S_GCUR2, S_GPART2, S_GPTS2, S_GIDX2, S_GLIST2, S_GNL2, S_SEGZ, S_SEGCUR, S_SEGBIG, S_SEGLIST, S_PROBE, S_QUEUE, S_COUNT
 };
@@ -1867,6 +1867,8 @@ gs_status_t run_registration(gs_ctx *ctx, Plan &P, int n_problems, const gs_opti
     GS_TRY(wsT(ctx, S_PIVOT, 3 * (size_t)nv, &pivot));
     GS_TRY(wsT(ctx, S_CCAM, 3 * (size_t)nv, &ccam));
     GS_TRY(wsT(ctx, S_CENT, 3 * (size_t)n_sets, &cent));
+    float2 *centp = nullptr;
+    GS_TRY(wsT(ctx, S_CENTP, 3 * gsl::kCentroidWarps * (size_t)n_sets, &centp));
     GS_TRY(wsT(ctx, S_LOSS, (size_t)nv, &lossd));
     GS_TRY(wsT(ctx, S_TF, npix, &tf));
     GS_TRY(wsT(ctx, S_LAST, npix, &last));
@@ -1898,6 +1900,7 @@ gs_status_t run_registration(gs_ctx *ctx, Plan &P, int n_problems, const gs_opti
     pa.pivot = pivot;
     pa.c_cam = ccam;
     pa.centroid = cent;
+    pa.cent_part = centp;
     pa.loss = lossd;
     pa.lr_rot = opt->lr_rot;
     pa.lr_trans = opt->lr_trans;
@@ -1938,7 +1941,7 @@ gs_status_t run_registration(gs_ctx *ctx, Plan &P, int n_problems, const gs_opti
         const long long l0 = gsl::g_launches;
         long long captured = 0, graph_kernels = 0, trial_kernels = 0;
         ctx->stats = gs_stats_t{};
-        gsl::centroids(D.vps, D.set_vp, n_sets, cent, s);
+        gsl::centroids(D.vps, D.set_vp, n_sets, centp, s);
         gsl::pose_init(pa, s);
         // size the duplicate lists at the initial poses (with headroom: the
         // count drifts as the poses move).  The asynchronous form takes the
@@ -2610,6 +2613,8 @@ gs_status_t srv_replan(gs_server *srv, cudaStream_t s)
     GS_TRY(wsT(ctx, S_PIVOT, 3 * (size_t)nv, &srv->pivot));
     GS_TRY(wsT(ctx, S_CCAM, 3 * (size_t)nv, &srv->ccam));
     GS_TRY(wsT(ctx, S_CENT, 3 * (size_t)std::max(n_sets, 1), &srv->cent));
+    float2 *centp = nullptr;
+    GS_TRY(wsT(ctx, S_CENTP, 3 * gsl::kCentroidWarps * (size_t)std::max(n_sets, 1), &centp));
     GS_TRY(wsT(ctx, S_LOSS, (size_t)nv, &srv->lossd));
     GS_TRY(wsT(ctx, S_TF, npix, &srv->tf));
     GS_TRY(wsT(ctx, S_LAST, npix, &srv->last));
@@ -2641,6 +2646,7 @@ gs_status_t srv_replan(gs_server *srv, cudaStream_t s)
     pa.pivot = srv->pivot;
     pa.c_cam = srv->ccam;
     pa.centroid = srv->cent;
+    pa.cent_part = centp;
     pa.loss = srv->lossd;
     pa.lr_rot = srv->opt.lr_rot;
     pa.lr_trans = srv->opt.lr_trans;
@@ -2654,7 +2660,7 @@ gs_status_t srv_replan(gs_server *srv, cudaStream_t s)
     GS_TRY(alloc_exposure(ctx, P, pa, expo_r));
 
     // fresh requests start at the identity; the others resume their state
-    gsl::centroids(D.vps, D.set_vp, n_sets, srv->cent, s);
+    gsl::centroids(D.vps, D.set_vp, n_sets, centp, s);
     gsl::pose_init(pa, s);
     for (int64_t id : srv->active) {
         const ServerReq &r = srv->reqs[id];

@@ -498,6 +498,7 @@ void nn_grid_search(const float4 *A, int na, const int32_t *order, const float4 
 // |K| and the pairs within tau from the nearest neighbours both ways
 void overlap_count(const OverlapArgs &a, cudaStream_t s);
 
+constexpr int kCentroidWarps = 32;
 struct PoseArgs {
     const gsk::VpDesc *vps;
     int n_vps;
@@ -508,7 +509,8 @@ struct PoseArgs {
     double *adam;              // [vp][13]
     double *pivot;             // [vp][3] world
     double *c_cam;             // [vp][3]
-    const double *centroid;    // [set][3]
+    double *centroid;          // [set][3] (written by pose_init)
+    const float2 *cent_part;   // [set][kCentroidWarps][3] (centroids)
     double *loss;              // [vp] last loss
     double *grad;              // [vp][6] last world gradient (may be null)
     double *expo;              // [vp][7] exposure a, b and Adam state (m_a, m_b, v_a, v_b, steps)
@@ -524,7 +526,8 @@ void exposure_floats(const double *expo, float *expo32, int n_vps, cudaStream_t 
 // per-keyframe sum of the tile losses (FP64, fixed order)
 void loss_reduce(const gsk::VpDesc *vps, int n_vps, const float *tile_loss, double *loss_out, cudaStream_t s);
 void pose_init(const PoseArgs &a, cudaStream_t s);
-void centroids(const gsk::VpDesc *vps, const int *set_vp, int n_sets, double *centroid, cudaStream_t s);
+// the 32 warp sums (hi, lo) of each set's means, [set][kCentroidWarps][3]; k_pose_init joins them
+void centroids(const gsk::VpDesc *vps, const int *set_vp, int n_sets, float2 *part, cudaStream_t s);
 
 struct FuseArgs {
     const double *pose64;      // [vp][12]

@@ -5,6 +5,7 @@
 // pose update about the moving submap's centroid (Sec. 3.2; learning rates
 // Supp. B), the standalone L1 loss, the Eq. 7 fusion and the Eq. 8/9 rigid
 // transform of a submap.  Latency-bound tiny kernels, FP64 state.
+#include <algorithm>
 #include <cmath>
 
 #include "gs_internal.cuh"
@@ -13,11 +14,11 @@ namespace {
 
 using namespace gsk;
 
-__device__ void so3_exp(const double *w, double R[3][3])
+// exp([w]x) = I + a [w]x + b [w]x^2
+__device__ __forceinline__ void so3_coef(const double *w, double &a, double &b)
 {
     const double th2 = w[0] * w[0] + w[1] * w[1] + w[2] * w[2];
     const double th = sqrt(th2);
-    double a, b;
     if (th < 1e-8) {
         a = 1.0 - th2 / 6.0;
         b = 0.5 - th2 / 24.0;
@@ -27,12 +28,21 @@ __device__ void so3_exp(const double *w, double R[3][3])
         a = sn / th;
         b = (1.0 - cs) / th2;
     }
-    const double K[3][3] = {{0, -w[2], w[1]}, {w[2], 0, -w[0]}, {-w[1], w[0], 0}};
-    for (int i = 0; i < 3; ++i)
-        for (int j = 0; j < 3; ++j) {
-            double k2 = K[i][0] * K[0][j] + K[i][1] * K[1][j] + K[i][2] * K[2][j];
-            R[i][j] = (i == j ? 1.0 : 0.0) + a * K[i][j] + b * k2;
-        }
+}
+
+// entry (i, j) of [w]x
+__device__ __forceinline__ double skew(const double *w, int i, int j)
+{
+    if (i == j)
+        return 0.0;
+    const double x = w[3 - i - j];
+    return (j - i + 3) % 3 == 1 ? -x : x;
+}
+
+__device__ __forceinline__ double so3_entry(const double *w, double a, double b, int i, int j)
+{
+    const double k2 = skew(w, i, 0) * skew(w, 0, j) + skew(w, i, 1) * skew(w, 1, j) + skew(w, i, 2) * skew(w, 2, j);
+    return (i == j ? 1.0 : 0.0) + a * skew(w, i, j) + b * k2;
 }
 
 // b^n for a step count n >= 1 (binary powering: a few multiplies instead of
@@ -50,21 +60,24 @@ __device__ __forceinline__ double pow_count(double b, double n)
     return r;
 }
 
-// Adam step of twist component i (0..2 rotation, 3..5 translation) with
-// gradient gi: updates its moments st[i], st[6 + i] and returns the step
-// xi_i.  k = iteration index in [0, iters) of the learning-rate schedule;
-// t = steps taken including this one (bias correction).
-__device__ double adam_component(double *st, int i, double gi, double t, int k, int iters, float lr_rot,
-                                 float lr_trans, float b1f, float b2f, float epsf, float lr_final)
+// Learning-rate schedule of iteration k in [0, iters).
+__device__ __forceinline__ double cosine_schedule(int k, int iters, float lr_final)
 {
     const double kPi = 3.14159265358979323846;
-    const double b1 = b1f, b2 = b2f, eps = epsf, f = lr_final;
-    const double sched = f + (1.0 - f) * 0.5 * (1.0 + cos(kPi * (double)k / (double)iters));
-    st[i] = b1 * st[i] + (1.0 - b1) * gi;
-    st[6 + i] = b2 * st[6 + i] + (1.0 - b2) * gi * gi;
-    const double mh = st[i] / (1.0 - pow_count(b1, t));
-    const double vh = st[6 + i] / (1.0 - pow_count(b2, t));
-    const double lr = (i < 3 ? (double)lr_rot : (double)lr_trans) * sched;
+    const double f = lr_final;
+    return f + (1.0 - f) * 0.5 * (1.0 + cos(kPi * (double)k / (double)iters));
+}
+
+// Adam step with gradient gi, learning rate lr and the bias corrections
+// bc = 1 - b^t: updates the moments m, v and returns the step.
+__device__ __forceinline__ double adam_step(double &m, double &v, double gi, double lr, double bc1, double bc2, float b1f,
+                                            float b2f, float epsf)
+{
+    const double b1 = b1f, b2 = b2f, eps = epsf;
+    m = b1 * m + (1.0 - b1) * gi;
+    v = b2 * v + (1.0 - b2) * gi * gi;
+    const double mh = m / bc1;
+    const double vh = v / bc2;
     return -lr * mh / (sqrt(vh) + eps);
 }
 
@@ -72,8 +85,11 @@ __device__ double adam_component(double *st, int i, double gi, double t, int k, 
 // R <- exp(-s_w) R, t <- exp(-s_w)(t - c) + c - s_v (xi carries the signs).
 __device__ void exp_update(double *pose, const double *xi, const double *c)
 {
-    double dR[3][3];
-    so3_exp(xi, dR);
+    double dR[3][3], ca, cb;
+    so3_coef(xi, ca, cb);
+    for (int i = 0; i < 3; ++i)
+        for (int j = 0; j < 3; ++j)
+            dR[i][j] = so3_entry(xi, ca, cb, i, j);
     double R[3][3], tt[3];
     for (int i = 0; i < 3; ++i) {
         for (int j = 0; j < 3; ++j)
@@ -94,9 +110,12 @@ __device__ void adam_exp_update(double *pose, double *st, const double *g, const
                                 float lr_rot, float lr_trans, float b1f, float b2f, float epsf, float lr_final)
 {
     const double t = st[12] + 1.0;
+    const double sched = cosine_schedule(k, iters, lr_final);
+    const double bc1 = 1.0 - pow_count(b1f, t), bc2 = 1.0 - pow_count(b2f, t);
     double xi[6];
     for (int i = 0; i < 6; ++i)
-        xi[i] = adam_component(st, i, g[i], t, k, iters, lr_rot, lr_trans, b1f, b2f, epsf, lr_final);
+        xi[i] = adam_step(st[i], st[6 + i], g[i], (i < 3 ? (double)lr_rot : (double)lr_trans) * sched, bc1, bc2, b1f,
+                          b2f, epsf);
     st[12] = t;
     exp_update(pose, xi, c);
 }
@@ -111,33 +130,43 @@ __device__ void pivots_of(const VpDesc &d, const double *pose, const double *mba
                   (double)d.w2c[4 * i + 3];
 }
 
-// mean of each Gaussian set's means (one 1024-thread block per set): FP32
-// TwoSum pairs per thread (two interleaved chains), TwoSum butterflies and a
-// fixed-order TwoSum of the warps, one FP64 division (FP64 sums over 10^5
-// means were latency-bound on the slow FP64 pipe)
-constexpr int kCentroidThreads = 1024;
+// Mean of each Gaussian set's means: 1024 running sums of two interleaved
+// FP32 TwoSum chains each, TwoSum butterflies over warps of 32 and a
+// fixed-order TwoSum of the 32 warps (in k_pose_init), one FP64 division
+// (FP64 sums over 10^5 means were latency-bound on the slow FP64 pipe).
+// One CTA per warp of the set, kCentUnroll pairs of loads in flight: the 32
+// warps on one SM took 75 us for 150k means (ncu), two loads in flight each.
+constexpr int kCentWarps = gsl::kCentroidWarps, kCentSums = 32 * kCentWarps, kCentUnroll = 8;
 
-__global__ void __launch_bounds__(kCentroidThreads) k_centroid(const VpDesc *vps, const int *set_vp, double *centroid)
+__global__ void __launch_bounds__(32) k_centroid(const VpDesc *vps, const int *set_vp, float2 *part)
 {
-    __shared__ float s[kCentroidThreads / 32][3][2];
-    const VpDesc &d = vps[set_vp[blockIdx.x]];
+    const VpDesc &d = vps[set_vp[blockIdx.y]];
+    const int n = d.n;
+    const float4 *means = d.means;
     float hs[2][3] = {{0.0f, 0.0f, 0.0f}, {0.0f, 0.0f, 0.0f}}, ls[2][3] = {{0.0f, 0.0f, 0.0f}, {0.0f, 0.0f, 0.0f}};
-    int i = threadIdx.x;
-    for (; i + kCentroidThreads < d.n; i += 2 * kCentroidThreads) {
-        const float4 m0 = d.means[i], m1 = d.means[i + kCentroidThreads];
-        two_sum_add(hs[0][0], ls[0][0], m0.x, 0.0f);
-        two_sum_add(hs[0][1], ls[0][1], m0.y, 0.0f);
-        two_sum_add(hs[0][2], ls[0][2], m0.z, 0.0f);
-        two_sum_add(hs[1][0], ls[1][0], m1.x, 0.0f);
-        two_sum_add(hs[1][1], ls[1][1], m1.y, 0.0f);
-        two_sum_add(hs[1][2], ls[1][2], m1.z, 0.0f);
+    auto add = [&](int c, const float4 &m) {
+        two_sum_add(hs[c][0], ls[c][0], m.x, 0.0f);
+        two_sum_add(hs[c][1], ls[c][1], m.y, 0.0f);
+        two_sum_add(hs[c][2], ls[c][2], m.z, 0.0f);
+    };
+    int64_t i = 32 * blockIdx.x + threadIdx.x;
+    for (; i + (2 * kCentUnroll - 1) * kCentSums < n; i += 2 * kCentUnroll * kCentSums) {
+        float4 m[2 * kCentUnroll];
+#pragma unroll
+        for (int u = 0; u < 2 * kCentUnroll; ++u)
+            m[u] = means[i + u * kCentSums];
+#pragma unroll
+        for (int u = 0; u < 2 * kCentUnroll; ++u)
+            add(u & 1, m[u]);
     }
-    if (i < d.n) {
-        const float4 m0 = d.means[i];
-        two_sum_add(hs[0][0], ls[0][0], m0.x, 0.0f);
-        two_sum_add(hs[0][1], ls[0][1], m0.y, 0.0f);
-        two_sum_add(hs[0][2], ls[0][2], m0.z, 0.0f);
+    for (; i + kCentSums < n; i += 2 * kCentSums) {
+        const float4 m0 = means[i], m1 = means[i + kCentSums];
+        add(0, m0);
+        add(1, m1);
     }
+    if (i < n)
+        add(0, means[i]);
+#pragma unroll
     for (int k = 0; k < 3; ++k) {
         float h = hs[0][k], l = ls[0][k];
         two_sum_add(h, l, hs[1][k], ls[1][k]);
@@ -146,17 +175,8 @@ __global__ void __launch_bounds__(kCentroidThreads) k_centroid(const VpDesc *vps
             const float bh = __shfl_xor_sync(0xffffffffu, h, o), bl = __shfl_xor_sync(0xffffffffu, l, o);
             two_sum_add(h, l, bh, bl);
         }
-        if ((threadIdx.x & 31) == 0) {
-            s[threadIdx.x >> 5][k][0] = h;
-            s[threadIdx.x >> 5][k][1] = l;
-        }
-    }
-    __syncthreads();
-    if (threadIdx.x < 3) {
-        float h = s[0][threadIdx.x][0], l = s[0][threadIdx.x][1];
-        for (int w = 1; w < kCentroidThreads / 32; ++w)
-            two_sum_add(h, l, s[w][threadIdx.x][0], s[w][threadIdx.x][1]);
-        centroid[3 * blockIdx.x + threadIdx.x] = d.n > 0 ? ((double)h + (double)l) / d.n : 0.0;
+        if (threadIdx.x == 0)
+            part[(blockIdx.y * kCentWarps + blockIdx.x) * 3 + k] = make_float2(h, l);
     }
 }
 
@@ -165,7 +185,35 @@ __global__ void k_pose_init(const gsl::PoseArgs a)
     const int vp = blockIdx.x * blockDim.x + threadIdx.x;
     if (vp >= a.n_vps)
         return;
-    const VpDesc &d = a.vps[vp];
+    {
+        // the set's centroid, joined by every keyframe that needs it and
+        // kept by the set's first (a set's keyframes are consecutive)
+        const VpDesc &d = a.vps[vp];
+        const float2 *part = a.cent_part + (size_t)d.set * kCentWarps * 3;
+        float h[3], l[3];
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            h[k] = part[k].x;
+            l[k] = part[k].y;
+        }
+#pragma unroll 8
+        for (int w = 1; w < kCentWarps; ++w)
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                const float2 v = part[3 * w + k];
+                two_sum_add(h[k], l[k], v.x, v.y);
+            }
+        double mbar[3];
+        for (int k = 0; k < 3; ++k)
+            mbar[k] = d.n > 0 ? ((double)h[k] + (double)l[k]) / d.n : 0.0;
+        if (vp == 0 || a.vps[vp - 1].set != d.set)
+            for (int k = 0; k < 3; ++k)
+                a.centroid[3 * d.set + k] = mbar[k];
+        double I[12];
+        for (int k = 0; k < 12; ++k)
+            I[k] = (k % 5 == 0) ? 1.0 : 0.0;
+        pivots_of(d, I, mbar, a.pivot + 3 * vp, a.c_cam + 3 * vp);
+    }
     double *P = a.pose64 + 12 * vp;
     for (int k = 0; k < 12; ++k) {
         P[k] = (k % 5 == 0) ? 1.0 : 0.0;
@@ -173,7 +221,6 @@ __global__ void k_pose_init(const gsl::PoseArgs a)
     }
     for (int k = 0; k < 13; ++k)
         a.adam[13 * vp + k] = 0.0;
-    pivots_of(d, P, a.centroid + 3 * d.set, a.pivot + 3 * vp, a.c_cam + 3 * vp);
     if (a.expo) {
         for (int k = 0; k < 7; ++k)
             a.expo[7 * vp + k] = 0.0;
@@ -182,129 +229,193 @@ __global__ void k_pose_init(const gsl::PoseArgs a)
     }
 }
 
-// Adam step on the exposure (a, b) with the pose's moments and schedule
-// (iteration k of iters); e = a, b, m_a, m_b, v_a, v_b, steps taken
-__device__ void exposure_step(double *e, const double *g, int k, int iters, float lr, float b1f, float b2f, float epsf,
-                              float lr_final)
-{
-    const double kPi = 3.14159265358979323846;
-    const double b1 = b1f, b2 = b2f, eps = epsf, f = lr_final;
-    const double t = e[6] + 1.0;
-    e[6] = t;
-    const double sched = f + (1.0 - f) * 0.5 * (1.0 + cos(kPi * (double)k / (double)iters));
-    for (int i = 0; i < 2; ++i) {
-        e[2 + i] = b1 * e[2 + i] + (1.0 - b1) * g[i];
-        e[4 + i] = b2 * e[4 + i] + (1.0 - b2) * g[i] * g[i];
-        const double mh = e[2 + i] / (1.0 - pow(b1, t));
-        const double vh = e[4 + i] / (1.0 - pow(b2, t));
-        e[i] -= (double)lr * sched * mh / (sqrt(vh) + eps);
-    }
-}
-
 // 1024 threads per block: a keyframe's 3,225 tile pairs (1200x680) are
 // about three loads deep per thread (256 threads waited on thirteen).
 constexpr int kPoseThreads = 1024, kPoseWarps = kPoseThreads / 32;
 
-// one block per keyframe: reduce the tile twists and losses in a fixed
+// One block per keyframe: reduce the tile twists and losses in a fixed
 // order, rotate the twist to the world frame, then (update) take the step.
-// The step's FP64 work runs on warp 0: Adam on the six twist components in
-// parallel (one lane each -- serially, their pow/sqrt chains dominated the
-// update, the FP64 pipe being a small fraction of the FP32 one), then the
-// exponential-map update, the exposure step and the pivots on lane 0.
+// Bound by the latency of the step's FP64 chain (this part issues an FP64
+// instruction of a warp every 16 clocks): so what needs no gradient -- the
+// schedule's cosine and the bias corrections -- is found by other warps
+// while the tiles are summed, and the 3x3 products of the exponential map
+// run one entry per lane instead of all on one.  Each entry's operations
+// and their order are those of exp_update.
 __global__ void __launch_bounds__(kPoseThreads) k_pose_update(const gsl::PoseArgs a)
 {
     __shared__ float s[kPoseWarps][9][2];
-    __shared__ double s_tot[9], s_g[6], s_xi[6];
+    __shared__ double s_tot[9], s_g[6], s_xi[6], s_pre[5], s_dR[9], s_P[12];
     const int vp = blockIdx.x;
     const VpDesc &d = a.vps[vp];
     const uint32_t nt = (uint32_t)d.TX * d.TY;
     const bool expo = d.exposure && a.tile_expo && a.expo;
-    // (hi, lo) FP32 pairs summed by TwoSum in a fixed order (per thread,
-    // then butterflies, then the warps); one FP64 value per component
-    float hs[9], ls[9];
-#pragma unroll
-    for (int i = 0; i < 9; ++i)
-        hs[i] = ls[i] = 0.0f;
-#pragma unroll 4
-    for (uint32_t k = threadIdx.x; k < nt; k += blockDim.x) {
-        const size_t t = d.tile_base + k;
-        if (a.tile_twist)
-#pragma unroll
-            for (int i = 0; i < 6; ++i) {
-                const float2 v = a.tile_twist[t * 6 + i];
-                two_sum_add(hs[i], ls[i], v.x, v.y);
-            }
-        two_sum_add(hs[6], ls[6], a.tile_loss[t], 0.0f);
-        if (expo) {
-            two_sum_add(hs[7], ls[7], a.tile_expo[2 * t], 0.0f);
-            two_sum_add(hs[8], ls[8], a.tile_expo[2 * t + 1], 0.0f);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    // (a gradient-only caller has neither pose nor optimiser state)
+    const bool update = a.update && a.tile_twist;
+    const int iters = d.iters > 0 ? d.iters : a.iters;
+    double *st = update ? a.adam + 13 * vp : nullptr;
+    // warp 0's operands of the step, loaded ahead of the sums
+    double m = 0.0, v = 0.0, P0 = 0.0, taken = 0.0;
+    if (update && (warp == 0 || warp >= kPoseWarps - 5)) {
+        taken = st[12];
+        if (warp == 0 && lane < 6) {
+            m = st[lane];
+            v = st[6 + lane];
         }
+        if (warp == 0 && lane < 12)
+            P0 = a.pose64[12 * vp + lane];
     }
+    if (update && (int)taken < iters) {
+        // s_pre: schedule, 1 - b1^t, 1 - b2^t of the pose and of the exposure
+        if (warp == kPoseWarps - 1 && lane == 0)
+            s_pre[0] = cosine_schedule((int)taken, iters, a.lr_final);
+        if (warp == kPoseWarps - 2 && lane == 0)
+            s_pre[1] = 1.0 - pow_count(a.beta1, taken + 1.0);
+        if (warp == kPoseWarps - 3 && lane == 0)
+            s_pre[2] = 1.0 - pow_count(a.beta2, taken + 1.0);
+        if (expo && warp == kPoseWarps - 4 && lane == 0)
+            s_pre[3] = 1.0 - pow((double)a.beta1, a.expo[7 * vp + 6] + 1.0);
+        if (expo && warp == kPoseWarps - 5 && lane == 0)
+            s_pre[4] = 1.0 - pow((double)a.beta2, a.expo[7 * vp + 6] + 1.0);
+    }
+    // (hi, lo) FP32 pairs summed by TwoSum in a fixed order (per thread,
+    // then butterflies, then the warps); one FP64 value per component.  A
+    // warp without tiles holds zeros, which leave a TwoSum as it is.
+    const int nw = (int)min((nt + 31) / 32, (uint32_t)kPoseWarps);
+    if (warp < nw) {
+        float hs[9], ls[9];
 #pragma unroll
-    for (int i = 0; i < 9; ++i) {
+        for (int i = 0; i < 9; ++i)
+            hs[i] = ls[i] = 0.0f;
+#pragma unroll 4
+        for (uint32_t k = threadIdx.x; k < nt; k += blockDim.x) {
+            const size_t t = d.tile_base + k;
+            if (a.tile_twist)
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            const float bh = __shfl_xor_sync(0xffffffffu, hs[i], o), bl = __shfl_xor_sync(0xffffffffu, ls[i], o);
-            two_sum_add(hs[i], ls[i], bh, bl);
+                for (int i = 0; i < 6; ++i) {
+                    const float2 w = a.tile_twist[t * 6 + i];
+                    two_sum_add(hs[i], ls[i], w.x, w.y);
+                }
+            two_sum_add(hs[6], ls[6], a.tile_loss[t], 0.0f);
+            if (expo) {
+                two_sum_add(hs[7], ls[7], a.tile_expo[2 * t], 0.0f);
+                two_sum_add(hs[8], ls[8], a.tile_expo[2 * t + 1], 0.0f);
+            }
         }
-        if ((threadIdx.x & 31) == 0) {
-            s[threadIdx.x >> 5][i][0] = hs[i];
-            s[threadIdx.x >> 5][i][1] = ls[i];
+#pragma unroll
+        for (int i = 0; i < 9; ++i) {
+            if ((i < 6 && !a.tile_twist) || (i > 6 && !expo))
+                continue;
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                const float bh = __shfl_xor_sync(0xffffffffu, hs[i], o), bl = __shfl_xor_sync(0xffffffffu, ls[i], o);
+                two_sum_add(hs[i], ls[i], bh, bl);
+            }
+            if (lane == 0) {
+                s[warp][i][0] = hs[i];
+                s[warp][i][1] = ls[i];
+            }
         }
     }
     __syncthreads();
-    if (threadIdx.x >= 32)
+    if (warp != 0)
         return;
-    const int lane = threadIdx.x;
-    if (lane < 9) {
+    if (lane < 9 && (lane >= 6 || a.tile_twist) && (lane <= 6 || expo)) {
         float h = s[0][lane][0], l = s[0][lane][1];
-        for (int w = 1; w < kPoseWarps; ++w)
+#pragma unroll 8
+        for (int w = 1; w < nw; ++w)
             two_sum_add(h, l, s[w][lane][0], s[w][lane][1]);
         s_tot[lane] = (double)h + (double)l;
+        if (lane == 6)
+            a.loss[vp] = s_tot[6];
     }
-    __syncwarp();
-    double tot[9];
-    for (int i = 0; i < 9; ++i)
-        tot[i] = s_tot[i];
-    if (lane == 0)
-        a.loss[vp] = tot[6];
     if (!a.tile_twist)
         return;
+    __syncwarp();
     // camera frame -> world frame: w = Rv^T w_c, v = Rv^T v_c
+    double gi = 0.0;
     if (lane < 6) {
         const int r = lane % 3, o = lane < 3 ? 0 : 3;
-        const double gi =
-            (double)d.w2c[r] * tot[o] + (double)d.w2c[4 + r] * tot[o + 1] + (double)d.w2c[8 + r] * tot[o + 2];
-        s_g[lane] = gi;
+        gi = (double)d.w2c[r] * s_tot[o] + (double)d.w2c[4 + r] * s_tot[o + 1] + (double)d.w2c[8 + r] * s_tot[o + 2];
         if (a.grad)
             a.grad[6 * vp + lane] = gi;
     }
-    if (!a.update)
-        return;  // (pose and optimiser state may be absent: gradient-only callers)
-    const int iters = d.iters > 0 ? d.iters : a.iters;
-    double *st = a.adam + 13 * vp;
-    const int k = (int)st[12];
+    if (!update)
+        return;
+    const int k = (int)taken;
     if (k >= iters)
         return;
-    const double t = st[12] + 1.0;
-    if (lane < 6)
-        s_xi[lane] = adam_component(st, lane, s_g[lane], t, k, iters, d.lr_rot, d.lr_trans, a.beta1, a.beta2,
-                                    a.eps, a.lr_final);
-    __syncwarp();
-    if (lane != 0)
-        return;
-    st[12] = t;
-    double *P = a.pose64 + 12 * vp;
-    exp_update(P, s_xi, a.pivot + 3 * vp);
-    if (expo) {
-        double *e = a.expo + 7 * vp;
-        exposure_step(e, tot + 7, k, iters, d.lr_exposure, a.beta1, a.beta2, a.eps, a.lr_final);
-        a.expo32[2 * vp] = (float)exp(e[0]);
-        a.expo32[2 * vp + 1] = (float)e[1];
+    if (lane < 6) {
+        s_xi[lane] = adam_step(m, v, gi, (lane < 3 ? (double)d.lr_rot : (double)d.lr_trans) * s_pre[0], s_pre[1],
+                               s_pre[2], a.beta1, a.beta2, a.eps);
+        st[lane] = m;
+        st[6 + lane] = v;
     }
-    for (int q = 0; q < 12; ++q)
-        a.pose32[12 * vp + q] = (float)P[q];
-    pivots_of(d, P, a.centroid + 3 * d.set, a.pivot + 3 * vp, a.c_cam + 3 * vp);
+    if (lane < 12)
+        s_P[lane] = P0;
+    if (lane == 6)
+        st[12] = taken + 1.0;
+    __syncwarp();
+    // R <- exp(xi_w) R, t <- exp(xi_w)(t - c) + c + xi_v (exp_update), entry
+    // (i, j) on lane 3 i + j, then on lane 4 i + j
+    double ca, cb;
+    so3_coef(s_xi, ca, cb);
+    if (lane < 9)
+        s_dR[lane] = so3_entry(s_xi, ca, cb, lane / 3, lane % 3);
+    __syncwarp();
+    const double *c = a.pivot + 3 * vp;
+    double Pn = 0.0;
+    if (lane < 12) {
+        const int i = lane >> 2, j = lane & 3;
+        double q[3];
+#pragma unroll
+        for (int r = 0; r < 3; ++r) {
+            q[r] = s_P[4 * r + j];
+            if (j == 3)
+                q[r] = q[r] - c[r];
+        }
+        Pn = s_dR[3 * i] * q[0] + s_dR[3 * i + 1] * q[1] + s_dR[3 * i + 2] * q[2];
+        if (j == 3)
+            Pn = Pn + c[i] + s_xi[3 + i];
+    }
+    __syncwarp();
+    if (lane < 12) {
+        s_P[lane] = Pn;
+        a.pose64[12 * vp + lane] = Pn;
+        a.pose32[12 * vp + lane] = (float)Pn;
+    }
+    if (expo && (lane == 16 || lane == 17)) {
+        // Adam on the exposure (a, b) with the pose's schedule; e = a, b,
+        // m_a, m_b, v_a, v_b, steps taken
+        const int i = lane - 16;
+        double *e = a.expo + 7 * vp;
+        const double t = e[6] + 1.0;
+        double em = e[2 + i], ev = e[4 + i];
+        const double b1 = a.beta1, b2 = a.beta2, eps = a.eps, g = s_tot[7 + i];
+        em = b1 * em + (1.0 - b1) * g;
+        ev = b2 * ev + (1.0 - b2) * g * g;
+        const double mh = em / s_pre[3], vh = ev / s_pre[4];
+        double x = e[i];
+        x -= (double)d.lr_exposure * s_pre[0] * mh / (sqrt(vh) + eps);
+        e[i] = x;
+        e[2 + i] = em;
+        e[4 + i] = ev;
+        a.expo32[2 * vp + i] = i == 0 ? (float)exp(x) : (float)x;
+        __syncwarp(0x30000u);  // both lanes have read the count
+        if (i == 0)
+            e[6] = t;
+    }
+    __syncwarp();
+    // the pivot R mu_bar + t and its camera-frame image (pivots_of)
+    if (lane < 3) {
+        const double *mb = a.centroid + 3 * d.set;
+        s_g[lane] = s_P[4 * lane] * mb[0] + s_P[4 * lane + 1] * mb[1] + s_P[4 * lane + 2] * mb[2] + s_P[4 * lane + 3];
+        a.pivot[3 * vp + lane] = s_g[lane];
+    }
+    __syncwarp();
+    if (lane < 3)
+        a.c_cam[3 * vp + lane] = (double)d.w2c[4 * lane] * s_g[0] + (double)d.w2c[4 * lane + 1] * s_g[1] +
+                                 (double)d.w2c[4 * lane + 2] * s_g[2] + (double)d.w2c[4 * lane + 3];
 }
 
 __global__ void k_expo32(const double *expo, float *expo32, int n)
@@ -365,65 +476,195 @@ __device__ void jacobi4(double A[4][4], double V[4][4])
     }
 }
 
-// T^-1 of a 3x4 rigid map
-__device__ void rigid_inverse(const double *T, double *Ti)
+// Eigenvectors (columns of V) and eigenvalues (diagonal of A) of a symmetric
+// 4x4 in FP32: cyclic Jacobi, unrolled so that everything stays in registers.
+__device__ __forceinline__ void jacobi4_f32(float (&A)[4][4], float (&V)[4][4])
 {
-    for (int i = 0; i < 3; ++i) {
-        for (int j = 0; j < 3; ++j)
-            Ti[4 * i + j] = T[4 * j + i];
-        Ti[4 * i + 3] = -(T[i] * T[3] + T[4 + i] * T[7] + T[8 + i] * T[11]);
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+            V[i][j] = i == j ? 1.0f : 0.0f;
+    for (int sweep = 0; sweep < 6; ++sweep) {
+        float off = 0.0f;
+#pragma unroll
+        for (int p = 0; p < 4; ++p)
+#pragma unroll
+            for (int q = p + 1; q < 4; ++q) {
+                off += fabsf(A[p][q]);
+                if (fabsf(A[p][q]) < 1e-30f)
+                    continue;
+                const float theta = (A[q][q] - A[p][p]) / (2.0f * A[p][q]);
+                const float t = copysignf(1.0f, theta) / (fabsf(theta) + sqrtf(fmaf(theta, theta, 1.0f)));
+                const float c = rsqrtf(fmaf(t, t, 1.0f)), s = t * c;
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    const float x = A[k][p], y = A[k][q];
+                    A[k][p] = c * x - s * y;
+                    A[k][q] = s * x + c * y;
+                }
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    const float x = A[p][k], y = A[q][k];
+                    A[p][k] = c * x - s * y;
+                    A[q][k] = s * x + c * y;
+                    const float u = V[k][p], v = V[k][q];
+                    V[k][p] = c * u - s * v;
+                    V[k][q] = s * u + c * v;
+                }
+            }
+        if (off < 1e-6f)
+            break;
     }
 }
 
-// one thread per problem: weighted chordal L2 mean of the rotations (the
-// quaternion maximising tr(R^T sum w_i R_i), i.e. the top eigenvector of
-// Horn's symmetric 4x4 matrix) and weighted mean of the translations
-__global__ void k_fuse(const gsl::FuseArgs a)
+// Top eigenvector of a symmetric 4x4: the FP32 eigenvectors, then FP64
+// residuals corrected along the other three eigenvectors in FP32 (each step
+// gains the FP32 factors' accuracy over the relative gap), until the
+// residual is FP64's own.  Returns false (x unspecified) where that is not
+// reached: a gap below 1e-3 of the largest entry, or values not finite.
+__device__ __forceinline__ bool top_eigenvector4(const double (&K)[4][4], double (&x)[4])
 {
-    const int p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= a.n_problems)
-        return;
-    double M[3][3] = {{0, 0, 0}, {0, 0, 0}, {0, 0, 0}}, ts[3] = {0, 0, 0}, wsum = 0.0;
-    const int first = a.prob_first[p], count = a.prob_count[p];
-    for (int e = first; e < first + count; ++e) {
-        double T[12];
-        const double *src = a.pose64 + 12 * e;
-        if (a.reverse[e])
-            rigid_inverse(src, T);
-        else
-            for (int k = 0; k < 12; ++k)
-                T[k] = src[k];
-        if (a.est_out)
-            for (int k = 0; k < 12; ++k)
-                a.est_out[12 * e + k] = T[k];
-        const double w = 1.0 / fmax(a.eps[e], 1e-12);
-        for (int i = 0; i < 3; ++i) {
-            for (int j = 0; j < 3; ++j)
-                M[i][j] += w * T[4 * i + j];
-            ts[i] += w * T[4 * i + 3];
+    double scale = 0.0;
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+            scale = fmax(scale, fabs(K[i][j]));
+    if (!(scale > 0.0) || !(scale < 1e300))
+        return false;
+    const double inv = 1.0 / scale;
+    float A[4][4], V[4][4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+            A[i][j] = (float)(K[i][j] * inv);
+    jacobi4_f32(A, V);
+    // the largest eigenvalue into column 0
+#pragma unroll
+    for (int i = 1; i < 4; ++i)
+        if (A[i][i] > A[0][0]) {
+            const float e = A[0][0];
+            A[0][0] = A[i][i];
+            A[i][i] = e;
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const float v = V[k][0];
+                V[k][0] = V[k][i];
+                V[k][i] = v;
+            }
         }
-        wsum += w;
+    float g[3];
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        if (!(A[0][0] - A[i + 1][i + 1] > 1e-3f))
+            return false;
+        g[i] = 1.0f / (A[0][0] - A[i + 1][i + 1]);
     }
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+        x[k] = V[k][0];
+    for (int it = 0; it < 8; ++it) {
+        double y[4], rho = 0.0, xx = 0.0;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            y[i] = (K[i][0] * x[0] + K[i][1] * x[1] + K[i][2] * x[2] + K[i][3] * x[3]) * inv;
+            rho += x[i] * y[i];
+            xx += x[i] * x[i];
+        }
+        rho /= xx;
+        float r[4], rmax = 0.0f;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            r[i] = (float)(y[i] - rho * x[i]);
+            rmax = fmaxf(rmax, fabsf(r[i]));
+        }
+        if (rmax < 1e-15f)
+            return true;
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+            float w = 0.0f;
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+                w = fmaf(V[k][i + 1], r[k], w);
+            w *= g[i];
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+                x[k] += (double)(w * V[k][i + 1]);
+        }
+    }
+    return false;
+}
+
+// One warp per problem: weighted chordal L2 mean of the rotations (the
+// quaternion maximising tr(R^T sum w_i R_i), i.e. the top eigenvector of
+// Horn's symmetric 4x4 matrix) and weighted mean of the translations.  Lane
+// 4 i + j sums entry (i, j) of the weighted estimates, in their order.
+// Latency only: the FP64 Jacobi sweeps of one thread, whose arrays were
+// indexed in local memory, took 92 to 385 us per call (ncu; most of it
+// sweeps after convergence, their threshold being absolute); they remain
+// for eigenvalues too close for the FP32 start.
+__global__ void __launch_bounds__(32) k_fuse(const gsl::FuseArgs a)
+{
+    __shared__ double s_m[12];
+    const int p = blockIdx.x, lane = threadIdx.x;
+    const int first = a.prob_first[p], count = a.prob_count[p];
+    const int i = lane >> 2, j = lane & 3;
+    double sum = 0.0, wsum = 0.0;
+    for (int e0 = first; e0 < first + count; e0 += 32) {
+        const int n = min(32, first + count - e0);
+        const double wl = lane < n ? 1.0 / fmax(a.eps[e0 + lane], 1e-12) : 0.0;
+        for (int q = 0; q < n; ++q) {
+            const int e = e0 + q;
+            const double w = __shfl_sync(0xffffffffu, wl, q);
+            if (lane < 12) {
+                const double *src = a.pose64 + 12 * (size_t)e;
+                double t;
+                if (!a.reverse[e])
+                    t = src[lane];
+                else if (j < 3)
+                    t = src[4 * j + i];
+                else
+                    t = -(src[i] * src[3] + src[4 + i] * src[7] + src[8 + i] * src[11]);
+                if (a.est_out)
+                    a.est_out[12 * (size_t)e + lane] = t;
+                sum += w * t;
+            }
+            wsum += w;
+        }
+    }
+    if (lane < 12)
+        s_m[lane] = sum;
+    __syncwarp();
+    if (lane != 0)
+        return;
+    const double M[3][3] = {{s_m[0], s_m[1], s_m[2]}, {s_m[4], s_m[5], s_m[6]}, {s_m[8], s_m[9], s_m[10]}};
     double K[4][4] = {
         {M[0][0] + M[1][1] + M[2][2], M[2][1] - M[1][2], M[0][2] - M[2][0], M[1][0] - M[0][1]},
         {M[2][1] - M[1][2], M[0][0] - M[1][1] - M[2][2], M[0][1] + M[1][0], M[0][2] + M[2][0]},
         {M[0][2] - M[2][0], M[0][1] + M[1][0], -M[0][0] + M[1][1] - M[2][2], M[1][2] + M[2][1]},
         {M[1][0] - M[0][1], M[0][2] + M[2][0], M[1][2] + M[2][1], -M[0][0] - M[1][1] + M[2][2]}};
-    double V[4][4];
-    jacobi4(K, V);
-    int best = 0;
-    for (int i = 1; i < 4; ++i)
-        if (K[i][i] > K[best][best])
-            best = i;
-    double w = V[0][best], x = V[1][best], y = V[2][best], z = V[3][best];
+    double v[4];
+    if (!top_eigenvector4(K, v)) {
+        double V[4][4];
+        jacobi4(K, V);
+        int best = 0;
+        for (int k = 1; k < 4; ++k)
+            if (K[k][k] > K[best][best])
+                best = k;
+        for (int k = 0; k < 4; ++k)
+            v[k] = V[k][best];
+    }
+    double w = v[0], x = v[1], y = v[2], z = v[3];
     const double nq = sqrt(w * w + x * x + y * y + z * z);
     w /= nq; x /= nq; y /= nq; z /= nq;
-    double *T = a.T_out + 12 * p;
+    double *T = a.T_out + 12 * (size_t)p;
     T[0] = 1 - 2 * (y * y + z * z); T[1] = 2 * (x * y - w * z); T[2] = 2 * (x * z + w * y);
     T[4] = 2 * (x * y + w * z); T[5] = 1 - 2 * (x * x + z * z); T[6] = 2 * (y * z - w * x);
     T[8] = 2 * (x * z - w * y); T[9] = 2 * (y * z + w * x); T[10] = 1 - 2 * (x * x + y * y);
-    for (int i = 0; i < 3; ++i)
-        T[4 * i + 3] = wsum > 0 ? ts[i] / wsum : 0.0;
+    for (int r = 0; r < 3; ++r)
+        T[4 * r + 3] = wsum > 0 ? s_m[4 * r + 3] / wsum : 0.0;
     a.conf[p] = count > 0 ? wsum / count : 0.0;
 }
 
@@ -629,10 +870,12 @@ __global__ void __launch_bounds__(kRigidThreads) k_transform_batch(const gsl::Ma
 
 namespace gsl {
 
-void centroids(const VpDesc *vps, const int *set_vp, int n_sets, double *centroid, cudaStream_t s)
+void centroids(const VpDesc *vps, const int *set_vp, int n_sets, float2 *part, cudaStream_t s)
 {
-    if (n_sets > 0) {
-        k_centroid<<<n_sets, kCentroidThreads, 0, s>>>(vps, set_vp, centroid);
+    // (grids are at most 65,535 high)
+    for (int f = 0; f < n_sets; f += 32768) {
+        k_centroid<<<dim3(kCentWarps, std::min(n_sets - f, 32768)), 32, 0, s>>>(vps, set_vp + f,
+                                                                              part + (size_t)f * kCentWarps * 3);
         ++g_launches;
     }
 }
@@ -666,7 +909,7 @@ void pose_step_raw(int n, double *pose, double *state, const double *grad, const
 void fuse(const FuseArgs &a, cudaStream_t s)
 {
     if (a.n_problems > 0) {
-        k_fuse<<<(a.n_problems + 63) / 64, 64, 0, s>>>(a);
+        k_fuse<<<a.n_problems, 32, 0, s>>>(a);
         ++g_launches;
     }
 }

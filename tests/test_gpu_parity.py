@@ -398,6 +398,32 @@ def test_fuse_parity(gs, ctx):
     assert float(conf) == pytest.approx(cr, rel=1e-12)
 
 
+@pytest.mark.parametrize("kind", ["one", "many", "gap_1e-2", "gap_1e-4", "weights"])
+def test_fuse_eigenvector_routes(gs, ctx, kind):
+    # one estimate, more than a warp's, two estimates half a turn apart whose
+    # weights leave a relative eigenvalue gap on either side of the FP32
+    # start's limit, and weights over eight decades; FP64 bars as above (an
+    # eigenvector of FP64 residual 1e-15 over a gap of 1e-4 is within 1e-11)
+    rng = np.random.default_rng(140)
+    n = {"one": 1, "many": 40}.get(kind, 2 if kind.startswith("gap") else 9)
+    T0 = synth.random_rigid(rng, 30.0, 0.5)
+    est = [synth.compose(synth.random_rigid(rng, 5.0, 0.05), T0) for _ in range(n)]
+    eps = rng.uniform(0.01, 0.2, n)
+    if kind.startswith("gap"):
+        turn = np.concatenate([synth.axis_angle_matrix((1, 2, 3), math.pi), np.zeros((3, 1))], 1)
+        est[1] = synth.compose(turn, est[0])
+        eps = np.array([0.1, 0.1 * (1.0 + float(kind[4:]))])
+    if kind == "weights":
+        eps = 10.0 ** rng.uniform(-8, 0, n)
+    rev = [k % 3 == 1 for k in range(n)]
+    given = [synth.inverse(E) if r else E for E, r in zip(est, rev)]
+    T, conf = gs.gs_fuse(ctx, dev(np.stack(given).reshape(n, 12), torch.float64),
+                         dev(np.array(rev, np.int32), torch.int32), dev(eps, torch.float64))
+    Tr, cr = O.fuse(np.stack(given), eps, rev)
+    np.testing.assert_allclose(T.cpu().numpy().reshape(3, 4), Tr, atol=1e-10)
+    assert float(conf) == pytest.approx(cr, rel=1e-12)
+
+
 def test_transform_parity(gs, ctx):
     gd, _ = plain_case()
     og = O.Gaussians.from_dict(gd)
