@@ -24,7 +24,7 @@ enum Slot {
     S_VPS, S_GROUPS, S_TILEVP, S_POSE32, S_REC, S_AUX, S_COUNTS, S_PARTIALS, S_NDUPS, S_K0, S_V0, S_RANGES, S_FLAGS, S_TF, S_LAST, S_CODE, S_TLOSS, S_TTWIST, S_POSE64, S_ADAM, S_PIVOT,
     S_CCAM, S_CENT, S_CENTP, S_LOSS, S_SETVP, S_REV, S_PFIRST, S_PCOUNT, S_TOUT, S_CONF, S_EST, S_GRAD, S_DUPG,
     S_PAIRS, S_RSLOT, S_RSLOTN, S_TERR, S_TCOL, S_TW,
-    S_TMED, S_TNV, S_TVPS, S_EXPO, S_EXPO32, S_TEXPO, S_OPT, S_ONN1, S_ONN2, S_OD2, S_OT, S_OCNT, S_MAPS, S_OS, S_ORDER, S_ORDC, S_SK, S_SV, S_SN, S_OBOX, S_GCELL, S_GSTART, S_GCUR, S_GPART, S_GPTS, S_GIDX, S_GLIST, S_GNL, S_GCELL2, S_GSTART2, S_GCUR2, S_GPART2, S_GPTS2, S_GIDX2, S_GLIST2, S_GNL2, S_SEGZ, S_SEGCUR, S_SEGBIG, S_SEGLIST, S_PROBE, S_QUEUE, S_COUNT
+    S_TMED, S_TNV, S_TVPS, S_EXPO, S_EXPO32, S_TEXPO, S_OPT, S_ONN1, S_ONN2, S_OD2, S_OHDR, S_MAPS, S_OS, S_ORDER, S_ORDC, S_SK, S_SV, S_SN, S_GCELL, S_GCOUNT, S_GSTART, S_GSUMS, S_GPTS, S_GLIST, S_SEGZ, S_SEGCUR, S_SEGBIG, S_SEGLIST, S_PROBE, S_QUEUE, S_COUNT
 };
 
 struct Buf {
@@ -1369,12 +1369,8 @@ gs_status_t gs_overlap_ratio(gs_ctx_t *ctx, const gs_gaussians_t *p, const gs_ga
     a.q = (const float4 *)q->means;
     a.np = (int)np;
     a.nq = (int)nq;
-    std::vector<float> T32(12);
     for (int k = 0; k < 12; ++k)
-        T32[k] = (float)T_host[k];
-    float *Td = nullptr;
-    GS_TRY(upload(ctx, S_OT, T32, &Td, s));
-    a.T32 = Td;
+        a.T32[k] = (float)T_host[k];
     GS_TRY(wsT(ctx, S_OPT, std::max<size_t>(np, 1), &a.pt));
     if (nn_pq)
         a.nn_pq = nn_pq;
@@ -1385,94 +1381,29 @@ gs_status_t gs_overlap_ratio(gs_ctx_t *ctx, const gs_gaussians_t *p, const gs_ga
     else
         GS_TRY(wsT(ctx, S_ONN2, std::max<size_t>(nq, 1), &a.nn_qp));
     GS_TRY(wsT(ctx, S_OD2, std::max<size_t>(np, 1), &a.d2));
-    GS_TRY(wsT(ctx, S_OCNT, 2, &a.counts));
+    GS_TRY(wsT(ctx, S_OHDR, 1, &a.hdr));
     a.tau2 = tau * tau;
-    if (np < 64 || nq < 64) {
-        gsl::overlap(a, s);  // brute force
+    const bool grid = np >= 64 && nq >= 64;
+    if (grid) {
+        const size_t nmax = std::max(np, nq);
+        a.max_cells = (uint32_t)std::min<size_t>(nmax * 11 / 5 + 64, (size_t)1 << 22);
+        GS_TRY(wsT(ctx, S_GCELL, np + nq, &a.cell));
+        GS_TRY(wsT(ctx, S_GCOUNT, 2 * (size_t)a.max_cells, &a.count));
+        GS_TRY(wsT(ctx, S_GSTART, 2 * (size_t)a.max_cells + 1, &a.start));
+        GS_TRY(wsT(ctx, S_GSUMS, gsl::overlap_sum_blocks(a.max_cells), &a.sums));
+        GS_TRY(wsT(ctx, S_GPTS, np + nq, &a.spts));
+        GS_TRY(wsT(ctx, S_GLIST, np + nq, &a.list));
+        gsl::overlap_grid(a, s);
     } else {
-        // uniform grid over the box of both point sets (read back once)
-        uint32_t *bbox = nullptr;
-        GS_TRY(wsT(ctx, S_OBOX, 6, &bbox));
-        gsl::overlap_moved_bbox(a, bbox, s);
-        uint32_t mm[6];
-        GS_CUDA(cudaMemcpyAsync(mm, bbox, sizeof mm, cudaMemcpyDeviceToHost, s));
-        GS_CUDA(cudaStreamSynchronize(s));
-        auto o2f = [](uint32_t u) {
-            const uint32_t b = (u & 0x80000000u) ? (u & 0x7fffffffu) : ~u;
-            float f;
-            std::memcpy(&f, &b, sizeof f);
-            return (double)f;
-        };
-        double lo[3], ext[3], emax = 0.0;
-        for (int k = 0; k < 3; ++k) {
-            lo[k] = o2f(mm[k]);
-            ext[k] = o2f(mm[3 + k]) - lo[k];
-            if (!std::isfinite(lo[k]) || !std::isfinite(ext[k]))
-                return fail(ctx, GS_ERR_NONFINITE, "gs_overlap_ratio: non-finite mean");
-            emax = std::max(emax, ext[k]);
-        }
-        const double pad = 1e-3 * emax + 1e-6;
-        double vol = 1.0;
-        for (int k = 0; k < 3; ++k) {
-            lo[k] -= pad;
-            ext[k] = std::max(ext[k] + 2.0 * pad, 1e-3 * emax + 1e-6);
-            vol *= ext[k];
-        }
-        // about two cells per target, at most 2^22 cells and 2048 per axis
-        double cell = std::cbrt(vol / (2.0 * (double)std::max(np, nq)));
-        cell = std::max(cell, (emax + 2.0 * pad) / 2048.0);
-        int dims[3];
-        for (;;) {
-            size_t cells = 1;
-            for (int k = 0; k < 3; ++k) {
-                dims[k] = std::max(1, (int)std::ceil(ext[k] / cell));
-                cells *= (size_t)dims[k];
-            }
-            if (cells <= ((size_t)1 << 22))
-                break;
-            cell *= 1.26;
-        }
-        gsl::NNGrid g{};
-        g.ox = (float)lo[0];
-        g.oy = (float)lo[1];
-        g.oz = (float)lo[2];
-        g.s = (float)cell;
-        g.inv_s = 1.0f / g.s;
-        g.nx = dims[0];
-        g.ny = dims[1];
-        g.nz = dims[2];
-        double amax = 0.0;  // largest coordinate magnitude in the box
-        for (int k = 0; k < 3; ++k)
-            amax = std::max(amax, std::max(std::fabs(lo[k]), std::fabs(lo[k] + ext[k])));
-        g.margin = (float)(4e-6 * (emax + amax) + 1e-7);
-        const size_t cells = (size_t)dims[0] * dims[1] * dims[2], nmax = std::max(np, nq);
-        // one grid per set; each set's points in cell order are then the
-        // query order of its search in the other set's grid (neighbouring
-        // threads search the same cells)
-        gsl::NNScratch sq{}, sp{};
-        const int sl[2][8] = {{S_GCELL, S_GSTART, S_GCUR, S_GPART, S_GPTS, S_GIDX, S_GLIST, S_GNL},
-                              {S_GCELL2, S_GSTART2, S_GCUR2, S_GPART2, S_GPTS2, S_GIDX2, S_GLIST2, S_GNL2}};
-        gsl::NNScratch *scs[2] = {&sq, &sp};
-        for (int k = 0; k < 2; ++k) {
-            gsl::NNScratch &sc = *scs[k];
-            GS_TRY(wsT(ctx, sl[k][0], nmax, &sc.cell));
-            GS_TRY(wsT(ctx, sl[k][1], cells + 1, &sc.start));
-            GS_TRY(wsT(ctx, sl[k][2], cells, &sc.cursor));
-            GS_TRY(wsT(ctx, sl[k][3], gsl::scan_partials(cells + 1), &sc.partials));
-            GS_TRY(wsT(ctx, sl[k][4], nmax, &sc.spts));
-            GS_TRY(wsT(ctx, sl[k][5], nmax, &sc.sidx));
-            GS_TRY(wsT(ctx, sl[k][6], nmax, &sc.list));
-            GS_TRY(wsT(ctx, sl[k][7], 1, &sc.n_list));
-        }
-        gsl::nn_grid_build(a.q, (int)nq, g, sq, s);
-        gsl::nn_grid_build(a.pt, (int)np, g, sp, s);
-        gsl::nn_grid_search(a.pt, (int)np, sp.sidx, a.q, (int)nq, g, sq, a.nn_pq, a.d2, s);
-        gsl::nn_grid_search(a.q, (int)nq, sq.sidx, a.pt, (int)np, g, sp, a.nn_qp, nullptr, s);
-        gsl::overlap_count(a, s);
+        gsl::overlap(a, s);
     }
-    unsigned long long c[2] = {0, 0};
-    GS_CUDA(cudaMemcpyAsync(c, a.counts, sizeof c, cudaMemcpyDeviceToHost, s));
+    GS_CUDA(cudaGetLastError());
+    gsl::NNHeader h;
+    GS_CUDA(cudaMemcpyAsync(&h, a.hdr, sizeof h, cudaMemcpyDeviceToHost, s));
     GS_CUDA(cudaStreamSynchronize(s));
+    if (grid && !h.ok)
+        return fail(ctx, GS_ERR_NONFINITE, "gs_overlap_ratio: non-finite mean");
+    const unsigned long long *c = h.counts;
     *ratio = c[0] ? (double)c[1] / (double)c[0] : 0.0;
     if (n_corr)
         *n_corr = (int64_t)c[0];

@@ -450,20 +450,6 @@ Rigid make_rigid(const double *T);
 unsigned transform_blocks(int64_t n);
 void transform_batch(const MapDesc *maps, int n_maps, unsigned blocks, cudaStream_t s);
 
-// Overlap ratio of two submaps (loop filter): moved means of P, exact
-// nearest neighbours both ways, reciprocal pairs and those within tau.
-struct OverlapArgs {
-    const float4 *p, *q;      // means [np], [nq]
-    int np, nq;
-    const float *T32;         // [12] device, T_{P->Q} rounded to FP32
-    float4 *pt;               // [np] scratch: T p
-    int32_t *nn_pq, *nn_qp;   // [np], [nq] out
-    float *d2;                // [np] out: squared distance to the nearest of Q
-    float tau2;               // tau * tau (FP32)
-    unsigned long long *counts;  // [2] out: |K|, pairs of K within tau
-};
-void overlap(const OverlapArgs &a, cudaStream_t s);
-
 // Uniform grid for exact nearest-neighbour search: cell of x is
 // floor((x - o) * inv_s) per axis (FP32, clamped to the grid), cells
 // numbered x-fastest.  margin bounds how far a cell boundary computed this
@@ -472,31 +458,37 @@ struct NNGrid {
     float ox, oy, oz, s, inv_s, margin;
     int nx, ny, nz;
 };
-// Scratch of one grid search (targets nt, queries na):
-//   cell [nt], start [cells + 1], cursor [cells], spts [nt], sidx [nt],
-//   list [na], n_list [1]
-struct NNScratch {
-    uint32_t *cell, *start, *cursor, *partials;
-    float4 *spts;
-    int32_t *sidx, *list;
-    uint32_t *n_list;
+// zeroed before each call
+struct NNHeader {
+    unsigned long long counts[2];  // |K|, pairs of K within tau
+    uint32_t box[6];               // of both sets: complemented minima, maxima (ordered integers)
+    uint32_t blocks_done, bad, n_list[2];
+    int ok;                        // the box is finite and the grid chosen
+    NNGrid grid;
 };
-// moved means pt = T p and the bounding box of pt and q as ordered-int
-// min x, y, z, max x, y, z in bbox[6]
-void overlap_moved_bbox(const OverlapArgs &a, uint32_t *bbox, cudaStream_t s);
-// exact nearest neighbour in targets B of every query in A (FP32 squared
-// distance, ties to the smaller index): a grid search that stops once no
-// unsearched cell can hold a nearer target, and the brute-force sweep for
-// the queries whose search would run past kNNMaxRing rings
-// the grid of the targets B: their cells, per-cell starts, and the targets
-// (sidx: their indices) in cell order
-void nn_grid_build(const float4 *B, int nb, const NNGrid &g, const NNScratch &sc, cudaStream_t s);
-// the search of every query of A in the grid of B built into sc; thread t
-// takes query order[t] when order is given (a permutation of 0..na-1)
-void nn_grid_search(const float4 *A, int na, const int32_t *order, const float4 *B, int nb, const NNGrid &g,
-                    const NNScratch &sc, int32_t *nn, float *d2, cudaStream_t s);
-// |K| and the pairs within tau from the nearest neighbours both ways
-void overlap_count(const OverlapArgs &a, cudaStream_t s);
+// Overlap ratio of two submaps (loop filter): moved means of P, exact
+// nearest neighbours both ways (FP32 squared distance, ties to the smaller
+// index), reciprocal pairs and those within tau.
+struct OverlapArgs {
+    const float4 *p, *q;      // means [np], [nq]
+    int np, nq;
+    float T32[12];            // T_{P->Q} rounded to FP32
+    float4 *pt;               // [np] scratch: T p
+    int32_t *nn_pq, *nn_qp;   // [np], [nq] out
+    float *d2;                // [np] out: squared distance to the nearest of Q
+    float tau2;               // tau * tau (FP32)
+    NNHeader *hdr;
+    // scratch of the grid search (overlap_grid)
+    uint32_t max_cells;       // cells a set's grid may have
+    uint32_t *cell;           // [np + nq]
+    uint32_t *count, *start;  // [2 max_cells], [2 max_cells + 1]: P's cells, then Q's
+    uint32_t *sums;           // [overlap_sum_blocks(max_cells)]
+    float4 *spts;             // [np + nq] in cell order, index in w
+    int32_t *list;            // [np + nq] queries left to the brute-force sweep
+};
+size_t overlap_sum_blocks(uint32_t max_cells);
+void overlap_grid(const OverlapArgs &a, cudaStream_t s);  // np, nq > 0
+void overlap(const OverlapArgs &a, cudaStream_t s);       // brute force
 
 constexpr int kCentroidWarps = 32;
 struct PoseArgs {

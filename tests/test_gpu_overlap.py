@@ -111,3 +111,41 @@ def test_overlap_grid_with_far_outliers(gs, ctx):
     y = np.concatenate([rng.uniform(-0.5, 0.5, (2500, 3)), rng.uniform(-80, -40, (10, 3))])
     r, k = check(gs, ctx, pts(x), pts(y), synth.random_rigid(rng, 5.0, 0.05), tau=0.05)
     assert 0.0 < r < 1.0 and k > 100
+
+
+@pytest.mark.parametrize("n,m", [(64, 64), (65, 2049), (1500, 700)])
+@pytest.mark.parametrize("kind", ["plane", "line", "point", "clusters", "far", "huge"])
+def test_overlap_grid_shapes(gs, ctx, n, m, kind):
+    # boxes with one, two or three flat axes, clusters at the box's corners
+    # (rows of cells clipped on every side), a box far from the origin and
+    # extents beyond float's products: the neighbours are the brute force's
+    rng = np.random.default_rng(n + m)
+    x, y = rng.uniform(-2, 2, (n, 3)), rng.uniform(-2, 2, (m, 3))
+    for a in (x, y):
+        if kind in ("plane", "line"):
+            a[:, 2] = 0.5
+        if kind == "line":
+            a[:, 0] = -1.0
+        if kind == "point":
+            a[:] = 0.25
+        if kind == "clusters":
+            a[:] = np.sign(a) * 2.0 + rng.normal(0, 0.01, a.shape)
+        if kind == "far":
+            a += (1000.0, -3000.0, 50.0)
+        if kind == "huge":
+            a *= 1e31
+    to = lambda a: O.Gaussians(np.concatenate([a, np.zeros((len(a), 1))], 1).astype(np.float32), np.zeros((len(a), 4)),
+                               np.tile([1.0, 0, 0, 0], (len(a), 1)), np.zeros(len(a)), np.zeros((len(a), 4)))
+    T = np.eye(3, 4) if kind in ("plane", "line", "point") else synth.random_rigid(rng, 1.0, 0.01)
+    check(gs, ctx, to(x), to(y), T)
+
+
+def test_overlap_non_finite_means_are_refused(gs, ctx):
+    g = gs.Gaussians.from_numpy(synth.gaussians_box(300, np.random.default_rng(3)))
+    for bad in (float("nan"), float("inf"), -float("inf")):
+        h = gs.Gaussians(g.means4.clone(), g.log_scales4, g.quats4, g.logits, g.rgb4)
+        h.means4[17, 1] = bad
+        for p, q in ((g, h), (h, g)):
+            with pytest.raises(gs.GsError, match="NONFINITE"):
+                gs.gs_overlap_ratio(ctx, p, q, np.eye(3, 4))
+    assert gs.gs_overlap_ratio(ctx, g, g, np.eye(3, 4)) == (1.0, 300)
