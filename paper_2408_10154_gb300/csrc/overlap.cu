@@ -413,6 +413,19 @@ __global__ void __launch_bounds__(256) k_nn_grid(const gsl::OverlapArgs o)
             }
         }
     };
+    // A row's targets are at least this far (squared): the gaps between the
+    // query and the row's cells in y and z, less the margin of their
+    // boundaries.  A row beyond the best so far is left out (a tie is not
+    // beyond: it may hold the smaller index).
+    const float fy = a.y - (g.oy + (float)cy * g.s), fz = a.z - (g.oz + (float)cz * g.s);
+    auto gap = [&](int d, float f) {
+        const float x = d > 0 ? (float)d * g.s - f : (d < 0 ? f - (float)(d + 1) * g.s : 0.0f);
+        return fmaxf(x - g.margin, 0.0f);
+    };
+    auto row_dist2 = [&](int dy, int dz) {
+        const float gy = gap(dy, fy), gz = gap(dz, fz);
+        return (gy * gy + gz * gz) * (1.0f - 1e-6f);
+    };
     auto row_of = [&](int y, int z) { return (uint32_t)g.nx * ((uint32_t)y + (uint32_t)g.ny * (uint32_t)z); };
     {
         const int x0 = max(cx - 1, 0), x1 = min(cx + 1, g.nx - 1);
@@ -424,9 +437,14 @@ __global__ void __launch_bounds__(256) k_nn_grid(const gsl::OverlapArgs o)
             j0[k] = in ? start[row_of(y, z) + x0] : 0u;
             j1[k] = in ? start[row_of(y, z) + x1 + 1] : 0u;
         }
+        // the query's own row first, then the others nearest first
+        constexpr int kOrder[9] = {4, 1, 3, 5, 7, 0, 2, 6, 8};
 #pragma unroll
-        for (int k = 0; k < 9; ++k)
-            scan_run(j0[k], j1[k]);
+        for (int q = 0; q < 9; ++q) {
+            const int k = kOrder[q];
+            if (k == 4 || row_dist2(k % 3 - 1, k / 3 - 1) <= best)
+                scan_run(j0[k], j1[k]);
+        }
     }
     for (int r = 1;;) {
         const bool covered = cx - r <= 0 && cx + r >= g.nx - 1 && cy - r <= 0 && cy + r >= g.ny - 1 &&
@@ -444,6 +462,8 @@ __global__ void __launch_bounds__(256) k_nn_grid(const gsl::OverlapArgs o)
         const int x0 = max(cx - r, 0), x1 = min(cx + r, g.nx - 1);
         for (int z = max(cz - r, 0); z <= min(cz + r, g.nz - 1); ++z)
             for (int y = max(cy - r, 0); y <= min(cy + r, g.ny - 1); ++y) {
+                if (row_dist2(y - cy, z - cz) > best)
+                    continue;
                 const uint32_t row = row_of(y, z);
                 if (z == cz - r || z == cz + r || y == cy - r || y == cy + r) {
                     scan_run(start[row + x0], start[row + x1 + 1]);
