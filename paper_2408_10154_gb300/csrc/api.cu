@@ -24,7 +24,7 @@ enum Slot {
     S_VPS, S_GROUPS, S_TILEVP, S_POSE32, S_REC, S_AUX, S_COUNTS, S_PARTIALS, S_NDUPS, S_K0, S_V0, S_RANGES, S_FLAGS, S_TF, S_LAST, S_CODE, S_TLOSS, S_TTWIST, S_POSE64, S_ADAM, S_PIVOT,
     S_CCAM, S_CENT, S_CENTP, S_LOSS, S_SETVP, S_REV, S_PFIRST, S_PCOUNT, S_TOUT, S_CONF, S_EST, S_GRAD, S_DUPG,
     S_PAIRS, S_RSLOT, S_RSLOTN, S_TERR, S_TCOL, S_TW,
-    S_TMED, S_TNV, S_TVPS, S_EXPO, S_EXPO32, S_TEXPO, S_OPT, S_ONN1, S_ONN2, S_OD2, S_OHDR, S_MAPS, S_OS, S_ORDER, S_ORDC, S_SK, S_SV, S_SN, S_GCELL, S_GCOUNT, S_GSTART, S_GSUMS, S_GPTS, S_GLIST, S_SEGZ, S_SEGCUR, S_SEGBIG, S_SEGLIST, S_PROBE, S_QUEUE, S_COUNT
+    S_TMED, S_TNV, S_TVPS, S_EXPO, S_EXPO32, S_TEXPO, S_OPT, S_ONN1, S_ONN2, S_OD2, S_OHDR, S_MAPS, S_OS, S_ORDER, S_ORDC, S_SK, S_SV, S_SN, S_GCELL, S_GCOUNT, S_GSTART, S_GSUMS, S_GPTS, S_GLIST, S_SEGZ, S_SEGCUR, S_SEGLIST, S_PROBE, S_QUEUE, S_COUNT
 };
 
 struct Buf {
@@ -337,7 +337,7 @@ struct Pipe {
     uint64_t n_records = 0;
     // segmented build
     unsigned long long *seg_hdr = nullptr;
-    uint32_t *seg_diff = nullptr, *seg_cursor = nullptr, *seg_big = nullptr;
+    uint32_t *seg_diff = nullptr, *seg_cursor = nullptr;
     uint4 *seg_list = nullptr;
     size_t seg_zero = 0;
 };
@@ -350,7 +350,7 @@ struct Pipe {
 // yield the same lists, which the tests cross-check.
 
 // scratch of the segmented build: cleared header + difference grids,
-// visible-record list, cursors, long-list queue
+// visible-record list, cursors
 gs_status_t alloc_seg(gs_ctx *ctx, const Plan &P, Pipe &p)
 {
     const size_t T = P.n_tiles ? P.n_tiles : 1, R = P.n_records ? P.n_records : 1;
@@ -358,10 +358,9 @@ gs_status_t alloc_seg(gs_ctx *ctx, const Plan &P, Pipe &p)
     uint8_t *z = nullptr;
     GS_TRY(wsT(ctx, S_SEGZ, p.seg_zero, &z));
     p.seg_hdr = (unsigned long long *)z;
-    p.seg_diff = (uint32_t *)(p.seg_hdr + 1 + P.vps.size());
+    p.seg_diff = (uint32_t *)(p.seg_hdr + P.vps.size());
     GS_TRY(wsT(ctx, S_SEGLIST, R, &p.seg_list));
     GS_TRY(wsT(ctx, S_SEGCUR, T, &p.seg_cursor));
-    GS_TRY(wsT(ctx, S_SEGBIG, T, &p.seg_big));
     return GS_OK;
 }
 
@@ -450,11 +449,12 @@ gsl::BinArgs bin_args(const Plan &P, const DevPlan &D, const Pipe &p)
     b.seg_diff = p.seg_diff;
     b.seg_zero_bytes = p.seg_zero;
     b.seg_cursor = p.seg_cursor;
-    b.seg_big = p.seg_big;
     b.seg_list = p.seg_list;
     b.seg_counted = 1;
-    for (const VpDesc &d : P.vps)
+    for (const VpDesc &d : P.vps) {
         b.seg_max_cells = std::max(b.seg_max_cells, (uint32_t)(d.TX * d.TY));
+        b.seg_max_rows = std::max(b.seg_max_rows, (uint32_t)d.TY);
+    }
     return b;
 }
 

@@ -5,8 +5,8 @@
 // difference grids of the records' rectangles give every tile's list length
 // and start without sorting the duplicates; records are placed into their
 // tiles through per-tile atomic cursors and each short list is then sorted
-// on its own (registers, shared memory, or global memory for the rare long
-// list).  One-stage route (gs_render_noalloc): exclusive scan of the
+// on its own (registers, shared memory, or global memory for the rare list
+// of thousands).  One-stage route (gs_render_noalloc): exclusive scan of the
 // tiles-touched counts, emission of 64-bit (tile << 32 | depth bits) keys,
 // stable LSD radix sort, per-tile ranges.  Also the one-sweep LSD radix sort
 // of 32-bit keys (gs_sort_u32) and the longest-first tile schedule.
@@ -587,6 +587,7 @@ __global__ void __launch_bounds__(kSegThreads) k_seg_collect(const gsl::BinArgs 
         atomicAdd(g + q.y1 * w1 + q.x0, 0xffffffffu);
         e = make_uint4(__float_as_uint(a.rec[3 * (size_t)r + 1].z), d.tile_base + q.y0 * (uint32_t)d.TX + q.x0,
                        (q.x1 - q.x0) | ((q.y1 - q.y0) << 16), (uint32_t)d.TX);
+        atomicAdd(a.seg_hdr + vp, (unsigned long long)c);
     }
     a.seg_list[r] = e;
 }
@@ -623,31 +624,127 @@ __device__ __forceinline__ unsigned long long block_incl_scan(unsigned long long
     return r;
 }
 
-// One CTA per keyframe: 2-D prefix sums of its difference grid (rows, then
-// columns) turn it into the tile counts, written back in place, and the
-// keyframe's duplicate total goes to seg_hdr[1 + v].  SMEM: the TY x TX
-// counting cells are summed in shared memory (dynamic, a.seg_max_cells
-// words); otherwise in place in global memory.
+// One CTA per keyframe: 2-D prefix sums of its difference grid give the tile
+// counts, an exclusive scan of them in tile order, offset by the totals of
+// the earlier keyframes (counted with the records), each tile's start.
+// Writes the ranges ((0, 0) when empty; clipped to the capacity), the
+// placement cursors, and (CTA 0) the duplicate total and the capacity flag.
+// Latency-bound: one launch of a few microseconds in place of two (counts,
+// then ranges: 3.3 + 4.0 us on a 160x120 view, 7.4 + 7.4 us on 1200x680, by
+// ncu), columns one thread each, rows one warp each.
+//
+// SMEM: the TY x TX cells are summed in shared memory (dynamic: a.seg_max_cells
+// + 1 words, then a.seg_max_rows 64-bit row offsets); otherwise in place in
+// global memory.
 template <bool SMEM>
-__global__ void __launch_bounds__(kSegTileThreads) k_seg_count(const gsl::BinArgs a)
+__global__ void __launch_bounds__(kSegTileThreads) k_seg_ranges(const gsl::BinArgs a)
 {
-    extern __shared__ uint32_t s_grid[];
+    extern __shared__ unsigned long long s_dyn64[];
     __shared__ unsigned long long s_w[kSegTileThreads / 32];
+    __shared__ unsigned long long s_base;
     const int v = blockIdx.x;
     const VpDesc &d = a.vps[v];
     const int TX = d.TX, TY = d.TY, w1 = TX + 1;
-    uint32_t *g = a.seg_diff + d.diff_base;
     const uint32_t nt = (uint32_t)TX * (uint32_t)TY;
-    uint32_t *c = SMEM ? s_grid : g;
-    const int pitch = SMEM ? TX : w1;
+    uint32_t *g = a.seg_diff + d.diff_base;
+    unsigned long long *s_row = s_dyn64;
+    uint32_t *s_grid = reinterpret_cast<uint32_t *>(s_dyn64 + a.seg_max_rows);
     if (SMEM) {
         for (uint32_t i = threadIdx.x; i < nt; i += blockDim.x)
             s_grid[i] = g[(size_t)(i / (uint32_t)TX) * w1 + i % (uint32_t)TX];
+    }
+    unsigned long long before = 0, all = 0;
+    for (int k = threadIdx.x; k < a.n_vps; k += blockDim.x) {
+        const unsigned long long t = a.seg_hdr[k];
+        before += k < v ? t : 0ull;
+        all += t;
+    }
+    const unsigned long long base_incl = block_incl_scan(before, s_w);
+    const unsigned long long grand = v == 0 ? block_incl_scan(all, s_w) : 0ull;
+    if (threadIdx.x == kSegTileThreads - 1) {
+        s_base = base_incl;
+        if (v == 0) {
+            *a.n_dups = grand < 0xffffffffull ? (uint32_t)grand : 0xffffffffu;
+            if (grand > a.capacity)
+                atomicOr(a.flags, kFlagCapacity);
+        }
+    }
+    __syncthreads();
+    const unsigned long long cap = a.capacity;
+    auto put = [&](uint32_t lt, unsigned long long st, unsigned long long en, bool any) {
+        const uint32_t t = d.tile_base + lt;
+        // (0, 0) for an empty tile
+        a.ranges[t] = any ? make_uint2((uint32_t)(st < cap ? st : cap), (uint32_t)(en < cap ? en : cap))
+                          : make_uint2(0u, 0u);
+        a.seg_cursor[t] = (uint32_t)(st < cap ? st : cap);
+    };
+    if (SMEM) {
+        for (int x = threadIdx.x; x < TX; x += blockDim.x) {
+            uint32_t acc = 0;
+#pragma unroll 8
+            for (int y = 0; y < TY; ++y) {
+                acc += s_grid[y * TX + x];
+                s_grid[y * TX + x] = acc;
+            }
+        }
         __syncthreads();
+        // a row: its counts (inclusive sums along x), then their inclusive
+        // sums, kept where they fit 32 bits (a larger one is past any
+        // capacity, and so clipped)
+        const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+        for (int y = warp; y < TY; y += kSegTileThreads / 32) {
+            uint32_t carry = 0;
+            unsigned long long total = 0;
+            for (int x0 = 0; x0 < TX; x0 += 32) {
+                const int x = x0 + lane;
+                uint32_t c = x < TX ? s_grid[y * TX + x] : 0u;
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const uint32_t u = __shfl_up_sync(0xffffffffu, c, o);
+                    if (lane >= o)
+                        c += u;
+                }
+                c += carry;
+                carry = __shfl_sync(0xffffffffu, c, 31);
+                unsigned long long run = x < TX ? c : 0u;
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const unsigned long long u = __shfl_up_sync(0xffffffffu, run, o);
+                    if (lane >= o)
+                        run += u;
+                }
+                run += total;
+                total = __shfl_sync(0xffffffffu, run, 31);
+                if (x < TX)
+                    s_grid[y * TX + x] = run < 0xffffffffull ? (uint32_t)run : 0xffffffffu;
+            }
+            if (lane == 0)
+                s_row[y] = total;
+        }
+        __syncthreads();
+        // the rows' starts
+        unsigned long long before_rows = s_base;
+        for (int y0 = 0; y0 < TY; y0 += kSegTileThreads) {
+            const int y = y0 + (int)threadIdx.x;
+            const unsigned long long t = y < TY ? s_row[y] : 0ull;
+            const unsigned long long incl = block_incl_scan(t, s_w);
+            if (y < TY)
+                s_row[y] = before_rows + incl - t;
+            if (threadIdx.x == kSegTileThreads - 1)
+                s_base = before_rows + incl;
+            __syncthreads();
+            before_rows = s_base;
+        }
+        for (uint32_t lt = threadIdx.x; lt < nt; lt += blockDim.x) {
+            const uint32_t y = lt / (uint32_t)TX, x = lt % (uint32_t)TX;
+            const uint32_t lo = x ? s_grid[lt - 1] : 0u, hi = s_grid[lt];
+            put(lt, s_row[y] + lo, s_row[y] + hi, hi != lo);
+        }
+        return;
     }
     for (int y = threadIdx.x; y < TY; y += blockDim.x) {
         uint32_t acc = 0;
-        uint32_t *row = c + (size_t)y * pitch;
+        uint32_t *row = g + (size_t)y * w1;
         for (int x = 0; x < TX; ++x) {
             acc += row[x];
             row[x] = acc;
@@ -657,56 +754,12 @@ __global__ void __launch_bounds__(kSegTileThreads) k_seg_count(const gsl::BinArg
     for (int x = threadIdx.x; x < TX; x += blockDim.x) {
         uint32_t acc = 0;
         for (int y = 0; y < TY; ++y) {
-            acc += c[(size_t)y * pitch + x];
-            c[(size_t)y * pitch + x] = acc;
-        }
-    }
-    __syncthreads();
-    unsigned long long sum = 0;
-    for (uint32_t i = threadIdx.x; i < nt; i += blockDim.x) {
-        const uint32_t y = i / (uint32_t)TX, x = i % (uint32_t)TX;
-        const uint32_t n = c[(size_t)y * pitch + x];
-        if (SMEM)
-            g[(size_t)y * w1 + x] = n;
-        sum += n;
-    }
-    const unsigned long long tot = block_incl_scan(sum, s_w);
-    if (threadIdx.x == kSegTileThreads - 1)
-        a.seg_hdr[1 + v] = tot;
-}
-
-// One CTA per keyframe: an exclusive scan of its tile counts in tile order,
-// offset by the totals of the earlier keyframes, gives each tile's start.
-// Writes the ranges ((0, 0) when empty; clipped to the capacity), the
-// placement cursors, and (CTA 0) the duplicate total and the capacity flag.
-__global__ void __launch_bounds__(kSegTileThreads) k_seg_ranges(const gsl::BinArgs a)
-{
-    __shared__ unsigned long long s_w[kSegTileThreads / 32];
-    __shared__ unsigned long long s_base;
-    const int v = blockIdx.x;
-    const VpDesc &d = a.vps[v];
-    const int TX = d.TX, w1 = TX + 1;
-    const uint32_t *g = a.seg_diff + d.diff_base;
-    const unsigned long long *tot = a.seg_hdr + 1;
-    unsigned long long before = 0, all = 0;
-    for (int k = threadIdx.x; k < a.n_vps; k += blockDim.x) {
-        const unsigned long long t = tot[k];
-        before += k < v ? t : 0ull;
-        all += t;
-    }
-    const unsigned long long base = block_incl_scan(before, s_w);
-    const unsigned long long grand = block_incl_scan(all, s_w);
-    if (threadIdx.x == kSegTileThreads - 1) {
-        s_base = base;
-        if (v == 0) {
-            *a.n_dups = grand < 0xffffffffull ? (uint32_t)grand : 0xffffffffu;
-            if (grand > a.capacity)
-                atomicOr(a.flags, kFlagCapacity);
+            acc += g[(size_t)y * w1 + x];
+            g[(size_t)y * w1 + x] = acc;
         }
     }
     __syncthreads();
     // each thread scans a contiguous run of tiles; one block scan joins the runs
-    const uint32_t nt = (uint32_t)TX * (uint32_t)d.TY;
     const uint32_t per = (nt + kSegTileThreads - 1) / kSegTileThreads;
     const uint32_t l0 = min(threadIdx.x * per, nt), l1 = min(l0 + per, nt);
     auto cell = [&](uint32_t lt) { return g[(size_t)(lt / (uint32_t)TX) * w1 + lt % (uint32_t)TX]; };
@@ -714,16 +767,10 @@ __global__ void __launch_bounds__(kSegTileThreads) k_seg_ranges(const gsl::BinAr
     for (uint32_t lt = l0; lt < l1; ++lt)
         run += cell(lt);
     unsigned long long st = s_base + block_incl_scan(run, s_w) - run;
-    const unsigned long long cap = a.capacity;
     for (uint32_t lt = l0; lt < l1; ++lt) {
         const uint32_t n = cell(lt);
-        const unsigned long long en = st + n;
-        const uint32_t t = d.tile_base + lt;
-        // (0, 0) for an empty tile
-        a.ranges[t] = n ? make_uint2((uint32_t)(st < cap ? st : cap), (uint32_t)(en < cap ? en : cap))
-                        : make_uint2(0u, 0u);
-        a.seg_cursor[t] = (uint32_t)(st < cap ? st : cap);
-        st = en;
+        put(lt, st, st + n, n != 0);
+        st += n;
     }
 }
 
@@ -928,77 +975,141 @@ __device__ __forceinline__ void cex(unsigned long long *s, int i, int p)
     }
 }
 
-constexpr int kSegSortWarps = 8;
-constexpr int kSegSortCap = 512;  // longest list sorted by one warp in shared memory
+constexpr int kSegSortWarps = 8, kSegSortThreads = kSegSortWarps * 32;
+constexpr int kSegSortWarpMax = 256;    // longest list sorted by one warp in registers
+constexpr int kSegSortChunk = 4096;     // entries the block sorts in shared memory
 
-// One warp per tile: lists of up to 256 entries are sorted in registers (up
-// to 8 per lane), up to kSegSortCap in shared memory (padded with ~0 to a
-// power of two);
-// longer lists are queued for k_seg_sort_big.  The sorted record indices
-// replace the tile's values in place.
-__global__ void __launch_bounds__(kSegSortWarps * 32) k_seg_sort(const gsl::BinArgs a)
+// Ascending sort of the first n (padded to a power of two N with ~0) keys in
+// shared memory by the block; first: from the size-2 merges on, else only
+// the half-cleaners below `size` (a bitonic sequence per block of `size`).
+__device__ __forceinline__ void block_bitonic(unsigned long long *sk, int N, bool first)
 {
-    __shared__ unsigned long long s_k[kSegSortWarps][kSegSortCap];
+    auto cleaners = [&](int j) {
+        for (; j >= 1; j >>= 1) {
+            for (int q = threadIdx.x; q < (N >> 1); q += kSegSortThreads) {
+                const int i = ((q & ~(j - 1)) << 1) | (q & (j - 1));
+                cex(sk, i, i | j);
+            }
+            __syncthreads();
+        }
+    };
+    if (!first) {
+        cleaners(N >> 1);
+        return;
+    }
+    for (int k = 2; k <= N; k <<= 1) {
+        const int h = k >> 1;
+        for (int q = threadIdx.x; q < (N >> 1); q += kSegSortThreads) {
+            const int i = (q / h) * k + (q & (h - 1));
+            cex(sk, i, i + k - 1 - 2 * (q & (h - 1)));
+        }
+        __syncthreads();
+        cleaners(k >> 2);
+    }
+}
+
+// One list of n > kSegSortWarpMax entries by the block: in shared memory, a
+// chunk at a time; the merges of a list longer than a chunk exchange
+// (key, value) pairs in global memory at distances of a chunk and more.
+__device__ void block_sort_list(uint32_t *keys, uint32_t *vals, uint32_t n, unsigned long long *sk)
+{
+    auto chunk = [&](uint32_t c0, bool first) {
+        const uint32_t cnt = min(n - c0, (uint32_t)kSegSortChunk);
+        int N = 512;
+        while ((uint32_t)N < cnt)
+            N <<= 1;
+        if (!first)
+            N = kSegSortChunk;
+        for (int i = threadIdx.x; i < N; i += kSegSortThreads)
+            sk[i] = (uint32_t)i < cnt ? (((unsigned long long)keys[c0 + i] << 32) | vals[c0 + i]) : ~0ull;
+        __syncthreads();
+        block_bitonic(sk, N, first);
+        for (uint32_t i = threadIdx.x; i < cnt; i += kSegSortThreads) {
+            keys[c0 + i] = (uint32_t)(sk[i] >> 32);
+            vals[c0 + i] = (uint32_t)sk[i];
+        }
+        __syncthreads();
+    };
+    for (uint32_t c0 = 0; c0 < n; c0 += kSegSortChunk)
+        chunk(c0, true);
+    if (n <= (uint32_t)kSegSortChunk)
+        return;
+    auto ce = [&](uint64_t i, uint64_t p) {
+        if (p >= n)
+            return;  // +infinity past the end
+        const unsigned long long u = ((unsigned long long)keys[i] << 32) | vals[i];
+        const unsigned long long w = ((unsigned long long)keys[p] << 32) | vals[p];
+        if (u > w) {
+            keys[i] = (uint32_t)(w >> 32);
+            vals[i] = (uint32_t)w;
+            keys[p] = (uint32_t)(u >> 32);
+            vals[p] = (uint32_t)u;
+        }
+    };
+    uint64_t N = kSegSortChunk;
+    while (N < n)
+        N <<= 1;
+    for (uint64_t k = 2 * kSegSortChunk; k <= N; k <<= 1) {
+        const uint64_t h = k >> 1;
+        for (uint64_t q = threadIdx.x; q < (N >> 1); q += kSegSortThreads) {
+            const uint64_t i = (q / h) * k + (q & (h - 1));
+            ce(i, i + k - 1 - 2 * (q & (h - 1)));
+        }
+        __syncthreads();
+        for (uint64_t j = k >> 2; j >= (uint64_t)kSegSortChunk; j >>= 1) {
+            for (uint64_t q = threadIdx.x; q < (N >> 1); q += kSegSortThreads) {
+                const uint64_t i = ((q & ~(j - 1)) << 1) | (q & (j - 1));
+                ce(i, i | j);
+            }
+            __syncthreads();
+        }
+        for (uint32_t c0 = 0; c0 < n; c0 += kSegSortChunk)
+            chunk(c0, false);
+    }
+}
+
+// One warp per tile sorts lists of up to kSegSortWarpMax entries in registers
+// (up to 8 per lane); the block's longer lists follow, one after another, by
+// the whole block.  (A long list used to be sorted by one warp in shared
+// memory up to 512 entries, and beyond that by a launch of its own in
+// global memory, stage by stage.)  The sorted record indices replace the
+// tile's values in place.
+__global__ void __launch_bounds__(kSegSortThreads) k_seg_sort(const gsl::BinArgs a)
+{
+    __shared__ unsigned long long s_k[kSegSortChunk];
+    __shared__ uint2 s_long[kSegSortWarps];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t t = blockIdx.x * kSegSortWarps + warp;
-    if (t >= a.n_tiles)
-        return;
-    const uint2 rg = a.ranges[t];
+    const uint2 rg = t < a.n_tiles ? a.ranges[t] : make_uint2(0u, 0u);
     const uint32_t n = rg.y - rg.x;
-    if (n <= 1)
-        return;
-    const uint32_t *keys = a.tkeys[0] + rg.x;
+    const bool is_long = n > (uint32_t)kSegSortWarpMax;
+    uint32_t *keys = a.tkeys[0] + rg.x;
     uint32_t *vals = a.vals[0] + rg.x;
-    if (n <= 32) {
+    if (lane == 0)
+        s_long[warp] = is_long ? rg : make_uint2(0u, 0u);
+    if (n <= 1 || is_long) {
+        // (nothing for the warp)
+    } else if (n <= 32) {
         unsigned long long x = ~0ull;
         if ((uint32_t)lane < n)
             x = ((unsigned long long)keys[lane] << 32) | vals[lane];
         x = warp_bitonic32(x, lane);
         if ((uint32_t)lane < n)
             vals[lane] = (uint32_t)x;
-        return;
-    }
-    if (n <= 64) {
+    } else if (n <= 64) {
         sort_list_reg<2>(keys, vals, n, lane);
-        return;
-    }
-    if (n <= 128) {
+    } else if (n <= 128) {
         sort_list_reg<4>(keys, vals, n, lane);
-        return;
-    }
-    if (n <= 256) {
+    } else {
         sort_list_reg<8>(keys, vals, n, lane);
+    }
+    if (!__syncthreads_or(is_long))
         return;
+    for (int w = 0; w < kSegSortWarps; ++w) {
+        const uint2 q = s_long[w];
+        if (q.y > q.x)
+            block_sort_list(a.tkeys[0] + q.x, a.vals[0] + q.x, q.y - q.x, s_k);
     }
-    if (n > (uint32_t)kSegSortCap) {
-        if (lane == 0)
-            a.seg_big[atomicAdd(a.seg_hdr, 1ull)] = t;
-        return;
-    }
-    int N = 512;
-    while ((uint32_t)N < n)
-        N <<= 1;
-    unsigned long long *sk = s_k[warp];
-    for (int i = lane; i < N; i += 32)
-        sk[i] = (uint32_t)i < n ? (((unsigned long long)keys[i] << 32) | vals[i]) : ~0ull;
-    __syncwarp();
-    for (int k = 2; k <= N; k <<= 1) {
-        const int h = k >> 1;
-        for (int q = lane; q < (N >> 1); q += 32) {
-            const int i = (q / h) * k + (q & (h - 1));
-            cex(sk, i, i + k - 1 - 2 * (q & (h - 1)));
-        }
-        __syncwarp();
-        for (int j = k >> 2; j >= 1; j >>= 1) {
-            for (int q = lane; q < (N >> 1); q += 32) {
-                const int i = ((q & ~(j - 1)) << 1) | (q & (j - 1));
-                cex(sk, i, i | j);
-            }
-            __syncwarp();
-        }
-    }
-    for (int i = lane; (uint32_t)i < n; i += 32)
-        vals[i] = (uint32_t)sk[i];
 }
 
 // 64-bit (tile << 32 | depth bits) keys of the segmented lists, one warp per tile (for gs_bin)
@@ -1010,52 +1121,6 @@ __global__ void __launch_bounds__(256) k_seg_keys64(const gsl::BinArgs a, uint64
     const uint2 rg = a.ranges[t];
     for (uint32_t i = rg.x + (threadIdx.x & 31); i < rg.y; i += 32)
         keys[i] = ((uint64_t)t << 32) | __float_as_uint(a.rec[3 * (size_t)a.vals[0][i] + 1].z);
-}
-
-// Lists longer than kSegSortCap (none on typical views; a splat-dense tile
-// close to the camera): one CTA per queued tile, the same network over the
-// list in global memory, (key, value) pairs exchanged in place, then the
-// values kept.  Slow per element but only ever reached by a few tiles.
-__global__ void __launch_bounds__(1024) k_seg_sort_big(const gsl::BinArgs a)
-{
-    const unsigned long long nb = a.seg_hdr[0];
-    for (unsigned long long b = blockIdx.x; b < nb; b += gridDim.x) {
-        const uint2 rg = a.ranges[a.seg_big[b]];
-        const uint32_t n = rg.y - rg.x;
-        uint32_t *keys = a.tkeys[0] + rg.x;
-        uint32_t *vals = a.vals[0] + rg.x;
-        uint64_t N = 1;
-        while (N < n)
-            N <<= 1;
-        auto ce = [&](uint64_t i, uint64_t p) {
-            if (p >= n)
-                return;  // +infinity past the end
-            const unsigned long long u = ((unsigned long long)keys[i] << 32) | vals[i];
-            const unsigned long long v = ((unsigned long long)keys[p] << 32) | vals[p];
-            if (u > v) {
-                keys[i] = (uint32_t)(v >> 32);
-                vals[i] = (uint32_t)v;
-                keys[p] = (uint32_t)(u >> 32);
-                vals[p] = (uint32_t)u;
-            }
-        };
-        for (uint64_t k = 2; k <= N; k <<= 1) {
-            const uint64_t h = k >> 1;
-            for (uint64_t q = threadIdx.x; q < (N >> 1); q += blockDim.x) {
-                const uint64_t i = (q / h) * k + (q & (h - 1));
-                ce(i, i + k - 1 - 2 * (q & (h - 1)));
-            }
-            __syncthreads();
-            for (uint64_t j = k >> 2; j >= 1; j >>= 1) {
-                for (uint64_t q = threadIdx.x; q < (N >> 1); q += blockDim.x) {
-                    const uint64_t i = ((q & ~(j - 1)) << 1) | (q & (j - 1));
-                    ce(i, i | j);
-                }
-                __syncthreads();
-            }
-        }
-        __syncthreads();
-    }
 }
 
 }  // namespace
@@ -1135,7 +1200,7 @@ int onesweep_u32(uint32_t *keys[2], uint32_t *vals[2], const uint32_t *n_dev, ui
 
 size_t seg_zero_bytes(int n_vps, uint64_t n_diff)
 {
-    return sizeof(unsigned long long) * (1 + (size_t)n_vps) + sizeof(uint32_t) * (size_t)n_diff;
+    return sizeof(unsigned long long) * (size_t)n_vps + sizeof(uint32_t) * (size_t)n_diff;
 }
 
 int bin_seg(const BinArgs &a, cudaStream_t s)
@@ -1150,20 +1215,19 @@ int bin_seg(const BinArgs &a, cudaStream_t s)
         k_seg_collect<<<div_up(a.n_records, kSegThreads), kSegThreads, 0, s>>>(a);
         ++g_launches;
     }
-    if (a.seg_max_cells * sizeof(uint32_t) <= 40 * 1024)
-        k_seg_count<true><<<a.n_vps, kSegTileThreads, a.seg_max_cells * sizeof(uint32_t), s>>>(a);
+    const size_t smem = sizeof(unsigned long long) * a.seg_max_rows + sizeof(uint32_t) * a.seg_max_cells;
+    if (smem <= 40 * 1024)
+        k_seg_ranges<true><<<a.n_vps, kSegTileThreads, smem, s>>>(a);
     else
-        k_seg_count<false><<<a.n_vps, kSegTileThreads, 0, s>>>(a);
-    k_seg_ranges<<<a.n_vps, kSegTileThreads, 0, s>>>(a);
-    g_launches += 2;
+        k_seg_ranges<false><<<a.n_vps, kSegTileThreads, 0, s>>>(a);
+    ++g_launches;
     if (a.n_records) {
         k_seg_place<<<div_up(a.n_records, kSegThreads * kSegPerThread), kSegThreads, 0, s>>>(a);
         ++g_launches;
     }
     if (a.n_tiles) {
-        k_seg_sort<<<div_up(a.n_tiles, kSegSortWarps), kSegSortWarps * 32, 0, s>>>(a);
-        k_seg_sort_big<<<152, 1024, 0, s>>>(a);
-        g_launches += 2;
+        k_seg_sort<<<div_up(a.n_tiles, kSegSortWarps), kSegSortThreads, 0, s>>>(a);
+        ++g_launches;
     }
     return 0;
 }

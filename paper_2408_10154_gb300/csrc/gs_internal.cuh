@@ -309,13 +309,12 @@ struct BinArgs {
     uint32_t n_tiles;
     int *flags;
     uint32_t *tkeys[2];             // [capacity] segmented build: depth bits of the placed entries (tkeys[0])
-    // segmented build (bin_seg): seg_hdr[0] counts the tiles queued for the
-    // long-list sort, seg_hdr[1 + v] holds keyframe v's duplicate total, and
-    // the difference grids (VpDesc::diff_base) follow in the same allocation
-    // of seg_zero_bytes, cleared at the start of every build.  seg_list: per
-    // record {depth bits, first tile, width | height << 16, tiles per row}
-    // (size 0: not visible).  seg_counted: the projection has already
-    // cleared, counted and written the entries (ProjectArgs::seg_*);
+    // segmented build (bin_seg): seg_hdr[v] holds keyframe v's duplicate
+    // total, and the difference grids (VpDesc::diff_base) follow in the same
+    // allocation of seg_zero_bytes, cleared at the start of every build.
+    // seg_list: per record {depth bits, first tile, width | height << 16,
+    // tiles per row} (size 0: not visible).  seg_counted: the projection has
+    // already cleared, counted and written the entries (ProjectArgs::seg_*);
     // otherwise bin_seg does it from rec / counts.
     unsigned long long *seg_hdr;
     uint32_t *seg_diff;
@@ -323,8 +322,8 @@ struct BinArgs {
     uint4 *seg_list;     // [n_records]
     int seg_counted;
     uint32_t *seg_cursor;  // [n_tiles] placement cursors
-    uint32_t *seg_big;     // [n_tiles] tiles whose lists exceed the warp sort
     uint32_t seg_max_cells;  // largest TX * TY over the keyframes
+    uint32_t seg_max_rows;   // largest TY
 };
 // emits, sorts and ranges; returns which buffer holds the sorted result
 int bin(const BinArgs &a, cudaStream_t s);

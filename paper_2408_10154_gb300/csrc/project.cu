@@ -70,7 +70,9 @@ __device__ __forceinline__ void tighten(float ca, float cb, float cc, float o, f
 // (y1, x1) and -1 (mod 2^32) at (y0, x1) and (y1, x0) of its keyframe's
 // (TY + 1) x (TX + 1) difference grid, whose 2-D prefix sum is the tile
 // count; every record writes its entry {depth bits, first tile, width |
-// height << 16, tiles per row} (size 0 when not visible).
+// height << 16, tiles per row} (size 0 when not visible).  The keyframe's
+// duplicate total is counted beside it (one atomic per block and keyframe),
+// so that the list ranges of all keyframes are found in one launch.
 __device__ __forceinline__ void seg_note(const gsl::ProjectArgs &a, const int *geo, uint32_t rec, float z, int count,
                                          int x0, int x1, int y0, int y1)
 {
@@ -92,10 +94,11 @@ __device__ __forceinline__ void seg_note(const gsl::ProjectArgs &a, const int *g
 
 // One (keyframe, Gaussian) pair: camera-space mean, covariance, the
 // dilated 2D covariance, conic, radius, pixel mean and tile rectangle (all
-// the contract's FP32 sequence), the record and its list entry.
-__device__ __forceinline__ void project_pair(const gsl::ProjectArgs &a, const float *M, const float *cam,
-                                             const int *geo, uint32_t i, const float4 &mu, const float (&Rq)[3][3],
-                                             const float (&sig)[3], float opa, const float4 &col, bool qok)
+// the contract's FP32 sequence), the record and its list entry.  Returns the
+// tiles touched.
+__device__ __forceinline__ int project_pair(const gsl::ProjectArgs &a, const float *M, const float *cam,
+                                            const int *geo, uint32_t i, const float4 &mu, const float (&Rq)[3][3],
+                                            const float (&sig)[3], float opa, const float4 &col, bool qok)
 {
     const uint32_t rec = (uint32_t)geo[2] + i;
     const float x = fma_rn(M[2], mu.z, fma_rn(M[1], mu.y, fma_rn(M[0], mu.x, M[3])));
@@ -180,6 +183,7 @@ __device__ __forceinline__ void project_pair(const gsl::ProjectArgs &a, const fl
         a.counts[rec] = count;
     if (a.seg_hdr)
         seg_note(a, geo, rec, z, count, x0, x1, y0, y1);
+    return count;
 }
 
 // keyframes per compaction round of a warp (its queue holds 32 per keyframe)
@@ -210,6 +214,7 @@ __global__ void __launch_bounds__(256) k_project(const gsl::ProjectArgs a)
     constexpr int kF = 21;
     __shared__ float sG[8][kF][32];
     __shared__ uint16_t sQ[8][kProjRound * 32];
+    __shared__ uint32_t sTot[kMaxVpPerGroup];  // the block's duplicates per keyframe
     for (int v = threadIdx.x; v < G.vp_count; v += blockDim.x) {
         const int vp = G.vp_first + v;
         const VpDesc &d = a.vps[vp];
@@ -232,13 +237,12 @@ __global__ void __launch_bounds__(256) k_project(const gsl::ProjectArgs a)
         sGeo[v][2] = (int)d.rec_base;
         sGeo[v][3] = (int)d.tile_base;
         sGeo[v][4] = (int)d.diff_base;
+        sTot[v] = 0;
     }
     __syncthreads();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int i = (int)(blockIdx.x - G.blk_base) * blockDim.x + threadIdx.x;
     const int i_warp = i - lane;  // the warp's first Gaussian
-    if (i_warp >= G.n)
-        return;  // the whole warp is past the group (warp-uniform)
     const bool mine = i < G.n;
     float4 mu = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
     bool qok = false;
@@ -320,12 +324,20 @@ __global__ void __launch_bounds__(256) k_project(const gsl::ProjectArgs a)
                                         {g[9 * 32], g[10 * 32], g[11 * 32]}};
                 const float sig[3] = {g[12 * 32], g[13 * 32], g[14 * 32]};
                 const float4 c4 = make_float4(g[16 * 32], g[17 * 32], g[18 * 32], 0.0f);
-                project_pair(a, sM[v], sCam[v], sGeo[v], (uint32_t)(i_warp + src), m4, Rq, sig, g[15 * 32], c4,
-                             g[19 * 32] != 0.0f);
+                const int count = project_pair(a, sM[v], sCam[v], sGeo[v], (uint32_t)(i_warp + src), m4, Rq, sig,
+                                               g[15 * 32], c4, g[19 * 32] != 0.0f);
+                if (a.seg_hdr && count)
+                    atomicAdd(&sTot[v], (uint32_t)count);
             }
         }
         __syncwarp();
     }
+    if (!a.seg_hdr)
+        return;
+    __syncthreads();
+    for (int v = threadIdx.x; v < G.vp_count; v += blockDim.x)
+        if (sTot[v])
+            atomicAdd(a.seg_hdr + G.vp_first + v, (unsigned long long)sTot[v]);
 }
 
 }  // namespace
