@@ -1921,7 +1921,9 @@ gs_status_t run_registration(gs_ctx *ctx, Plan &P, int n_problems, const gs_opti
         };
         auto iteration = [&](cudaStream_t st) {
             mark(0, st);
-            gsl::project(project_args(P, D, p, pose32, opt, false), st);
+            gsl::ProjectArgs pj = project_args(P, D, p, pose32, opt, false);
+            pj.seg_zero_bytes = 0;  // cleared below, and by every build
+            gsl::project(pj, st);
             mark(1, st);
             const int c = run_bin(b, st);
             if (ordered)
@@ -1968,6 +1970,7 @@ gs_status_t run_registration(gs_ctx *ctx, Plan &P, int n_problems, const gs_opti
         // queue over every keyframe problem) -- timed on trial iterations
         // 1 2 3 4 4 3 2 1 from the initial poses, then the poses start over.
         // Every schedule gives the same results.
+        GS_CUDA(cudaMemsetAsync(p.seg_hdr, 0, p.seg_zero, s));
         int sched = opt->tile_schedule;
         if (sched == 0) {
             const auto it = ctx->schedule.find(key);
@@ -2631,8 +2634,11 @@ gs_status_t srv_replan(gs_server *srv, cudaStream_t s)
     r.exposure = any_exposure(P);
     gsl::TrackArgs ta;
     GS_TRY(alloc_track(ctx, P, D, r, ta, srv->tloss, s));
+    GS_CUDA(cudaMemsetAsync(p.seg_hdr, 0, p.seg_zero, s));
+    gsl::ProjectArgs pj = project_args(P, D, p, srv->pose32, &srv->opt, false);
+    pj.seg_zero_bytes = 0;  // cleared above, and by every build
     GS_CUDA(cudaStreamBeginCapture(ctx->cap, cudaStreamCaptureModeThreadLocal));
-    gsl::project(project_args(P, D, p, srv->pose32, &srv->opt, false), ctx->cap);
+    gsl::project(pj, ctx->cap);
     r.vals = p.vals[run_bin(b, ctx->cap)];
     if (srv->opt.fuse_compositing && ta.n_track == 0) {
         gsl::forward_backward(r, ctx->cap);

@@ -628,8 +628,9 @@ __device__ __forceinline__ unsigned long long block_incl_scan(unsigned long long
 // counts, an exclusive scan of them in tile order, offset by the totals of
 // the earlier keyframes (counted with the records), each tile's start.
 // Writes the ranges ((0, 0) when empty; clipped to the capacity), the
-// placement cursors, and (CTA 0) the duplicate total and the capacity flag.
-// Latency-bound: one launch of a few microseconds in place of two (counts,
+// placement cursors, and (CTA 0) the duplicate total and the capacity flag,
+// and leaves the grid clear for the next build (the totals, which every CTA
+// reads, are cleared by the placement).  Latency-bound: one launch of a few microseconds in place of two (counts,
 // then ranges: 3.3 + 4.0 us on a 160x120 view, 7.4 + 7.4 us on 1200x680, by
 // ncu), columns one thread each, rows one warp each.
 //
@@ -647,11 +648,18 @@ __global__ void __launch_bounds__(kSegTileThreads) k_seg_ranges(const gsl::BinAr
     const int TX = d.TX, TY = d.TY, w1 = TX + 1;
     const uint32_t nt = (uint32_t)TX * (uint32_t)TY;
     uint32_t *g = a.seg_diff + d.diff_base;
+    pdl_wait();
     unsigned long long *s_row = s_dyn64;
     uint32_t *s_grid = reinterpret_cast<uint32_t *>(s_dyn64 + a.seg_max_rows);
     if (SMEM) {
-        for (uint32_t i = threadIdx.x; i < nt; i += blockDim.x)
-            s_grid[i] = g[(size_t)(i / (uint32_t)TX) * w1 + i % (uint32_t)TX];
+        // every cell is cleared for the next build as it is read
+        for (uint32_t i = threadIdx.x; i < nt + TX + TY + 1; i += blockDim.x) {
+            const uint32_t y = i / (uint32_t)w1, x = i % (uint32_t)w1;
+            const uint32_t c = g[i];
+            g[i] = 0;
+            if (x < (uint32_t)TX && y < (uint32_t)TY)
+                s_grid[y * TX + x] = c;
+        }
     }
     unsigned long long before = 0, all = 0;
     for (int k = threadIdx.x; k < a.n_vps; k += blockDim.x) {
@@ -772,6 +780,9 @@ __global__ void __launch_bounds__(kSegTileThreads) k_seg_ranges(const gsl::BinAr
         put(lt, st, st + n, n != 0);
         st += n;
     }
+    __syncthreads();
+    for (uint32_t i = threadIdx.x; i < nt + TX + TY + 1; i += blockDim.x)
+        g[i] = 0;  // for the next build
 }
 
 constexpr uint32_t kSegSmall = 4;  // tiles of a record placed by its own thread; more: by the whole warp
@@ -792,6 +803,10 @@ constexpr int kSegRounds = 8;       // a large record: rounds of 32 tiles whose 
 __global__ void __launch_bounds__(kSegThreads) k_seg_place(const gsl::BinArgs a)
 {
     const int lane = threadIdx.x & 31;
+    pdl_wait();
+    if (blockIdx.x == 0)
+        for (int v = threadIdx.x; v < a.n_vps; v += kSegThreads)
+            a.seg_hdr[v] = 0;
     uint32_t cnt[kSegPerThread], t0[kSegPerThread], w[kSegPerThread], tx[kSegPerThread], zb[kSegPerThread],
         rr[kSegPerThread];
 #pragma unroll
@@ -1080,6 +1095,7 @@ __global__ void __launch_bounds__(kSegSortThreads) k_seg_sort(const gsl::BinArgs
     __shared__ uint2 s_long[kSegSortWarps];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t t = blockIdx.x * kSegSortWarps + warp;
+    pdl_wait();
     const uint2 rg = t < a.n_tiles ? a.ranges[t] : make_uint2(0u, 0u);
     const uint32_t n = rg.y - rg.x;
     const bool is_long = n > (uint32_t)kSegSortWarpMax;
@@ -1217,18 +1233,13 @@ int bin_seg(const BinArgs &a, cudaStream_t s)
     }
     const size_t smem = sizeof(unsigned long long) * a.seg_max_rows + sizeof(uint32_t) * a.seg_max_cells;
     if (smem <= 40 * 1024)
-        k_seg_ranges<true><<<a.n_vps, kSegTileThreads, smem, s>>>(a);
+        launch_pdl(k_seg_ranges<true>, a.n_vps, kSegTileThreads, smem, s, a);
     else
-        k_seg_ranges<false><<<a.n_vps, kSegTileThreads, 0, s>>>(a);
-    ++g_launches;
-    if (a.n_records) {
-        k_seg_place<<<div_up(a.n_records, kSegThreads * kSegPerThread), kSegThreads, 0, s>>>(a);
-        ++g_launches;
-    }
-    if (a.n_tiles) {
-        k_seg_sort<<<div_up(a.n_tiles, kSegSortWarps), kSegSortThreads, 0, s>>>(a);
-        ++g_launches;
-    }
+        launch_pdl(k_seg_ranges<false>, a.n_vps, kSegTileThreads, 0, s, a);
+    if (a.n_records)
+        launch_pdl(k_seg_place, div_up(a.n_records, kSegThreads * kSegPerThread), kSegThreads, 0, s, a);
+    if (a.n_tiles)
+        launch_pdl(k_seg_sort, div_up(a.n_tiles, kSegSortWarps), kSegSortThreads, 0, s, a);
     return 0;
 }
 

@@ -188,6 +188,17 @@ __device__ __forceinline__ void compose_ct(const float *V, const float *T, float
 }
 
 // ------------------------------------------------------------------------
+// Programmatic dependent launch.  The kernels of an iteration are launched
+// so that each may start as its predecessor's last blocks end, before the
+// predecessor has completed (launch_pdl); pdl_wait() holds it until every
+// kernel before it has completed and its stores are visible (a no-op in an
+// ordinary launch).  Ahead of it a kernel touches only its inputs and what
+// the iteration's kernels before its predecessor wrote: every kernel waits
+// before it ends, so those have completed.
+// ------------------------------------------------------------------------
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+// ------------------------------------------------------------------------
 // small utilities
 // ------------------------------------------------------------------------
 __device__ __forceinline__ unsigned lanemask_lt()
@@ -253,6 +264,30 @@ namespace gsl {
 // site adds one
 extern long long g_launches;
 
+// Launches k (which calls gsk::pdl_wait) so that it may start before its
+// predecessor on the stream has completed: between two small kernels that
+// hides most of the launch.  50 iterations of a four-view, 160x120 edge (six
+// kernels each): 3.58 -> 3.50 ms; 40 of a tracking frame (ten kernels):
+// 7.01 -> 6.83 ms.  (Letting the successor in earlier, as soon as every
+// block has started, measured 3.50 and 7.19 ms: its blocks then wait in the
+// slots that the running kernel's neighbours could use.)
+template <typename... P, typename... A>
+inline void launch_pdl(void (*k)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A... args)
+{
+    cudaLaunchConfig_t c{};
+    c.gridDim = grid;
+    c.blockDim = block;
+    c.dynamicSmemBytes = smem;
+    c.stream = s;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    c.attrs = &at;
+    c.numAttrs = 1;
+    cudaLaunchKernelEx(&c, k, P(args)...);
+    ++g_launches;
+}
+
 struct ProjectArgs {
     const gsk::VpDesc *vps;
     const gsk::GroupDesc *groups;
@@ -276,7 +311,7 @@ struct ProjectArgs {
     int tight;
     float alpha_min;          // the threshold of the tight rectangles
     // segmented tile lists (null: not built here): clears seg_hdr/seg_diff
-    // (seg_zero_bytes), then every visible record adds its rectangle to its
+    // (seg_zero_bytes, unless 0: a build before left them clear), then every visible record adds its rectangle to its
     // keyframe's difference grid, and every record writes its seg_list
     // entry (see BinArgs)
     unsigned long long *seg_hdr;
@@ -311,7 +346,8 @@ struct BinArgs {
     uint32_t *tkeys[2];             // [capacity] segmented build: depth bits of the placed entries (tkeys[0])
     // segmented build (bin_seg): seg_hdr[v] holds keyframe v's duplicate
     // total, and the difference grids (VpDesc::diff_base) follow in the same
-    // allocation of seg_zero_bytes, cleared at the start of every build.
+    // allocation of seg_zero_bytes, cleared before the first build and left
+    // clear by every build.
     // seg_list: per record {depth bits, first tile, width | height << 16,
     // tiles per row} (size 0: not visible).  seg_counted: the projection has
     // already cleared, counted and written the entries (ProjectArgs::seg_*);

@@ -278,6 +278,7 @@ __global__ void __launch_bounds__(kPoseThreads) k_pose_update(const gsl::PoseArg
         if (expo && warp == kPoseWarps - 5 && lane == 0)
             s_pre[4] = 1.0 - pow((double)a.beta2, a.expo[7 * vp + 6] + 1.0);
     }
+    pdl_wait();  // (what is above reads only the state of the update before)
     // (hi, lo) FP32 pairs summed by TwoSum in a fixed order (per thread,
     // then butterflies, then the warps); one FP64 value per component.  A
     // warp without tiles holds zeros, which leave a TwoSum as it is.
@@ -890,10 +891,8 @@ void pose_init(const PoseArgs &a, cudaStream_t s)
 
 void pose_update(const PoseArgs &a, cudaStream_t s)
 {
-    if (a.n_vps > 0) {
-        k_pose_update<<<a.n_vps, kPoseThreads, 0, s>>>(a);
-        ++g_launches;
-    }
+    if (a.n_vps > 0)
+        launch_pdl(k_pose_update, a.n_vps, kPoseThreads, 0, s, a);
 }
 
 void pose_step_raw(int n, double *pose, double *state, const double *grad, const double *pivot, int k, int iters,

@@ -215,6 +215,22 @@ __global__ void __launch_bounds__(256) k_project(const gsl::ProjectArgs a)
     __shared__ float sG[8][kF][32];
     __shared__ uint16_t sQ[8][kProjRound * 32];
     __shared__ uint32_t sTot[kMaxVpPerGroup];  // the block's duplicates per keyframe
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int i = (int)(blockIdx.x - G.blk_base) * blockDim.x + threadIdx.x;
+    const int i_warp = i - lane;  // the warp's first Gaussian
+    const bool mine = i < G.n;
+    // the Gaussian (an input: loaded ahead of the kernels before)
+    float4 mu = make_float4(0.0f, 0.0f, 0.0f, 0.0f), sc = mu, q = mu, col = mu;
+    float logit = 0.0f;
+    if (mine) {
+        const VpDesc &d0 = a.vps[G.vp_first];
+        mu = __ldg(d0.means + i);
+        sc = __ldg(d0.scales + i);
+        q = __ldg(d0.quats + i);
+        logit = __ldg(d0.logits + i);
+        col = __ldg(d0.rgb + i);
+    }
+    pdl_wait();
     for (int v = threadIdx.x; v < G.vp_count; v += blockDim.x) {
         const int vp = G.vp_first + v;
         const VpDesc &d = a.vps[vp];
@@ -240,19 +256,8 @@ __global__ void __launch_bounds__(256) k_project(const gsl::ProjectArgs a)
         sTot[v] = 0;
     }
     __syncthreads();
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int i = (int)(blockIdx.x - G.blk_base) * blockDim.x + threadIdx.x;
-    const int i_warp = i - lane;  // the warp's first Gaussian
-    const bool mine = i < G.n;
-    float4 mu = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
     bool qok = false;
     if (mine) {
-        const VpDesc &d0 = a.vps[G.vp_first];
-        mu = __ldg(d0.means + i);
-        const float4 sc = __ldg(d0.scales + i);
-        const float4 q = __ldg(d0.quats + i);
-        const float logit = __ldg(d0.logits + i);
-        const float4 col = __ldg(d0.rgb + i);
         const bool finite = isfinite(mu.x) && isfinite(mu.y) && isfinite(mu.z) && isfinite(sc.x) &&
                             isfinite(sc.y) && isfinite(sc.z) && isfinite(q.x) && isfinite(q.y) && isfinite(q.z) &&
                             isfinite(q.w) && isfinite(logit);
@@ -346,12 +351,11 @@ namespace gsl {
 
 void project(const ProjectArgs &a, cudaStream_t s)
 {
-    if (a.seg_hdr)
+    if (a.seg_hdr && a.seg_zero_bytes)
         cudaMemsetAsync(a.seg_hdr, 0, a.seg_zero_bytes, s);
     if (a.n_blocks == 0)
         return;
-    k_project<<<a.n_blocks, 256, 0, s>>>(a);
-    ++g_launches;
+    launch_pdl(k_project, a.n_blocks, 256, 0, s, a);
 }
 
 }  // namespace gsl

@@ -566,6 +566,7 @@ __device__ __forceinline__ void fwd_tile(const gsl::RasterArgs &a, const uint32_
 template <bool REG, int X>
 __global__ void __launch_bounds__(kFwdThreads, 8) k_forward(const gsl::RasterArgs a)
 {
+    pdl_wait();
     fwd_tile<REG, X>(a, a.tile_order ? a.tile_order[blockIdx.x] : blockIdx.x);
 }
 
@@ -601,6 +602,7 @@ __device__ __forceinline__ void run_queue(const gsl::RasterArgs &a, Tile &&tile)
 template <int X>
 __global__ void __launch_bounds__(kFwdThreads, 8) k_forward_q(const gsl::RasterArgs a)
 {
+    pdl_wait();
     run_queue(a, [&](uint32_t t) { fwd_tile<true, X>(a, t); });
 }
 
@@ -1134,6 +1136,7 @@ __device__ __forceinline__ void bwd_tile(const gsl::RasterArgs &a, const uint32_
 template <bool REG, bool FULL>
 __global__ void __launch_bounds__(kBwd2Threads, kBwd2MinBlocks) k_backward2(const gsl::RasterArgs a)
 {
+    pdl_wait();
     bwd_tile<REG, FULL>(a, a.tile_order ? a.tile_order[blockIdx.x] : blockIdx.x);
 }
 
@@ -1141,6 +1144,7 @@ __global__ void __launch_bounds__(kBwd2Threads, kBwd2MinBlocks) k_backward2(cons
 template <bool REG, bool FULL>
 __global__ void __launch_bounds__(kBwd2Threads, kBwd2MinBlocks) k_backward2_q(const gsl::RasterArgs a)
 {
+    pdl_wait();
     run_queue(a, [&](uint32_t t) { bwd_tile<REG, FULL>(a, t); });
 }
 
@@ -1295,12 +1299,14 @@ __device__ __forceinline__ void fused_adjoint(const gsl::RasterArgs &a, uint32_t
 template <int X>
 __global__ void __launch_bounds__(kFwdThreads, 8) k_fwdbwd(const gsl::RasterArgs a)
 {
+    pdl_wait();
     fwd_tile<true, X, true>(a, a.tile_order ? a.tile_order[blockIdx.x] : blockIdx.x);
 }
 
 template <int X>
 __global__ void __launch_bounds__(kFwdThreads, 8) k_fwdbwd_q(const gsl::RasterArgs a)
 {
+    pdl_wait();
     run_queue(a, [&](uint32_t t) { fwd_tile<true, X, true>(a, t); });
 }
 
@@ -1322,14 +1328,12 @@ void launch_backward(const gsl::RasterArgs &a, cudaStream_t s)
     if constexpr (REG && !FULL) {
         if (a.queue && g_bwd_q_ctas > 0) {
             cudaMemsetAsync(a.queue, 0, sizeof(uint32_t), s);
-            k_backward2_q<REG, FULL><<<(unsigned)std::min<uint32_t>(a.n_tiles, g_bwd_q_ctas), kBwd2Threads,
-                                       bwd2_smem<REG, FULL>(), s>>>(a);
-            ++gsl::g_launches;
+            gsl::launch_pdl(k_backward2_q<REG, FULL>, (unsigned)std::min<uint32_t>(a.n_tiles, g_bwd_q_ctas),
+                            kBwd2Threads, bwd2_smem<REG, FULL>(), s, a);
             return;
         }
     }
-    k_backward2<REG, FULL><<<a.n_tiles, kBwd2Threads, bwd2_smem<REG, FULL>(), s>>>(a);
-    ++gsl::g_launches;
+    gsl::launch_pdl(k_backward2<REG, FULL>, a.n_tiles, kBwd2Threads, bwd2_smem<REG, FULL>(), s, a);
 }
 
 template <int X>
@@ -1338,9 +1342,9 @@ void launch_fwdbwd(const gsl::RasterArgs &a, cudaStream_t s)
     constexpr size_t smem = bwd2_smem<true, false>();
     if (a.queue && g_fb_q_ctas > 0) {
         cudaMemsetAsync(a.queue, 0, sizeof(uint32_t), s);
-        k_fwdbwd_q<X><<<(unsigned)std::min<uint32_t>(a.n_tiles, g_fb_q_ctas), kFwdThreads, smem, s>>>(a);
+        gsl::launch_pdl(k_fwdbwd_q<X>, (unsigned)std::min<uint32_t>(a.n_tiles, g_fb_q_ctas), kFwdThreads, smem, s, a);
     } else {
-        k_fwdbwd<X><<<a.n_tiles, kFwdThreads, smem, s>>>(a);
+        gsl::launch_pdl(k_fwdbwd<X>, a.n_tiles, kFwdThreads, smem, s, a);
     }
 }
 
@@ -1349,9 +1353,9 @@ void launch_forward_reg(const gsl::RasterArgs &a, cudaStream_t s)
 {
     if (a.queue && g_fwd_q_ctas > 0) {
         cudaMemsetAsync(a.queue, 0, sizeof(uint32_t), s);
-        k_forward_q<X><<<(unsigned)std::min<uint32_t>(a.n_tiles, g_fwd_q_ctas), kFwdThreads, 0, s>>>(a);
+        gsl::launch_pdl(k_forward_q<X>, (unsigned)std::min<uint32_t>(a.n_tiles, g_fwd_q_ctas), kFwdThreads, 0, s, a);
     } else {
-        k_forward<true, X><<<a.n_tiles, kFwdThreads, 0, s>>>(a);
+        gsl::launch_pdl(k_forward<true, X>, a.n_tiles, kFwdThreads, 0, s, a);
     }
 }
 
@@ -1393,7 +1397,7 @@ void forward(const RasterArgs &a, bool registration, cudaStream_t s)
     // packed operations two pixels per thread had measured slower, 0.82
     // against 0.76 ms, as the early stop favours one pixel per thread)
     if (!registration)
-        k_forward<false, 0><<<a.n_tiles, kFwdThreads, 0, s>>>(a);
+        launch_pdl(k_forward<false, 0>, a.n_tiles, kFwdThreads, 0, s, a);
     else if (a.exposure && a.count_contrib)
         launch_forward_reg<kFwdExposure | kFwdCount>(a, s);
     else if (a.exposure)
@@ -1402,7 +1406,6 @@ void forward(const RasterArgs &a, bool registration, cudaStream_t s)
         launch_forward_reg<kFwdCount>(a, s);
     else
         launch_forward_reg<0>(a, s);
-    ++g_launches;
 }
 
 void backward(const RasterArgs &a, bool registration, bool full, cudaStream_t s)
@@ -1429,7 +1432,6 @@ void forward_backward(const RasterArgs &a, cudaStream_t s)
         launch_fwdbwd<kFwdCount>(a, s);
     else
         launch_fwdbwd<0>(a, s);
-    ++g_launches;
 }
 
 }  // namespace gsl

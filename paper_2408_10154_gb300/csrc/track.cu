@@ -65,6 +65,7 @@ __global__ void __cluster_dims__(kMedCluster, 1, 1) __launch_bounds__(kMedThread
     const uint32_t *v = reinterpret_cast<const uint32_t *>(a.err) + d.pix_base;
     for (int b = threadIdx.x; b < 3 * kMedBins; b += kMedThreads)
         (&hist[0][0])[b] = 0;
+    pdl_wait();
     __syncthreads();
     uint32_t prefix = 0, mask = 0, k = 0, m = 0;
 #pragma unroll
@@ -125,6 +126,7 @@ __global__ void __launch_bounds__(256) k_track_loss(const gsl::TrackArgs a)
     const uint32_t t = blockIdx.x;
     const int vp = (int)a.tile_vp[t];
     const VpDesc &d = a.vps[vp];
+    pdl_wait();
     if (d.loss_kind != 1)
         return;
     const uint32_t lt = t - d.tile_base;
@@ -194,9 +196,8 @@ void track_loss(const TrackArgs &a, cudaStream_t s)
 {
     if (a.n_track <= 0 || a.n_tiles == 0)
         return;
-    k_track_median<<<a.n_track * kMedCluster, kMedThreads, 0, s>>>(a);
-    k_track_loss<<<a.n_tiles, 256, 0, s>>>(a);
-    g_launches += 2;
+    launch_pdl(k_track_median, a.n_track * kMedCluster, kMedThreads, 0, s, a);
+    launch_pdl(k_track_loss, a.n_tiles, 256, 0, s, a);
 }
 
 void track_prep(const TrackArgs &a, const float *rgb, const float *depth, float *err, float *col, cudaStream_t s)
