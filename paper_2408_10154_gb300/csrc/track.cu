@@ -20,7 +20,8 @@ constexpr uint32_t kInfBits = 0x7f800000u;  // +inf marks a pixel without input 
 constexpr int kMedThreads = 1024;
 constexpr int kMedBins = 2048;
 constexpr int kMedCluster = 8;  // CTAs per keyframe (the portable cluster size)
-constexpr int kMedUnroll = 8;   // pixel loads in flight per thread
+constexpr int kMedKeep = 38;    // pixels per thread held in registers (640x480: 37.5)
+constexpr int kMedUnroll = 8;   // pixel loads in flight per thread otherwise
 // the three digits, high to low, of a non-negative float's 31 bits
 __device__ __forceinline__ constexpr int med_shift(int pass) { return pass == 0 ? 20 : (pass == 1 ? 10 : 0); }
 __device__ __forceinline__ constexpr uint32_t med_mask(int pass) { return pass == 0 ? 0x7ffu : 0x3ffu; }
@@ -46,11 +47,14 @@ __device__ __forceinline__ uint2 cluster_load2(const uint32_t *p, uint32_t rank)
 // pass, cleared together up front), and after one cluster barrier every CTA
 // adds the eight histograms through distributed shared memory and finds the
 // digit that holds the median's rank -- the same on all of them, so nothing
-// is sent back.  Bound by latency (one frame is 1.2 MB, read three times
-// from L2).  One CTA per keyframe took 346 us on a 640x480 frame, by ncu:
+// is sent back.  KEEP: a slice of at most kMedKeep pixels per thread is read
+// once and kept in registers over the three passes; a larger one is read by
+// each.  Bound by latency (one frame is 1.2 MB; reading it three times took
+// 7 us more of a tracking iteration).  One CTA per keyframe took 346 us on a 640x480 frame, by ncu:
 // each pass one dependent load and one match_any per 1024 pixels; the
 // tracking iteration spent two thirds of its time there (40 iterations of a
 // 640x480 frame on 150k Gaussians: 18.97 -> 7.06 ms with this kernel).
+template <bool KEEP>
 __global__ void __cluster_dims__(kMedCluster, 1, 1) __launch_bounds__(kMedThreads) k_track_median(const gsl::TrackArgs a)
 {
     __shared__ __align__(8) uint32_t hist[3][kMedBins];
@@ -66,20 +70,35 @@ __global__ void __cluster_dims__(kMedCluster, 1, 1) __launch_bounds__(kMedThread
     for (int b = threadIdx.x; b < 3 * kMedBins; b += kMedThreads)
         (&hist[0][0])[b] = 0;
     pdl_wait();
+    uint32_t kept[KEEP ? kMedKeep : 1];
+    if (KEEP) {
+#pragma unroll
+        for (int u = 0; u < kMedKeep; ++u) {
+            const int64_t i = i0 + u * kMedThreads + threadIdx.x;
+            kept[u] = i < i1 ? v[i] : kInfBits;
+        }
+    }
     __syncthreads();
     uint32_t prefix = 0, mask = 0, k = 0, m = 0;
 #pragma unroll
     for (int pass = 0; pass < 3; ++pass) {
         uint32_t *h = hist[pass];
-        for (int64_t base = i0 + threadIdx.x; base < i1; base += kMedUnroll * kMedThreads) {
-            uint32_t x[kMedUnroll];
+        if (KEEP) {
 #pragma unroll
-            for (int u = 0; u < kMedUnroll; ++u)
-                x[u] = base + u * kMedThreads < i1 ? v[base + u * kMedThreads] : kInfBits;
+            for (int u = 0; u < kMedKeep; ++u)
+                if (kept[u] < kInfBits && (kept[u] & mask) == prefix)
+                    atomicAdd(&h[(kept[u] >> med_shift(pass)) & med_mask(pass)], 1u);
+        } else {
+            for (int64_t base = i0 + threadIdx.x; base < i1; base += kMedUnroll * kMedThreads) {
+                uint32_t x[kMedUnroll];
 #pragma unroll
-            for (int u = 0; u < kMedUnroll; ++u)
-                if (x[u] < kInfBits && (x[u] & mask) == prefix)
-                    atomicAdd(&h[(x[u] >> med_shift(pass)) & med_mask(pass)], 1u);
+                for (int u = 0; u < kMedUnroll; ++u)
+                    x[u] = base + u * kMedThreads < i1 ? v[base + u * kMedThreads] : kInfBits;
+#pragma unroll
+                for (int u = 0; u < kMedUnroll; ++u)
+                    if (x[u] < kInfBits && (x[u] & mask) == prefix)
+                        atomicAdd(&h[(x[u] >> med_shift(pass)) & med_mask(pass)], 1u);
+            }
         }
         cluster_sync();
         // the cluster's counts of bins 2t and 2t + 1, their exclusive scan,
@@ -196,7 +215,8 @@ void track_loss(const TrackArgs &a, cudaStream_t s)
 {
     if (a.n_track <= 0 || a.n_tiles == 0)
         return;
-    launch_pdl(k_track_median, a.n_track * kMedCluster, kMedThreads, 0, s, a);
+    launch_pdl(a.max_pix <= (int64_t)kMedCluster * kMedKeep * kMedThreads ? k_track_median<true> : k_track_median<false>,
+               a.n_track * kMedCluster, kMedThreads, 0, s, a);
     launch_pdl(k_track_loss, a.n_tiles, 256, 0, s, a);
 }
 
