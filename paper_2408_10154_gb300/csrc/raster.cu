@@ -208,14 +208,65 @@ constexpr int kBwdSlotRow = kBwd2Chunk + 1;
 constexpr int kBwd2MinBlocks = kBwdPPT == 2 ? 8 : 12;
 static_assert(kBwdPPT * kBwdRowStep == 8 && kTile % kBwdPatchW == 0, "warp patches of 8 rows tile the 16x16 tile");
 
+// ---------------------------------------------------------------------------
+// Tensor memory as the fused tile's alpha stash.  The adjoint evaluates again
+// what the forward has just evaluated for the same pixels; the forward keeps
+// the alphas of each warp's first kStash records there, two 32-bit columns
+// per record in the warp's own 32 lanes (registers and shared memory are
+// full at eight CTAs per SM; 8 x 64 columns are all of an SM's 512).
+// ---------------------------------------------------------------------------
+constexpr int kStash = 32, kStashCols = 2 * kStash;
+
+// all lanes of one warp; the address lands in *dst (shared memory)
+__device__ __forceinline__ void tmem_alloc(uint32_t *dst)
+{
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
+                 :: "r"((uint32_t)__cvta_generic_to_shared(dst)), "n"(kStashCols)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+}
+// by all threads behind their last access, with the CTA's barrier inside
+__device__ __forceinline__ void tmem_free(const uint32_t *addr)
+{
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    if (threadIdx.x >= 32)
+        return;
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    __syncwarp();
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" :: "r"(*addr), "n"(kStashCols) : "memory");
+}
+// behind a barrier after tmem_alloc: the warp's own lanes of the allocation
+__device__ __forceinline__ uint32_t tmem_of_warp(const uint32_t *addr, int warp)
+{
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    return *addr + ((uint32_t)warp << 21);  // lanes 32 w .. 32 w + 31 (bits 16 and up)
+}
+// each lane's two values to or from columns addr, addr + 1 of its own lane
+__device__ __forceinline__ void tmem_store2(uint32_t addr, float v0, float v1)
+{
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x2.b32 [%0], {%1, %2};" :: "r"(addr), "f"(v0), "f"(v1) : "memory");
+}
+__device__ __forceinline__ void tmem_store_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
+__device__ __forceinline__ void tmem_load2(uint32_t addr, float &v0, float &v1)
+{
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x2.b32 {%0, %1}, [%2];\n\ttcgen05.wait::ld.sync.aligned;"
+                 : "=f"(v0), "=f"(v1)
+                 : "r"(addr)
+                 : "memory");
+}
+
 // the adjoint half of the fused registration tile (defined with the adjoint)
 __device__ __forceinline__ void fused_adjoint(const gsl::RasterArgs &a, uint32_t t, const VpDesc &d, uint2 rg,
                                               float4 *s0, float4 *s1, float4 *s2, const uint32_t *s_v,
                                               uint8_t *s_selw, float xa, float ya, PixAdj2 &P2, int maxl,
-                                              int wmaxl, const float *cc, bool fgen);
+                                              int wmaxl, const float *cc, bool fgen, int fsel, uint32_t tmem);
 
+// s_tmem: fused, where the stash's address is (written before the tile's
+// first barrier)
 template <bool REG, int X, bool FUSED = false>
-__device__ __forceinline__ void fwd_tile(const gsl::RasterArgs &a, const uint32_t t)
+__device__ __forceinline__ void fwd_tile(const gsl::RasterArgs &a, const uint32_t t, const uint32_t *s_tmem = nullptr)
 {
     static_assert(REG || !FUSED, "only the registration forward is fused with the adjoint");
     __shared__ float4 s0[kFwdBatch], s1[kFwdBatch], s2[kFwdBatch];
@@ -268,6 +319,11 @@ __device__ __forceinline__ void fwd_tile(const gsl::RasterArgs &a, const uint32_
     // opacity exceeds alpha_max (only those can reach the clamp: x = o e with
     // e <= 1 for every exponent <= 0) or whose exponent could round above 0
     bool gen = false;
+    // fused: the records the warp walked (of a list staged whole), and the
+    // warp's stash
+    int fsel = 0;
+    uint32_t tmem = 0;
+    const bool stash = FUSED && rg.y - rg.x <= (uint32_t)kFwdBatch;
     for (uint32_t b = rg.x; b < rg.y; b += kFwdBatch) {
         if (b != rg.x) {
             if (__syncthreads_count(done0 && done1) == kFwdThreads)
@@ -291,6 +347,8 @@ __device__ __forceinline__ void fwd_tile(const gsl::RasterArgs &a, const uint32_
             }
             gen = __syncthreads_or(hot) != 0;
         }
+        if (FUSED)
+            tmem = tmem_of_warp(s_tmem, warp);
         const int cnt = (int)min((uint32_t)kFwdBatch, rg.y - b);
         int nsel = 0;
         if (!__all_sync(0xffffffffu, done0 && done1)) {
@@ -354,6 +412,11 @@ __device__ __forceinline__ void fwd_tile(const gsl::RasterArgs &a, const uint32_
                     last1 = ok1 ? base + j : last1;
                     if (X & kFwdCount)
                         nc += (int)ok0 + (int)ok1;
+                    if (FUSED && !GEN && stash && k < kStash) {
+                        float v0, v1;
+                        x2_split(al, v0, v1);
+                        tmem_store2(tmem + 2 * k, v0, v1);
+                    }
                     continue;
                 }
                 // a stopping pixel is done: its pair adds nothing, T stays
@@ -372,6 +435,8 @@ __device__ __forceinline__ void fwd_tile(const gsl::RasterArgs &a, const uint32_
                 last1 = c1 ? base + j : last1;
                 if (X & kFwdCount)
                     nc += (int)c0 + (int)c1;
+                if (FUSED && !GEN && stash && k < kStash)
+                    tmem_store2(tmem + 2 * k, c0 ? al0 : 0.0f, c1 ? al1 : 0.0f);
                 if (__all_sync(0xffffffffu, done0 && done1))
                     break;
             }
@@ -381,6 +446,8 @@ __device__ __forceinline__ void fwd_tile(const gsl::RasterArgs &a, const uint32_
             else
                 walk(std::false_type{});
         }
+        if (FUSED)
+            fsel = nsel;
     }
     float Tk[2], C0k[2], C1k[2], C2k[2], Dk[2];
     x2_split(T, Tk[0], Tk[1]);
@@ -557,7 +624,7 @@ __device__ __forceinline__ void fwd_tile(const gsl::RasterArgs &a, const uint32_
         P2.gd = x2(g[0][3], g[1][3]);
         P2.last0 = last0;
         P2.last1 = last1;
-        fused_adjoint(a, t, d, rg, s0, s1, s2, s_v, s_sel[warp], xa, ya, P2, maxl, wmaxl, cc, gen);
+        fused_adjoint(a, t, d, rg, s0, s1, s2, s_v, s_sel[warp], xa, ya, P2, maxl, wmaxl, cc, gen, fsel, tmem);
     }
 }
 
@@ -837,24 +904,29 @@ __device__ __forceinline__ void pix_adj_init(PixAdj &P, const VpDesc &d, const g
 // every sum with weight 0 (so every value is the one-pixel walk's, up to the
 // sign of zero sums).  ALPHA: the alpha image has a cotangent (render mode).
 // FULL: also the opacity and colour gradients (ng[6..9]).  Returns whether
-// either pixel contributed.
-template <bool ALPHA, bool FULL, bool GEN = true>
+// either pixel contributed.  STASH: st0, st1 are the alphas the forward
+// blended (0: the pair did not contribute), and nothing is decided or
+// evaluated again (never with GEN or FULL).
+template <bool ALPHA, bool FULL, bool GEN = true, bool STASH = false>
 __device__ __forceinline__ bool pix_adj_x2(PixAdj2 &P, int jj, const RecX2 &R, float amax, float namax,
-                                           float namin, float (&ng)[FULL ? 10 : 6])
+                                           float namin, float (&ng)[FULL ? 10 : 6], float st0 = 0.0f, float st1 = 0.0f)
 {
+    static_assert(!STASH || (!GEN && !FULL), "the stash holds unclamped alphas only");
     f32x2 dx, h, ky;
     const f32x2 power = exponent_x2(R, P.pxf, P.pyf, dx, h, ky);
-    float p0, p1, e0, e1;
-    x2_split(power, p0, p1);
-    exp_ct_nonpos_x2(p0, p1, e0, e1);
-    // -x = (-o) e; clamped: x > alpha_max; -alpha; the alpha test
-    float nx0, nx1;
-    x2_split(mul2(R.co.y, x2(e0, e1)), nx0, nx1);
+    float p0 = 0.0f, p1 = 0.0f, e0 = 0.0f, e1 = 0.0f, nx0 = -st0, nx1 = -st1;
+    if (!STASH) {
+        x2_split(power, p0, p1);
+        exp_ct_nonpos_x2(p0, p1, e0, e1);
+        // -x = (-o) e
+        x2_split(mul2(R.co.y, x2(e0, e1)), nx0, nx1);
+    }
+    // clamped: x > alpha_max; -alpha; the alpha test
     const bool cl0 = GEN && nx0 < namax, cl1 = GEN && nx1 < namax;
     const float na0 = GEN ? fmaxf(nx0, namax) : nx0, na1 = GEN ? fmaxf(nx1, namax) : nx1;
-    const bool live0 = jj < P.last0 && (!GEN || !(p0 > 0.0f)) && !(na0 > namin);
-    const bool live1 = jj < P.last1 && (!GEN || !(p1 > 0.0f)) && !(na1 > namin);
-    const f32x2 nal = x2(live0 ? na0 : 0.0f, live1 ? na1 : 0.0f);
+    const bool live0 = STASH ? st0 != 0.0f : jj < P.last0 && (!GEN || !(p0 > 0.0f)) && !(na0 > namin);
+    const bool live1 = STASH ? st1 != 0.0f : jj < P.last1 && (!GEN || !(p1 > 0.0f)) && !(na1 > namin);
+    const f32x2 nal = STASH ? x2(na0, na1) : x2(live0 ? na0 : 0.0f, live1 ? na1 : 0.0f);
     const f32x2 nag = GEN ? x2(live0 && !cl0 ? na0 : 0.0f, live1 && !cl1 ? na1 : 0.0f) : nal;
     // 1 - alpha, its reciprocal, T_i = T / (1 - alpha)
     float om0, om1;
@@ -1154,10 +1226,16 @@ __global__ void __launch_bounds__(kBwd2Threads, kBwd2MinBlocks) k_backward2_q(co
 // there, chunk position j at list position lo + j; a longer one is
 // restaged chunk by chunk into the first kBwd2Chunk slots.  Only the
 // records' camera-frame mean and covariance are loaded per chunk.
+//
+// A list staged whole that needs no general walk is walked by the forward's
+// selection and its stashed alphas (kStash): of the adjoint's pair that
+// leaves out the exponential, the alpha test and the last-contributor test,
+// about 25 of 140 instructions (the kernel issues in 76 % of its slots).
+// STASH_NOW
 __device__ __forceinline__ void fused_adjoint(const gsl::RasterArgs &a, uint32_t t, const VpDesc &d, uint2 rg,
                                               float4 *s0, float4 *s1, float4 *s2, const uint32_t *s_v,
                                               uint8_t *s_selw, float xa, float ya, PixAdj2 &P2, int maxl,
-                                              int wmaxl, const float *cc, bool fgen)
+                                              int wmaxl, const float *cc, bool fgen, int fsel, uint32_t tmem)
 {
     constexpr int NG = 6;
     extern __shared__ float4 s_dyn[];
@@ -1175,6 +1253,36 @@ __device__ __forceinline__ void fused_adjoint(const gsl::RasterArgs &a, uint32_t
     const bool whole = n_list <= kFwdBatch;
     const bool cull = a.alpha_min > 0.0f;
     const int twist_warps = (min(maxl, kBwd2Chunk) + 31) / 32;
+    // the stashed walk: the warp's selection behind its last contributor is
+    // left out (it is in list order), and k runs down over all chunks
+    const bool stashed = whole && !fgen;
+    int k_next = -1;
+    if (stashed) {
+        __syncwarp();
+        for (int i0 = 0; i0 < fsel; i0 += 32)
+            k_next += __popc(__ballot_sync(0xffffffffu, i0 + lane < fsel && (int)s_selw[i0 + lane] < wmaxl));
+        tmem_store_wait();
+    }
+    auto sum_to_slot = [&](float (&g)[NG], int j) {
+        float v[8];
+#pragma unroll
+        for (int k2 = 0; k2 < 8; ++k2)
+            v[k2] = k2 < NG ? g[k2] : 0.0f;
+        const float sum = warp_sum_transpose<8, NG>(v, lane);
+        const int kk = lane / 4;
+        if ((lane % 4) == 0 && kk < NG)
+            s_slots[(kk * kBwd2Warps + warp) * kBwdSlotRow + j] = sum;
+    };
+    auto record = [&](int p) {
+        const float4 q0 = s0[p], q1 = s1[p], q2 = s2[p];
+        RecX2 R;
+        R.uv = make_ulonglong2(bc2(q0.x), bc2(q0.y));
+        R.ab = make_ulonglong2(bc2(q0.z), bc2(q0.w));
+        R.co = make_ulonglong2(bc2(q1.x), bc2(q2.w));
+        R.zr = make_ulonglong2(bc2(q1.z), bc2(q2.x));
+        R.gb = make_ulonglong2(bc2(q2.y), bc2(q2.z));
+        return R;
+    };
     for (int hi = maxl; hi > 0; hi -= kBwd2Chunk) {
         const int lo = max(hi - kBwd2Chunk, 0), cnt = hi - lo;
         const int sb = whole ? lo : 0;  // staging slot of chunk position 0
@@ -1219,51 +1327,61 @@ __device__ __forceinline__ void fused_adjoint(const gsl::RasterArgs &a, uint32_t
             if (!whole)
                 gen = any_hot;
         }
-        const int wl = min(wmaxl - lo, cnt);
-        int nsel = 0;
-        for (int j0 = 0; j0 < wl; j0 += 32) {
-            const int j = j0 + lane;
-            bool keep = false;
-            if (j < wl) {
-                const float4 t1 = s1[sb + j];
-                keep = !cull || patch_may_hit(s0[sb + j], t1.x, t1.w, xa, xa + 7.0f, ya, ya + 7.0f);
+        if (stashed) {
+            __syncwarp();  // (the staging above may have split the warp)
+            for (; k_next >= kStash; --k_next) {
+                const int j = s_selw[k_next];
+                if (j < lo)
+                    break;
+                float g[NG];
+                if (__any_sync(0xffffffffu, pix_adj_x2<false, false, false>(P2, j, record(j), a.alpha_max, -a.alpha_max,
+                                                                            -a.alpha_min, g)))
+                    sum_to_slot(g, j - lo);
             }
-            const unsigned m = __ballot_sync(0xffffffffu, keep);
-            if (keep)
-                s_selw[nsel + __popc(m & lanemask_lt())] = (uint8_t)j;
-            nsel += __popc(m);
-        }
-        __syncwarp();
-        auto walk = [&](auto gen_tag) {
-        constexpr bool GEN = decltype(gen_tag)::value;
-        for (int k = nsel - 1; k >= 0; --k) {
-            const int j = s_selw[k];
-            float g[NG];
-            const float4 q0 = s0[sb + j], q1 = s1[sb + j], q2 = s2[sb + j];
-            RecX2 R;
-            R.uv = make_ulonglong2(bc2(q0.x), bc2(q0.y));
-            R.ab = make_ulonglong2(bc2(q0.z), bc2(q0.w));
-            R.co = make_ulonglong2(bc2(q1.x), bc2(q2.w));
-            R.zr = make_ulonglong2(bc2(q1.z), bc2(q2.x));
-            R.gb = make_ulonglong2(bc2(q2.y), bc2(q2.z));
-            const bool contrib =
-                pix_adj_x2<false, false, GEN>(P2, lo + j, R, a.alpha_max, -a.alpha_max, -a.alpha_min, g);
-            if (__any_sync(0xffffffffu, contrib)) {
-                float v[8];
-#pragma unroll
-                for (int k2 = 0; k2 < 8; ++k2)
-                    v[k2] = k2 < NG ? g[k2] : 0.0f;
-                const float sum = warp_sum_transpose<8, NG>(v, lane);
-                const int kk = lane / 4;
-                if ((lane % 4) == 0 && kk < NG)
-                    s_slots[(kk * kBwd2Warps + warp) * kBwdSlotRow + j] = sum;
+            if (k_next < kStash) {
+                for (; k_next >= 0; --k_next) {
+                    const int j = s_selw[k_next];
+                    if (j < lo)
+                        break;
+                    const RecX2 R = record(j);
+                    float g[NG], st0, st1;
+                    tmem_load2(tmem + 2 * k_next, st0, st1);
+                    if (__any_sync(0xffffffffu, pix_adj_x2<false, false, false, true>(P2, 0, R, 0.0f, 0.0f, 0.0f, g, st0,
+                                                                                      st1)))
+                        sum_to_slot(g, j - lo);
+                }
             }
+        } else {
+            const int wl = min(wmaxl - lo, cnt);
+            int nsel = 0;
+            for (int j0 = 0; j0 < wl; j0 += 32) {
+                const int j = j0 + lane;
+                bool keep = false;
+                if (j < wl) {
+                    const float4 t1 = s1[sb + j];
+                    keep = !cull || patch_may_hit(s0[sb + j], t1.x, t1.w, xa, xa + 7.0f, ya, ya + 7.0f);
+                }
+                const unsigned m = __ballot_sync(0xffffffffu, keep);
+                if (keep)
+                    s_selw[nsel + __popc(m & lanemask_lt())] = (uint8_t)j;
+                nsel += __popc(m);
+            }
+            __syncwarp();
+            auto walk = [&](auto gen_tag) {
+                constexpr bool GEN = decltype(gen_tag)::value;
+                for (int k = nsel - 1; k >= 0; --k) {
+                    const int j = s_selw[k];
+                    float g[NG];
+                    if (__any_sync(0xffffffffu, pix_adj_x2<false, false, GEN>(P2, lo + j, record(sb + j), a.alpha_max,
+                                                                              -a.alpha_max, -a.alpha_min, g)))
+                        sum_to_slot(g, j);
+                }
+            };
+            if (gen)
+                walk(std::true_type{});
+            else
+                walk(std::false_type{});
         }
-        };
-        if (gen)
-            walk(std::true_type{});
-        else
-            walk(std::false_type{});
         __syncthreads();
         if ((int)threadIdx.x < cnt) {
             float G[NG];
@@ -1299,15 +1417,23 @@ __device__ __forceinline__ void fused_adjoint(const gsl::RasterArgs &a, uint32_t
 template <int X>
 __global__ void __launch_bounds__(kFwdThreads, 8) k_fwdbwd(const gsl::RasterArgs a)
 {
+    __shared__ uint32_t s_tmem;
+    if (threadIdx.x < 32)
+        tmem_alloc(&s_tmem);
     pdl_wait();
-    fwd_tile<true, X, true>(a, a.tile_order ? a.tile_order[blockIdx.x] : blockIdx.x);
+    fwd_tile<true, X, true>(a, a.tile_order ? a.tile_order[blockIdx.x] : blockIdx.x, &s_tmem);
+    tmem_free(&s_tmem);
 }
 
 template <int X>
 __global__ void __launch_bounds__(kFwdThreads, 8) k_fwdbwd_q(const gsl::RasterArgs a)
 {
+    __shared__ uint32_t s_tmem;
+    if (threadIdx.x < 32)
+        tmem_alloc(&s_tmem);
     pdl_wait();
-    run_queue(a, [&](uint32_t t) { fwd_tile<true, X, true>(a, t); });
+    run_queue(a, [&](uint32_t t) { fwd_tile<true, X, true>(a, t, &s_tmem); });
+    tmem_free(&s_tmem);
 }
 
 template <bool REG, bool FULL>
