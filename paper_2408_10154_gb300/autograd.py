@@ -26,13 +26,14 @@ class Rasterize(torch.autograd.Function):
         out, saved = gsreg.gs_render_saved(gsctx, g, poses, cams)
         fctx.gsctx, fctx.saved = gsctx, saved
         fctx.save_for_backward(pivots)
+        fctx.set_materialize_grads(False)  # an image without a cotangent needs no zeros (None: NULL, taken as 0)
         return out["rgb"], out["depth"], out["alpha"]
 
     @staticmethod
     def backward(fctx, d_rgb, d_depth, d_alpha):
         (pivots,) = fctx.saved_tensors
-        pg, gr = gsreg.gs_render_backward_saved(fctx.gsctx, fctx.saved, d_rgb.contiguous(), d_depth.contiguous(),
-                                                d_alpha.contiguous(), pivots, params=True)
+        d_rgb, d_depth, d_alpha = [None if d is None else d.contiguous() for d in (d_rgb, d_depth, d_alpha)]
+        pg, gr = gsreg.gs_render_backward_saved(fctx.gsctx, fctx.saved, d_rgb, d_depth, d_alpha, pivots, params=True)
         fctx.saved.close()
         return (None, None, None, None, gr["means4"], gr["log_scales4"], gr["quats4"], gr["logits"], gr["rgb4"], pg)
 

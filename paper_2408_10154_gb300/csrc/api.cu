@@ -21,8 +21,8 @@
 namespace {
 
 enum Slot {
-    S_VPS, S_GROUPS, S_TILEVP, S_POSE32, S_REC, S_AUX, S_COUNTS, S_PARTIALS, S_NDUPS, S_K0, S_V0, S_RANGES, S_FLAGS, S_TF, S_LAST, S_CODE, S_TLOSS, S_TTWIST, S_POSE64, S_ADAM, S_PIVOT,
-    S_CCAM, S_CENT, S_CENTP, S_LOSS, S_SETVP, S_REV, S_PFIRST, S_PCOUNT, S_TOUT, S_CONF, S_EST, S_GRAD, S_DUPG,
+    S_VPS, S_GROUPS, S_TILEVP, S_POSE32, S_REC, S_AUX, S_COUNTS, S_PARTIALS, S_K0, S_V0, S_RANGES, S_FLAGS, S_TF, S_LAST, S_CODE, S_TLOSS, S_TTWIST, S_POSE64, S_ADAM, S_PIVOT,
+    S_CCAM, S_CENT, S_CENTP, S_LOSS, S_SETVP, S_REV, S_PFIRST, S_PCOUNT, S_RESULT, S_TOUT, S_CONF, S_EST, S_GRAD, S_DUPG,
     S_PAIRS, S_RSLOT, S_RSLOTN, S_TERR, S_TCOL, S_TW,
     S_TMED, S_TNV, S_TVPS, S_EXPO, S_EXPO32, S_TEXPO, S_OPT, S_ONN1, S_ONN2, S_OD2, S_OHDR, S_MAPS, S_OS, S_ORDER, S_ORDC, S_SK, S_SV, S_SN, S_GCELL, S_GCOUNT, S_GSTART, S_GSUMS, S_GPTS, S_GLIST, S_SEGZ, S_SEGCUR, S_SEGLIST, S_PROBE, S_QUEUE, S_COUNT
 };
@@ -56,6 +56,13 @@ struct gs_ctx {
     // largest tile-duplicate count seen at the initial poses per plan shape
     // (sizes the lists of the asynchronous registration calls)
     std::map<std::tuple<uint64_t, size_t, uint64_t>, uint32_t> dups_seen;
+    // the same for the forward passes kept for their adjoint
+    std::map<std::tuple<uint64_t, size_t, uint64_t>, uint32_t> saved_seen;
+    // whether the list builds' counting grids may hold counts (a projection
+    // whose lists were not built, or a new buffer): every build leaves them clear
+    bool seg_dirty = true;
+    void *host = nullptr;  // page-locked block the results are read back into
+    size_t host_bytes = 0;
 };
 
 namespace {
@@ -152,6 +159,23 @@ gs_status_t upload(gs_ctx *ctx, int slot, const std::vector<T> &v, T **out, cuda
     return GS_OK;
 }
 
+// page-locked host block of at least `bytes` (grown, never shrunk; every use
+// of it ends before the call that made it returns)
+gs_status_t host_block(gs_ctx *ctx, size_t bytes, void **out)
+{
+    if (ctx->host_bytes < bytes) {
+        if (ctx->host)
+            cudaFreeHost(ctx->host);
+        ctx->host = nullptr;
+        ctx->host_bytes = 0;
+        const size_t want = (bytes + bytes / 4 + 4095) & ~(size_t)4095;
+        GS_CUDA(cudaMallocHost(&ctx->host, want));
+        ctx->host_bytes = want;
+    }
+    *out = ctx->host;
+    return GS_OK;
+}
+
 bool aligned16(const void *p) { return ((uintptr_t)p & 15u) == 0; }
 
 gs_status_t check_gaussians(gs_ctx *ctx, const gs_gaussians_t *g, const char *what)
@@ -212,7 +236,6 @@ gs_status_t check_options(gs_ctx *ctx, const gs_options_t *o)
 struct Plan {
     std::vector<VpDesc> vps;
     std::vector<GroupDesc> groups;
-    std::vector<uint32_t> tile_vp;
     std::vector<int> set_vp;  // a vp of each Gaussian set
     uint64_t n_records = 0, n_tiles = 0, n_diff = 0;
     int64_t n_pix = 0;
@@ -252,8 +275,6 @@ void add_vp(Plan &P, const gs_gaussians_t *g, const gs_camera_t &c, int set, int
     d.problem = problem;
     d.reverse = reverse;
     const int vp = (int)P.vps.size();
-    for (int k = 0; k < d.TX * d.TY; ++k)
-        P.tile_vp.push_back((uint32_t)vp);
     P.n_records += (uint64_t)d.n;
     P.n_tiles += (uint64_t)d.TX * d.TY;
     P.n_diff += (uint64_t)(d.TX + 1) * (d.TY + 1);
@@ -305,20 +326,110 @@ float skip_threshold(const gs_options_t *o)
     return o->alpha_min > 0 ? logf(o->alpha_min) - 0.05f : -3.0e38f;
 }
 
-// device copies of a plan's tables
+// device copies of a plan's tables, and of the registration problems' (or null)
 struct DevPlan {
     VpDesc *vps = nullptr;
     GroupDesc *groups = nullptr;
     uint32_t *tile_vp = nullptr;
     int *set_vp = nullptr;
+    int32_t *rev = nullptr, *prob_first = nullptr, *prob_count = nullptr;
 };
 
-gs_status_t upload_plan(gs_ctx *ctx, const Plan &P, DevPlan &D, cudaStream_t s)
+// The tables travel as kernel arguments, 16 keyframes per launch: a launch
+// costs the host less than the copies of seven small tables, needs no
+// staging memory to outlive the call, and fills the tile -> keyframe table
+// (100 kB on eight 1200x680 views) on the device.
+constexpr int kPlanChunk = 16;
+struct PlanChunk {
+    VpDesc vps[kPlanChunk];
+    GroupDesc groups[kPlanChunk];
+    int32_t set_vp[kPlanChunk], rev[kPlanChunk], prob_first[kPlanChunk], prob_count[kPlanChunk];
+    int v0, n_vps, n_groups, n_sets, n_probs;
+    DevPlan D;
+    int *flags;  // cleared by the first chunk (or null)
+};
+
+__global__ void __launch_bounds__(256) k_plan(const __grid_constant__ PlanChunk c)
 {
-    GS_TRY(upload(ctx, S_VPS, P.vps, &D.vps, s));
-    GS_TRY(upload(ctx, S_GROUPS, P.groups, &D.groups, s));
-    GS_TRY(upload(ctx, S_TILEVP, P.tile_vp, &D.tile_vp, s));
-    GS_TRY(upload(ctx, S_SETVP, P.set_vp, &D.set_vp, s));
+    const int v = blockIdx.y, i = threadIdx.x;
+    if (v < c.n_vps) {
+        const VpDesc &d = c.vps[v];
+        if (blockIdx.x == 0 && i < (int)(sizeof(VpDesc) / 4))
+            reinterpret_cast<uint32_t *>(c.D.vps + c.v0 + v)[i] = reinterpret_cast<const uint32_t *>(&d)[i];
+        const uint32_t nt = (uint32_t)d.TX * (uint32_t)d.TY;
+        for (uint32_t t = blockIdx.x * 256 + i; t < nt; t += gridDim.x * 256)
+            c.D.tile_vp[d.tile_base + t] = (uint32_t)(c.v0 + v);
+    }
+    if (blockIdx.x != 0 || v != 0)
+        return;
+    if (i < c.n_groups)
+        c.D.groups[c.v0 + i] = c.groups[i];
+    if (c.D.set_vp && i < c.n_sets)
+        c.D.set_vp[c.v0 + i] = c.set_vp[i];
+    if (c.D.rev && i < c.n_vps)
+        c.D.rev[c.v0 + i] = c.rev[i];
+    if (c.D.rev && i < c.n_probs) {
+        c.D.prob_first[c.v0 + i] = c.prob_first[i];
+        c.D.prob_count[c.v0 + i] = c.prob_count[i];
+    }
+    if (i == 0 && c.v0 == 0 && c.flags)
+        *c.flags = 0;
+}
+static_assert(sizeof(VpDesc) % 4 == 0 && sizeof(VpDesc) / 4 <= 256, "one thread copies one word of a descriptor");
+
+// (groups, sets and problems are at most as many as keyframes)
+void send_plan(const Plan &P, const DevPlan &D, int n_problems, int *flags, cudaStream_t s)
+{
+    std::vector<int32_t> pf(n_problems, 0), pc(n_problems, 0);
+    if (n_problems > 0)
+        for (int v = 0; v < (int)P.vps.size(); ++v)
+            if (pc[P.vps[v].problem]++ == 0)
+                pf[P.vps[v].problem] = v;
+    const int nv = (int)P.vps.size();
+    for (int v0 = 0; v0 == 0 || v0 < nv; v0 += kPlanChunk) {
+        PlanChunk c;
+        auto part = [&](size_t n) { return std::max(0, std::min(kPlanChunk, (int)n - v0)); };
+        c.v0 = v0;
+        c.n_vps = part(P.vps.size());
+        c.n_groups = part(P.groups.size());
+        c.n_sets = part(P.set_vp.size());
+        c.n_probs = part((size_t)n_problems);
+        c.D = D;
+        c.flags = flags;
+        uint32_t nt = 1;
+        for (int i = 0; i < c.n_vps; ++i) {
+            c.vps[i] = P.vps[v0 + i];
+            c.rev[i] = P.vps[v0 + i].reverse;
+            nt = std::max(nt, (uint32_t)c.vps[i].TX * (uint32_t)c.vps[i].TY);
+        }
+        for (int i = 0; i < c.n_groups; ++i)
+            c.groups[i] = P.groups[v0 + i];
+        for (int i = 0; i < c.n_sets; ++i)
+            c.set_vp[i] = P.set_vp[v0 + i];
+        for (int i = 0; i < c.n_probs; ++i) {
+            c.prob_first[i] = pf[v0 + i];
+            c.prob_count[i] = pc[v0 + i];
+        }
+        k_plan<<<dim3(std::min<uint32_t>((nt + 1023) / 1024, 64), std::max(c.n_vps, 1)), 256, 0, s>>>(c);
+        ++gsl::g_launches;
+    }
+}
+
+// n_problems > 0: the registration problems' tables too; flags: a device
+// word to clear (or null)
+gs_status_t upload_plan(gs_ctx *ctx, const Plan &P, DevPlan &D, cudaStream_t s, int n_problems = 0, int *flags = nullptr)
+{
+    GS_TRY(wsT(ctx, S_VPS, P.vps.size(), &D.vps));
+    GS_TRY(wsT(ctx, S_GROUPS, P.groups.size(), &D.groups));
+    GS_TRY(wsT(ctx, S_TILEVP, (size_t)P.n_tiles, &D.tile_vp));
+    GS_TRY(wsT(ctx, S_SETVP, P.set_vp.size(), &D.set_vp));
+    if (n_problems > 0) {
+        GS_TRY(wsT(ctx, S_REV, P.vps.size(), &D.rev));
+        GS_TRY(wsT(ctx, S_PFIRST, (size_t)n_problems, &D.prob_first));
+        GS_TRY(wsT(ctx, S_PCOUNT, (size_t)n_problems, &D.prob_count));
+    }
+    send_plan(P, D, n_problems, flags, s);
+    GS_CUDA(cudaGetLastError());
     return GS_OK;
 }
 
@@ -339,7 +450,6 @@ struct Pipe {
     unsigned long long *seg_hdr = nullptr;
     uint32_t *seg_diff = nullptr, *seg_cursor = nullptr;
     uint4 *seg_list = nullptr;
-    size_t seg_zero = 0;
 };
 
 // Binning routes.  The context-based entry points and gs_bin use the
@@ -354,9 +464,12 @@ struct Pipe {
 gs_status_t alloc_seg(gs_ctx *ctx, const Plan &P, Pipe &p)
 {
     const size_t T = P.n_tiles ? P.n_tiles : 1, R = P.n_records ? P.n_records : 1;
-    p.seg_zero = gsl::seg_zero_bytes((int)P.vps.size(), P.n_diff);
+    const size_t zero = gsl::seg_zero_bytes((int)P.vps.size(), P.n_diff);
     uint8_t *z = nullptr;
-    GS_TRY(wsT(ctx, S_SEGZ, p.seg_zero, &z));
+    const void *before = ctx->bufs[S_SEGZ].p;
+    GS_TRY(wsT(ctx, S_SEGZ, zero, &z));
+    if (z != before)
+        ctx->seg_dirty = true;
     p.seg_hdr = (unsigned long long *)z;
     p.seg_diff = (uint32_t *)(p.seg_hdr + P.vps.size());
     GS_TRY(wsT(ctx, S_SEGLIST, R, &p.seg_list));
@@ -372,9 +485,9 @@ gs_status_t alloc_pipe(gs_ctx *ctx, const Plan &P, bool aux, Pipe &p)
         GS_TRY(wsT(ctx, S_AUX, 2 * R, &p.aux));
     GS_TRY(wsT(ctx, S_COUNTS, R, &p.counts));
     GS_TRY(wsT(ctx, S_PARTIALS, gsl::scan_partials(R), &p.partials));
-    GS_TRY(wsT(ctx, S_NDUPS, 4, &p.ndups));
     GS_TRY(wsT(ctx, S_RANGES, P.n_tiles ? P.n_tiles : 1, &p.ranges));
-    GS_TRY(wsT(ctx, S_FLAGS, 4, &p.flags));
+    GS_TRY(wsT(ctx, S_FLAGS, 4, &p.flags));  // {flags, n_dups}: read back together
+    p.ndups = (uint32_t *)p.flags + 1;
     GS_TRY(alloc_seg(ctx, P, p));
     p.n_records = R;
     return GS_OK;
@@ -391,7 +504,22 @@ gs_status_t alloc_sort(gs_ctx *ctx, uint64_t want, Pipe &p)
     return GS_OK;
 }
 
-int run_bin(const gsl::BinArgs &b, cudaStream_t s) { return gsl::bin_seg(b, s); }
+// Ahead of a projection that counts: clears the counting grids unless the
+// last build left them clear.
+gs_status_t begin_lists(gs_ctx *ctx, cudaStream_t s)
+{
+    if (ctx->seg_dirty)
+        GS_CUDA(cudaMemsetAsync(ctx->bufs[S_SEGZ].p, 0, ctx->bufs[S_SEGZ].bytes, s));
+    ctx->seg_dirty = true;
+    return GS_OK;
+}
+
+int run_bin(gs_ctx *ctx, const gsl::BinArgs &b, cudaStream_t s)
+{
+    const int cur = gsl::bin_seg(b, s);
+    ctx->seg_dirty = false;
+    return cur;
+}
 
 // counts = false: the per-record tile counts are not written (the
 // segmented lists read the records' seg_list entries; only the scan for the
@@ -418,7 +546,6 @@ gsl::ProjectArgs project_args(const Plan &P, const DevPlan &D, const Pipe &p, co
     // the projection counts and lists for the segmented build (run_bin follows every projection here)
     a.seg_hdr = p.seg_hdr;
     a.seg_diff = p.seg_diff;
-    a.seg_zero_bytes = p.seg_zero;
     a.seg_list = p.seg_list;
     return a;
 }
@@ -447,7 +574,6 @@ gsl::BinArgs bin_args(const Plan &P, const DevPlan &D, const Pipe &p)
     b.tkeys[0] = p.tkeys[0];
     b.seg_hdr = p.seg_hdr;
     b.seg_diff = p.seg_diff;
-    b.seg_zero_bytes = p.seg_zero;
     b.seg_cursor = p.seg_cursor;
     b.seg_list = p.seg_list;
     b.seg_counted = 1;
@@ -483,6 +609,7 @@ gs_status_t project_and_bin(gs_ctx *ctx, const Plan &P, const DevPlan &D, Pipe &
                             const gs_options_t *o, cudaStream_t s, int *cur, uint32_t *n_dups_out)
 {
     GS_CUDA(cudaMemsetAsync(p.flags, 0, sizeof(int), s));
+    GS_TRY(begin_lists(ctx, s));
     gsl::project(project_args(P, D, p, pose32, o), s);
     gsl::BinArgs b = bin_args(P, D, p);
     gsl::bin_count(b, s);
@@ -491,21 +618,41 @@ gs_status_t project_and_bin(gs_ctx *ctx, const Plan &P, const DevPlan &D, Pipe &
     GS_CUDA(cudaStreamSynchronize(s));
     if (nd == 0xffffffffu)
         return fail(ctx, GS_ERR_CAPACITY, "more than 2^32 tile duplicates");
-    if (p.cap < nd || !p.tkeys[0])
+    if (p.cap < nd || p.cap == 0)
         GS_TRY(alloc_sort(ctx, nd, p));
     b = bin_args(P, D, p);
-    *cur = run_bin(b, s);
+    *cur = run_bin(ctx, b, s);
     if (n_dups_out)
         *n_dups_out = nd;
     GS_CUDA(cudaGetLastError());
     return GS_OK;
 }
 
-gs_status_t read_flags(gs_ctx *ctx, const Pipe &p, cudaStream_t s, int *flags)
+// waits for the stream and reads the status word, and the duplicate total
+// (n_dups or null) that lies beside it where alloc_pipe made both
+gs_status_t read_flags(gs_ctx *ctx, const Pipe &p, cudaStream_t s, int *flags, uint32_t *n_dups = nullptr)
 {
-    GS_CUDA(cudaMemcpyAsync(flags, p.flags, sizeof(int), cudaMemcpyDeviceToHost, s));
+    void *h = nullptr;
+    GS_TRY(host_block(ctx, 2 * sizeof(int), &h));
+    GS_CUDA(cudaMemcpyAsync(h, p.flags, (n_dups ? 2 : 1) * sizeof(int), cudaMemcpyDeviceToHost, s));
     GS_CUDA(cudaStreamSynchronize(s));
+    *flags = ((const int *)h)[0];
+    if (n_dups)
+        *n_dups = ((const uint32_t *)h)[1];
     return GS_OK;
+}
+
+// the list buffers an earlier call left on the context, if any
+bool lists_at_hand(const gs_ctx *ctx, Pipe &p)
+{
+    const Buf &k = ctx->bufs[S_K0], &v = ctx->bufs[S_V0];
+    const size_t cap = std::min(std::min(k.bytes, v.bytes) / sizeof(uint32_t), (size_t)0xfff00000u);
+    if (cap == 0)
+        return false;
+    p.tkeys[0] = (uint32_t *)k.p;
+    p.vals[0] = (uint32_t *)v.p;
+    p.cap = (uint32_t)cap;
+    return true;
 }
 
 gs_status_t check_common(gs_ctx *ctx, const gs_gaussians_t *g, const gs_camera_t *cams, int n_cams,
@@ -791,6 +938,8 @@ gs_status_t gs_ctx_destroy(gs_ctx_t *ctx)
         cudaEventDestroy(e);
     if (ctx->cap)
         cudaStreamDestroy(ctx->cap);
+    if (ctx->host)
+        cudaFreeHost(ctx->host);
     delete ctx;
     return GS_OK;
 }
@@ -864,8 +1013,8 @@ gs_status_t gs_bin(gs_ctx_t *ctx, const float *records, const int32_t *counts, c
     p.rec = (float4 *)records;
     p.counts = (int32_t *)counts;
     GS_TRY(wsT(ctx, S_PARTIALS, gsl::scan_partials(P.n_records ? P.n_records : 1), &p.partials));
-    GS_TRY(wsT(ctx, S_NDUPS, 4, &p.ndups));
     GS_TRY(wsT(ctx, S_FLAGS, 4, &p.flags));
+    p.ndups = (uint32_t *)p.flags + 1;
     GS_CUDA(cudaMemsetAsync(p.flags, 0, sizeof(int), s));
     p.ranges = (uint2 *)ranges;
     const size_t R = P.n_records ? P.n_records : 1;
@@ -882,7 +1031,8 @@ gs_status_t gs_bin(gs_ctx_t *ctx, const float *records, const int32_t *counts, c
     GS_TRY(alloc_sort(ctx, nd, p));
     b = bin_args(P, D, p);
     b.seg_counted = 0;  // the caller's records: collect them here
-    const int cur = gsl::bin_seg(b, s);
+    GS_TRY(begin_lists(ctx, s));
+    const int cur = run_bin(ctx, b, s);
     if (nd > 0) {
         gsl::seg_keys64(b, keys, s);
         GS_CUDA(cudaMemcpyAsync(vals, p.vals[cur], sizeof(uint32_t) * nd, cudaMemcpyDeviceToDevice, s));
@@ -907,27 +1057,44 @@ gs_status_t gs_render(gs_ctx_t *ctx, const gs_gaussians_t *g, const float *poses
     Plan P = plan_for(g, cams, n_cams);
     GS_TRY(finalize(ctx, P));
     DevPlan D;
-    GS_TRY(upload_plan(ctx, P, D, s));
     Pipe p;
     GS_TRY(alloc_pipe(ctx, P, false, p));
+    const long long l0 = gsl::g_launches;
+    GS_TRY(upload_plan(ctx, P, D, s, 0, p.flags));
     int cur = 0;
     uint32_t nd = 0;
-    const long long l0 = gsl::g_launches;
-    GS_TRY(project_and_bin(ctx, P, D, p, poses, opt, s, &cur, &nd));
-    gsl::RasterArgs r = raster_args(P, D, p, cur, opt);
-    r.out_rgb = rgb;
-    r.out_depth = depth;
-    r.out_alpha = alpha;
-    r.t_final = t_final;
-    r.last = last;
-    gsl::forward(r, false, s);
-    GS_CUDA(cudaGetLastError());
+    int flags = 0;
+    auto composite = [&]() {
+        gsl::RasterArgs r = raster_args(P, D, p, cur, opt);
+        r.out_rgb = rgb;
+        r.out_depth = depth;
+        r.out_alpha = alpha;
+        r.t_final = t_final;
+        r.last = last;
+        gsl::forward(r, false, s);
+    };
+    // With lists left by an earlier call the whole pass is enqueued at once
+    // and redone, with the lists counted first, if they are too short.
+    bool done = false;
+    if (lists_at_hand(ctx, p)) {
+        GS_TRY(begin_lists(ctx, s));
+        gsl::project(project_args(P, D, p, poses, opt, false), s);
+        cur = run_bin(ctx, bin_args(P, D, p), s);
+        composite();
+        GS_TRY(read_flags(ctx, p, s, &flags, &nd));
+        done = !(flags & gsk::kFlagCapacity);
+    }
+    if (!done) {
+        p.cap = 0;
+        GS_TRY(project_and_bin(ctx, P, D, p, poses, opt, s, &cur, &nd));
+        composite();
+        GS_CUDA(cudaGetLastError());
+        GS_TRY(read_flags(ctx, p, s, &flags, nullptr));
+    }
     ctx->stats = gs_stats_t{};
     ctx->stats.kernel_launches = gsl::g_launches - l0;
     ctx->stats.n_dups = nd;
     ctx->stats.n_pixels = P.n_pix;
-    int flags = 0;
-    GS_TRY(read_flags(ctx, p, s, &flags));
     if (flags & gsk::kFlagNonFinite)
         return fail(ctx, GS_ERR_NONFINITE, "non-finite Gaussian parameter");
     if (flags & gsk::kFlagTimeout)
@@ -1068,9 +1235,9 @@ gs_status_t gs_render_backward(gs_ctx_t *ctx, const gs_gaussians_t *g, const flo
 // A forward pass kept for its adjoint: the plan (host), and in two
 // stream-ordered device blocks the plan tables, the pose copy, the records
 // and their auxiliary camera-frame mean and covariance, the counts, tile
-// ranges, the duplicate count, per-pixel final transmittance and last
-// contributor (block 1, sized from the plan), and the sorted tile lists
-// (block 2, sized after counting).
+// ranges, per-pixel final transmittance and last contributor (block 1, sized
+// from the plan), and the sorted tile lists (block 2, sized from the
+// duplicates counted, or from what a pass of the shape had before).
 struct gs_saved {
     int device = 0;
     Plan P;
@@ -1082,7 +1249,7 @@ struct gs_saved {
     float4 *rec = nullptr, *aux = nullptr;
     int32_t *counts = nullptr, *last = nullptr;
     uint2 *ranges = nullptr;
-    uint32_t *vals = nullptr, *ndups = nullptr;
+    uint32_t *vals = nullptr;
     uint32_t cap = 0;
 };
 
@@ -1128,10 +1295,10 @@ gs_status_t gs_render_saved(gs_ctx_t *ctx, const gs_gaussians_t *g, const float 
                  px = (size_t)std::max<int64_t>(P.n_pix, 1);
     Layout L;
     const size_t o_vps = L.take(sizeof(VpDesc) * nv), o_grp = L.take(sizeof(GroupDesc) * P.groups.size()),
-                 o_tvp = L.take(sizeof(uint32_t) * P.tile_vp.size()), o_pose = L.take(sizeof(float) * 12 * nv),
+                 o_tvp = L.take(sizeof(uint32_t) * (size_t)P.n_tiles), o_pose = L.take(sizeof(float) * 12 * nv),
                  o_rec = L.take(sizeof(float4) * 3 * R), o_aux = L.take(sizeof(float4) * 2 * R),
                  o_cnt = L.take(sizeof(int32_t) * R), o_rng = L.take(sizeof(uint2) * T),
-                 o_nd = L.take(sizeof(uint32_t) * 4), o_tf = L.take(sizeof(float) * px),
+                 o_tf = L.take(sizeof(float) * px),
                  o_last = L.take(sizeof(int32_t) * px);
     auto cleanup = [&](gs_status_t st) {
         for (void *b : sv->blk)
@@ -1154,24 +1321,19 @@ gs_status_t gs_render_saved(gs_ctx_t *ctx, const gs_gaussians_t *g, const float 
     sv->aux = (float4 *)(b0 + o_aux);
     sv->counts = (int32_t *)(b0 + o_cnt);
     sv->ranges = (uint2 *)(b0 + o_rng);
-    sv->ndups = (uint32_t *)(b0 + o_nd);
     sv->t_final = (float *)(b0 + o_tf);
     sv->last = (int32_t *)(b0 + o_last);
     auto copy = [&](void *dst, const void *src, size_t bytes, cudaMemcpyKind k) {
         return bytes == 0 || cudaMemcpyAsync(dst, src, bytes, k, s) == cudaSuccess;
     };
-    if (!copy(sv->D.vps, P.vps.data(), sizeof(VpDesc) * nv, cudaMemcpyHostToDevice) ||
-        !copy(sv->D.groups, P.groups.data(), sizeof(GroupDesc) * P.groups.size(), cudaMemcpyHostToDevice) ||
-        !copy(sv->D.tile_vp, P.tile_vp.data(), sizeof(uint32_t) * P.tile_vp.size(), cudaMemcpyHostToDevice) ||
-        !copy(sv->pose32, poses, sizeof(float) * 12 * nv, cudaMemcpyDeviceToDevice))
-        return cleanup(fail(ctx, GS_ERR_CUDA, "gs_render_saved: copy of the plan"));
+    if (!copy(sv->pose32, poses, sizeof(float) * 12 * nv, cudaMemcpyDeviceToDevice))
+        return cleanup(fail(ctx, GS_ERR_CUDA, "gs_render_saved: copy of the poses"));
     // projection into the saved block, list building scratch in the arena
     Pipe p;
     p.rec = sv->rec;
     p.aux = sv->aux;
     p.counts = sv->counts;
     p.ranges = sv->ranges;
-    p.ndups = sv->ndups;
     p.n_records = R;
     gs_status_t st = wsT(ctx, S_PARTIALS, gsl::scan_partials(R), &p.partials);
     if (st == GS_OK)
@@ -1180,43 +1342,72 @@ gs_status_t gs_render_saved(gs_ctx_t *ctx, const gs_gaussians_t *g, const float 
         st = alloc_seg(ctx, P, p);
     if (st != GS_OK)
         return cleanup(st);
-    if (cudaMemsetAsync(p.flags, 0, sizeof(int), s) != cudaSuccess)
-        return cleanup(fail(ctx, GS_ERR_CUDA, "gs_render_saved: memset"));
-    gsl::project(project_args(P, sv->D, p, sv->pose32, opt), s);
-    gsl::BinArgs b = bin_args(P, sv->D, p);
-    gsl::bin_count(b, s);
+    p.ndups = (uint32_t *)p.flags + 1;
+    send_plan(P, sv->D, 0, p.flags, s);
+    // With the duplicates an earlier pass of this shape had as a guide, the
+    // whole pass is enqueued at once, and redone if its lists were too short;
+    // a shape not seen before has its duplicates counted first.
+    const auto key = std::make_tuple((uint64_t)P.n_tiles, P.vps.size(), (uint64_t)P.n_records);
+    const auto seen = ctx->saved_seen.find(key);
     uint32_t nd = 0;
-    if (cudaMemcpyAsync(&nd, p.ndups, sizeof nd, cudaMemcpyDeviceToHost, s) != cudaSuccess ||
-        cudaStreamSynchronize(s) != cudaSuccess)
-        return cleanup(fail(ctx, GS_ERR_CUDA, "gs_render_saved: duplicate count"));
-    if (nd == 0xffffffffu)
-        return cleanup(fail(ctx, GS_ERR_CAPACITY, "more than 2^32 tile duplicates"));
-    st = alloc_sort(ctx, nd, p);
-    if (st != GS_OK)
-        return cleanup(st);
-    if (cudaMallocAsync(&sv->blk[1], sizeof(uint32_t) * (size_t)p.cap, s) != cudaSuccess) {
-        cudaGetLastError();
-        sv->blk[1] = nullptr;
-        return cleanup(fail(ctx, GS_ERR_OOM, "gs_render_saved: cudaMallocAsync failed"));
-    }
-    sv->vals = (uint32_t *)sv->blk[1];
-    sv->cap = p.cap;
-    p.vals[0] = sv->vals;  // the sorted lists land in the saved block
-    b = bin_args(P, sv->D, p);
-    const int cur = run_bin(b, s);
-    gsl::RasterArgs r = raster_args(P, sv->D, p, cur, opt);
-    r.out_rgb = rgb;
-    r.out_depth = depth;
-    r.out_alpha = alpha;
-    r.t_final = sv->t_final;
-    r.last = sv->last;
-    gsl::forward(r, false, s);
-    if (cudaGetLastError() != cudaSuccess)
-        return cleanup(fail(ctx, GS_ERR_CUDA, "gs_render_saved: launch"));
     int flags = 0;
-    st = read_flags(ctx, p, s, &flags);
-    if (st != GS_OK)
-        return cleanup(st);
+    bool count_first = seen == ctx->saved_seen.end();
+    uint64_t want = count_first ? 0 : (uint64_t)seen->second + seen->second / 8 + 1024;
+    for (;;) {
+        if (count_first || want > 0xfff00000ull) {
+            if (cudaMemsetAsync(p.flags, 0, sizeof(int), s) != cudaSuccess)
+                return cleanup(fail(ctx, GS_ERR_CUDA, "gs_render_saved: memset"));
+            st = begin_lists(ctx, s);
+            if (st != GS_OK)
+                return cleanup(st);
+            gsl::project(project_args(P, sv->D, p, sv->pose32, opt), s);
+            gsl::BinArgs b = bin_args(P, sv->D, p);
+            gsl::bin_count(b, s);
+            st = read_flags(ctx, p, s, &flags, &nd);
+            if (st != GS_OK)
+                return cleanup(st);
+            if (nd == 0xffffffffu)
+                return cleanup(fail(ctx, GS_ERR_CAPACITY, "more than 2^32 tile duplicates"));
+            want = nd;
+        } else {
+            st = begin_lists(ctx, s);
+            if (st != GS_OK)
+                return cleanup(st);
+            gsl::project(project_args(P, sv->D, p, sv->pose32, opt), s);
+        }
+        st = alloc_sort(ctx, want, p);
+        if (st != GS_OK)
+            return cleanup(st);
+        if (cudaMallocAsync(&sv->blk[1], sizeof(uint32_t) * (size_t)p.cap, s) != cudaSuccess) {
+            cudaGetLastError();
+            sv->blk[1] = nullptr;
+            return cleanup(fail(ctx, GS_ERR_OOM, "gs_render_saved: cudaMallocAsync failed"));
+        }
+        sv->vals = (uint32_t *)sv->blk[1];
+        sv->cap = p.cap;
+        p.vals[0] = sv->vals;  // the sorted lists land in the saved block
+        const int cur = run_bin(ctx, bin_args(P, sv->D, p), s);
+        gsl::RasterArgs r = raster_args(P, sv->D, p, cur, opt);
+        r.out_rgb = rgb;
+        r.out_depth = depth;
+        r.out_alpha = alpha;
+        r.t_final = sv->t_final;
+        r.last = sv->last;
+        gsl::forward(r, false, s);
+        if (cudaGetLastError() != cudaSuccess)
+            return cleanup(fail(ctx, GS_ERR_CUDA, "gs_render_saved: launch"));
+        st = read_flags(ctx, p, s, &flags, &nd);
+        if (st != GS_OK)
+            return cleanup(st);
+        if (!(flags & gsk::kFlagCapacity))
+            break;
+        // the guess was too short
+        cudaFreeAsync(sv->blk[1], s);
+        sv->blk[1] = nullptr;
+        count_first = true;
+    }
+    uint32_t &most = ctx->saved_seen[key];
+    most = std::max(most, nd);
     if (flags & gsk::kFlagNonFinite)
         return cleanup(fail(ctx, GS_ERR_NONFINITE, "non-finite Gaussian parameter"));
     ctx->stats = gs_stats_t{};
@@ -1255,7 +1446,6 @@ gs_status_t gs_render_backward_saved(gs_ctx_t *ctx, const gs_saved_t *saved, con
     p.counts = saved->counts;
     p.ranges = saved->ranges;
     p.vals[0] = saved->vals;
-    p.ndups = saved->ndups;
     p.cap = saved->cap;
     p.n_records = std::max<uint64_t>(P.n_records, 1);
     const bool full = wants_params(grads);
@@ -1776,13 +1966,56 @@ __global__ void k_async_status(const int *flags, const double *eps, int nv, int3
     *status = st;
 }
 
+// The host's results of a registration as one block: {flags, pairs walked,
+// pairs contributing (integers in the doubles' places)}, then the parts.
+struct RegResult {
+    static constexpr int kParts = 5, kHead = 3;
+    const int *flags;
+    const unsigned long long *pairs;  // [2][n_tiles]
+    uint32_t n_tiles;
+    const double *src[kParts];
+    int n[kParts];
+    double *out;
+};
+
+__global__ void __launch_bounds__(1024) k_reg_result(const __grid_constant__ RegResult q)
+{
+    __shared__ unsigned long long s_sum[2][32];
+    unsigned long long sum[2] = {0, 0};
+    for (uint32_t t = threadIdx.x; t < q.n_tiles; t += 1024) {
+        sum[0] += q.pairs[t];
+        sum[1] += q.pairs[q.n_tiles + t];
+    }
+    for (int k = 0; k < 2; ++k) {
+        const unsigned long long w = gsk::warp_sum(sum[k]);
+        if ((threadIdx.x & 31) == 0)
+            s_sum[k][threadIdx.x >> 5] = w;
+    }
+    __syncthreads();
+    unsigned long long *head = reinterpret_cast<unsigned long long *>(q.out);
+    if (threadIdx.x < 2) {
+        unsigned long long w = 0;
+        for (int k = 0; k < 32; ++k)
+            w += s_sum[threadIdx.x][k];
+        head[1 + threadIdx.x] = w;
+    }
+    if (threadIdx.x == 0)
+        q.out[0] = (double)*q.flags;
+    double *out = q.out + RegResult::kHead;
+    for (int k = 0; k < RegResult::kParts; ++k) {
+        for (int i = threadIdx.x; i < q.n[k]; i += 1024)
+            out[i] = q.src[k][i];
+        out += q.n[k];
+    }
+}
+
 gs_status_t run_registration(gs_ctx *ctx, Plan &P, int n_problems, const gs_options_t *opt, int iters,
                              cudaStream_t s, double *T_out, double *conf_out, double *eps_out, double *est_out,
                              const AsyncOut *ao, double *grad_out)
 {
     GS_TRY(finalize(ctx, P));
     DevPlan D;
-    GS_TRY(upload_plan(ctx, P, D, s));
+    GS_TRY(upload_plan(ctx, P, D, s, n_problems));
     const int nv = (int)P.vps.size();
     const int n_sets = (int)P.set_vp.size();
     Pipe p;
@@ -1791,7 +2024,7 @@ gs_status_t run_registration(gs_ctx *ctx, Plan &P, int n_problems, const gs_opti
     double *pose64 = nullptr, *adam = nullptr, *pivot = nullptr, *ccam = nullptr, *cent = nullptr, *lossd = nullptr,
            *Tdev = nullptr, *confd = nullptr, *est = nullptr;
     float2 *ttw = nullptr;
-    int32_t *last = nullptr, *rev = nullptr, *pf = nullptr, *pc = nullptr;
+    int32_t *last = nullptr;
     uint8_t *code = nullptr;
     const size_t npix = (size_t)std::max<int64_t>(P.n_pix, 1), ntl = (size_t)std::max<uint64_t>(P.n_tiles, 1);
     GS_TRY(wsT(ctx, S_POSE32, 12 * (size_t)nv, &pose32));
@@ -1811,17 +2044,6 @@ gs_status_t run_registration(gs_ctx *ctx, Plan &P, int n_problems, const gs_opti
     GS_TRY(wsT(ctx, S_TOUT, 12 * (size_t)n_problems, &Tdev));
     GS_TRY(wsT(ctx, S_CONF, (size_t)n_problems, &confd));
     GS_TRY(wsT(ctx, S_EST, 12 * (size_t)nv, &est));
-    std::vector<int32_t> revh(nv), pfh(n_problems, 0), pch(n_problems, 0);
-    for (int v = 0; v < nv; ++v) {
-        revh[v] = P.vps[v].reverse;
-        const int q = P.vps[v].problem;
-        if (pch[q]++ == 0)
-            pfh[q] = v;
-    }
-    GS_TRY(upload(ctx, S_REV, revh, &rev, s));
-    GS_TRY(upload(ctx, S_PFIRST, pfh, &pf, s));
-    GS_TRY(upload(ctx, S_PCOUNT, pch, &pc, s));
-
     gsl::PoseArgs pa{};
     pa.vps = D.vps;
     pa.n_vps = nv;
@@ -1923,11 +2145,9 @@ gs_status_t run_registration(gs_ctx *ctx, Plan &P, int n_problems, const gs_opti
         };
         auto iteration = [&](cudaStream_t st) {
             mark(0, st);
-            gsl::ProjectArgs pj = project_args(P, D, p, pose32, opt, false);
-            pj.seg_zero_bytes = 0;  // cleared below, and by every build
-            gsl::project(pj, st);
+            gsl::project(project_args(P, D, p, pose32, opt, false), st);
             mark(1, st);
-            const int c = run_bin(b, st);
+            const int c = run_bin(ctx, b, st);
             if (ordered)
                 gsl::tile_order(p.ranges, (uint32_t)P.n_tiles, order, order_cnt, st);
             mark(2, st);
@@ -1972,7 +2192,7 @@ gs_status_t run_registration(gs_ctx *ctx, Plan &P, int n_problems, const gs_opti
         // queue over every keyframe problem) -- timed on trial iterations
         // 1 2 3 4 4 3 2 1 from the initial poses, then the poses start over.
         // Every schedule gives the same results.
-        GS_CUDA(cudaMemsetAsync(p.seg_hdr, 0, p.seg_zero, s));
+        GS_TRY(begin_lists(ctx, s));
         int sched = opt->tile_schedule;
         if (sched == 0) {
             const auto it = ctx->schedule.find(key);
@@ -2081,7 +2301,7 @@ gs_status_t run_registration(gs_ctx *ctx, Plan &P, int n_problems, const gs_opti
         r.tile_order = nullptr;
         r.queue = nullptr;
         gsl::project(project_args(P, D, p, pose32, opt, false), s);
-        r.vals = p.vals[run_bin(b, s)];
+        r.vals = p.vals[run_bin(ctx, b, s)];
         gsl::forward(r, true, s);
         gsl::track_loss(ta, s);
         gsl::PoseArgs fa = pa;
@@ -2091,9 +2311,9 @@ gs_status_t run_registration(gs_ctx *ctx, Plan &P, int n_problems, const gs_opti
         gsl::FuseArgs f{};
         f.pose64 = pose64;
         f.eps = lossd;
-        f.reverse = rev;
-        f.prob_first = pf;
-        f.prob_count = pc;
+        f.reverse = D.rev;
+        f.prob_first = D.prob_first;
+        f.prob_count = D.prob_count;
         f.n_problems = n_problems;
         f.T_out = Tdev;
         f.conf = confd;
@@ -2120,8 +2340,32 @@ gs_status_t run_registration(gs_ctx *ctx, Plan &P, int n_problems, const gs_opti
             st.schedule = sched_run;
             return GS_OK;
         }
-        int flags = 0;
-        GS_TRY(read_flags(ctx, p, s, &flags));
+        // everything the host wants, gathered and read back in one copy
+        RegResult q{};
+        q.flags = p.flags;
+        q.pairs = pairs;
+        q.n_tiles = (uint32_t)ntl;
+        const struct {
+            const double *src;
+            int n;
+        } part[RegResult::kParts] = {
+            {Tdev, 12 * n_problems}, {confd, n_problems}, {lossd, nv}, {est_out ? est : nullptr, 12 * nv},
+            {grad_out ? gradd : nullptr, 6 * nv}};
+        int total = RegResult::kHead;
+        for (int k = 0; k < RegResult::kParts; ++k) {
+            q.src[k] = part[k].src;
+            q.n[k] = part[k].src ? part[k].n : 0;
+            total += q.n[k];
+        }
+        GS_TRY(wsT(ctx, S_RESULT, (size_t)total, &q.out));
+        k_reg_result<<<1, 1024, 0, s>>>(q);
+        ++gsl::g_launches;
+        void *hostp = nullptr;
+        GS_TRY(host_block(ctx, total * sizeof(double), &hostp));
+        GS_CUDA(cudaMemcpyAsync(hostp, q.out, total * sizeof(double), cudaMemcpyDeviceToHost, s));
+        GS_CUDA(cudaStreamSynchronize(s));
+        const double *res = (const double *)hostp;
+        const int flags = (int)res[0];
         if (flags & gsk::kFlagNonFinite)
             return fail(ctx, GS_ERR_NONFINITE, "non-finite Gaussian parameter");
         if (flags & gsk::kFlagTimeout)
@@ -2130,28 +2374,23 @@ gs_status_t run_registration(gs_ctx *ctx, Plan &P, int n_problems, const gs_opti
             headroom = std::max(2.0 * headroom, 1.5);  // the lists outgrew the headroom: redo with more
             continue;
         }
-        std::vector<double> epsh(nv);
-        std::vector<unsigned long long> pairs_h(2 * ntl);
-        GS_CUDA(cudaMemcpyAsync(T_out, Tdev, 12 * sizeof(double) * n_problems, cudaMemcpyDeviceToHost, s));
-        GS_CUDA(cudaMemcpyAsync(conf_out, confd, sizeof(double) * n_problems, cudaMemcpyDeviceToHost, s));
-        GS_CUDA(cudaMemcpyAsync(epsh.data(), lossd, nv * sizeof(double), cudaMemcpyDeviceToHost, s));
-        GS_CUDA(cudaMemcpyAsync(pairs_h.data(), pairs, 2 * ntl * sizeof(unsigned long long), cudaMemcpyDeviceToHost,
-                                s));
-        if (est_out)
-            GS_CUDA(cudaMemcpyAsync(est_out, est, 12 * nv * sizeof(double), cudaMemcpyDeviceToHost, s));
-        if (grad_out)
-            GS_CUDA(cudaMemcpyAsync(grad_out, gradd, 6 * nv * sizeof(double), cudaMemcpyDeviceToHost, s));
-        GS_CUDA(cudaStreamSynchronize(s));
+        double *dst[RegResult::kParts] = {T_out, conf_out, eps_out, est_out, grad_out};
+        const double *at = res + RegResult::kHead, *epsh = nullptr;
+        for (int k = 0; k < RegResult::kParts; ++k) {
+            if (k == 2)
+                epsh = at;
+            if (dst[k] && q.n[k])
+                std::memcpy(dst[k], at, q.n[k] * sizeof(double));
+            at += q.n[k];
+        }
         gs_stats_t &st = ctx->stats;
         st.kernel_launches = (gsl::g_launches - l0) - captured + graph_kernels * iters + trial_kernels;
         st.n_dups = nd;
         st.n_pixels = P.n_pix;
         st.iterations = iters;
         st.schedule = sched_run;
-        for (size_t k = 0; k < ntl; ++k) {
-            st.pairs += (int64_t)pairs_h[k];
-            st.contributing += (int64_t)pairs_h[ntl + k];
-        }
+        st.pairs = (int64_t)((const unsigned long long *)res)[1];
+        st.contributing = (int64_t)((const unsigned long long *)res)[2];
         if (prof)
             for (int it = 0; it < iters; ++it)
                 for (int k = 0; k < kPhases; ++k) {
@@ -2160,10 +2399,8 @@ gs_status_t run_registration(gs_ctx *ctx, Plan &P, int n_problems, const gs_opti
                                              ctx->pool[(size_t)it * (kPhases + 1) + k + 1]) == cudaSuccess)
                         st.phase_ms[k] += ms;
                 }
-        if (eps_out)
-            std::memcpy(eps_out, epsh.data(), nv * sizeof(double));
-        for (double e : epsh)
-            if (!std::isfinite(e))
+        for (int v = 0; v < nv; ++v)
+            if (!std::isfinite(epsh[v]))
                 return fail(ctx, GS_ERR_DIVERGED, "registration residual is not finite");
         return GS_OK;
     }
@@ -2286,7 +2523,7 @@ extern "C" gs_status_t gs_render_noalloc(const gs_gaussians_t *g, const float *p
     const size_t R = P.n_records ? P.n_records : 1;
     VpDesc *vps = cv.take<VpDesc>(P.vps.size());
     GroupDesc *groups = cv.take<GroupDesc>(P.groups.size());
-    uint32_t *tile_vp = cv.take<uint32_t>(P.tile_vp.size());
+    uint32_t *tile_vp = cv.take<uint32_t>((size_t)P.n_tiles);
     Pipe p;
     p.rec = cv.take<float4>(3 * R);
     p.counts = cv.take<int32_t>(R);
@@ -2296,21 +2533,14 @@ extern "C" gs_status_t gs_render_noalloc(const gs_gaussians_t *g, const float *p
     p.ranges = cv.take<uint2>(P.n_tiles ? P.n_tiles : 1);
     if (!vps || !groups || !tile_vp || !p.rec || !p.counts || !p.partials || !p.ndups || !p.flags || !p.ranges)
         return GS_ERR_CAPACITY;
-    if (!P.vps.empty() && cudaMemcpyAsync(vps, P.vps.data(), P.vps.size() * sizeof(VpDesc), cudaMemcpyHostToDevice,
-                                          s) != cudaSuccess)
-        return GS_ERR_CUDA;
-    if (!P.groups.empty() && cudaMemcpyAsync(groups, P.groups.data(), P.groups.size() * sizeof(GroupDesc),
-                                             cudaMemcpyHostToDevice, s) != cudaSuccess)
-        return GS_ERR_CUDA;
-    if (!P.tile_vp.empty() && cudaMemcpyAsync(tile_vp, P.tile_vp.data(), P.tile_vp.size() * sizeof(uint32_t),
-                                              cudaMemcpyHostToDevice, s) != cudaSuccess)
-        return GS_ERR_CUDA;
     DevPlan D;
     D.vps = vps;
     D.groups = groups;
     D.tile_vp = tile_vp;
-    // the scratch keeps the previous call's contents: clear the status word
-    if (cudaMemsetAsync(p.flags, 0, sizeof(int), s) != cudaSuccess)
+    // the scratch keeps the previous call's contents: the status word is
+    // cleared with the plan's tables
+    send_plan(P, D, 0, p.flags, s);
+    if (cudaGetLastError() != cudaSuccess)
         return GS_ERR_CUDA;
     gsl::project(project_args(P, D, p, poses, opt), s);
     gsl::BinArgs b = bin_args(P, D, p);
@@ -2404,7 +2634,7 @@ struct gs_server {
     double *pose64 = nullptr, *adam = nullptr, *pivot = nullptr, *ccam = nullptr, *cent = nullptr,
            *lossd = nullptr, *Tdev = nullptr, *confd = nullptr;
     float2 *ttw = nullptr;
-    int32_t *last = nullptr, *rev = nullptr, *pf = nullptr, *pc = nullptr;
+    int32_t *last = nullptr;
     uint8_t *code = nullptr;
     gsl::PoseArgs pa{};
     cudaGraphExec_t exec = nullptr;
@@ -2469,6 +2699,7 @@ gs_status_t srv_measure(gs_server *srv, ServerReq &r)
     float *pose32 = nullptr;
     GS_TRY(upload(ctx, S_POSE32, ident, &pose32, s));
     GS_CUDA(cudaMemsetAsync(p.flags, 0, sizeof(int), s));
+    GS_TRY(begin_lists(ctx, s));
     gsl::project(project_args(P, D, p, pose32, &r.opt), s);
     gsl::BinArgs b = bin_args(P, D, p);
     gsl::bin_count(b, s);
@@ -2535,7 +2766,7 @@ gs_status_t srv_replan(gs_server *srv, cudaStream_t s)
     }
     GS_TRY(finalize(ctx, P));
     DevPlan &D = srv->D;
-    GS_TRY(upload_plan(ctx, P, D, s));
+    GS_TRY(upload_plan(ctx, P, D, s, (int)srv->active.size()));
     const int nv = (int)P.vps.size(), n_sets = (int)P.set_vp.size(), np = (int)srv->active.size();
     srv->n_vps = nv;
     srv->n_problems = np;
@@ -2559,17 +2790,6 @@ gs_status_t srv_replan(gs_server *srv, cudaStream_t s)
     GS_TRY(wsT(ctx, S_TTWIST, 6 * ntl, &srv->ttw));
     GS_TRY(wsT(ctx, S_TOUT, 12 * (size_t)np, &srv->Tdev));
     GS_TRY(wsT(ctx, S_CONF, (size_t)np, &srv->confd));
-    std::vector<int32_t> revh(nv), pfh(np, 0), pch(np, 0);
-    for (int v = 0; v < nv; ++v) {
-        revh[v] = P.vps[v].reverse;
-        const int q = P.vps[v].problem;
-        if (pch[q]++ == 0)
-            pfh[q] = v;
-    }
-    GS_TRY(upload(ctx, S_REV, revh, &srv->rev, s));
-    GS_TRY(upload(ctx, S_PFIRST, pfh, &srv->pf, s));
-    GS_TRY(upload(ctx, S_PCOUNT, pch, &srv->pc, s));
-
     gsl::PoseArgs &pa = srv->pa;
     pa = gsl::PoseArgs{};
     pa.vps = D.vps;
@@ -2636,12 +2856,10 @@ gs_status_t srv_replan(gs_server *srv, cudaStream_t s)
     r.exposure = any_exposure(P);
     gsl::TrackArgs ta;
     GS_TRY(alloc_track(ctx, P, D, r, ta, srv->tloss, s));
-    GS_CUDA(cudaMemsetAsync(p.seg_hdr, 0, p.seg_zero, s));
-    gsl::ProjectArgs pj = project_args(P, D, p, srv->pose32, &srv->opt, false);
-    pj.seg_zero_bytes = 0;  // cleared above, and by every build
+    GS_TRY(begin_lists(ctx, s));
     GS_CUDA(cudaStreamBeginCapture(ctx->cap, cudaStreamCaptureModeThreadLocal));
-    gsl::project(pj, ctx->cap);
-    r.vals = p.vals[run_bin(b, ctx->cap)];
+    gsl::project(project_args(P, D, p, srv->pose32, &srv->opt, false), ctx->cap);
+    r.vals = p.vals[run_bin(ctx, b, ctx->cap)];
     if (srv->opt.fuse_compositing && ta.n_track == 0) {
         gsl::forward_backward(r, ctx->cap);
     } else {
@@ -2733,9 +2951,9 @@ gs_status_t srv_round(gs_server *srv, cudaStream_t s, int64_t *done_ids, int max
         gsl::FuseArgs f{};
         f.pose64 = srv->pose64;
         f.eps = srv->lossd;
-        f.reverse = srv->rev;
-        f.prob_first = srv->pf;
-        f.prob_count = srv->pc;
+        f.reverse = srv->D.rev;
+        f.prob_first = srv->D.prob_first;
+        f.prob_count = srv->D.prob_count;
         f.n_problems = srv->n_problems;
         f.T_out = srv->Tdev;
         f.conf = srv->confd;

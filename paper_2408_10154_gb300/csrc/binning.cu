@@ -1221,8 +1221,6 @@ size_t seg_zero_bytes(int n_vps, uint64_t n_diff)
 
 int bin_seg(const BinArgs &a, cudaStream_t s)
 {
-    if (!a.seg_counted)
-        cudaMemsetAsync(a.seg_hdr, 0, a.seg_zero_bytes, s);
     if (a.n_vps == 0) {
         cudaMemsetAsync(a.n_dups, 0, sizeof(uint32_t), s);
         return 0;

@@ -188,7 +188,8 @@ __device__ __forceinline__ void compose_ct(const float *V, const float *T, float
 }
 
 // ------------------------------------------------------------------------
-// Programmatic dependent launch.  The kernels of an iteration are launched
+// Programmatic dependent launch.  The kernels of an iteration (all but its
+// first, which follows the tables' upload or another iteration) are launched
 // so that each may start as its predecessor's last blocks end, before the
 // predecessor has completed (launch_pdl); pdl_wait() holds it until every
 // kernel before it has completed and its stores are visible (a no-op in an
@@ -310,13 +311,11 @@ struct ProjectArgs {
     // (and list positions such as `last`) are shorter.
     int tight;
     float alpha_min;          // the threshold of the tight rectangles
-    // segmented tile lists (null: not built here): clears seg_hdr/seg_diff
-    // (seg_zero_bytes, unless 0: a build before left them clear), then every visible record adds its rectangle to its
-    // keyframe's difference grid, and every record writes its seg_list
-    // entry (see BinArgs)
+    // segmented tile lists (null: not built here): every visible record adds
+    // its rectangle to its keyframe's difference grid (clear before), and
+    // every record writes its seg_list entry (see BinArgs)
     unsigned long long *seg_hdr;
     uint32_t *seg_diff;
-    size_t seg_zero_bytes;
     uint4 *seg_list;
 };
 void project(const ProjectArgs &a, cudaStream_t s);
@@ -346,15 +345,14 @@ struct BinArgs {
     uint32_t *tkeys[2];             // [capacity] segmented build: depth bits of the placed entries (tkeys[0])
     // segmented build (bin_seg): seg_hdr[v] holds keyframe v's duplicate
     // total, and the difference grids (VpDesc::diff_base) follow in the same
-    // allocation of seg_zero_bytes, cleared before the first build and left
+    // allocation (seg_zero_bytes), clear before the first build and left
     // clear by every build.
     // seg_list: per record {depth bits, first tile, width | height << 16,
     // tiles per row} (size 0: not visible).  seg_counted: the projection has
-    // already cleared, counted and written the entries (ProjectArgs::seg_*);
+    // already counted and written the entries (ProjectArgs::seg_*);
     // otherwise bin_seg does it from rec / counts.
     unsigned long long *seg_hdr;
     uint32_t *seg_diff;
-    size_t seg_zero_bytes;
     uint4 *seg_list;     // [n_records]
     int seg_counted;
     uint32_t *seg_cursor;  // [n_tiles] placement cursors

@@ -219,7 +219,7 @@ __global__ void __launch_bounds__(256) k_project(const gsl::ProjectArgs a)
     const int i = (int)(blockIdx.x - G.blk_base) * blockDim.x + threadIdx.x;
     const int i_warp = i - lane;  // the warp's first Gaussian
     const bool mine = i < G.n;
-    // the Gaussian (an input: loaded ahead of the kernels before)
+    // the Gaussian, loaded while the keyframes' poses are composed
     float4 mu = make_float4(0.0f, 0.0f, 0.0f, 0.0f), sc = mu, q = mu, col = mu;
     float logit = 0.0f;
     if (mine) {
@@ -230,7 +230,6 @@ __global__ void __launch_bounds__(256) k_project(const gsl::ProjectArgs a)
         logit = __ldg(d0.logits + i);
         col = __ldg(d0.rgb + i);
     }
-    pdl_wait();
     for (int v = threadIdx.x; v < G.vp_count; v += blockDim.x) {
         const int vp = G.vp_first + v;
         const VpDesc &d = a.vps[vp];
@@ -351,11 +350,10 @@ namespace gsl {
 
 void project(const ProjectArgs &a, cudaStream_t s)
 {
-    if (a.seg_hdr && a.seg_zero_bytes)
-        cudaMemsetAsync(a.seg_hdr, 0, a.seg_zero_bytes, s);
     if (a.n_blocks == 0)
         return;
-    launch_pdl(k_project, a.n_blocks, 256, 0, s, a);
+    k_project<<<a.n_blocks, 256, 0, s>>>(a);
+    ++g_launches;
 }
 
 }  // namespace gsl

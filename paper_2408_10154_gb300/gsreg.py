@@ -184,19 +184,22 @@ def default_options(**kw) -> gs_options_t:
     return o
 
 
+def _camera_words(cams):
+    """cam18 rows as gs_camera_t words: the float32 row with the image size
+    (columns 4 and 5) as int32."""
+    c = np.array(cams, np.float32).reshape(-1, 18)
+    c.view(np.int32)[:, 4:6] = c[:, 4:6].astype(np.int32)
+    return c
+
+
 def camera(cam18) -> gs_camera_t:
-    c = np.asarray(cam18, np.float32).reshape(18)
-    out = gs_camera_t(float(c[0]), float(c[1]), float(c[2]), float(c[3]), int(c[4]), int(c[5]))
-    out.world_to_cam = (ctypes.c_float * 12)(*[float(v) for v in c[6:]])
-    return out
+    return gs_camera_t.from_buffer(_camera_words(np.asarray(cam18, np.float32).reshape(18)))
 
 
 def cameras(cams):
-    cams = np.asarray(cams, np.float32).reshape(-1, 18)
-    arr = (gs_camera_t * len(cams))()
-    for k, c in enumerate(cams):
-        arr[k] = camera(c)
-    return arr, len(cams)
+    c = _camera_words(cams)
+    n = len(c)
+    return ((gs_camera_t * n).from_buffer(c) if n else (gs_camera_t * 0)()), n
 
 
 @dataclass
@@ -257,8 +260,8 @@ class Context:
 
 
 def _npix(cams):
-    c = np.asarray(cams, np.float32).reshape(-1, 18)
-    return int(sum(int(x[4]) * int(x[5]) for x in c))
+    c = np.asarray(cams, np.float32).reshape(-1, 18)[:, 4:6].astype(np.int64)
+    return int((c[:, 0] * c[:, 1]).sum())
 
 
 def gs_project(ctx: Context, g: Gaussians, poses: torch.Tensor, cams, opt=None, with_aux=True):
@@ -462,9 +465,14 @@ def gs_fuse(ctx: Context, est, reverse, eps):
 
 
 def _views(views):
-    arr = (gs_view_t * max(len(views), 1))()
-    for k, (cam18, rgb, depth) in enumerate(views):
-        arr[k] = gs_view_t(rgb.data_ptr(), depth.data_ptr(), camera(cam18))
+    n = len(views)
+    arr = (gs_view_t * max(n, 1))()
+    if n:
+        # gs_view_t: two pointers, then the camera's 18 words (and 8 bytes to the next)
+        w = np.frombuffer(arr, np.uint8).reshape(n, -1)
+        w[:, :16] = np.array([(rgb.data_ptr(), depth.data_ptr()) for _, rgb, depth in views],
+                             np.uint64).view(np.uint8).reshape(n, 16)
+        w[:, 16:88] = _camera_words([np.asarray(c, np.float32).reshape(18) for c, _, _ in views]).view(np.uint8)
     return arr
 
 
@@ -538,12 +546,14 @@ def gs_transform_batch(ctx: Context, maps, Ts):
     """Map adjustment: every submap of ``maps`` moved by its own T (Eq. 8/9)
     in one launch.  Returns new Gaussians per map."""
     n = len(maps)
-    arr = (gs_gaussians_t * max(n, 1))(*[g.c_struct() for g in maps])
     Th = np.ascontiguousarray(np.asarray(Ts, np.float64).reshape(n, 12))
     outs = [(torch.empty_like(g.means4), torch.empty_like(g.quats4)) for g in maps]
-    om = (ctypes.c_void_p * max(n, 1))(*[m.data_ptr() for m, _ in outs])
-    oq = (ctypes.c_void_p * max(n, 1))(*[q.data_ptr() for _, q in outs])
-    ctx.check(ctx._lib.gs_transform_batch(ctx.handle, arr, n, Th.ctypes.data_as(ctypes.c_void_p), om, oq, _stream()))
+    # gs_gaussians_t rows (five pointers and n), and the output pointers
+    arr = np.array([(g.means4.data_ptr(), g.log_scales4.data_ptr(), g.quats4.data_ptr(), g.logits.data_ptr(),
+                     g.rgb4.data_ptr(), g.n) for g in maps], np.uint64).reshape(n, 6)
+    out = np.array([[m.data_ptr() for m, _ in outs], [q.data_ptr() for _, q in outs]], np.uint64)
+    d = lambda a: a.ctypes.data_as(ctypes.c_void_p)
+    ctx.check(ctx._lib.gs_transform_batch(ctx.handle, d(arr), n, d(Th), d(out[0]), d(out[1]), _stream()))
     return [Gaussians(m, g.log_scales4, q, g.logits, g.rgb4) for g, (m, q) in zip(maps, outs)]
 
 
