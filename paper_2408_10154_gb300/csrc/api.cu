@@ -24,7 +24,7 @@ enum Slot {
     S_VPS, S_GROUPS, S_TILEVP, S_POSE32, S_REC, S_AUX, S_COUNTS, S_PARTIALS, S_K0, S_V0, S_RANGES, S_FLAGS, S_TF, S_LAST, S_CODE, S_TLOSS, S_TTWIST, S_POSE64, S_ADAM, S_PIVOT,
     S_CCAM, S_CENT, S_CENTP, S_LOSS, S_SETVP, S_REV, S_PFIRST, S_PCOUNT, S_RESULT, S_TOUT, S_CONF, S_EST, S_GRAD, S_DUPG,
     S_PAIRS, S_RSLOT, S_RSLOTN, S_TERR, S_TCOL, S_TW,
-    S_TMED, S_TNV, S_TVPS, S_EXPO, S_EXPO32, S_TEXPO, S_OPT, S_ONN1, S_ONN2, S_OD2, S_OHDR, S_MAPS, S_OS, S_ORDER, S_ORDC, S_SK, S_SV, S_SN, S_GCELL, S_GCOUNT, S_GSTART, S_GSUMS, S_GPTS, S_GLIST, S_SEGZ, S_SEGCUR, S_SEGLIST, S_PROBE, S_QUEUE, S_COUNT
+    S_TMED, S_TNV, S_TVPS, S_EXPO, S_EXPO32, S_TEXPO, S_OPT, S_ONN1, S_ONN2, S_OD2, S_OHDR, S_MAPS, S_OS, S_ORDER, S_ORDC, S_SK, S_SV, S_SN, S_GCELL, S_GCOUNT, S_GSTART, S_GSUMS, S_GPTS, S_GLIST, S_SEGZ, S_SEGCUR, S_SEGEXT, S_SEGLIST, S_PROBE, S_QUEUE, S_COUNT
 };
 
 struct Buf {
@@ -444,11 +444,11 @@ struct Pipe {
     uint2 *ranges = nullptr;
     int *flags = nullptr;
     uint32_t cap = 0;
-    uint32_t *tkeys[2] = {nullptr, nullptr};
+    uint64_t *ents = nullptr;
     uint64_t n_records = 0;
     // segmented build
     unsigned long long *seg_hdr = nullptr;
-    uint32_t *seg_diff = nullptr, *seg_cursor = nullptr;
+    uint32_t *seg_diff = nullptr, *seg_ext = nullptr, *seg_cursor = nullptr;
     uint4 *seg_list = nullptr;
 };
 
@@ -472,6 +472,7 @@ gs_status_t alloc_seg(gs_ctx *ctx, const Plan &P, Pipe &p)
         ctx->seg_dirty = true;
     p.seg_hdr = (unsigned long long *)z;
     p.seg_diff = (uint32_t *)(p.seg_hdr + P.vps.size());
+    GS_TRY(wsT(ctx, S_SEGEXT, R, &p.seg_ext));
     GS_TRY(wsT(ctx, S_SEGLIST, R, &p.seg_list));
     GS_TRY(wsT(ctx, S_SEGCUR, T, &p.seg_cursor));
     return GS_OK;
@@ -498,7 +499,7 @@ gs_status_t alloc_sort(gs_ctx *ctx, uint64_t want, Pipe &p)
     if (want > 0xfff00000ull)
         return fail(ctx, GS_ERR_CAPACITY, "more than 2^32 tile duplicates");
     const uint32_t cap = (uint32_t)std::max<uint64_t>(want, 1024);
-    GS_TRY(wsT(ctx, S_K0, cap, &p.tkeys[0]));
+    GS_TRY(wsT(ctx, S_K0, cap, &p.ents));
     GS_TRY(wsT(ctx, S_V0, cap, &p.vals[0]));
     p.cap = cap;
     return GS_OK;
@@ -546,6 +547,7 @@ gsl::ProjectArgs project_args(const Plan &P, const DevPlan &D, const Pipe &p, co
     // the projection counts and lists for the segmented build (run_bin follows every projection here)
     a.seg_hdr = p.seg_hdr;
     a.seg_diff = p.seg_diff;
+    a.seg_ext = p.seg_ext;
     a.seg_list = p.seg_list;
     return a;
 }
@@ -571,10 +573,11 @@ gsl::BinArgs bin_args(const Plan &P, const DevPlan &D, const Pipe &p)
     b.ranges = p.ranges;
     b.n_tiles = (uint32_t)P.n_tiles;
     b.flags = p.flags;
-    b.tkeys[0] = p.tkeys[0];
+    b.ents = p.ents;
     b.seg_hdr = p.seg_hdr;
     b.seg_diff = p.seg_diff;
     b.seg_cursor = p.seg_cursor;
+    b.seg_ext = p.seg_ext;
     b.seg_list = p.seg_list;
     b.seg_counted = 1;
     for (const VpDesc &d : P.vps) {
@@ -646,10 +649,10 @@ gs_status_t read_flags(gs_ctx *ctx, const Pipe &p, cudaStream_t s, int *flags, u
 bool lists_at_hand(const gs_ctx *ctx, Pipe &p)
 {
     const Buf &k = ctx->bufs[S_K0], &v = ctx->bufs[S_V0];
-    const size_t cap = std::min(std::min(k.bytes, v.bytes) / sizeof(uint32_t), (size_t)0xfff00000u);
+    const size_t cap = std::min(std::min(k.bytes / sizeof(uint64_t), v.bytes / sizeof(uint32_t)), (size_t)0xfff00000u);
     if (cap == 0)
         return false;
-    p.tkeys[0] = (uint32_t *)k.p;
+    p.ents = (uint64_t *)k.p;
     p.vals[0] = (uint32_t *)v.p;
     p.cap = (uint32_t)cap;
     return true;
@@ -2650,9 +2653,8 @@ double srv_now(const gs_server *srv)
 // Scratch of a request in a plan, from its measured tile duplicates nd:
 // per record 100 B (record 48, auxiliary 32, count 4, list entry 16); per
 // list entry of capacity (headroom x nd; a plan's 64 Ki spare entries come
-// out of the arena's slack) 12.5 B (depth bits, value, and 4.5 B to
-// spare); per pixel 9 B (final transmittance,
-// last contributor, loss sign code), 12 B more for tracking masks; per tile
+// out of the arena's slack) 12.5 B (entry 8, sorted value 4); per pixel 9 B
+// (final transmittance, last contributor, loss sign code), 12 B more for tracking masks; per tile
 // 92 B (range, keyframe, loss, twist, counters, cursors, order); per
 // keyframe problem its FP64 optimiser state.
 size_t footprint_bytes(const ServerReq &r, int64_t nd, double headroom)

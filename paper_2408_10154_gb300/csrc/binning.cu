@@ -567,7 +567,7 @@ constexpr int kSegThreads = 256;
 // context paths do this inside the projection): a valid visible record adds
 // its rectangle to its keyframe's difference grid (+1 at (y0, x0) and
 // (y1, x1), -1 mod 2^32 at (y0, x1) and (y1, x0));
-// every record writes its entry (size 0 when not taking part).
+// every record writes its extent (0 when not taking part).
 __global__ void __launch_bounds__(kSegThreads) k_seg_collect(const gsl::BinArgs a)
 {
     const uint32_t r = blockIdx.x * kSegThreads + threadIdx.x;
@@ -577,7 +577,7 @@ __global__ void __launch_bounds__(kSegThreads) k_seg_collect(const gsl::BinArgs 
     const int vp = c > 0 ? vp_of_record(a.vps, a.n_vps, r) : 0;
     const VpDesc &d = a.vps[vp];
     const SegRect q = c > 0 ? seg_rect(a.rec, r) : SegRect{0, 0, 0, 0};
-    uint4 e = make_uint4(0u, 0u, 0u, 0u);
+    uint32_t ext = 0;
     if (c > 0 && seg_valid(q, d, c)) {
         const uint32_t w1 = (uint32_t)d.TX + 1;
         uint32_t *g = a.seg_diff + d.diff_base;
@@ -585,11 +585,12 @@ __global__ void __launch_bounds__(kSegThreads) k_seg_collect(const gsl::BinArgs 
         atomicAdd(g + q.y1 * w1 + q.x1, 1u);
         atomicAdd(g + q.y0 * w1 + q.x1, 0xffffffffu);
         atomicAdd(g + q.y1 * w1 + q.x0, 0xffffffffu);
-        e = make_uint4(__float_as_uint(a.rec[3 * (size_t)r + 1].z), d.tile_base + q.y0 * (uint32_t)d.TX + q.x0,
-                       (q.x1 - q.x0) | ((q.y1 - q.y0) << 16), (uint32_t)d.TX);
+        ext = (q.x1 - q.x0) | ((q.y1 - q.y0) << 16);
+        a.seg_list[r] = make_uint4(__float_as_uint(a.rec[3 * (size_t)r + 1].z),
+                                   d.tile_base + q.y0 * (uint32_t)d.TX + q.x0, (uint32_t)d.TX, 0u);
         atomicAdd(a.seg_hdr + vp, (unsigned long long)c);
     }
-    a.seg_list[r] = e;
+    a.seg_ext[r] = ext;
 }
 
 constexpr int kSegTileThreads = 512;
@@ -786,20 +787,22 @@ __global__ void __launch_bounds__(kSegTileThreads) k_seg_ranges(const gsl::BinAr
 }
 
 constexpr uint32_t kSegSmall = 4;  // tiles of a record placed by its own thread; more: by the whole warp
-constexpr int kSegPerThread = 2;    // records per thread (more cursor atomics in flight per warp)
 constexpr int kSegRounds = 8;       // a large record: rounds of 32 tiles whose atomics are in flight together
 
-// kSegPerThread records per thread (kSegThreads apart, so each load is
-// coalesced): a visible one writes (depth bits, record) into the lists of
-// the tiles of its rectangle (from its seg_list entry) at positions taken
-// from the tiles' cursors, all cursor atomics of the thread in flight
-// before its stores.  Records with more than kSegSmall tiles are spread over
-// the lanes of their warp, one record at a time, so a splat covering
-// thousands of tiles does not serialise one thread, kSegRounds rounds of 32
-// tiles with all their atomics in flight before the stores (a record over a
-// whole 1200x680 frame is 101 rounds: one atomic round trip each made it
-// the kernel's critical path).  Positions at or past the capacity are
-// dropped (the capacity flag is already set).
+// PER records per thread (kSegThreads apart, so each load is coalesced): a
+// visible one writes its entry (depth bits << 32 | record, one 8 B store)
+// into the lists of the tiles of its rectangle at positions taken from the
+// tiles' cursors, all cursor atomics of the thread in flight before its
+// stores.  Records with more than kSegSmall tiles are spread over the lanes
+// of their warp, one record at a time, so a splat covering thousands of tiles
+// does not serialise one thread, kSegRounds rounds of 32 tiles with all their
+// atomics in flight before the stores (a record over a whole 1200x680 frame
+// is 101 rounds: one atomic round trip each made it the kernel's critical
+// path).  Positions at or past the capacity are dropped (the capacity flag
+// is already set).  Bound by the cursor atomics' latency: 60.6 us for the room
+// edge's 2.4 M records (66.9 with two 4 B stores per entry and 16 B read per
+// record), 5.9 us (6.8) for 8,000.
+template <int PER>
 __global__ void __launch_bounds__(kSegThreads) k_seg_place(const gsl::BinArgs a)
 {
     const int lane = threadIdx.x & 31;
@@ -807,31 +810,25 @@ __global__ void __launch_bounds__(kSegThreads) k_seg_place(const gsl::BinArgs a)
     if (blockIdx.x == 0)
         for (int v = threadIdx.x; v < a.n_vps; v += kSegThreads)
             a.seg_hdr[v] = 0;
-    uint32_t cnt[kSegPerThread], t0[kSegPerThread], w[kSegPerThread], tx[kSegPerThread], zb[kSegPerThread],
-        rr[kSegPerThread];
+    uint32_t ext[PER], cnt[PER], t0[PER], w[PER], tx[PER], zb[PER], rr[PER];
 #pragma unroll
-    for (int q = 0; q < kSegPerThread; ++q) {
-        const uint32_t r = (blockIdx.x * kSegPerThread + q) * kSegThreads + threadIdx.x;
-        rr[q] = r;
-        cnt[q] = 0;
-        t0[q] = 0;
-        w[q] = 1;
-        tx[q] = 0;
-        zb[q] = 0;
-        if (r < a.n_records) {
-            const uint4 e = a.seg_list[r];
-            if (e.z) {
-                zb[q] = e.x;
-                t0[q] = e.y;
-                w[q] = e.z & 0xffffu;
-                cnt[q] = w[q] * (e.z >> 16);
-                tx[q] = e.w;
-            }
-        }
+    for (int q = 0; q < PER; ++q) {
+        rr[q] = (blockIdx.x * PER + q) * kSegThreads + threadIdx.x;
+        ext[q] = rr[q] < a.n_records ? a.seg_ext[rr[q]] : 0u;
     }
-    uint32_t pos[kSegPerThread][kSegSmall];
 #pragma unroll
-    for (int q = 0; q < kSegPerThread; ++q) {
+    for (int q = 0; q < PER; ++q) {
+        w[q] = max(ext[q] & 0xffffu, 1u);
+        cnt[q] = w[q] * (ext[q] >> 16);
+        const uint4 e = cnt[q] ? a.seg_list[rr[q]] : make_uint4(0u, 0u, 0u, 0u);
+        zb[q] = e.x;
+        t0[q] = e.y;
+        tx[q] = e.z;
+    }
+    uint64_t *ents = a.ents;
+    uint32_t pos[PER][kSegSmall];
+#pragma unroll
+    for (int q = 0; q < PER; ++q) {
         if (cnt[q] > kSegSmall)
             continue;
         uint32_t col = 0, row = t0[q];
@@ -847,19 +844,16 @@ __global__ void __launch_bounds__(kSegThreads) k_seg_place(const gsl::BinArgs a)
         }
     }
 #pragma unroll
-    for (int q = 0; q < kSegPerThread; ++q) {
+    for (int q = 0; q < PER; ++q) {
         if (cnt[q] > kSegSmall)
             continue;
 #pragma unroll
-        for (uint32_t k = 0; k < kSegSmall; ++k) {
-            if (k < cnt[q] && pos[q][k] < a.capacity) {
-                a.tkeys[0][pos[q][k]] = zb[q];
-                a.vals[0][pos[q][k]] = rr[q];
-            }
-        }
+        for (uint32_t k = 0; k < kSegSmall; ++k)
+            if (k < cnt[q] && pos[q][k] < a.capacity)
+                ents[pos[q][k]] = ((uint64_t)zb[q] << 32) | rr[q];
     }
 #pragma unroll
-    for (int q = 0; q < kSegPerThread; ++q) {
+    for (int q = 0; q < PER; ++q) {
         unsigned m = __ballot_sync(0xffffffffu, cnt[q] > kSegSmall);
         while (m) {
             const int src = __ffs(m) - 1;
@@ -868,20 +862,18 @@ __global__ void __launch_bounds__(kSegThreads) k_seg_place(const gsl::BinArgs a)
             const uint32_t ww = __shfl_sync(0xffffffffu, w[q], src), tt = __shfl_sync(0xffffffffu, tx[q], src);
             const uint32_t z = __shfl_sync(0xffffffffu, zb[q], src), r = __shfl_sync(0xffffffffu, rr[q], src);
             for (uint32_t k0 = 0; k0 < c; k0 += 32 * kSegRounds) {
-                uint32_t pos[kSegRounds];
+                uint32_t at[kSegRounds];
 #pragma unroll
                 for (int u = 0; u < kSegRounds; ++u) {
                     const uint32_t k = k0 + 32 * u + lane;
                     if (k < c)
-                        pos[u] = atomicAdd(a.seg_cursor + b + (k / ww) * tt + k % ww, 1u);
+                        at[u] = atomicAdd(a.seg_cursor + b + (k / ww) * tt + k % ww, 1u);
                 }
 #pragma unroll
                 for (int u = 0; u < kSegRounds; ++u) {
                     const uint32_t k = k0 + 32 * u + lane;
-                    if (k < c && pos[u] < a.capacity) {
-                        a.tkeys[0][pos[u]] = z;
-                        a.vals[0][pos[u]] = r;
-                    }
+                    if (k < c && at[u] < a.capacity)
+                        ents[at[u]] = ((uint64_t)z << 32) | r;
                 }
             }
         }
@@ -964,13 +956,13 @@ __device__ __forceinline__ void warp_bitonic_reg(unsigned long long (&x)[K], int
 }
 
 template <int K>
-__device__ __forceinline__ void sort_list_reg(const uint32_t *keys, uint32_t *vals, uint32_t n, int lane)
+__device__ __forceinline__ void sort_list_reg(const uint64_t *ents, uint32_t *vals, uint32_t n, int lane)
 {
     unsigned long long x[K];
 #pragma unroll
     for (int k = 0; k < K; ++k) {
         const uint32_t e = (uint32_t)(k * 32 + lane);
-        x[k] = e < n ? (((unsigned long long)keys[e] << 32) | vals[e]) : ~0ull;
+        x[k] = e < n ? ents[e] : ~0ull;
     }
     warp_bitonic_reg<K>(x, lane);
 #pragma unroll
@@ -1024,11 +1016,11 @@ __device__ __forceinline__ void block_bitonic(unsigned long long *sk, int N, boo
 }
 
 // One list of n > kSegSortWarpMax entries by the block: in shared memory, a
-// chunk at a time; the merges of a list longer than a chunk exchange
-// (key, value) pairs in global memory at distances of a chunk and more.
-__device__ void block_sort_list(uint32_t *keys, uint32_t *vals, uint32_t n, unsigned long long *sk)
+// chunk at a time; the merges of a list longer than a chunk exchange entries
+// in global memory at distances of a chunk and more.
+__device__ void block_sort_list(uint64_t *ents, uint32_t *vals, uint32_t n, unsigned long long *sk)
 {
-    auto chunk = [&](uint32_t c0, bool first) {
+    auto chunk = [&](uint32_t c0, bool first, bool last) {
         const uint32_t cnt = min(n - c0, (uint32_t)kSegSortChunk);
         int N = 512;
         while ((uint32_t)N < cnt)
@@ -1036,34 +1028,31 @@ __device__ void block_sort_list(uint32_t *keys, uint32_t *vals, uint32_t n, unsi
         if (!first)
             N = kSegSortChunk;
         for (int i = threadIdx.x; i < N; i += kSegSortThreads)
-            sk[i] = (uint32_t)i < cnt ? (((unsigned long long)keys[c0 + i] << 32) | vals[c0 + i]) : ~0ull;
+            sk[i] = (uint32_t)i < cnt ? ents[c0 + i] : ~0ull;
         __syncthreads();
         block_bitonic(sk, N, first);
         for (uint32_t i = threadIdx.x; i < cnt; i += kSegSortThreads) {
-            keys[c0 + i] = (uint32_t)(sk[i] >> 32);
-            vals[c0 + i] = (uint32_t)sk[i];
+            if (last)
+                vals[c0 + i] = (uint32_t)sk[i];
+            else
+                ents[c0 + i] = sk[i];
         }
         __syncthreads();
-    };
-    for (uint32_t c0 = 0; c0 < n; c0 += kSegSortChunk)
-        chunk(c0, true);
-    if (n <= (uint32_t)kSegSortChunk)
-        return;
-    auto ce = [&](uint64_t i, uint64_t p) {
-        if (p >= n)
-            return;  // +infinity past the end
-        const unsigned long long u = ((unsigned long long)keys[i] << 32) | vals[i];
-        const unsigned long long w = ((unsigned long long)keys[p] << 32) | vals[p];
-        if (u > w) {
-            keys[i] = (uint32_t)(w >> 32);
-            vals[i] = (uint32_t)w;
-            keys[p] = (uint32_t)(u >> 32);
-            vals[p] = (uint32_t)u;
-        }
     };
     uint64_t N = kSegSortChunk;
     while (N < n)
         N <<= 1;
+    for (uint32_t c0 = 0; c0 < n; c0 += kSegSortChunk)
+        chunk(c0, true, N == kSegSortChunk);
+    auto ce = [&](uint64_t i, uint64_t p) {
+        if (p >= n)
+            return;  // +infinity past the end
+        const uint64_t u = ents[i], w = ents[p];
+        if (u > w) {
+            ents[i] = w;
+            ents[p] = u;
+        }
+    };
     for (uint64_t k = 2 * kSegSortChunk; k <= N; k <<= 1) {
         const uint64_t h = k >> 1;
         for (uint64_t q = threadIdx.x; q < (N >> 1); q += kSegSortThreads) {
@@ -1079,7 +1068,7 @@ __device__ void block_sort_list(uint32_t *keys, uint32_t *vals, uint32_t n, unsi
             __syncthreads();
         }
         for (uint32_t c0 = 0; c0 < n; c0 += kSegSortChunk)
-            chunk(c0, false);
+            chunk(c0, false, k == N);
     }
 }
 
@@ -1087,8 +1076,8 @@ __device__ void block_sort_list(uint32_t *keys, uint32_t *vals, uint32_t n, unsi
 // (up to 8 per lane); the block's longer lists follow, one after another, by
 // the whole block.  (A long list used to be sorted by one warp in shared
 // memory up to 512 entries, and beyond that by a launch of its own in
-// global memory, stage by stage.)  The sorted record indices replace the
-// tile's values in place.
+// global memory, stage by stage.)  The sorted entries' record indices are the
+// tile's values.
 __global__ void __launch_bounds__(kSegSortThreads) k_seg_sort(const gsl::BinArgs a)
 {
     __shared__ unsigned long long s_k[kSegSortChunk];
@@ -1099,32 +1088,31 @@ __global__ void __launch_bounds__(kSegSortThreads) k_seg_sort(const gsl::BinArgs
     const uint2 rg = t < a.n_tiles ? a.ranges[t] : make_uint2(0u, 0u);
     const uint32_t n = rg.y - rg.x;
     const bool is_long = n > (uint32_t)kSegSortWarpMax;
-    uint32_t *keys = a.tkeys[0] + rg.x;
+    const uint64_t *ents = a.ents + rg.x;
     uint32_t *vals = a.vals[0] + rg.x;
     if (lane == 0)
         s_long[warp] = is_long ? rg : make_uint2(0u, 0u);
-    if (n <= 1 || is_long) {
+    if (n == 0 || is_long) {
         // (nothing for the warp)
     } else if (n <= 32) {
-        unsigned long long x = ~0ull;
-        if ((uint32_t)lane < n)
-            x = ((unsigned long long)keys[lane] << 32) | vals[lane];
-        x = warp_bitonic32(x, lane);
+        unsigned long long x = (uint32_t)lane < n ? ents[lane] : ~0ull;
+        if (n > 1)
+            x = warp_bitonic32(x, lane);
         if ((uint32_t)lane < n)
             vals[lane] = (uint32_t)x;
     } else if (n <= 64) {
-        sort_list_reg<2>(keys, vals, n, lane);
+        sort_list_reg<2>(ents, vals, n, lane);
     } else if (n <= 128) {
-        sort_list_reg<4>(keys, vals, n, lane);
+        sort_list_reg<4>(ents, vals, n, lane);
     } else {
-        sort_list_reg<8>(keys, vals, n, lane);
+        sort_list_reg<8>(ents, vals, n, lane);
     }
     if (!__syncthreads_or(is_long))
         return;
     for (int w = 0; w < kSegSortWarps; ++w) {
         const uint2 q = s_long[w];
         if (q.y > q.x)
-            block_sort_list(a.tkeys[0] + q.x, a.vals[0] + q.x, q.y - q.x, s_k);
+            block_sort_list(a.ents + q.x, a.vals[0] + q.x, q.y - q.x, s_k);
     }
 }
 
@@ -1234,8 +1222,12 @@ int bin_seg(const BinArgs &a, cudaStream_t s)
         launch_pdl(k_seg_ranges<true>, a.n_vps, kSegTileThreads, smem, s, a);
     else
         launch_pdl(k_seg_ranges<false>, a.n_vps, kSegTileThreads, 0, s, a);
-    if (a.n_records)
-        launch_pdl(k_seg_place, div_up(a.n_records, kSegThreads * kSegPerThread), kSegThreads, 0, s, a);
+    // one record per thread while that many threads are resident at once
+    // (2048 per SM), two beyond (more cursor atomics in flight per warp)
+    if (a.n_records > 0 && a.n_records <= 152 * 2048)
+        launch_pdl(k_seg_place<1>, div_up(a.n_records, kSegThreads), kSegThreads, 0, s, a);
+    else if (a.n_records > 0)
+        launch_pdl(k_seg_place<2>, div_up(a.n_records, kSegThreads * 2), kSegThreads, 0, s, a);
     if (a.n_tiles)
         launch_pdl(k_seg_sort, div_up(a.n_tiles, kSegSortWarps), kSegSortThreads, 0, s, a);
     return 0;

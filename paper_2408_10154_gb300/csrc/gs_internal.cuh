@@ -313,9 +313,9 @@ struct ProjectArgs {
     float alpha_min;          // the threshold of the tight rectangles
     // segmented tile lists (null: not built here): every visible record adds
     // its rectangle to its keyframe's difference grid (clear before), and
-    // every record writes its seg_list entry (see BinArgs)
+    // every record writes its extent and a visible one its entry (see BinArgs)
     unsigned long long *seg_hdr;
-    uint32_t *seg_diff;
+    uint32_t *seg_diff, *seg_ext;
     uint4 *seg_list;
 };
 void project(const ProjectArgs &a, cudaStream_t s);
@@ -342,17 +342,18 @@ struct BinArgs {
     uint2 *ranges;            // [total tiles]
     uint32_t n_tiles;
     int *flags;
-    uint32_t *tkeys[2];             // [capacity] segmented build: depth bits of the placed entries (tkeys[0])
+    uint64_t *ents;                 // [capacity] segmented build: placed entries, depth bits << 32 | record
     // segmented build (bin_seg): seg_hdr[v] holds keyframe v's duplicate
     // total, and the difference grids (VpDesc::diff_base) follow in the same
     // allocation (seg_zero_bytes), clear before the first build and left
-    // clear by every build.
-    // seg_list: per record {depth bits, first tile, width | height << 16,
-    // tiles per row} (size 0: not visible).  seg_counted: the projection has
-    // already counted and written the entries (ProjectArgs::seg_*);
-    // otherwise bin_seg does it from rec / counts.
+    // clear by every build.  seg_ext: per record width | height << 16 of its
+    // tile rectangle (0: not visible); seg_list: per visible record {depth
+    // bits, first tile, tiles per row}.  seg_counted: the projection has
+    // already counted and written them (ProjectArgs::seg_*); otherwise
+    // bin_seg does it from rec / counts.
     unsigned long long *seg_hdr;
     uint32_t *seg_diff;
+    uint32_t *seg_ext;   // [n_records]
     uint4 *seg_list;     // [n_records]
     int seg_counted;
     uint32_t *seg_cursor;  // [n_tiles] placement cursors

@@ -6,7 +6,7 @@
 // rigid transform of Eq. 8/9 composed with the keyframe's world -> camera
 // transform), one record per visible pair.  56 B read per Gaussian per
 // pass, 48 B record + 32 B auxiliary written per visible (keyframe,
-// Gaussian), 16 B list entry per pair.
+// Gaussian) with its 16 B list entry, a 4 B extent word per pair.
 //
 // Every value that decides an integer outcome follows a fixed FP32
 // operation sequence (see gs_internal.cuh): camera-space mean, quaternion
@@ -69,15 +69,18 @@ __device__ __forceinline__ void tighten(float ca, float cb, float cc, float o, f
 // Segmented lists: a visible record (count > 0) adds +1 at (y0, x0) and
 // (y1, x1) and -1 (mod 2^32) at (y0, x1) and (y1, x0) of its keyframe's
 // (TY + 1) x (TX + 1) difference grid, whose 2-D prefix sum is the tile
-// count; every record writes its entry {depth bits, first tile, width |
-// height << 16, tiles per row} (size 0 when not visible).  The keyframe's
-// duplicate total is counted beside it (one atomic per block and keyframe),
-// so that the list ranges of all keyframes are found in one launch.
+// count.  Every record writes its extent word (width | height << 16; 0 when
+// not visible), and a visible one its entry {depth bits, first tile, tiles
+// per row} (a 16 B entry for all, nine in ten of them empty, was most of the
+// kernel's stores).  The keyframe's duplicate total is counted beside it
+// (one atomic per block and keyframe), so that the list ranges of all
+// keyframes are found in one launch.
 __device__ __forceinline__ void seg_note(const gsl::ProjectArgs &a, const int *geo, uint32_t rec, float z, int count,
                                          int x0, int x1, int y0, int y1)
 {
     const bool vis = count > 0;
     const int TX = geo[0];
+    a.seg_ext[rec] = vis ? (uint32_t)(x1 - x0) | ((uint32_t)(y1 - y0) << 16) : 0u;
     if (vis) {
         const uint32_t w1 = (uint32_t)TX + 1;
         uint32_t *g = a.seg_diff + (uint32_t)geo[4];
@@ -85,11 +88,9 @@ __device__ __forceinline__ void seg_note(const gsl::ProjectArgs &a, const int *g
         atomicAdd(g + (uint32_t)y1 * w1 + (uint32_t)x1, 1u);
         atomicAdd(g + (uint32_t)y0 * w1 + (uint32_t)x1, 0xffffffffu);
         atomicAdd(g + (uint32_t)y1 * w1 + (uint32_t)x0, 0xffffffffu);
+        a.seg_list[rec] = make_uint4(__float_as_uint(z), (uint32_t)geo[3] + (uint32_t)y0 * (uint32_t)TX + (uint32_t)x0,
+                                     (uint32_t)TX, 0u);
     }
-    a.seg_list[rec] = vis ? make_uint4(__float_as_uint(z),
-                                           (uint32_t)geo[3] + (uint32_t)y0 * (uint32_t)TX + (uint32_t)x0,
-                                           (uint32_t)(x1 - x0) | ((uint32_t)(y1 - y0) << 16), (uint32_t)TX)
-                              : make_uint4(0u, 0u, 0u, 0u);
 }
 
 // One (keyframe, Gaussian) pair: camera-space mean, covariance, the
@@ -198,7 +199,7 @@ constexpr int kProjRound = 8;
 // view-independent parts in shared memory and, kProjRound keyframes at a
 // time, queues the pairs in front of the camera (ballot compaction) and
 // projects them 32 at a time on all of its lanes.  A pair behind the near
-// plane writes its empty list entry in the first pass.  Every value is
+// plane writes its empty extent in the first pass.  Every value is
 // computed by the same operations as in a per-thread loop.
 __global__ void __launch_bounds__(256) k_project(const gsl::ProjectArgs a)
 {
@@ -303,7 +304,7 @@ __global__ void __launch_bounds__(256) k_project(const gsl::ProjectArgs a)
                 const float z = fma_rn(M[10], mu.z, fma_rn(M[9], mu.y, fma_rn(M[8], mu.x, M[11])));
                 front = z > a.z_near && qok;
                 if (!front) {
-                    // behind the near plane: no record, an empty list entry
+                    // behind the near plane: no record, an empty extent
                     const uint32_t rec = (uint32_t)sGeo[v][2] + (uint32_t)i;
                     if (a.counts)
                         a.counts[rec] = 0;
