@@ -23,7 +23,7 @@ namespace {
 enum Slot {
     S_VPS, S_GROUPS, S_TILEVP, S_POSE32, S_REC, S_AUX, S_COUNTS, S_PARTIALS, S_K0, S_V0, S_RANGES, S_FLAGS, S_TF, S_LAST, S_CODE, S_TLOSS, S_TTWIST, S_POSE64, S_ADAM, S_PIVOT,
     S_CCAM, S_CENT, S_CENTP, S_LOSS, S_SETVP, S_REV, S_PFIRST, S_PCOUNT, S_RESULT, S_TOUT, S_CONF, S_EST, S_GRAD, S_DUPG,
-    S_PAIRS, S_RSLOT, S_RSLOTN, S_TERR, S_TCOL, S_TW,
+    S_PAIRS, S_RSLOT, S_RSLOTN, S_RLONG, S_TERR, S_TCOL, S_TW,
     S_TMED, S_TNV, S_TVPS, S_EXPO, S_EXPO32, S_TEXPO, S_OPT, S_ONN1, S_ONN2, S_OD2, S_OHDR, S_MAPS, S_OS, S_ORDER, S_ORDC, S_SK, S_SV, S_SN, S_GCELL, S_GCOUNT, S_GSTART, S_GSUMS, S_GPTS, S_GLIST, S_SEGZ, S_SEGCUR, S_SEGEXT, S_SEGLIST, S_PROBE, S_QUEUE, S_COUNT
 };
 
@@ -1138,17 +1138,18 @@ gs_status_t backward_core(gs_ctx *ctx, const Plan &P, const DevPlan &D, Pipe &p,
         ++gsl::g_launches;
     }
     r.c_cam = ccam;
-    uint32_t *slots = nullptr;
+    uint32_t *slots = nullptr, *totals = nullptr, *longs = nullptr;
     if (full) {
-        uint32_t *total = nullptr;
         GS_TRY(wsT(ctx, S_DUPG, 12 * (size_t)p.cap, &r.dup_grads));
         GS_TRY(wsT(ctx, S_RSLOT, (size_t)std::max<uint64_t>(P.n_records, 1), &slots));
-        GS_TRY(wsT(ctx, S_RSLOTN, 1, &total));
-        gsl::rec_slots(p.counts, (uint32_t)P.n_records, total, slots, s);
+        GS_TRY(wsT(ctx, S_RSLOTN, 2, &totals));
+        GS_TRY(wsT(ctx, S_RLONG, gsl::long_records(p.cap), &longs));
+        gsl::rec_slots(p.counts, (uint32_t)P.n_records, totals, slots, longs, s);
         r.rec_slot = slots;
     }
     gsl::backward(r, false, full, s);
     if (full) {
+        gsl::long_sums(totals, longs, p.cap, p.counts, slots, r.dup_grads, s);
         gsl::ParamArgs pa{};
         pa.vps = D.vps;
         pa.n_vps = nv;

@@ -588,8 +588,15 @@ struct ParamArgs {
     const float *logits;
     float *g_means, *g_scales, *g_quats, *g_logits, *g_rgb;  // outputs (any may be null)
 };
-// first slots of the records from their tile counts; total: device scratch word
-void rec_slots(const int32_t *counts, uint32_t n_records, uint32_t *total, uint32_t *first, cudaStream_t s);
+// First slots of the records from their tile counts, and the list of the
+// long records (long_records(cap) of them at most); totals: two device words.
+// long_sums: a long record's slots are summed into its first, ahead of
+// param_grads.
+size_t long_records(uint32_t cap);
+void rec_slots(const int32_t *counts, uint32_t n_records, uint32_t *totals, uint32_t *first, uint32_t *longs,
+               cudaStream_t s);
+void long_sums(const uint32_t *totals, const uint32_t *longs, uint32_t cap, const int32_t *counts, const uint32_t *first,
+               float *dup_grads, cudaStream_t s);
 void param_grads(const ParamArgs &a, cudaStream_t s);
 
 }  // namespace gsl

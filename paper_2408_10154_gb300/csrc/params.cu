@@ -5,11 +5,17 @@
 // through the projection, the rigid transform (Eq. 8/9) and the scale /
 // rotation / opacity parameterisation.  Fixed summation order, no atomics
 // on the gradients.
+#include <algorithm>
+
 #include "gs_internal.cuh"
 
 namespace {
 
 using namespace gsk;
+
+constexpr int kParamThreads = 128, kParamWarps = kParamThreads / 32;
+constexpr uint32_t kShortSlots = 32;  // a record of more slots is summed by a warp of k_long_sums
+constexpr int kStage = 64;            // slots staged at a time there (two per lane)
 
 // First slot of every record's (tile, record) gradients: the record of tile
 // rectangle [x0, x1) x [y0, y1) owns (x1 - x0)(y1 - y0) consecutive slots,
@@ -17,8 +23,9 @@ using namespace gsk;
 // slot from the record alone and nothing has to be sorted by record.  A
 // block's records are consecutive; where the block's slots start follows
 // the order in which the blocks ask (no result depends on it).
-__global__ void __launch_bounds__(kScanThreads) k_rec_slots(const int32_t *counts, uint32_t n, uint32_t *total,
-                                                           uint32_t *first)
+// Records of more than kShortSlots tiles are also listed (totals[1] of them).
+__global__ void __launch_bounds__(kScanThreads) k_rec_slots(const int32_t *counts, uint32_t n, uint32_t *totals,
+                                                           uint32_t *first, uint32_t *longs)
 {
     __shared__ uint32_t s_warp[kScanThreads / 32 + 1];
     __shared__ uint32_t s_base;
@@ -33,56 +40,93 @@ __global__ void __launch_bounds__(kScanThreads) k_rec_slots(const int32_t *count
     uint32_t tot;
     uint32_t ex = block_excl_scan<kScanThreads>(sum, s_warp, tot);
     if (threadIdx.x == 0)
-        s_base = tot ? atomicAdd(total, tot) : 0u;
+        s_base = tot ? atomicAdd(totals, tot) : 0u;
     __syncthreads();
     ex += s_base;
 #pragma unroll
     for (int k = 0; k < K; ++k) {
         if (c[k])
             first[base + k] = ex;
+        if (c[k] > kShortSlots)
+            longs[atomicAdd(totals + 1, 1u)] = base + k;
         ex += c[k];
     }
 }
 
-constexpr int kParamThreads = 128, kParamWarps = kParamThreads / 32;
-// a record of more slots is staged through shared memory
-constexpr uint32_t kShortSlots = 32;
-constexpr int kStage = 64;  // slots staged at a time (two per lane)
-
-// One thread per Gaussian chains its records' gradients.  The sum over a
-// record's tiles before that runs in tile order (an FP32 sum of a splat
+// The sum over a record's tiles runs in tile order (an FP32 sum of a splat
 // over thousands of tiles cancels by 1e4, so another order shows at 1e-4 of
-// the gradient), one lane per component: a short record by loads straight
-// from its slots, several in flight, three records per warp; a long one by
-// a whole warp that stages 64 slots in shared memory while the next 64 are
-// loading.  Most visible records cover a handful of tiles, a few near the
-// camera all of a frame's 3,225: one thread summing its own records, each
-// slot's load waiting for the last, took 646 us on the 300k-Gaussian,
-// 4 x 1200x680 step (ncu), 33 MB or 5 us of HBM traffic, and grouping the
-// slots by record took 14 launches of radix sort.  That step: 1.86 -> 1.21 ms.
+// the gradient), one lane per component.  A long record's is taken by a warp
+// here, which stages 64 slots in shared memory while the next 64 are
+// loading, and left in its first slot: a splat over a whole 1200x680 frame
+// (3,225 slots) is a chain of 3,225 additions per component, and several of
+// them in one block of k_param_grads, camera after camera, were its tail
+// (300k Gaussians, 4 x 1200x680: 95 us in one kernel, 29 + 50 in two).
+__global__ void __launch_bounds__(kParamThreads) k_long_sums(const uint32_t *totals, const uint32_t *longs,
+                                                            const int32_t *counts, const uint32_t *first, float *dup)
+{
+    __shared__ __align__(16) float s_stage[kParamWarps][kStage * 12];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const uint32_t n_long = totals[1];
+    for (uint32_t l = blockIdx.x * kParamWarps + warp; l < n_long; l += gridDim.x * kParamWarps) {
+        const uint32_t r = longs[l], n = (uint32_t)counts[r];
+        float4 *p = reinterpret_cast<float4 *>(dup) + 3 * (size_t)first[r];
+        float4 *st = reinterpret_cast<float4 *>(s_stage[warp]);
+        // batch b: float4s [192 b, 192 b + 192) of the record's 3 n
+        float4 v[6];
+        const uint32_t n4 = 3 * n;
+#pragma unroll
+        for (int u = 0; u < 6; ++u)
+            if (32u * u + lane < n4)
+                v[u] = p[32 * u + lane];
+        float G = 0.0f;
+        for (uint32_t b = 0; b < n; b += kStage) {
+#pragma unroll
+            for (int u = 0; u < 6; ++u)
+                st[32 * u + lane] = v[u];
+            __syncwarp();
+#pragma unroll
+            for (int u = 0; u < 6; ++u) {
+                const uint32_t q = 3 * (b + kStage) + 32 * u + lane;
+                if (q < n4)
+                    v[u] = p[q];
+            }
+            const int cntb = (int)min((uint32_t)kStage, n - b);
+            if (lane < 10) {
+#pragma unroll 8
+                for (int k = 0; k < cntb; ++k)
+                    G += s_stage[warp][12 * k + lane];
+            }
+            __syncwarp();
+        }
+        if (lane < 10)
+            reinterpret_cast<float *>(p)[lane] = G;
+    }
+}
+
+// One thread per Gaussian chains its records' gradients; a short record's
+// sum over its tiles before that is taken by one lane per component, three
+// records per warp, straight from its slots with several loads in flight.
+// Most visible records cover a handful of tiles.  One thread summing its own
+// records, each slot's load waiting for the last, took 646 us on the
+// 300k-Gaussian, 4 x 1200x680 step (ncu), 33 MB or 5 us of HBM traffic, and
+// grouping the slots by record took 14 launches of radix sort: the step's
+// 1.86 ms became 1.21 with the slots alone.
 __global__ void __launch_bounds__(kParamThreads) k_param_grads(const gsl::ParamArgs a)
 {
     __shared__ float s_G[kParamThreads][10];
-    __shared__ __align__(16) float s_stage[kParamWarps][kStage * 12];
-    __shared__ uint8_t s_long[kParamThreads];
-    __shared__ int s_n_long;
-    static_assert(kParamThreads <= 256, "s_long holds thread indices in a byte");
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int i0 = blockIdx.x * kParamThreads, i = i0 + threadIdx.x;
+    const int i = blockIdx.x * kParamThreads + threadIdx.x;
     const int comp = lane % 10, sub = lane / 10;  // lanes 30 and 31 sum nothing
     // object-frame accumulators over cameras
     float gmu[3] = {0, 0, 0}, GS[3][3] = {{0, 0, 0}, {0, 0, 0}, {0, 0, 0}}, dop = 0.0f, drgb[3] = {0, 0, 0};
     for (int c = 0; c < a.n_vps; ++c) {
         const VpDesc &d = a.vps[c];
         const uint32_t r = d.rec_base + (uint32_t)i;
-        const uint32_t cnt = i < a.n ? (uint32_t)a.counts[r] : 0u;
+        uint32_t cnt = i < a.n ? (uint32_t)a.counts[r] : 0u;
         const uint32_t off = cnt ? a.rec_slot[r] : 0u;
-        if (threadIdx.x == 0)
-            s_n_long = 0;
-        __syncthreads();
         if (cnt > kShortSlots)
-            s_long[atomicAdd(&s_n_long, 1)] = (uint8_t)threadIdx.x;
-        unsigned m = __ballot_sync(0xffffffffu, cnt > 0 && cnt <= kShortSlots);
+            cnt = 1;  // summed by k_long_sums
+        unsigned m = __ballot_sync(0xffffffffu, cnt > 0);
         while (m) {
             int src = -1;
 #pragma unroll
@@ -102,53 +146,14 @@ __global__ void __launch_bounds__(kParamThreads) k_param_grads(const gsl::ParamA
                 s_G[32 * warp + src][comp] = G;
             }
         }
-        __syncthreads();
-        // the block's long records, dealt to its warps
-        const int n_long = s_n_long;
-        for (int l = warp; l < n_long; l += kParamWarps) {
-            const int src = s_long[l];
-            const uint32_t rl = d.rec_base + (uint32_t)(i0 + src);
-            const uint32_t n = (uint32_t)a.counts[rl];
-            const float4 *p = reinterpret_cast<const float4 *>(a.dup_grads) + 3 * (size_t)a.rec_slot[rl];
-            float4 *st = reinterpret_cast<float4 *>(s_stage[warp]);
-            // batch b: float4s [192 b, 192 b + 192) of the record's 3 n
-            float4 v[6];
-            const uint32_t n4 = 3 * n;
-#pragma unroll
-            for (int u = 0; u < 6; ++u)
-                if (32u * u + lane < n4)
-                    v[u] = p[32 * u + lane];
-            float G = 0.0f;
-            for (uint32_t b = 0; b < n; b += kStage) {
-#pragma unroll
-                for (int u = 0; u < 6; ++u)
-                    st[32 * u + lane] = v[u];
-                __syncwarp();
-#pragma unroll
-                for (int u = 0; u < 6; ++u) {
-                    const uint32_t q = 3 * (b + kStage) + 32 * u + lane;
-                    if (q < n4)
-                        v[u] = p[q];
-                }
-                const int cntb = (int)min((uint32_t)kStage, n - b);
-                if (lane < 10) {
-#pragma unroll 8
-                    for (int k = 0; k < cntb; ++k)
-                        G += s_stage[warp][12 * k + lane];
-                }
-                __syncwarp();
-            }
-            if (lane < 10)
-                s_G[src][lane] = G;
-        }
-        if (n_long > 0)
-            __syncthreads();
-        if (cnt == 0)
-            continue;
+        __syncwarp();
         float G[10];
 #pragma unroll
         for (int k = 0; k < 10; ++k)
             G[k] = s_G[threadIdx.x][k];
+        __syncwarp();  // (the next camera's sums take their place)
+        if (cnt == 0)
+            continue;
         const float4 q1 = a.rec[3 * (size_t)r + 1];
         const float4 x0 = a.aux[2 * (size_t)r], x1 = a.aux[2 * (size_t)r + 1];
         const float fx = d.fx, fy = d.fy;
@@ -256,12 +261,23 @@ inline uint32_t div_up(size_t a, size_t b) { return (uint32_t)((a + b - 1) / b);
 
 namespace gsl {
 
-void rec_slots(const int32_t *counts, uint32_t n_records, uint32_t *total, uint32_t *first, cudaStream_t s)
+size_t long_records(uint32_t cap) { return cap / (kShortSlots + 1) + 1; }
+
+void rec_slots(const int32_t *counts, uint32_t n_records, uint32_t *totals, uint32_t *first, uint32_t *longs,
+               cudaStream_t s)
 {
-    cudaMemsetAsync(total, 0, sizeof(uint32_t), s);
+    cudaMemsetAsync(totals, 0, 2 * sizeof(uint32_t), s);
     if (n_records == 0)
         return;
-    k_rec_slots<<<div_up(n_records, kScanTile), kScanThreads, 0, s>>>(counts, n_records, total, first);
+    k_rec_slots<<<div_up(n_records, kScanTile), kScanThreads, 0, s>>>(counts, n_records, totals, first, longs);
+    ++g_launches;
+}
+
+void long_sums(const uint32_t *totals, const uint32_t *longs, uint32_t cap, const int32_t *counts, const uint32_t *first,
+               float *dup_grads, cudaStream_t s)
+{
+    const uint32_t blocks = std::min<uint32_t>(div_up(long_records(cap), kParamWarps), 152 * 8);
+    k_long_sums<<<blocks, kParamThreads, 0, s>>>(totals, longs, counts, first, dup_grads);
     ++g_launches;
 }
 
