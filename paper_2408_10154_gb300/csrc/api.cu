@@ -466,10 +466,10 @@ gs_status_t alloc_seg(gs_ctx *ctx, const Plan &P, Pipe &p)
     const size_t T = P.n_tiles ? P.n_tiles : 1, R = P.n_records ? P.n_records : 1;
     const size_t zero = gsl::seg_zero_bytes((int)P.vps.size(), P.n_diff);
     uint8_t *z = nullptr;
-    const void *before = ctx->bufs[S_SEGZ].p;
+    const size_t before = ctx->bufs[S_SEGZ].bytes;
     GS_TRY(wsT(ctx, S_SEGZ, zero, &z));
-    if (z != before)
-        ctx->seg_dirty = true;
+    if (ctx->bufs[S_SEGZ].bytes != before)
+        ctx->seg_dirty = true;  // a new buffer (which may lie where the old one did)
     p.seg_hdr = (unsigned long long *)z;
     p.seg_diff = (uint32_t *)(p.seg_hdr + P.vps.size());
     GS_TRY(wsT(ctx, S_SEGEXT, R, &p.seg_ext));

@@ -1218,10 +1218,16 @@ int bin_seg(const BinArgs &a, cudaStream_t s)
         ++g_launches;
     }
     const size_t smem = sizeof(unsigned long long) * a.seg_max_rows + sizeof(uint32_t) * a.seg_max_cells;
-    if (smem <= 40 * 1024)
-        launch_pdl(k_seg_ranges<true>, a.n_vps, kSegTileThreads, smem, s, a);
-    else
-        launch_pdl(k_seg_ranges<false>, a.n_vps, kSegTileThreads, 0, s, a);
+    const auto ranges = smem <= 40 * 1024 ? k_seg_ranges<true> : k_seg_ranges<false>;
+    const size_t dyn = smem <= 40 * 1024 ? smem : 0;
+    if (a.n_records) {
+        launch_pdl(ranges, a.n_vps, kSegTileThreads, dyn, s, a);
+    } else {
+        // without records nothing may have run since the keyframe table was
+        // written, which the kernel reads ahead of its wait
+        ranges<<<a.n_vps, kSegTileThreads, dyn, s>>>(a);
+        ++g_launches;
+    }
     // one record per thread while that many threads are resident at once
     // (2048 per SM), two beyond (more cursor atomics in flight per warp)
     if (a.n_records > 0 && a.n_records <= 152 * 2048)
