@@ -1349,16 +1349,18 @@ gs_status_t gs_render_saved(gs_ctx_t *ctx, const gs_gaussians_t *g, const float 
     p.ndups = (uint32_t *)p.flags + 1;
     send_plan(P, sv->D, 0, p.flags, s);
     // With the duplicates an earlier pass of this shape had as a guide, the
-    // whole pass is enqueued at once, and redone if its lists were too short;
-    // a shape not seen before has its duplicates counted first.
+    // whole pass is enqueued at once, within the scratch at hand, and redone
+    // if its lists were too short; a shape not seen before has its duplicates
+    // counted first.
     const auto key = std::make_tuple((uint64_t)P.n_tiles, P.vps.size(), (uint64_t)P.n_records);
     const auto seen = ctx->saved_seen.find(key);
     uint32_t nd = 0;
     int flags = 0;
-    bool count_first = seen == ctx->saved_seen.end();
-    uint64_t want = count_first ? 0 : (uint64_t)seen->second + seen->second / 8 + 1024;
+    bool count_first = seen == ctx->saved_seen.end() || !lists_at_hand(ctx, p);
+    if (!count_first)
+        p.cap = (uint32_t)std::min<uint64_t>(p.cap, std::max<uint64_t>((uint64_t)seen->second + seen->second / 8, 1024));
     for (;;) {
-        if (count_first || want > 0xfff00000ull) {
+        if (count_first) {
             if (cudaMemsetAsync(p.flags, 0, sizeof(int), s) != cudaSuccess)
                 return cleanup(fail(ctx, GS_ERR_CUDA, "gs_render_saved: memset"));
             st = begin_lists(ctx, s);
@@ -1372,20 +1374,24 @@ gs_status_t gs_render_saved(gs_ctx_t *ctx, const gs_gaussians_t *g, const float 
                 return cleanup(st);
             if (nd == 0xffffffffu)
                 return cleanup(fail(ctx, GS_ERR_CAPACITY, "more than 2^32 tile duplicates"));
-            want = nd;
-        } else {
+            st = alloc_sort(ctx, nd, p);
+            if (st != GS_OK)
+                return cleanup(st);
+        }
+        if (cudaMallocAsync(&sv->blk[1], sizeof(uint32_t) * (size_t)p.cap, s) != cudaSuccess) {
+            cudaGetLastError();
+            sv->blk[1] = nullptr;
+            if (!count_first) {
+                count_first = true;  // the count may ask for less
+                continue;
+            }
+            return cleanup(fail(ctx, GS_ERR_OOM, "gs_render_saved: cudaMallocAsync failed"));
+        }
+        if (!count_first) {
             st = begin_lists(ctx, s);
             if (st != GS_OK)
                 return cleanup(st);
             gsl::project(project_args(P, sv->D, p, sv->pose32, opt), s);
-        }
-        st = alloc_sort(ctx, want, p);
-        if (st != GS_OK)
-            return cleanup(st);
-        if (cudaMallocAsync(&sv->blk[1], sizeof(uint32_t) * (size_t)p.cap, s) != cudaSuccess) {
-            cudaGetLastError();
-            sv->blk[1] = nullptr;
-            return cleanup(fail(ctx, GS_ERR_OOM, "gs_render_saved: cudaMallocAsync failed"));
         }
         sv->vals = (uint32_t *)sv->blk[1];
         sv->cap = p.cap;

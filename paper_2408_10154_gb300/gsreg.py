@@ -187,7 +187,7 @@ def default_options(**kw) -> gs_options_t:
 def _camera_words(cams):
     """cam18 rows as gs_camera_t words: the float32 row with the image size
     (columns 4 and 5) as int32."""
-    c = np.array(cams, np.float32).reshape(-1, 18)
+    c = np.array(cams, np.float32, order="C").reshape(-1, 18)
     c.view(np.int32)[:, 4:6] = c[:, 4:6].astype(np.int32)
     return c
 

@@ -86,3 +86,16 @@ def test_missing_library_fails_loudly(monkeypatch, tmp_path):
         gsreg.load()
     with pytest.raises(RuntimeError, match="not built"):
         gsreg.Context(0)
+
+
+def test_cameras_of_any_memory_order(lib):
+    # camera rows in row-major, column-major, strided and reversed memory
+    from paper_2408_10154_gb300 import gsreg, synth
+    rows = np.stack([synth.camera(30.0 + k, 31.0, 32.0, 8.0, 64 + k, 16, np.eye(3, 4)) for k in range(3)])
+    want = bytes(gsreg.cameras(rows)[0])
+    wide = np.zeros((3, 36), np.float32)
+    wide[:, ::2] = rows
+    for same in (np.asfortranarray(rows), rows.T.copy().T, wide[:, ::2], rows[::-1][::-1], rows.astype(np.float64),
+                 rows.tolist()):
+        assert bytes(gsreg.cameras(same)[0]) == want
+    assert bytes(gsreg.camera(np.asfortranarray(rows)[1])) == want[72:144]

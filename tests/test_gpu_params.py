@@ -165,3 +165,34 @@ def test_parameter_adjoint_ignores_earlier_calls(env):
         for k in want:
             assert torch.equal(got[k], want[k]), k
     fresh.close()
+
+
+def test_saved_forward_repeats_at_the_smallest_budget(env):
+    # a repeated forward (whose lists are sized by what the shape had before)
+    # needs no more scratch than the first
+    gs, _, _ = env
+    c = synth.small_case(2500, 120, 88, 100.0, n_views=2, seed=79, ls_mean=-3.0)
+    g = gs.Gaussians.from_numpy(c["gaussians"])
+    P = dev(np.tile(np.eye(3, 4).reshape(1, 12), (2, 1)))
+    want, sv = gs.gs_render_saved(gs.Context(0), g, P, c["cams"])
+    sv.close()
+
+    def passes(budget, times):
+        ctx = gs.Context(0, budget)
+        try:
+            for _ in range(times):
+                out, saved = gs.gs_render_saved(ctx, g, P, c["cams"])
+                saved.close()
+                assert all(torch.equal(out[k], want[k]) for k in want)
+            return True
+        except gs.GsError:
+            return False
+        finally:
+            ctx.close()
+
+    lo, hi = 1 << 12, 1 << 26
+    assert not passes(lo, 1) and passes(hi, 1)
+    while hi - lo > 256:
+        mid = (lo + hi) // 2
+        lo, hi = (lo, mid) if passes(mid, 1) else (mid, hi)
+    assert passes(hi, 3)
