@@ -449,7 +449,7 @@ struct Pipe {
     // segmented build
     unsigned long long *seg_hdr = nullptr;
     uint32_t *seg_diff = nullptr, *seg_ext = nullptr, *seg_cursor = nullptr;
-    uint4 *seg_list = nullptr;
+    gsl::SegEntry *seg_list = nullptr;
 };
 
 // Binning routes.  The context-based entry points and gs_bin use the
@@ -2658,12 +2658,13 @@ double srv_now(const gs_server *srv)
 }
 
 // Scratch of a request in a plan, from its measured tile duplicates nd:
-// per record 100 B (record 48, auxiliary 32, count 4, list entry 16); per
-// list entry of capacity (headroom x nd; a plan's 64 Ki spare entries come
-// out of the arena's slack) 12.5 B (entry 8, sorted value 4); per pixel 9 B
-// (final transmittance, last contributor, loss sign code), 12 B more for tracking masks; per tile
-// 92 B (range, keyframe, loss, twist, counters, cursors, order); per
-// keyframe problem its FP64 optimiser state.
+// per record 100 B (record 48, auxiliary 32, count 4, extent 4, list entry
+// 12); per list entry of capacity (headroom x nd; a plan's 64 Ki spare
+// entries come out of the arena's slack) 12.5 B (entry 8, sorted value 4, and
+// some slack); per pixel 9 B (final transmittance, last contributor, loss
+// sign code), 12 B more for tracking masks; per tile 92 B (range, keyframe,
+// loss, twist, counters, cursors, order); per keyframe problem its FP64
+// optimiser state.
 size_t footprint_bytes(const ServerReq &r, int64_t nd, double headroom)
 {
     double rec = 0, px = 0, tiles = 0;

@@ -586,8 +586,8 @@ __global__ void __launch_bounds__(kSegThreads) k_seg_collect(const gsl::BinArgs 
         atomicAdd(g + q.y0 * w1 + q.x1, 0xffffffffu);
         atomicAdd(g + q.y1 * w1 + q.x0, 0xffffffffu);
         ext = (q.x1 - q.x0) | ((q.y1 - q.y0) << 16);
-        a.seg_list[r] = make_uint4(__float_as_uint(a.rec[3 * (size_t)r + 1].z),
-                                   d.tile_base + q.y0 * (uint32_t)d.TX + q.x0, (uint32_t)d.TX, 0u);
+        a.seg_list[r] = gsl::SegEntry{__float_as_uint(a.rec[3 * (size_t)r + 1].z),
+                                      d.tile_base + q.y0 * (uint32_t)d.TX + q.x0, (uint32_t)d.TX};
         atomicAdd(a.seg_hdr + vp, (unsigned long long)c);
     }
     a.seg_ext[r] = ext;
@@ -631,9 +631,10 @@ __device__ __forceinline__ unsigned long long block_incl_scan(unsigned long long
 // Writes the ranges ((0, 0) when empty; clipped to the capacity), the
 // placement cursors, and (CTA 0) the duplicate total and the capacity flag,
 // and leaves the grid clear for the next build (the totals, which every CTA
-// reads, are cleared by the placement).  Latency-bound: one launch of a few microseconds in place of two (counts,
-// then ranges: 3.3 + 4.0 us on a 160x120 view, 7.4 + 7.4 us on 1200x680, by
-// ncu), columns one thread each, rows one warp each.
+// reads, are cleared by the placement).  Latency-bound: one launch of a few
+// microseconds in place of two (counts, then ranges: 3.3 + 4.0 us on a
+// 160x120 view, 7.4 + 7.4 us on 1200x680, by ncu), columns one thread each,
+// rows one warp each.
 //
 // SMEM: the TY x TX cells are summed in shared memory (dynamic: a.seg_max_cells
 // + 1 words, then a.seg_max_rows 64-bit row offsets); otherwise in place in
@@ -820,10 +821,10 @@ __global__ void __launch_bounds__(kSegThreads) k_seg_place(const gsl::BinArgs a)
     for (int q = 0; q < PER; ++q) {
         w[q] = max(ext[q] & 0xffffu, 1u);
         cnt[q] = w[q] * (ext[q] >> 16);
-        const uint4 e = cnt[q] ? a.seg_list[rr[q]] : make_uint4(0u, 0u, 0u, 0u);
-        zb[q] = e.x;
-        t0[q] = e.y;
-        tx[q] = e.z;
+        const gsl::SegEntry e = cnt[q] ? a.seg_list[rr[q]] : gsl::SegEntry{0u, 0u, 0u};
+        zb[q] = e.depth;
+        t0[q] = e.tile;
+        tx[q] = e.tx;
     }
     uint64_t *ents = a.ents;
     uint32_t pos[PER][kSegSmall];

@@ -289,6 +289,11 @@ inline void launch_pdl(void (*k)(P...), dim3 grid, dim3 block, size_t smem, cuda
     ++g_launches;
 }
 
+// a visible record's part of the segmented lists: depth bits, first tile, tiles per row
+struct SegEntry {
+    uint32_t depth, tile, tx;
+};
+
 struct ProjectArgs {
     const gsk::VpDesc *vps;
     const gsk::GroupDesc *groups;
@@ -316,7 +321,7 @@ struct ProjectArgs {
     // every record writes its extent and a visible one its entry (see BinArgs)
     unsigned long long *seg_hdr;
     uint32_t *seg_diff, *seg_ext;
-    uint4 *seg_list;
+    SegEntry *seg_list;
 };
 void project(const ProjectArgs &a, cudaStream_t s);
 
@@ -347,14 +352,14 @@ struct BinArgs {
     // total, and the difference grids (VpDesc::diff_base) follow in the same
     // allocation (seg_zero_bytes), clear before the first build and left
     // clear by every build.  seg_ext: per record width | height << 16 of its
-    // tile rectangle (0: not visible); seg_list: per visible record {depth
-    // bits, first tile, tiles per row}.  seg_counted: the projection has
+    // tile rectangle (0: not visible); seg_list: an entry per visible record.
+    // seg_counted: the projection has
     // already counted and written them (ProjectArgs::seg_*); otherwise
     // bin_seg does it from rec / counts.
     unsigned long long *seg_hdr;
     uint32_t *seg_diff;
     uint32_t *seg_ext;   // [n_records]
-    uint4 *seg_list;     // [n_records]
+    SegEntry *seg_list;  // [n_records]
     int seg_counted;
     uint32_t *seg_cursor;  // [n_tiles] placement cursors
     uint32_t seg_max_cells;  // largest TX * TY over the keyframes

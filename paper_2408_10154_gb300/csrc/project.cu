@@ -6,7 +6,7 @@
 // rigid transform of Eq. 8/9 composed with the keyframe's world -> camera
 // transform), one record per visible pair.  56 B read per Gaussian per
 // pass, 48 B record + 32 B auxiliary written per visible (keyframe,
-// Gaussian) with its 16 B list entry, a 4 B extent word per pair.
+// Gaussian) with its 12 B list entry, a 4 B extent word per pair.
 //
 // Every value that decides an integer outcome follows a fixed FP32
 // operation sequence (see gs_internal.cuh): camera-space mean, quaternion
@@ -71,7 +71,7 @@ __device__ __forceinline__ void tighten(float ca, float cb, float cc, float o, f
 // (TY + 1) x (TX + 1) difference grid, whose 2-D prefix sum is the tile
 // count.  Every record writes its extent word (width | height << 16; 0 when
 // not visible), and a visible one its entry {depth bits, first tile, tiles
-// per row} (a 16 B entry for all, nine in ten of them empty, was most of the
+// per row} (an entry for all, nine in ten of them empty, was most of the
 // kernel's stores).  The keyframe's duplicate total is counted beside it
 // (one atomic per block and keyframe), so that the list ranges of all
 // keyframes are found in one launch.
@@ -88,8 +88,8 @@ __device__ __forceinline__ void seg_note(const gsl::ProjectArgs &a, const int *g
         atomicAdd(g + (uint32_t)y1 * w1 + (uint32_t)x1, 1u);
         atomicAdd(g + (uint32_t)y0 * w1 + (uint32_t)x1, 0xffffffffu);
         atomicAdd(g + (uint32_t)y1 * w1 + (uint32_t)x0, 0xffffffffu);
-        a.seg_list[rec] = make_uint4(__float_as_uint(z), (uint32_t)geo[3] + (uint32_t)y0 * (uint32_t)TX + (uint32_t)x0,
-                                     (uint32_t)TX, 0u);
+        a.seg_list[rec] = gsl::SegEntry{__float_as_uint(z),
+                                        (uint32_t)geo[3] + (uint32_t)y0 * (uint32_t)TX + (uint32_t)x0, (uint32_t)TX};
     }
 }
 

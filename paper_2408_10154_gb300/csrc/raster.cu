@@ -1230,8 +1230,9 @@ __global__ void __launch_bounds__(kBwd2Threads, kBwd2MinBlocks) k_backward2_q(co
 // A list staged whole that needs no general walk is walked by the forward's
 // selection and its stashed alphas (kStash): of the adjoint's pair that
 // leaves out the exponential, the alpha test and the last-contributor test,
-// about 25 of 140 instructions (the kernel issues in 76 % of its slots).
-// STASH_NOW
+// about 25 of 140 instructions, and the second cull (the kernel issues in
+// 76 % of its slots): room edge (100 iterations of 16 keyframes of 1200x680)
+// 137.3 -> 128.8 ms.
 __device__ __forceinline__ void fused_adjoint(const gsl::RasterArgs &a, uint32_t t, const VpDesc &d, uint2 rg,
                                               float4 *s0, float4 *s1, float4 *s2, const uint32_t *s_v,
                                               uint8_t *s_selw, float xa, float ya, PixAdj2 &P2, int maxl,

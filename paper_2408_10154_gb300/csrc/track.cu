@@ -50,10 +50,11 @@ __device__ __forceinline__ uint2 cluster_load2(const uint32_t *p, uint32_t rank)
 // is sent back.  KEEP: a slice of at most kMedKeep pixels per thread is read
 // once and kept in registers over the three passes; a larger one is read by
 // each.  Bound by latency (one frame is 1.2 MB; reading it three times took
-// 7 us more of a tracking iteration).  One CTA per keyframe took 346 us on a 640x480 frame, by ncu:
-// each pass one dependent load and one match_any per 1024 pixels; the
-// tracking iteration spent two thirds of its time there (40 iterations of a
-// 640x480 frame on 150k Gaussians: 18.97 -> 7.06 ms with this kernel).
+// 7 us more of a tracking iteration).  One CTA per keyframe took 346 us on a
+// 640x480 frame, by ncu: each pass one dependent load and one match_any per
+// 1024 pixels; the tracking iteration spent two thirds of its time there (40
+// iterations of a 640x480 frame on 150k Gaussians: 18.97 -> 7.06 ms with
+// this kernel).
 template <bool KEEP>
 __global__ void __cluster_dims__(kMedCluster, 1, 1) __launch_bounds__(kMedThreads) k_track_median(const gsl::TrackArgs a)
 {
