@@ -126,8 +126,8 @@ typedef struct {
     /* CTA schedule of the compositing kernels in gs_register* and the
      * server (results are identical either way): 0 = picked by the
      * autotuner (the first registration of a plan shape on a context times
-     * the four below on trial iterations from the initial poses, keeps the
-     * fastest per shape and starts over); one CTA per tile in 1 = natural
+     * the four below on its first eight iterations and keeps the fastest per
+     * shape); one CTA per tile in 1 = natural
      * tile order, 2 = longest tile lists first; persistent CTAs (as many as
      * fit on the GPU) pulling tiles of every keyframe problem from one work
      * queue in 3 = natural order, 4 = longest lists first */

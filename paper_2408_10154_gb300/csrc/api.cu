@@ -2199,11 +2199,16 @@ gs_status_t run_registration(gs_ctx *ctx, Plan &P, int n_problems, const gs_opti
         // Autotuner: the CTA schedule of the compositing kernels for this
         // plan shape -- tile order (natural, or longest lists first) x launch
         // (one CTA per tile, or persistent CTAs pulling tiles from one work
-        // queue over every keyframe problem) -- timed on trial iterations
-        // 1 2 3 4 4 3 2 1 from the initial poses, then the poses start over.
-        // Every schedule gives the same results.
+        // queue over every keyframe problem) -- timed on the first eight
+        // iterations, 1 2 3 4 4 3 2 1.  Every schedule gives the same results,
+        // so they count (a first call on the room edge used to run 108
+        // iterations for 100, 152 -> 140 ms), unless a profile wants every
+        // iteration's phases: the poses start over then.
         GS_TRY(begin_lists(ctx, s));
-        int sched = opt->tile_schedule;
+        GS_CUDA(cudaMemsetAsync(p.flags, 0, sizeof(int), s));
+        GS_CUDA(cudaMemsetAsync(pairs, 0, sizeof(unsigned long long) * 2 * ntl, s));
+        int sched = opt->tile_schedule, iters_left = iters;
+        cudaGraphExec_t exec = nullptr;
         if (sched == 0) {
             const auto it = ctx->schedule.find(key);
             if (it != ctx->schedule.end()) {
@@ -2211,14 +2216,16 @@ gs_status_t run_registration(gs_ctx *ctx, Plan &P, int n_problems, const gs_opti
             } else if (iters >= 8 && P.n_tiles >= 2048 && !ao) {
                 marking = false;
                 cudaGraphExec_t g[4] = {};
-                const long long t0 = gsl::g_launches;
+                long long kernels[4] = {};
                 gs_status_t st = GS_OK;
                 for (int k = 0; k < 4 && st == GS_OK; ++k) {
                     ordered = (k & 1) != 0;
                     persistent = (k & 2) != 0;
+                    const long long t0 = gsl::g_launches;
                     st = capture(&g[k], nullptr);
+                    kernels[k] = gsl::g_launches - t0;
+                    trial_kernels += kernels[k];  // each graph runs twice: count them once more
                 }
-                trial_kernels = gsl::g_launches - t0;  // each graph runs twice: count them once more
                 cudaEvent_t e[9] = {};
                 for (cudaEvent_t &x : e)
                     if (st == GS_OK && cudaEventCreate(&x) != cudaSuccess)
@@ -2239,18 +2246,26 @@ gs_status_t run_registration(gs_ctx *ctx, Plan &P, int n_problems, const gs_opti
                 for (cudaEvent_t x : e)
                     if (x)
                         cudaEventDestroy(x);
-                for (cudaGraphExec_t x : g)
-                    if (x)
-                        cudaGraphExecDestroy(x);
-                GS_TRY(st);
                 int best = 0;
                 for (int k = 1; k < 4; ++k)
                     if (ms[k] < ms[best])
                         best = k;
+                for (int k = 0; k < 4; ++k)
+                    if (g[k] && (st != GS_OK || prof || k != best))
+                        cudaGraphExecDestroy(g[k]);
+                GS_TRY(st);
                 sched = best + 1;
                 ctx->schedule[key] = sched;
                 ++ctx->tuned;
-                gsl::pose_init(pa, s);  // back to the initial poses
+                if (prof) {
+                    gsl::pose_init(pa, s);  // back to the initial poses
+                    GS_CUDA(cudaMemsetAsync(p.flags, 0, sizeof(int), s));
+                    GS_CUDA(cudaMemsetAsync(pairs, 0, sizeof(unsigned long long) * 2 * ntl, s));
+                } else {
+                    exec = g[best];
+                    graph_kernels = kernels[best];
+                    iters_left -= 8;
+                }
                 marking = prof;
             } else {
                 sched = 1;
@@ -2259,12 +2274,15 @@ gs_status_t run_registration(gs_ctx *ctx, Plan &P, int n_problems, const gs_opti
         ordered = sched == 2 || sched == 4;
         persistent = sched >= 3;
         const int sched_run = sched;
-        GS_CUDA(cudaMemsetAsync(p.flags, 0, sizeof(int), s));
-        GS_CUDA(cudaMemsetAsync(pairs, 0, sizeof(unsigned long long) * 2 * ntl, s));
-        if (iters > 0) {
+        cudaError_t le = cudaSuccess;
+        if (exec) {
+            // the trial's graph of the schedule goes on
+            for (int it = 0; it < iters_left && le == cudaSuccess; ++it)
+                le = cudaGraphLaunch(exec, s);
+            cudaGraphExecDestroy(exec);
+        } else if (iters > 0) {
             const long long c0 = gsl::g_launches;
             cudaGraph_t graph = nullptr;
-            cudaGraphExec_t exec = nullptr;
             GS_TRY(capture(&exec, &graph));
             captured = gsl::g_launches - c0;
             if (mark_err != cudaSuccess) {
@@ -2291,7 +2309,6 @@ gs_status_t run_registration(gs_ctx *ctx, Plan &P, int n_problems, const gs_opti
                             evnode[k] = nd_;
                 }
             }
-            cudaError_t le = cudaSuccess;
             for (int it = 0; it < iters && le == cudaSuccess; ++it) {
                 if (prof)
                     for (int k = 0; k <= kPhases && le == cudaSuccess; ++k)
@@ -2303,9 +2320,9 @@ gs_status_t run_registration(gs_ctx *ctx, Plan &P, int n_problems, const gs_opti
             }
             cudaGraphExecDestroy(exec);
             cudaGraphDestroy(graph);
-            if (le != cudaSuccess)
-                return fail(ctx, GS_ERR_CUDA, std::string("graph launch: ") + cudaGetErrorString(le));
         }
+        if (le != cudaSuccess)
+            return fail(ctx, GS_ERR_CUDA, std::string("graph launch: ") + cudaGetErrorString(le));
         // residual eps at the final poses, then Eq. 7
         r.tile_pairs = nullptr;
         r.tile_order = nullptr;
@@ -2394,7 +2411,7 @@ gs_status_t run_registration(gs_ctx *ctx, Plan &P, int n_problems, const gs_opti
             at += q.n[k];
         }
         gs_stats_t &st = ctx->stats;
-        st.kernel_launches = (gsl::g_launches - l0) - captured + graph_kernels * iters + trial_kernels;
+        st.kernel_launches = (gsl::g_launches - l0) - captured + graph_kernels * iters_left + trial_kernels;
         st.n_dups = nd;
         st.n_pixels = P.n_pix;
         st.iterations = iters;

@@ -771,6 +771,31 @@ def test_transform_is_fp64_rounded_once(gs, ctx, kind, n):
     np.testing.assert_array_equal(out.quats4.cpu().numpy(), wq)
 
 
+@pytest.mark.parametrize("iters", [7, 8, 9, 20])
+def test_first_call_of_a_shape_equals_the_next(gs, iters):
+    # the first call of a shape times the schedules on its first eight
+    # iterations: the same estimate, residuals and statistics as a call whose
+    # schedule is given, and as a profiled one
+    import ctypes
+    c = synth.small_case(400, 1024, 512, 900.0, n_views=1, seed=81)
+    g = gs.Gaussians.from_numpy(c["gaussians"])
+    rng = np.random.default_rng(81)
+    views = [(c["cams"][0], dev(rng.random((3, 512, 1024)).astype(np.float32)),
+              dev(rng.uniform(1.0, 4.0, (512, 1024)).astype(np.float32)))]
+    out = []
+    for kw in (dict(tile_schedule=1), dict(), dict(profile=1)):
+        cx = gs.Context(0)
+        for _ in range(2):
+            T, conf, eps, est = gs.gs_register(cx, g, g, [], views, iters, gs.default_options(**kw))
+            st = gs.gsreg.gs_stats_t()
+            cx.check(cx._lib.gs_ctx_stats(cx.handle, ctypes.byref(st)))
+            out.append((T, conf, eps, est, st.pairs, st.iterations))
+        cx.close()
+    for o in out[1:]:
+        for x, y in zip(o, out[0]):
+            np.testing.assert_array_equal(x, y)
+
+
 def test_tile_schedules_give_identical_registrations(gs, ctx):
     # two full-size room keyframes (3225 tiles each): natural tile order,
     # longest lists first, either of them through the persistent kernels'
