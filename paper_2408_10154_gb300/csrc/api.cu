@@ -533,6 +533,8 @@ gsl::ProjectArgs project_args(const Plan &P, const DevPlan &D, const Pipe &p, co
     a.groups = D.groups;
     a.n_groups = (int)P.groups.size();
     a.n_blocks = P.proj_blocks;
+    for (const GroupDesc &g : P.groups)
+        a.max_vps = std::max(a.max_vps, g.vp_count);
     a.pose32 = pose32;
     a.z_near = o->z_near;
     a.dilation = o->dilation;

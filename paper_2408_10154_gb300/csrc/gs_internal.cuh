@@ -299,6 +299,7 @@ struct ProjectArgs {
     const gsk::GroupDesc *groups;
     int n_groups;
     uint32_t n_blocks;
+    int max_vps;              // most keyframes of a group
     const float *pose32;      // [vp][12]
     float z_near, dilation;
     int smooth;

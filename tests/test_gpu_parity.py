@@ -771,6 +771,25 @@ def test_transform_is_fp64_rounded_once(gs, ctx, kind, n):
     np.testing.assert_array_equal(out.quats4.cpu().numpy(), wq)
 
 
+@pytest.mark.parametrize("n,views", [(1, 2), (255, 3), (2000, 9), (5000, 64), (5000, 67), (40000, 3)])
+def test_projection_of_many_keyframes_equals_one_each(gs, ctx, n, views):
+    # keyframes of one submap, whole in a block or spread over several:
+    # the records of the keyframes projected one by one, bit for bit
+    c = synth.small_case(n, 64, 48, 56.0, n_views=views, seed=n + views)
+    g = gs.Gaussians.from_numpy(c["gaussians"])
+    rng = np.random.default_rng(n)
+    P = dev(np.stack([synth.random_rigid(rng, 3.0, 0.03) for _ in range(views)]).reshape(-1, 12).astype(np.float32))
+    together = gs.gs_project(ctx, g, P, c["cams"])
+    for v in range(views):
+        alone = gs.gs_project(ctx, g, P[v:v + 1].contiguous(), c["cams"][v:v + 1])
+        seen = alone[2] > 0
+        for a, b in zip(together, alone):
+            a = a.reshape(views, n, -1)[v]
+            b = b.reshape(n, -1)
+            assert torch.equal(a[seen], b[seen])
+        assert torch.equal(together[2].reshape(views, n)[v], alone[2])
+
+
 @pytest.mark.parametrize("iters", [7, 8, 9, 20])
 def test_first_call_of_a_shape_equals_the_next(gs, iters):
     # the first call of a shape times the schedules on its first eight
