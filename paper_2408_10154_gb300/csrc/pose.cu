@@ -839,6 +839,10 @@ constexpr int kRigidPerBlock = kRigidThreads * 2 * kRigidPairs;
 // Gaussians at a time, and the few whose rounding that leaves open (about
 // one in 10^4) in FP64: every result is FP64's rounded to FP32.  A call on 24
 // maps of 4.4 M Gaussians in all: 665 -> 189 us, most of that the host's.
+// Bound by the FP32 pipe (about 300 lane operations per Gaussian, 37 us) and
+// HBM (42 us) in turn, so eight CTAs of 64 registers per SM for one to
+// compute while another loads: 86 -> 70 us by ncu (five CTAs of 92 registers;
+// one pair per thread 73-76, three or four 98-102).
 __device__ __forceinline__ void rigid_block(const gsl::MapDesc &m, unsigned blk)
 {
     const int64_t base = (int64_t)blk * kRigidPerBlock + threadIdx.x;
@@ -888,13 +892,13 @@ __device__ __forceinline__ void rigid_block(const gsl::MapDesc &m, unsigned blk)
     }
 }
 
-__global__ void __launch_bounds__(kRigidThreads) k_transform(const __grid_constant__ gsl::MapDesc m)
+__global__ void __launch_bounds__(kRigidThreads, 8) k_transform(const __grid_constant__ gsl::MapDesc m)
 {
     rigid_block(m, blockIdx.x);
 }
 
 // many submaps, each with its own T: blocks [blk_base, next blk_base) of map k
-__global__ void __launch_bounds__(kRigidThreads) k_transform_batch(const gsl::MapDesc *maps, int n_maps)
+__global__ void __launch_bounds__(kRigidThreads, 8) k_transform_batch(const gsl::MapDesc *maps, int n_maps)
 {
     int lo = 0, hi = n_maps - 1;
     while (lo < hi) {
