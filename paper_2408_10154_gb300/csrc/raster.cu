@@ -173,6 +173,26 @@ __device__ __forceinline__ f32x2 exponent_x2(const RecX2 &R, f32x2 pxf, f32x2 py
     return fma2(h, dx, mul2(ky, dy));
 }
 
+// both pixels' alphas of a staged record {u, v, ca, cb}, {cc, o, ...} that
+// needs neither the clamp nor the positive-exponent test; 0 where the pixel
+// is done or the alpha test fails (ok)
+__device__ __forceinline__ f32x2 fast_alpha_x2(const float4 &q0, const float4 &q1, f32x2 pxf, f32x2 pyf,
+                                               float alpha_min, bool done0, bool done1, bool &ok0, bool &ok1)
+{
+    RecX2 R;
+    R.uv = make_ulonglong2(bc2(q0.x), bc2(q0.y));
+    R.ab = make_ulonglong2(bc2(q0.z), bc2(q0.w));
+    R.co.x = bc2(q1.x);
+    f32x2 dx, h, ky;
+    float p0, p1, e0, e1, x0, x1;
+    x2_split(exponent_x2(R, pxf, pyf, dx, h, ky), p0, p1);
+    exp_ct_nonpos_x2(p0, p1, e0, e1);
+    x2_split(mul2(bc2(q1.y), x2(e0, e1)), x0, x1);
+    ok0 = !done0 && !(x0 < alpha_min);
+    ok1 = !done1 && !(x1 < alpha_min);
+    return x2(ok0 ? x0 : 0.0f, ok1 ? x1 : 0.0f);
+}
+
 // forward variants (registration mode): exposure compensation, and the
 // count of pairs that pass the alpha test (statistics runs only: the counter
 // costs the common variant a register)
@@ -188,7 +208,9 @@ constexpr int kFwdExposure = 1, kFwdCount = 2;
 // so every output is the one-pixel walk's.  Records are staged 256 at a
 // time (two per thread) with the exponent cutoff in the tile rectangle's
 // slot (stage_cutoff); only the warp cull uses it: a pair below it fails the
-// alpha test.
+// alpha test.  Records are walked two at a time (one vote, two exponentials
+// in flight; not in the fused kernel, see kPairedCtas): eight 1200x680 views
+// 253 -> 248 us, four on 300k Gaussians 143 -> 139, one 160x120 11.0 -> 9.9.
 // ---------------------------------------------------------------------------
 constexpr int kFwdThreads = 128, kFwdBatch = 256;
 
@@ -217,6 +239,13 @@ static_assert(kBwdPPT * kBwdRowStep == 8 && kTile % kBwdPatchW == 0, "warp patch
 // ---------------------------------------------------------------------------
 constexpr int kStash = 32, kStashCols = 2 * kStash;
 constexpr int kFusedCtas = 8;  // per SM: 64 registers x 128 threads and 26 KB of shared memory each
+// Walking two records at a time (PAIRED: one vote in the forward, the shuffle
+// sums of two in the adjoint side by side) takes 101 registers, four CTAs per
+// SM.  While all tiles are resident at that, the kernel is the latency of a
+// tile's walk: 320 tiles (four 160x120 views) 30.9 -> 26.2 us.  With more
+// tiles the other CTAs hide that latency, and at 64 registers the pairs
+// spill (room edge: 1.22 -> 1.25 ms), so they are walked one by one.
+constexpr int kPairedCtas = 4;
 static_assert(kFusedCtas * kStashCols <= 512, "the resident CTAs' stashes fit an SM's tensor memory");
 
 // all lanes of one warp; the address lands in *dst (shared memory)
@@ -259,7 +288,16 @@ __device__ __forceinline__ void tmem_load2(uint32_t addr, float &v0, float &v1)
                  : "memory");
 }
 
+__device__ __forceinline__ void tmem_load4(uint32_t addr, float (&v)[4])
+{
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0, %1, %2, %3}, [%4];\n\ttcgen05.wait::ld.sync.aligned;"
+                 : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3])
+                 : "r"(addr)
+                 : "memory");
+}
+
 // the adjoint half of the fused registration tile (defined with the adjoint)
+template <bool PAIRED>
 __device__ __forceinline__ void fused_adjoint(const gsl::RasterArgs &a, uint32_t t, const VpDesc &d, uint2 rg,
                                               float4 *s0, float4 *s1, float4 *s2, const uint32_t *s_v,
                                               uint8_t *s_selw, float xa, float ya, PixAdj2 &P2, int maxl,
@@ -267,7 +305,7 @@ __device__ __forceinline__ void fused_adjoint(const gsl::RasterArgs &a, uint32_t
 
 // s_tmem: fused, where the stash's address is (written before the tile's
 // first barrier)
-template <bool REG, int X, bool FUSED = false>
+template <bool REG, int X, bool FUSED = false, bool PAIRED = !FUSED>
 __device__ __forceinline__ void fwd_tile(const gsl::RasterArgs &a, const uint32_t t, const uint32_t *s_tmem = nullptr)
 {
     static_assert(REG || !FUSED, "only the registration forward is fused with the adjoint");
@@ -379,6 +417,41 @@ __device__ __forceinline__ void fwd_tile(const gsl::RasterArgs &a, const uint32_
             auto walk = [&](auto gen_tag) {
             constexpr bool GEN = decltype(gen_tag)::value;
             for (int k = 0; k < nsel; ++k) {
+                if (!GEN && PAIRED && k + 1 < nsel) {
+                    // two records in which no pixel of the warp stops: their
+                    // exponentials side by side, one vote (T only falls, so
+                    // the second's stands for both)
+                    const int ja = s_sel[warp][k], jb = s_sel[warp][k + 1];
+                    bool oa0, oa1, ob0, ob1;
+                    const f32x2 aa = fast_alpha_x2(s0[ja], s1[ja], pxf, pyf, a.alpha_min, done0, done1, oa0, oa1);
+                    const f32x2 ab = fast_alpha_x2(s0[jb], s1[jb], pxf, pyf, a.alpha_min, done0, done1, ob0, ob1);
+                    const f32x2 ta = mul2(T, sub2(bc2(1.0f), aa)), tb = mul2(ta, sub2(bc2(1.0f), ab));
+                    float tb0, tb1;
+                    x2_split(tb, tb0, tb1);
+                    if (!__any_sync(0xffffffffu, !(tb0 >= a.t_min) || !(tb1 >= a.t_min))) {
+                        const f32x2 wa = mul2(aa, T), wb = mul2(ab, ta);
+                        const float4 ca = s2[ja], cb = s2[jb];
+                        C0 = fma2(bc2(cb.x), wb, fma2(bc2(ca.x), wa, C0));
+                        C1 = fma2(bc2(cb.y), wb, fma2(bc2(ca.y), wa, C1));
+                        C2 = fma2(bc2(cb.z), wb, fma2(bc2(ca.z), wa, C2));
+                        D = fma2(bc2(s1[jb].z), wb, fma2(bc2(s1[ja].z), wa, D));
+                        T = tb;
+                        last0 = ob0 ? base + jb : (oa0 ? base + ja : last0);
+                        last1 = ob1 ? base + jb : (oa1 ? base + ja : last1);
+                        if (X & kFwdCount)
+                            nc += (int)oa0 + (int)oa1 + (int)ob0 + (int)ob1;
+                        if (FUSED && stash && k < kStash) {
+                            float v0, v1, u0, u1;
+                            x2_split(aa, v0, v1);
+                            x2_split(ab, u0, u1);
+                            tmem_store2(tmem + 2 * k, v0, v1);
+                            if (k + 1 < kStash)
+                                tmem_store2(tmem + 2 * k + 2, u0, u1);
+                        }
+                        ++k;
+                        continue;
+                    }
+                }
                 const int j = s_sel[warp][k];
                 const float4 q0 = s0[j], q1 = s1[j], q2 = s2[j];
                 RecX2 R;
@@ -626,7 +699,7 @@ __device__ __forceinline__ void fwd_tile(const gsl::RasterArgs &a, const uint32_
         P2.gd = x2(g[0][3], g[1][3]);
         P2.last0 = last0;
         P2.last1 = last1;
-        fused_adjoint(a, t, d, rg, s0, s1, s2, s_v, s_sel[warp], xa, ya, P2, maxl, wmaxl, cc, gen, fsel, tmem);
+        fused_adjoint<PAIRED>(a, t, d, rg, s0, s1, s2, s_v, s_sel[warp], xa, ya, P2, maxl, wmaxl, cc, gen, fsel, tmem);
     }
 }
 
@@ -1235,6 +1308,7 @@ __global__ void __launch_bounds__(kBwd2Threads, kBwd2MinBlocks) k_backward2_q(co
 // about 25 of 140 instructions, and the second cull (the kernel issues in
 // 76 % of its slots): room edge (100 iterations of 16 keyframes of 1200x680)
 // 137.3 -> 128.8 ms.
+template <bool PAIRED>
 __device__ __forceinline__ void fused_adjoint(const gsl::RasterArgs &a, uint32_t t, const VpDesc &d, uint2 rg,
                                               float4 *s0, float4 *s1, float4 *s2, const uint32_t *s_v,
                                               uint8_t *s_selw, float xa, float ya, PixAdj2 &P2, int maxl,
@@ -1346,6 +1420,24 @@ __device__ __forceinline__ void fused_adjoint(const gsl::RasterArgs &a, uint32_t
                     const int j = s_selw[k_next];
                     if (j < lo)
                         break;
+                    if (PAIRED && k_next > 0) {
+                        const int j2 = s_selw[k_next - 1];
+                        if (j2 >= lo) {
+                            // two records, whose sums' shuffles run side by side
+                            float g[NG], g2[NG], st[4];
+                            tmem_load4(tmem + 2 * k_next - 2, st);
+                            const bool c =
+                                pix_adj_x2<false, false, false, true>(P2, 0, record(j), 0.0f, 0.0f, 0.0f, g, st[2], st[3]);
+                            const bool c2 =
+                                pix_adj_x2<false, false, false, true>(P2, 0, record(j2), 0.0f, 0.0f, 0.0f, g2, st[0], st[1]);
+                            if (__any_sync(0xffffffffu, c || c2)) {
+                                sum_to_slot(g, j - lo);
+                                sum_to_slot(g2, j2 - lo);
+                            }
+                            --k_next;
+                            continue;
+                        }
+                    }
                     const RecX2 R = record(j);
                     float g[NG], st0, st1;
                     tmem_load2(tmem + 2 * k_next, st0, st1);
@@ -1417,14 +1509,14 @@ __device__ __forceinline__ void fused_adjoint(const gsl::RasterArgs &a, uint32_t
 // set-up of its own (descriptor, pixel state, pivot, first chunk): one
 // launch in place of the forward and the adjoint, with the same values
 // bit for bit (the same operations in the same order).
-template <int X>
-__global__ void __launch_bounds__(kFwdThreads, kFusedCtas) k_fwdbwd(const gsl::RasterArgs a)
+template <int X, bool PAIRED>
+__global__ void __launch_bounds__(kFwdThreads, PAIRED ? kPairedCtas : kFusedCtas) k_fwdbwd(const gsl::RasterArgs a)
 {
     __shared__ uint32_t s_tmem;
     if (threadIdx.x < 32)
         tmem_alloc(&s_tmem);
     pdl_wait();
-    fwd_tile<true, X, true>(a, a.tile_order ? a.tile_order[blockIdx.x] : blockIdx.x, &s_tmem);
+    fwd_tile<true, X, true, PAIRED>(a, a.tile_order ? a.tile_order[blockIdx.x] : blockIdx.x, &s_tmem);
     tmem_free(&s_tmem);
 }
 
@@ -1447,7 +1539,7 @@ constexpr size_t bwd2_smem()
 
 // CTAs of the persistent kernels: as many as can be resident at once
 // (occupancy x SMs), found once by raster_init
-int g_fwd_q_ctas = 0, g_bwd_q_ctas = 0, g_fb_q_ctas = 0;
+int g_fwd_q_ctas = 0, g_bwd_q_ctas = 0, g_fb_q_ctas = 0, g_sms = 0;
 
 // (a one-pixel-per-thread adjoint with 256-thread CTAs measured 2.00 ms
 // against 1.43 ms for this one on the room workload)
@@ -1473,7 +1565,8 @@ void launch_fwdbwd(const gsl::RasterArgs &a, cudaStream_t s)
         cudaMemsetAsync(a.queue, 0, sizeof(uint32_t), s);
         gsl::launch_pdl(k_fwdbwd_q<X>, (unsigned)std::min<uint32_t>(a.n_tiles, g_fb_q_ctas), kFwdThreads, smem, s, a);
     } else {
-        gsl::launch_pdl(k_fwdbwd<X>, a.n_tiles, kFwdThreads, smem, s, a);
+        const bool paired = !(X & kFwdCount) && a.n_tiles <= (uint32_t)(kPairedCtas * g_sms);
+        gsl::launch_pdl(paired ? k_fwdbwd<X, !(X & kFwdCount)> : k_fwdbwd<X, false>, a.n_tiles, kFwdThreads, smem, s, a);
     }
 }
 
@@ -1508,6 +1601,7 @@ void raster_init()
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&f, k_forward_q<0>, kFwdThreads, 0) == cudaSuccess &&
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_backward2_q<true, false>, kBwd2Threads,
                                                       bwd2_smem<true, false>()) == cudaSuccess) {
+        g_sms = sms;
         g_fwd_q_ctas = std::max(f, 1) * sms;
         g_bwd_q_ctas = std::max(b, 1) * sms;
         // (the query answers 1 for a kernel that allocates tensor memory; with

@@ -183,3 +183,18 @@ def test_fused_at_list_length_boundaries(gs, ctx, n):
     lb, gb = gs.gs_register_gradient(ctx, g, g, [], views, gs.default_options(fuse_compositing=0))
     np.testing.assert_array_equal(ga, gb)
     np.testing.assert_array_equal(la, lb)
+
+
+@pytest.mark.parametrize("n", [1, 2, 31, 32, 33, 34, 64, 65, 97, 129, 256, 257])
+def test_fused_records_by_pairs(gs, ctx, n):
+    # up to 608 tiles the fused kernel walks two records at a time, beyond
+    # one: both equal the two kernels bit for bit, at odd and even list
+    # lengths, around the kept alphas (32), the chunk (64) and the staging (256)
+    gd, cams = one_tile(n, 90 + n)
+    g = gs.Gaussians.from_numpy(gd)
+    views = views_of(gd, cams, 100 + n, angle=1.0, trans=0.01)
+    lb, gb = gs.gs_register_gradient(ctx, g, g, [], views, gs.default_options(fuse_compositing=0))
+    for copies in (1, 608, 609):
+        la, ga = gs.gs_register_gradient(ctx, g, g, [], views * copies)
+        np.testing.assert_array_equal(ga, np.repeat(gb, copies, 0))
+        np.testing.assert_array_equal(la, np.repeat(lb, copies, 0))
