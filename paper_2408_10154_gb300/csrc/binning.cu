@@ -787,22 +787,22 @@ __global__ void __launch_bounds__(kSegTileThreads) k_seg_ranges(const gsl::BinAr
         g[i] = 0;  // for the next build
 }
 
-constexpr uint32_t kSegSmall = 4;  // tiles of a record placed by its own thread; more: by the whole warp
-constexpr int kSegRounds = 8;       // a large record: rounds of 32 tiles whose atomics are in flight together
+constexpr uint32_t kSegSmall = 4;  // tiles of a record placed by its own thread; more: by the whole block
+constexpr int kSegRounds = 4;       // tiles of larger records per thread whose atomics are in flight together
 
 // PER records per thread (kSegThreads apart, so each load is coalesced): a
 // visible one writes its entry (depth bits << 32 | record, one 8 B store)
 // into the lists of the tiles of its rectangle at positions taken from the
 // tiles' cursors, all cursor atomics of the thread in flight before its
-// stores.  Records with more than kSegSmall tiles are spread over the lanes
-// of their warp, one record at a time, so a splat covering thousands of tiles
-// does not serialise one thread, kSegRounds rounds of 32 tiles with all their
-// atomics in flight before the stores (a record over a whole 1200x680 frame
-// is 101 rounds: one atomic round trip each made it the kernel's critical
-// path).  Positions at or past the capacity are dropped (the capacity flag
-// is already set).  Bound by the cursor atomics' latency: 60.6 us for the room
-// edge's 2.4 M records (66.9 with two 4 B stores per entry and 16 B read per
-// record), 5.9 us (6.8) for 8,000.
+// stores.  The block's records with more than kSegSmall tiles are one run of
+// tiles, which its threads share out evenly, kSegRounds at a time with all
+// their atomics in flight before the stores: taken by its warp, one record
+// after another, a splat over a whole 1200x680 frame (3,225 tiles) was 13
+// atomic round trips and a warp with several of them the kernel's tail.
+// Positions at or past the capacity are dropped (the capacity flag is already
+// set).  Bound by the cursor atomics' latency: 39 us for the room edge's 2.4 M
+// records (56.8 by warps), 19.6 us (26.7) for four views of 300k Gaussians,
+// 8.7 us (11.9) for one 640x480 view of 150k.
 template <int PER>
 __global__ void __launch_bounds__(kSegThreads) k_seg_place(const gsl::BinArgs a)
 {
@@ -853,31 +853,74 @@ __global__ void __launch_bounds__(kSegThreads) k_seg_place(const gsl::BinArgs a)
             if (k < cnt[q] && pos[q][k] < a.capacity)
                 ents[pos[q][k]] = ((uint64_t)zb[q] << 32) | rr[q];
     }
+    // the block's larger records, as one run of tiles shared by its threads
+    __shared__ uint4 s_rec[kSegThreads * PER];  // {first of its run, first tile, width | tiles per row << 16, record}
+    __shared__ uint32_t s_z[kSegThreads * PER];
+    __shared__ uint2 s_warp[kSegThreads / 32];
+    uint32_t mine = 0, tiles = 0;
 #pragma unroll
-    for (int q = 0; q < PER; ++q) {
-        unsigned m = __ballot_sync(0xffffffffu, cnt[q] > kSegSmall);
-        while (m) {
-            const int src = __ffs(m) - 1;
-            m &= m - 1;
-            const uint32_t c = __shfl_sync(0xffffffffu, cnt[q], src), b = __shfl_sync(0xffffffffu, t0[q], src);
-            const uint32_t ww = __shfl_sync(0xffffffffu, w[q], src), tt = __shfl_sync(0xffffffffu, tx[q], src);
-            const uint32_t z = __shfl_sync(0xffffffffu, zb[q], src), r = __shfl_sync(0xffffffffu, rr[q], src);
-            for (uint32_t k0 = 0; k0 < c; k0 += 32 * kSegRounds) {
-                uint32_t at[kSegRounds];
-#pragma unroll
-                for (int u = 0; u < kSegRounds; ++u) {
-                    const uint32_t k = k0 + 32 * u + lane;
-                    if (k < c)
-                        at[u] = atomicAdd(a.seg_cursor + b + (k / ww) * tt + k % ww, 1u);
-                }
-#pragma unroll
-                for (int u = 0; u < kSegRounds; ++u) {
-                    const uint32_t k = k0 + 32 * u + lane;
-                    if (k < c && at[u] < a.capacity)
-                        ents[at[u]] = ((uint64_t)z << 32) | r;
-                }
-            }
+    for (int q = 0; q < PER; ++q)
+        if (cnt[q] > kSegSmall) {
+            ++mine;
+            tiles += cnt[q];
         }
+    // both scans over the block at once
+    uint32_t at = mine, run = tiles;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t x = __shfl_up_sync(0xffffffffu, at, o), y = __shfl_up_sync(0xffffffffu, run, o);
+        if (lane >= o) {
+            at += x;
+            run += y;
+        }
+    }
+    const int warp = threadIdx.x >> 5;
+    if (lane == 31)
+        s_warp[warp] = make_uint2(at, run);
+    __syncthreads();
+    at -= mine;
+    run -= tiles;
+    uint32_t n = 0, total = 0;
+#pragma unroll
+    for (int k = 0; k < kSegThreads / 32; ++k) {
+        const uint2 x = s_warp[k];
+        at += k < warp ? x.x : 0u;
+        run += k < warp ? x.y : 0u;
+        n += x.x;
+        total += x.y;
+    }
+    if (total == 0)
+        return;
+#pragma unroll
+    for (int q = 0; q < PER; ++q)
+        if (cnt[q] > kSegSmall) {
+            s_rec[at] = make_uint4(run, t0[q], w[q] | (tx[q] << 16), rr[q]);
+            s_z[at] = zb[q];
+            ++at;
+            run += cnt[q];
+        }
+    __syncthreads();
+    for (uint32_t k0 = threadIdx.x; k0 < total; k0 += kSegThreads * kSegRounds) {
+        uint32_t to[kSegRounds], e[kSegRounds];
+#pragma unroll
+        for (int u = 0; u < kSegRounds; ++u) {
+            const uint32_t k = k0 + kSegThreads * u;
+            if (k >= total)
+                break;
+            // the last record whose run starts at or before k
+            e[u] = 0;
+#pragma unroll
+            for (uint32_t h = kSegThreads * PER / 2; h > 0; h >>= 1)
+                if (e[u] + h < n && s_rec[e[u] + h].x <= k)
+                    e[u] += h;
+            const uint4 q = s_rec[e[u]];
+            const uint32_t ww = q.z & 0xffffu, l = k - q.x;
+            to[u] = atomicAdd(a.seg_cursor + q.y + (l / ww) * (q.z >> 16) + l % ww, 1u);
+        }
+#pragma unroll
+        for (int u = 0; u < kSegRounds; ++u)
+            if (k0 + kSegThreads * u < total && to[u] < a.capacity)
+                ents[to[u]] = ((uint64_t)s_z[e[u]] << 32) | s_rec[e[u]].w;
     }
 }
 

@@ -83,3 +83,20 @@ def test_frame_shapes(env, sizes):
         r[(r[:, 0] == r[:, 1]) | (r[:, 2] == r[:, 3])] = 0
         rects.append(r)
     check(env, cams, n, np.concatenate(rects), rng.uniform(0.3, 5.0, n * len(sizes)).astype(np.float32))
+
+
+@pytest.mark.parametrize("n,large", [(1, 1.0), (3, 1.0), (257, 0.5), (300, 1.0), (2000, 0.05), (311_297, 0.002)])
+def test_records_of_many_tiles(env, n, large):
+    # records of more than four tiles share their block's threads: none, one
+    # and all of a block, runs around 1,024 tiles, one and two records a thread
+    rng = np.random.default_rng(n)
+    w, h = 16 * 33, 16 * 32
+    cams = np.stack([synth.camera(50.0, 50.0, w / 2, h / 2, w, h, np.eye(3, 4))])
+    x, y = rng.integers(0, 33, n), rng.integers(0, 32, n)
+    rects = np.stack([x, np.minimum(x + rng.integers(1, 3, n), 33), y, np.minimum(y + rng.integers(1, 3, n), 32)], 1)
+    big = np.flatnonzero(rng.random(n) < large)
+    rects[big, 0], rects[big, 2] = rng.integers(0, 2, (2, len(big)))
+    rects[big, 1], rects[big, 3] = rng.integers(7, 34, len(big)), rng.integers(2, 33, len(big))
+    rects[big, 3] = np.maximum(rects[big, 3], rects[big, 2] + 1)
+    rects[big[::3]] = [0, 33, 0, 32]
+    check(env, cams, n, rects, np.round(rng.uniform(0.3, 5.0, n), 3))
