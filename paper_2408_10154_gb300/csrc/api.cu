@@ -24,7 +24,7 @@ enum Slot {
     S_VPS, S_GROUPS, S_TILEVP, S_POSE32, S_REC, S_AUX, S_COUNTS, S_PARTIALS, S_K0, S_V0, S_RANGES, S_FLAGS, S_TF, S_LAST, S_CODE, S_TLOSS, S_TTWIST, S_POSE64, S_ADAM, S_PIVOT,
     S_CCAM, S_CENT, S_CENTP, S_LOSS, S_SETVP, S_REV, S_PFIRST, S_PCOUNT, S_RESULT, S_TOUT, S_CONF, S_EST, S_GRAD, S_DUPG,
     S_PAIRS, S_RSLOT, S_RSLOTN, S_RLONG, S_TERR, S_TCOL, S_TW,
-    S_TMED, S_TNV, S_TVPS, S_EXPO, S_EXPO32, S_TEXPO, S_OPT, S_ONN1, S_ONN2, S_OD2, S_OHDR, S_MAPS, S_OS, S_ORDER, S_ORDC, S_SK, S_SV, S_SN, S_GCELL, S_GCOUNT, S_GSTART, S_GSUMS, S_GPTS, S_GLIST, S_SEGZ, S_SEGCUR, S_SEGEXT, S_SEGLIST, S_PROBE, S_QUEUE, S_COUNT
+    S_TMED, S_TNV, S_TVPS, S_EXPO, S_EXPO32, S_TEXPO, S_OPT, S_ONN1, S_ONN2, S_OD2, S_OHDR, S_MAPS, S_OS, S_ORDER, S_SK, S_SV, S_SN, S_GCELL, S_GCOUNT, S_GSTART, S_GSUMS, S_GPTS, S_GLIST, S_SEGZ, S_SEGCUR, S_SEGEXT, S_SEGLIST, S_PROBE, S_QUEUE, S_COUNT
 };
 
 struct Buf {
@@ -2144,9 +2144,8 @@ gs_status_t run_registration(gs_ctx *ctx, Plan &P, int n_problems, const gs_opti
         r.count_contrib = opt->profile >= 2;
         gsl::TrackArgs ta;
         GS_TRY(alloc_track(ctx, P, D, r, ta, tloss, s));
-        uint32_t *order = nullptr, *order_cnt = nullptr, *queue = nullptr;
+        uint32_t *order = nullptr, *queue = nullptr;
         GS_TRY(wsT(ctx, S_ORDER, ntl, &order));
-        GS_TRY(wsT(ctx, S_ORDC, 128, &order_cnt));
         GS_TRY(wsT(ctx, S_QUEUE, 4, &queue));
         bool ordered = false, persistent = false, marking = prof;
         cudaError_t mark_err = cudaSuccess;
@@ -2161,7 +2160,7 @@ gs_status_t run_registration(gs_ctx *ctx, Plan &P, int n_problems, const gs_opti
             mark(1, st);
             const int c = run_bin(ctx, b, st);
             if (ordered)
-                gsl::tile_order(p.ranges, (uint32_t)P.n_tiles, order, order_cnt, st);
+                gsl::tile_order(p.ranges, (uint32_t)P.n_tiles, order, st);
             mark(2, st);
             r.vals = p.vals[c];
             r.tile_order = ordered ? order : nullptr;

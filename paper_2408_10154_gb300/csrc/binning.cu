@@ -486,37 +486,63 @@ __global__ void __launch_bounds__(kSortThreads) k_os_pass(const uint32_t *kin, c
 // bucket of a list length: 0 holds the longest (top bit 31), 32 the empty
 __device__ __forceinline__ uint32_t len_bucket(const uint2 r) { return (uint32_t)__clz((int)(r.y - r.x)); }
 
-__global__ void k_order_hist(const uint2 *ranges, uint32_t n, uint32_t *counts)
-{
-    __shared__ uint32_t h[33];
-    if (threadIdx.x < 33)
-        h[threadIdx.x] = 0;
-    __syncthreads();
-    const uint32_t t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t < n)
-        atomicAdd(&h[len_bucket(ranges[t])], 1u);
-    __syncthreads();
-    if (threadIdx.x < 33 && h[threadIdx.x])
-        atomicAdd(&counts[threadIdx.x], h[threadIdx.x]);
-}
+constexpr int kOrderCluster = 8, kOrderThreads = 1024;
 
-// exclusive scan of the 33 bucket counts into the cursors (one warp)
-__global__ void k_order_scan(const uint32_t *counts, uint32_t *cursors)
+// The tile order in one launch, by one cluster: each CTA counts the buckets of
+// its eighth of the tiles, takes the other CTAs' counts through distributed
+// shared memory and places its tiles, a warp's tiles of one bucket with one
+// shared atomic.  Latency-bound: 3.3 us for 3,200 tiles and 8.3 for 51,600,
+// in place of three launches and a clear whose scatter took one global atomic
+// per tile on a handful of addresses (8 and 30 us): 50 iterations of a 20k
+// edge 6.07 -> 5.68 ms, 100 of the room edge 137.0 -> 135.4 (longest first
+// through the work queue is now its fastest schedule).
+__global__ void __cluster_dims__(kOrderCluster, 1, 1) __launch_bounds__(kOrderThreads)
+    k_tile_order(const uint2 *ranges, uint32_t n, uint32_t *order)
 {
-    if (threadIdx.x == 0) {
-        uint32_t s = 0;
-        for (int b = 0; b < 33; ++b) {
-            cursors[b] = s;
-            s += counts[b];
-        }
+    constexpr uint32_t kBuckets = 33, kNone = 64;
+    __shared__ uint32_t s_h[kBuckets], s_all[kBuckets], s_cur[kBuckets];
+    const uint32_t rank = blockIdx.x % kOrderCluster, lane = threadIdx.x & 31;
+    const uint32_t per = (n + kOrderCluster - 1) / kOrderCluster;
+    const uint32_t i0 = min(rank * per, n), i1 = min(i0 + per, n);
+    if (threadIdx.x < kBuckets)
+        s_h[threadIdx.x] = 0;
+    pdl_wait();
+    __syncthreads();
+    for (uint32_t i = i0; i < i1; i += kOrderThreads) {
+        const uint32_t t = i + threadIdx.x, b = t < i1 ? len_bucket(ranges[t]) : kNone;
+        const unsigned m = __match_any_sync(0xffffffffu, b);
+        if (b < kBuckets && lane == (uint32_t)__ffs(m) - 1)
+            atomicAdd(&s_h[b], (uint32_t)__popc(m));
     }
-}
-
-__global__ void k_order_scatter(const uint2 *ranges, uint32_t n, uint32_t *cursors, uint32_t *order)
-{
-    const uint32_t t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t < n)
-        order[atomicAdd(&cursors[len_bucket(ranges[t])], 1u)] = t;
+    cluster_sync();
+    uint32_t before = 0, all = 0;
+    if (threadIdx.x < kBuckets) {
+#pragma unroll
+        for (uint32_t c = 0; c < kOrderCluster; ++c) {
+            const uint32_t x = cluster_load(&s_h[threadIdx.x], c);
+            before += c < rank ? x : 0u;
+            all += x;
+        }
+        s_all[threadIdx.x] = all;
+    }
+    __syncthreads();
+    if (threadIdx.x < kBuckets) {
+        for (uint32_t b = 0; b < threadIdx.x; ++b)
+            before += s_all[b];
+        s_cur[threadIdx.x] = before;
+    }
+    cluster_sync();  // (and every CTA has read this one's counts)
+    for (uint32_t i = i0; i < i1; i += kOrderThreads) {
+        const uint32_t t = i + threadIdx.x, b = t < i1 ? len_bucket(ranges[t]) : kNone;
+        const unsigned m = __match_any_sync(0xffffffffu, b);
+        const int first = __ffs(m) - 1;
+        uint32_t at = 0;
+        if (b < kBuckets && (int)lane == first)
+            at = atomicAdd(&s_cur[b], (uint32_t)__popc(m));
+        at = __shfl_sync(0xffffffffu, at, first);
+        if (b < kBuckets)
+            order[at + __popc(m & lanemask_lt())] = t;
+    }
 }
 
 // --------------------------------------------------------- segmented build
@@ -1196,15 +1222,10 @@ void bin_count(const BinArgs &a, cudaStream_t s)
     g_launches += 2;
 }
 
-void tile_order(const uint2 *ranges, uint32_t n_tiles, uint32_t *order, uint32_t *counters, cudaStream_t s)
+void tile_order(const uint2 *ranges, uint32_t n_tiles, uint32_t *order, cudaStream_t s)
 {
-    if (n_tiles == 0)
-        return;
-    cudaMemsetAsync(counters, 0, 64 * sizeof(uint32_t), s);
-    k_order_hist<<<div_up(n_tiles, 256), 256, 0, s>>>(ranges, n_tiles, counters);
-    k_order_scan<<<1, 32, 0, s>>>(counters, counters + 64);
-    k_order_scatter<<<div_up(n_tiles, 256), 256, 0, s>>>(ranges, n_tiles, counters + 64, order);
-    g_launches += 3;
+    if (n_tiles)
+        launch_pdl(k_tile_order, kOrderCluster, kOrderThreads, 0, s, ranges, n_tiles, order);
 }
 
 size_t onesweep_scratch_bytes(uint32_t cap, int bits)

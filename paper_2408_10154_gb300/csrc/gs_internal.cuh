@@ -209,6 +209,31 @@ __device__ __forceinline__ unsigned lanemask_lt()
     return m;
 }
 
+__device__ __forceinline__ void cluster_sync()
+{
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+// The address of the word at p's shared-memory offset in CTA `rank` of the cluster
+__device__ __forceinline__ uint32_t cluster_addr(const uint32_t *p, uint32_t rank)
+{
+    uint32_t r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(rank));
+    return r;
+}
+__device__ __forceinline__ uint32_t cluster_load(const uint32_t *p, uint32_t rank)
+{
+    uint32_t v;
+    asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(cluster_addr(p, rank)) : "memory");
+    return v;
+}
+__device__ __forceinline__ uint2 cluster_load2(const uint32_t *p, uint32_t rank)
+{
+    uint2 v;
+    asm volatile("ld.shared::cluster.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(cluster_addr(p, rank)) : "memory");
+    return v;
+}
+
 template <typename T>
 __device__ __forceinline__ T warp_sum(T v)
 {
@@ -379,8 +404,8 @@ void seg_keys64(const BinArgs &a, uint64_t *out, cudaStream_t s);
 // Tile schedule for the compositing kernels: tiles ordered by decreasing
 // list length (bucketed by the position of the length's top bit; order
 // within a bucket arbitrary), so the longest tiles start first and do not
-// form the tail of a launch.  counters: 128 uint32 of scratch.
-void tile_order(const uint2 *ranges, uint32_t n_tiles, uint32_t *order, uint32_t *counters, cudaStream_t s);
+// form the tail of a launch.
+void tile_order(const uint2 *ranges, uint32_t n_tiles, uint32_t *order, cudaStream_t s);
 
 // One-sweep LSD radix sort of 32-bit keys (8-bit digits): one histogram
 // kernel for every digit, one scan of the digit counts, one scatter per

@@ -26,22 +26,6 @@ constexpr int kMedUnroll = 8;   // pixel loads in flight per thread otherwise
 __device__ __forceinline__ constexpr int med_shift(int pass) { return pass == 0 ? 20 : (pass == 1 ? 10 : 0); }
 __device__ __forceinline__ constexpr uint32_t med_mask(int pass) { return pass == 0 ? 0x7ffu : 0x3ffu; }
 
-__device__ __forceinline__ void cluster_sync()
-{
-    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-
-// The word at the same shared-memory offset as p in CTA `rank` of the cluster
-__device__ __forceinline__ uint2 cluster_load2(const uint32_t *p, uint32_t rank)
-{
-    const uint32_t a = (uint32_t)__cvta_generic_to_shared(p);
-    uint32_t r;
-    uint2 v;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
-    asm volatile("ld.shared::cluster.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(r) : "memory");
-    return v;
-}
-
 // One cluster of kMedCluster CTAs per tracking keyframe: each CTA counts the
 // digits of its eighth of the pixels in its own shared histogram (one per
 // pass, cleared together up front), and after one cluster barrier every CTA
