@@ -478,8 +478,8 @@ gs_status_t gs_register_gradient(gs_ctx_t *ctx, const gs_gaussians_t *src, const
  * counts them first, which synchronises `stream` once.  Growing the
  * context's scratch (a larger plan than before) frees and allocates device
  * memory, which synchronises the device.  The CTA schedule is the one the
- * autotuner chose earlier for the shape, else natural order (no trial
- * runs); profile is ignored.  Calls on one context must use one stream. */
+ * autotuner chose earlier for the shape, else longest tile lists first where
+ * the tiles are more than the GPU holds at once (no trial runs); profile is ignored.  Calls on one context must use one stream. */
 gs_status_t gs_register_async(gs_ctx_t *ctx, const gs_gaussians_t *src, const gs_gaussians_t *tgt,
                               const gs_view_t *src_views, int n_src_views, const gs_view_t *tgt_views,
                               int n_tgt_views, const gs_options_t *opt, int iters, double *T_dev, double *conf_dev,

@@ -198,3 +198,18 @@ def test_fused_records_by_pairs(gs, ctx, n):
         la, ga = gs.gs_register_gradient(ctx, g, g, [], views * copies)
         np.testing.assert_array_equal(ga, np.repeat(gb, copies, 0))
         np.testing.assert_array_equal(la, np.repeat(lb, copies, 0))
+
+
+@pytest.mark.parametrize("copies", [1, 9, 1217, 8193])
+def test_every_tile_is_in_the_order(gs, ctx, copies):
+    # longest lists first: one tile per keyframe, fewer and more tiles than
+    # the ordering cluster's CTAs and threads, every keyframe's estimate that
+    # of the keyframe alone in natural order
+    gd, cams = one_tile(40, 120)
+    g = gs.Gaussians.from_numpy(gd)
+    views = views_of(gd, cams, 121, angle=1.0, trans=0.01)
+    ref = gs.gs_register(ctx, g, g, [], views, 3, gs.default_options(tile_schedule=1))
+    for sched in (0, 2):
+        _, _, eps, est = gs.gs_register(ctx, g, g, [], views * copies, 3, gs.default_options(tile_schedule=sched))
+        np.testing.assert_array_equal(est, np.repeat(ref[3], copies, 0))
+        np.testing.assert_array_equal(eps, np.repeat(ref[2], copies, 0))
