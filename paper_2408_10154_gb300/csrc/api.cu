@@ -668,6 +668,8 @@ bool lists_at_hand(const gs_ctx *ctx, Pipe &p)
 // that (139 -> 135.5) and keeps the natural order.  Registrations time both
 // unless they are small or asynchronous.
 constexpr uint64_t kOneWave = 8 * 152;
+// runs of keyframes of one loss up to which a served mix is composited run by run
+constexpr size_t kMaxRuns = 4;
 
 // scratch of the tile order, where one pays (else *order stays null)
 gs_status_t alloc_order(gs_ctx *ctx, const Plan &P, uint32_t **order)
@@ -680,8 +682,35 @@ gs_status_t alloc_order(gs_ctx *ctx, const Plan &P, uint32_t **order)
 void order_tiles(const Plan &P, gsl::RasterArgs &r, uint32_t *order, cudaStream_t s)
 {
     if (order)
-        gsl::tile_order(r.ranges, (uint32_t)P.n_tiles, order, s);
+        gsl::tile_order(r.ranges, (uint32_t)P.n_tiles, order, 0, s);
     r.tile_order = order;
+}
+
+// The tiles of consecutive keyframes of one loss, each run with its own part
+// of the tile order
+struct TileRun {
+    uint32_t first, n;
+    bool track;
+};
+
+std::vector<TileRun> tile_runs(const Plan &P)
+{
+    std::vector<TileRun> runs;
+    for (const VpDesc &d : P.vps) {
+        const bool track = d.loss_kind == 1;
+        if (runs.empty() || runs.back().track != track)
+            runs.push_back({d.tile_base, 0, track});
+        runs.back().n += (uint32_t)(d.TX * d.TY);
+    }
+    return runs;
+}
+
+gsl::RasterArgs run_args(const gsl::RasterArgs &r, const TileRun &t, uint32_t *order)
+{
+    gsl::RasterArgs a = r;
+    a.tile_order = order + t.first;
+    a.n_tiles = t.n;
+    return a;
 }
 
 gs_status_t check_common(gs_ctx *ctx, const gs_gaussians_t *g, const gs_camera_t *cams, int n_cams,
@@ -2187,7 +2216,7 @@ gs_status_t run_registration(gs_ctx *ctx, Plan &P, int n_problems, const gs_opti
             mark(1, st);
             const int c = run_bin(ctx, b, st);
             if (ordered)
-                gsl::tile_order(p.ranges, (uint32_t)P.n_tiles, order, st);
+                gsl::tile_order(p.ranges, (uint32_t)P.n_tiles, order, 0, st);
             mark(2, st);
             r.vals = p.vals[c];
             r.tile_order = ordered ? order : nullptr;
@@ -2917,10 +2946,37 @@ gs_status_t srv_replan(gs_server *srv, cudaStream_t s)
     GS_CUDA(cudaStreamBeginCapture(ctx->cap, cudaStreamCaptureModeThreadLocal));
     gsl::project(project_args(P, D, p, srv->pose32, &srv->opt, false), ctx->cap);
     r.vals = p.vals[run_bin(ctx, b, ctx->cap)];
-    order_tiles(P, r, order, ctx->cap);
-    if (srv->opt.fuse_compositing && ta.n_track == 0) {
+    // Tracking frames and loop edges served together: the edges' tiles run
+    // fused, as they do alone, and only the tracking frames' as a forward, the
+    // median and an adjoint (five 640x480 frames and an edge of about as many
+    // tiles: 402 us of compositing per iteration in one run, 391 in two, and
+    // the tracking loss of only its own tiles 17 -> 13).  Many short runs
+    // would each end in a tail of their own.
+    const std::vector<TileRun> runs = tile_runs(P);
+    const bool split = srv->opt.fuse_compositing && order && runs.size() > 1 && runs.size() <= kMaxRuns;
+    if (split) {
+        for (const TileRun &t : runs)
+            gsl::tile_order(r.ranges + t.first, t.n, order + t.first, t.first, ctx->cap);
+        for (const TileRun &t : runs)
+            if (t.track)
+                gsl::forward(run_args(r, t, order), true, ctx->cap);
+            else
+                gsl::forward_backward(run_args(r, t, order), ctx->cap);
+        gsl::track_median(ta, ctx->cap);
+        for (const TileRun &t : runs)
+            if (t.track) {
+                ta.first_tile = t.first;
+                ta.n_tiles = t.n;
+                gsl::track_tiles(ta, ctx->cap);
+            }
+        for (const TileRun &t : runs)
+            if (t.track)
+                gsl::backward(run_args(r, t, order), true, false, ctx->cap);
+    } else if (srv->opt.fuse_compositing && ta.n_track == 0) {
+        order_tiles(P, r, order, ctx->cap);
         gsl::forward_backward(r, ctx->cap);
     } else {
+        order_tiles(P, r, order, ctx->cap);
         gsl::forward(r, true, ctx->cap);
         gsl::track_loss(ta, ctx->cap);
         gsl::backward(r, true, false, ctx->cap);

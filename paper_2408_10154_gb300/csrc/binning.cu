@@ -497,7 +497,7 @@ constexpr int kOrderCluster = 8, kOrderThreads = 1024;
 // edge 6.07 -> 5.68 ms, 100 of the room edge 137.0 -> 135.4 (longest first
 // through the work queue is now its fastest schedule).
 __global__ void __cluster_dims__(kOrderCluster, 1, 1) __launch_bounds__(kOrderThreads)
-    k_tile_order(const uint2 *ranges, uint32_t n, uint32_t *order)
+    k_tile_order(const uint2 *ranges, uint32_t n, uint32_t *order, uint32_t first_tile)
 {
     constexpr uint32_t kBuckets = 33, kNone = 64;
     __shared__ uint32_t s_h[kBuckets], s_all[kBuckets], s_cur[kBuckets];
@@ -541,7 +541,7 @@ __global__ void __cluster_dims__(kOrderCluster, 1, 1) __launch_bounds__(kOrderTh
             at = atomicAdd(&s_cur[b], (uint32_t)__popc(m));
         at = __shfl_sync(0xffffffffu, at, first);
         if (b < kBuckets)
-            order[at + __popc(m & lanemask_lt())] = t;
+            order[at + __popc(m & lanemask_lt())] = first_tile + t;
     }
 }
 
@@ -1222,10 +1222,10 @@ void bin_count(const BinArgs &a, cudaStream_t s)
     g_launches += 2;
 }
 
-void tile_order(const uint2 *ranges, uint32_t n_tiles, uint32_t *order, cudaStream_t s)
+void tile_order(const uint2 *ranges, uint32_t n_tiles, uint32_t *order, uint32_t first, cudaStream_t s)
 {
     if (n_tiles)
-        launch_pdl(k_tile_order, kOrderCluster, kOrderThreads, 0, s, ranges, n_tiles, order);
+        launch_pdl(k_tile_order, kOrderCluster, kOrderThreads, 0, s, ranges, n_tiles, order, first);
 }
 
 size_t onesweep_scratch_bytes(uint32_t cap, int bits)

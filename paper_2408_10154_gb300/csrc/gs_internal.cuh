@@ -404,8 +404,9 @@ void seg_keys64(const BinArgs &a, uint64_t *out, cudaStream_t s);
 // Tile schedule for the compositing kernels: tiles ordered by decreasing
 // list length (bucketed by the position of the length's top bit; order
 // within a bucket arbitrary), so the longest tiles start first and do not
-// form the tail of a launch.
-void tile_order(const uint2 *ranges, uint32_t n_tiles, uint32_t *order, cudaStream_t s);
+// form the tail of a launch.  The tiles are first .. first + n_tiles - 1;
+// their ranges and their places in the order start at ranges and order.
+void tile_order(const uint2 *ranges, uint32_t n_tiles, uint32_t *order, uint32_t first, cudaStream_t s);
 
 // One-sweep LSD radix sort of 32-bit keys (8-bit digits): one histogram
 // kernel for every digit, one scan of the digit counts, one scatter per
@@ -478,7 +479,7 @@ void forward_backward(const RasterArgs &a, cudaStream_t s);
 struct TrackArgs {
     const gsk::VpDesc *vps;
     const uint32_t *tile_vp;
-    uint32_t n_tiles;
+    uint32_t first_tile, n_tiles;  // the tiles whose losses and weights are found
     const int *track_vps;     // [n_track] vp indices with loss_kind 1
     int n_track;
     int64_t max_pix;          // pixels of the largest of them
@@ -494,6 +495,9 @@ struct TrackArgs {
     uint8_t *inlier;
 };
 void track_loss(const TrackArgs &a, cudaStream_t s);
+// its two parts: every tracking keyframe's median, then the tiles of a
+void track_median(const TrackArgs &a, cudaStream_t s);
+void track_tiles(const TrackArgs &a, cudaStream_t s);
 // err / col of rendered images (standalone gs_track_loss)
 void track_prep(const TrackArgs &a, const float *rgb, const float *depth, float *err, float *col, cudaStream_t s);
 

@@ -127,7 +127,7 @@ __global__ void __cluster_dims__(kMedCluster, 1, 1) __launch_bounds__(kMedThread
 __global__ void __launch_bounds__(256) k_track_loss(const gsl::TrackArgs a)
 {
     __shared__ float s_red[8];
-    const uint32_t t = blockIdx.x;
+    const uint32_t t = a.first_tile + blockIdx.x;
     const int vp = (int)a.tile_vp[t];
     const VpDesc &d = a.vps[vp];
     pdl_wait();
@@ -200,10 +200,17 @@ void track_loss(const TrackArgs &a, cudaStream_t s)
 {
     if (a.n_track <= 0 || a.n_tiles == 0)
         return;
+    track_median(a, s);
+    track_tiles(a, s);
+}
+
+void track_median(const TrackArgs &a, cudaStream_t s)
+{
     launch_pdl(a.max_pix <= (int64_t)kMedCluster * kMedKeep * kMedThreads ? k_track_median<true> : k_track_median<false>,
                a.n_track * kMedCluster, kMedThreads, 0, s, a);
-    launch_pdl(k_track_loss, a.n_tiles, 256, 0, s, a);
 }
+
+void track_tiles(const TrackArgs &a, cudaStream_t s) { launch_pdl(k_track_loss, a.n_tiles, 256, 0, s, a); }
 
 void track_prep(const TrackArgs &a, const float *rgb, const float *depth, float *err, float *col, cudaStream_t s)
 {

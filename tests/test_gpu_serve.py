@@ -208,3 +208,19 @@ def test_admission_by_measured_footprint(gs, ctx, splats):
     for i, p in zip(ids, probs):
         same(srv.poll(i), gs.gs_register(ctx, *p, 8))
     srv.close()
+
+
+@pytest.mark.parametrize("order", ["tte", "ete", "tetet"])
+def test_mix_of_losses_larger_than_a_wave(gs, ctx, order):
+    # tracking frames and loop edges of more tiles than the GPU holds at once,
+    # in up to four runs of one loss (composited run by run) and in five:
+    # every result is gs_register's
+    track_opt = gs.default_options(tracking_loss=1)
+    reqs = [(tracking(gs, 800, 640, 480, 500.0, 50 + k), 6, track_opt) if c == "t" else
+            (edge(gs, 700, 640, 480, 500.0, 1, 1, 60 + k), 8, gs.default_options()) for k, c in enumerate(order)]
+    srv = gs.Server(0, max_round_iters=4)
+    ids = [srv.submit(*prob, iters, opt) for prob, iters, opt in reqs]
+    drain(srv)
+    for rid, (prob, iters, opt) in zip(ids, reqs):
+        same(srv.poll(rid), gs.gs_register(ctx, *prob, iters, opt))
+    srv.close()
