@@ -23,7 +23,8 @@
 //
 // Registration iterations (the registration loss) run both in one CTA per
 // tile (k_fwdbwd): the adjoint walks the forward's pixels from registers
-// and, for lists of at most 256 entries, the forward's staging.
+// and, for lists of at most 256 entries, the forward's staging, selection and
+// (the first 32 records of each warp) alphas.
 #include <float.h>
 
 #include <algorithm>
