@@ -518,7 +518,8 @@ gs_status_t begin_lists(gs_ctx *ctx, cudaStream_t s)
 int run_bin(gs_ctx *ctx, const gsl::BinArgs &b, cudaStream_t s)
 {
     const int cur = gsl::bin_seg(b, s);
-    ctx->seg_dirty = false;
+    // (behind a refused launch the grids may hold counts)
+    ctx->seg_dirty = cudaPeekAtLastError() != cudaSuccess;
     return cur;
 }
 
@@ -1139,6 +1140,7 @@ gs_status_t gs_render(gs_ctx_t *ctx, const gs_gaussians_t *g, const float *poses
         gsl::project(project_args(P, D, p, poses, opt, false), s);
         cur = run_bin(ctx, bin_args(P, D, p), s);
         composite();
+        GS_CUDA(cudaGetLastError());
         GS_TRY(read_flags(ctx, p, s, &flags, &nd));
         done = !(flags & gsk::kFlagCapacity);
     }

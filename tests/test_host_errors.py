@@ -1,0 +1,134 @@
+"""Host code of the library over a CUDA runtime without a GPU (fake_cudart.c,
+linked with the library's own objects): a launch that the runtime refuses is
+reported by the call that made it."""
+import ctypes
+import os
+import shutil
+import subprocess
+
+import numpy as np
+import pytest
+import torch
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+
+
+@pytest.fixture(scope="module")
+def fake_lib(tmp_path_factory):
+    if shutil.which("nvcc") is None and not os.path.exists("/usr/local/cuda/bin/nvcc"):
+        pytest.skip("nvcc not available")
+    from paper_2408_10154_gb300 import build
+    build.build()
+    d = tmp_path_factory.mktemp("fake")
+    obj, so = str(d / "fake_cudart.o"), str(d / "libgsreg_fake.so")
+    subprocess.run(["gcc", "-std=gnu11", "-w", "-fPIC", "-c", os.path.join(HERE, "fake_cudart.c"), "-o", obj], check=True)
+    objs = [os.path.join(build.BUILD, s.replace(".cu", ".o")) for s in build.SOURCES]
+    subprocess.run(["g++", "-shared", "-Wl,-Bsymbolic", "-Wl,-z,defs", "-o", so, *objs, obj], check=True)
+    return so
+
+
+@pytest.fixture
+def fake(fake_lib, monkeypatch):
+    """(package module, fake runtime) with the binding on the fake library."""
+    from paper_2408_10154_gb300 import build, gsreg
+    monkeypatch.setattr(build, "LIB", fake_lib)
+    monkeypatch.setattr(gsreg, "_lib", None)
+    monkeypatch.setattr(gsreg, "_stream", lambda: None)
+    monkeypatch.setattr(gsreg, "_ptr", lambda t: None if t is None else t.data_ptr())
+    rt = gsreg.load()
+    rt.fake_refuse(-1)
+    rt.fake_dups(0)
+    yield gsreg, rt
+    rt.fake_refuse(-1)
+
+
+class Image:
+    """A host tensor that the binding takes for a device tensor."""
+
+    def __init__(self, *shape):
+        self.t, self.is_cuda, self.is_contiguous = torch.zeros(shape), True, lambda: True
+        self.data_ptr = self.t.data_ptr
+
+
+def scene(gs, n=70):
+    z = lambda k: torch.zeros((n, k))
+    g = gs.Gaussians(z(4), z(4), z(4), torch.zeros(n), z(4))
+    cam = np.array([30, 30, 16, 16, 32, 32, 1, 0, 0, 0, 0, 1, 0, 0, 0, 0, 1, 0], np.float32)
+    return g, torch.eye(3, 4).reshape(1, 12), cam[None], (cam, Image(3, 32, 32), Image(32, 32))
+
+
+def calls(gs, ctx):
+    g, P, cams, view = scene(gs)
+    few = gs.Gaussians(*[t[:40].contiguous() for t in (g.means4, g.log_scales4, g.quats4, g.logits, g.rgb4)])
+
+    def saved():
+        _, sv = gs.gs_render_saved(ctx, g, P, cams)
+        try:
+            gs.gs_render_backward_saved(ctx, sv, params=True)
+        finally:
+            sv.close()
+
+    return {
+        "render": lambda: gs.gs_render(ctx, g, P, cams),
+        "saved": saved,
+        "loss": lambda: gs.gs_loss(ctx, cams, torch.zeros(3 * 1024), torch.zeros(1024), torch.zeros(3 * 1024),
+                                   torch.zeros(1024)),
+        "register": lambda: gs.gs_register(ctx, g, g, [view], [view], 2),
+        "batch": lambda: gs.gs_register_batch(ctx, [(g, g, [view], [view])], 2),
+        "overlap": lambda: gs.gs_overlap_ratio(ctx, few, few, np.eye(3, 4)),
+        "transform": lambda: gs.gs_transform(ctx, g, np.eye(3, 4)),
+        "transform_batch": lambda: gs.gs_transform_batch(ctx, [g, g], np.stack([np.eye(3, 4)] * 2)),
+    }
+
+
+@pytest.mark.parametrize("name", ["render", "saved", "loss", "overlap", "transform", "transform_batch"])
+def test_a_refused_launch_is_reported(fake, name):
+    # every launch of a call in turn, on a first call and on the later ones
+    # of a context (which take what the first left)
+    gs, rt = fake
+    for warm in (0, 2):
+        n = 0
+        while True:
+            ctx = gs.Context(0)
+            call = calls(gs, ctx)[name]
+            for _ in range(warm):
+                call()
+            rt.fake_refuse(n)
+            try:
+                call()
+                reported = False
+            except gs.GsError as e:
+                reported = True
+                assert e.status == 3, e  # GS_ERR_CUDA
+            launched = rt.fake_launches()
+            rt.fake_refuse(-1)
+            ctx.close()
+            if launched <= n:
+                break
+            assert reported, (warm, n)
+            n += 1
+        assert n > 0 and not reported
+
+
+def test_counting_grids_are_cleared_behind_a_refused_launch(fake):
+    # a repeated render clears nothing (each list build leaves the counting
+    # grids clear), but the one behind a call whose list build was refused does
+    gs, rt = fake
+    ctx = gs.Context(0)
+    render = calls(gs, ctx)["render"]
+
+    def memsets():
+        before = rt.fake_memsets()
+        render()
+        return rt.fake_memsets() - before
+
+    memsets()
+    usual = memsets()
+    for n in (2, 3):  # tables, projection, then the ranges and the placement
+        rt.fake_refuse(n)
+        with pytest.raises(gs.GsError):
+            render()
+        rt.fake_refuse(-1)
+        assert memsets() == usual + 1
+        assert memsets() == usual
+    ctx.close()
