@@ -2446,6 +2446,7 @@ gs_status_t run_registration(gs_ctx *ctx, Plan &P, int n_problems, const gs_opti
         GS_TRY(wsT(ctx, S_RESULT, (size_t)total, &q.out));
         k_reg_result<<<1, 1024, 0, s>>>(q);
         ++gsl::g_launches;
+        GS_CUDA(cudaGetLastError());
         void *hostp = nullptr;
         GS_TRY(host_block(ctx, total * sizeof(double), &hostp));
         GS_CUDA(cudaMemcpyAsync(hostp, q.out, total * sizeof(double), cudaMemcpyDeviceToHost, s));

@@ -81,7 +81,8 @@ def calls(gs, ctx):
     }
 
 
-@pytest.mark.parametrize("name", ["render", "saved", "loss", "overlap", "transform", "transform_batch"])
+@pytest.mark.parametrize("name", ["render", "saved", "loss", "register", "batch", "overlap", "transform",
+                                  "transform_batch"])
 def test_a_refused_launch_is_reported(fake, name):
     # every launch of a call in turn, on a first call and on the later ones
     # of a context (which take what the first left)
