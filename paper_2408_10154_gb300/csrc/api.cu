@@ -1454,7 +1454,6 @@ gs_status_t gs_render_saved(gs_ctx_t *ctx, const gs_gaussians_t *g, const float 
             gsl::project(project_args(P, sv->D, p, sv->pose32, opt), s);
         }
         sv->vals = (uint32_t *)sv->blk[1];
-        sv->cap = p.cap;
         p.vals[0] = sv->vals;  // the sorted lists land in the saved block
         const int cur = run_bin(ctx, bin_args(P, sv->D, p), s);
         gsl::RasterArgs r = raster_args(P, sv->D, p, cur, opt);
@@ -1478,6 +1477,22 @@ gs_status_t gs_render_saved(gs_ctx_t *ctx, const gs_gaussians_t *g, const float 
     }
     uint32_t &most = ctx->saved_seen[key];
     most = std::max(most, nd);
+    // the adjoint's slots are those of the duplicates there are, whatever the
+    // guess was, and a block that the guess made much too long is not kept
+    sv->cap = std::max(nd, 1u);
+    if (p.cap > (uint64_t)nd + nd / 2 + 65536) {
+        void *b = nullptr;
+        if (cudaMallocAsync(&b, sizeof(uint32_t) * (size_t)sv->cap, s) == cudaSuccess) {
+            const bool ok = copy(b, sv->vals, sizeof(uint32_t) * (size_t)nd, cudaMemcpyDeviceToDevice);
+            cudaFreeAsync(sv->blk[1], s);
+            sv->blk[1] = b;
+            sv->vals = (uint32_t *)b;
+            if (!ok)
+                return cleanup(fail(ctx, GS_ERR_CUDA, "gs_render_saved: copy of the lists"));
+        } else {
+            cudaGetLastError();  // (kept as it is)
+        }
+    }
     if (flags & gsk::kFlagNonFinite)
         return cleanup(fail(ctx, GS_ERR_NONFINITE, "non-finite Gaussian parameter"));
     ctx->stats = gs_stats_t{};

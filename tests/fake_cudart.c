@@ -37,10 +37,26 @@ const char *cudaGetErrorString() { return "refused"; }
 static int take(void **p, size_t n) { return (*p = calloc(n ? n : 1, 1)) ? 0 : 2; }
 int cudaMalloc(void **p, size_t n) { return take(p, n); }
 int cudaMallocHost(void **p, size_t n) { return take(p, n); }
-int cudaMallocAsync(void **p, size_t n) { return take(p, n); }
 int cudaFree(void *p) { return free(p), 0; }
 int cudaFreeHost(void *p) { return free(p), 0; }
-int cudaFreeAsync(void *p) { return free(p), 0; }
+
+/* stream-ordered blocks, their bytes counted */
+static size_t g_pool;
+size_t fake_pool_bytes(void) { return g_pool; }
+int cudaMallocAsync(void **p, size_t n)
+{
+    size_t *b = calloc(n + 64, 1);
+    if (!b)
+        return 2;
+    *b = n;
+    g_pool += n;
+    return *p = (char *)b + 64, 0;
+}
+int cudaFreeAsync(void *p)
+{
+    size_t *b = (size_t *)((char *)p - 64);
+    return g_pool -= *b, free(b), 0;
+}
 int cudaMemcpyAsync(void *dst, const void *src, size_t n, int kind)
 {
     memcpy(dst, src, n);

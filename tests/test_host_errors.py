@@ -1,6 +1,7 @@
 """Host code of the library over a CUDA runtime without a GPU (fake_cudart.c,
 linked with the library's own objects): a launch that the runtime refuses is
-reported by the call that made it."""
+reported by the call that made it, and a saved forward's adjoint takes the
+scratch of its own duplicates."""
 import ctypes
 import os
 import shutil
@@ -36,6 +37,7 @@ def fake(fake_lib, monkeypatch):
     monkeypatch.setattr(gsreg, "_stream", lambda: None)
     monkeypatch.setattr(gsreg, "_ptr", lambda t: None if t is None else t.data_ptr())
     rt = gsreg.load()
+    rt.fake_pool_bytes.restype = ctypes.c_size_t
     rt.fake_refuse(-1)
     rt.fake_dups(0)
     yield gsreg, rt
@@ -133,3 +135,69 @@ def test_counting_grids_are_cleared_behind_a_refused_launch(fake):
         assert memsets() == usual + 1
         assert memsets() == usual
     ctx.close()
+
+
+def train(gs, ctx, adjoint=True):
+    g, P, cams, _ = scene(gs)
+    _, sv = gs.gs_render_saved(ctx, g, P, cams)
+    try:
+        if adjoint:
+            gs.gs_render_backward_saved(ctx, sv, params=True)
+    finally:
+        sv.close()
+
+
+def test_a_repeated_training_step_fits_the_first_ones_budget(fake):
+    # the lists of a repeated pass are sized by a guess; its adjoint's slots
+    # are those of the duplicates it has
+    gs, rt = fake
+    rt.fake_dups(400_000)
+
+    def passes(budget, times):
+        ctx = gs.Context(0, budget)
+        try:
+            for _ in range(times):
+                train(gs, ctx)
+            return True
+        except gs.GsError as e:
+            assert e.status == 2, e  # GS_ERR_OOM
+            return False
+        finally:
+            ctx.close()
+
+    lo, hi = 1 << 16, 1 << 28
+    assert not passes(lo, 1) and passes(hi, 1)
+    while hi - lo > 256:
+        mid = (lo + hi) // 2
+        lo, hi = (lo, mid) if passes(mid, 1) else (mid, hi)
+    assert passes(hi, 3)
+
+
+def test_a_pass_with_many_duplicates_does_not_inflate_later_ones(fake):
+    gs, rt = fake
+
+    def after(dups):
+        """scratch of the adjoint, and bytes of the saved forward, of a pass
+        with 100,000 duplicates behind passes with dups of them"""
+        ctx = gs.Context(0)
+        for d in dups:
+            rt.fake_dups(d)
+            train(gs, ctx, adjoint=False)
+        rt.fake_dups(100_000)
+        g, P, cams, _ = scene(gs)
+        before, pool = ctx.bytes(), rt.fake_pool_bytes()
+        _, sv = gs.gs_render_saved(ctx, g, P, cams)
+        pool = rt.fake_pool_bytes() - pool
+        lists = ctx.bytes()
+        gs.gs_render_backward_saved(ctx, sv, params=True)
+        scratch = ctx.bytes() - lists
+        assert lists == before or not dups
+        sv.close()
+        ctx.close()
+        return scratch, pool
+
+    alone = after([])
+    many = after([3_000_000, 3_000_000])
+    assert many[0] == alone[0]
+    # (a block that is at most half as long again, and 64 Ki entries, is kept)
+    assert many[1] <= alone[1] + 4 * (50_000 + 65_536)
