@@ -1,11 +1,13 @@
 """Host code of the library over a CUDA runtime without a GPU (fake_cudart.c,
 linked with the library's own objects): a launch that the runtime refuses is
-reported by the call that made it, and a saved forward's adjoint takes the
-scratch of its own duplicates."""
+reported by the call that made it, a saved forward's adjoint takes the scratch
+of its own duplicates, and the binding's marshalling costs no more than the
+plain ctypes arrays."""
 import ctypes
 import os
 import shutil
 import subprocess
+import time
 
 import numpy as np
 import pytest
@@ -201,3 +203,31 @@ def test_a_pass_with_many_duplicates_does_not_inflate_later_ones(fake):
     assert many[0] == alone[0]
     # (a block that is at most half as long again, and 64 Ki entries, is kept)
     assert many[1] <= alone[1] + 4 * (50_000 + 65_536)
+
+
+@pytest.mark.parametrize("n", [1, 2, 4, 8, 24])
+def test_transform_batch_marshalling_cost(fake, n):
+    # the host time of a call on a few maps, against the same call through
+    # one ctypes array per argument (best of many, in turn)
+    gs, rt = fake
+    ctx = gs.Context(0)
+    maps, Ts = [scene(gs, 8)[0] for _ in range(n)], np.stack([np.eye(3, 4)] * n)
+
+    def plain():
+        arr = (gs.gs_gaussians_t * n)(*[g.c_struct() for g in maps])
+        Th = np.ascontiguousarray(np.asarray(Ts, np.float64).reshape(n, 12))
+        outs = [(torch.empty_like(g.means4), torch.empty_like(g.quats4)) for g in maps]
+        om = (ctypes.c_void_p * n)(*[m.data_ptr() for m, _ in outs])
+        oq = (ctypes.c_void_p * n)(*[q.data_ptr() for _, q in outs])
+        ctx.check(rt.gs_transform_batch(ctx.handle, arr, n, Th.ctypes.data_as(ctypes.c_void_p), om, oq, None))
+        return [gs.Gaussians(m, g.log_scales4, q, g.logits, g.rgb4) for g, (m, q) in zip(maps, outs)]
+
+    def best(f):
+        t = time.perf_counter()
+        for _ in range(20):
+            f()
+        return time.perf_counter() - t
+
+    times = [(best(lambda: gs.gs_transform_batch(ctx, maps, Ts)), best(plain)) for _ in range(60)]
+    ctx.close()
+    assert min(t for t, _ in times) <= 1.1 * min(t for _, t in times)
