@@ -196,3 +196,43 @@ def test_saved_forward_repeats_at_the_smallest_budget(env):
         mid = (lo + hi) // 2
         lo, hi = (lo, mid) if passes(mid, 1) else (mid, hi)
     assert passes(hi, 3)
+
+
+def test_lists_too_short_for_the_next_scene(env):
+    # a scene whose duplicates exceed what the context's lists hold is
+    # composited again once they are counted, and a smaller one behind it
+    # keeps no more than its own lists: outputs and gradients as on a fresh
+    # context, before and after
+    gs, _, _ = env
+    rng = np.random.default_rng(80)
+    few = synth.gaussians_box(900, rng, half=1.2, ls_mean=-5.0, ls_std=0.2)
+    many = {k: v.copy() for k, v in few.items()}
+    many["log_scales4"][:, :3] += 4.2
+    many["logits"][:] = -3.0
+    cams = synth.circle_cameras(2, 0.25, (0.0, 0.0, 2.5), 640, 480, 500.0)
+    P = dev(np.stack([np.eye(3, 4).reshape(12)] * 2))
+    npx = 2 * 640 * 480
+    cr, cd = dev(rng.standard_normal(3 * npx)), dev(rng.standard_normal(npx))
+
+    def render(ctx, gd):
+        out = gs.gs_render(ctx, gs.Gaussians.from_numpy(gd), P, cams)
+        return [out[k] for k in ("rgb", "depth", "alpha", "t_final", "last")]
+
+    def step(ctx, gd):
+        out, sv = gs.gs_render_saved(ctx, gs.Gaussians.from_numpy(gd), P, cams)
+        pg, gr = gs.gs_render_backward_saved(ctx, sv, cr, cd, params=True)
+        sv.close()
+        return [out[k] for k in ("rgb", "depth", "alpha")] + [pg] + [gr[k] for k in sorted(gr)]
+
+    for f in (render, step):
+        want = {}
+        for name, gd in (("few", few), ("many", many)):
+            fresh = gs.Context(0)
+            want[name] = f(fresh, gd)
+            fresh.close()
+        ctx = gs.Context(0)
+        for name, gd in (("few", few), ("many", many), ("few", few), ("few", few), ("many", many)):
+            got = f(ctx, gd)
+            for k, (x, y) in enumerate(zip(got, want[name])):
+                assert torch.equal(x, y), (f.__name__, name, k)
+        ctx.close()
