@@ -880,8 +880,6 @@ gs_status_t alloc_track(gs_ctx *ctx, const Plan &P, const DevPlan &D, gsl::Raste
     ta.n_tiles = (uint32_t)P.n_tiles;
     ta.track_vps = tvd;
     ta.n_track = (int)tv.size();
-    for (int v : tv)
-        ta.max_pix = std::max(ta.max_pix, (int64_t)P.vps[v].W * P.vps[v].H);
     ta.t_final = r.t_final;
     ta.err = r.trk_err;
     ta.col = r.trk_col;

@@ -482,7 +482,6 @@ struct TrackArgs {
     uint32_t first_tile, n_tiles;  // the tiles whose losses and weights are found
     const int *track_vps;     // [n_track] vp indices with loss_kind 1
     int n_track;
-    int64_t max_pix;          // pixels of the largest of them
     const float *t_final;     // [pix]
     const float *err, *col;   // [pix] from the forward (or k_track_prep)
     float *med;               // [vp] median depth error

@@ -20,8 +20,14 @@ constexpr uint32_t kInfBits = 0x7f800000u;  // +inf marks a pixel without input 
 constexpr int kMedThreads = 1024;
 constexpr int kMedBins = 2048;
 constexpr int kMedCluster = 8;  // CTAs per keyframe (the portable cluster size)
-constexpr int kMedKeep = 38;    // pixels per thread held in registers (640x480: 37.5)
-constexpr int kMedUnroll = 8;   // pixel loads in flight per thread otherwise
+constexpr int kMedUnroll = 8;   // pixel loads in flight per thread beyond the kept ones
+// pixels per thread held in registers over the passes: of the 64 that 1024
+// threads leave each, eight for those loads and 16 to work with (with 48 kept:
+// 18.7 us for 640x480, 17.9 with 40, and 20.2 against 20.4 for 768x512, where
+// 48 hold the whole slice)
+constexpr int kMedKeep = 65536 / kMedThreads - kMedUnroll - 16;
+constexpr int kMedGroup = 4;    // of those, taken or left out together
+static_assert(kMedKeep % kMedGroup == 0, "the kept pixels are whole groups");
 // the three digits, high to low, of a non-negative float's 31 bits
 __device__ __forceinline__ constexpr int med_shift(int pass) { return pass == 0 ? 20 : (pass == 1 ? 10 : 0); }
 __device__ __forceinline__ constexpr uint32_t med_mask(int pass) { return pass == 0 ? 0x7ffu : 0x3ffu; }
@@ -31,15 +37,16 @@ __device__ __forceinline__ constexpr uint32_t med_mask(int pass) { return pass =
 // pass, cleared together up front), and after one cluster barrier every CTA
 // adds the eight histograms through distributed shared memory and finds the
 // digit that holds the median's rank -- the same on all of them, so nothing
-// is sent back.  KEEP: a slice of at most kMedKeep pixels per thread is read
-// once and kept in registers over the three passes; a larger one is read by
-// each.  Bound by latency (one frame is 1.2 MB; reading it three times took
-// 7 us more of a tracking iteration).  One CTA per keyframe took 346 us on a
+// is sent back.  The first kMedKeep pixels per thread of its slice
+// are read once and kept in registers over the three passes; what lies beyond
+// (frames of more than 327,680 pixels) is read by each.  Bound by latency (one
+// 640x480 frame is 1.2 MB): 14.1, 17.9, 17.8 and 34.0 us for 320x240, 640x480,
+// 660x480 and 1200x680 by ncu; with one limit for a whole slice, 38 pixels, and
+// none left out, 16.7, 18.1, 22.8 and 38.6.  One CTA per keyframe took 346 us on a
 // 640x480 frame, by ncu: each pass one dependent load and one match_any per
 // 1024 pixels; the tracking iteration spent two thirds of its time there (40
 // iterations of a 640x480 frame on 150k Gaussians: 18.97 -> 7.06 ms with
 // this kernel).
-template <bool KEEP>
 __global__ void __cluster_dims__(kMedCluster, 1, 1) __launch_bounds__(kMedThreads) k_track_median(const gsl::TrackArgs a)
 {
     __shared__ __align__(8) uint32_t hist[3][kMedBins];
@@ -48,42 +55,48 @@ __global__ void __cluster_dims__(kMedCluster, 1, 1) __launch_bounds__(kMedThread
     const uint32_t rank = blockIdx.x % kMedCluster;
     const int vp = a.track_vps[blockIdx.x / kMedCluster];
     const VpDesc &d = a.vps[vp];
-    const int64_t n = (int64_t)d.W * d.H;
-    const int64_t per = (n + kMedCluster - 1) / kMedCluster;
-    const int64_t i0 = min((int64_t)rank * per, n), i1 = min(i0 + per, n);
-    const uint32_t *v = reinterpret_cast<const uint32_t *>(a.err) + d.pix_base;
+    // (a keyframe has at most 2^30 pixels)
+    const uint32_t n = (uint32_t)d.W * (uint32_t)d.H, per = (n + kMedCluster - 1) / kMedCluster;
+    const uint32_t i0 = min(rank * per, n), len = min(i0 + per, n) - i0;
+    const uint32_t *v = reinterpret_cast<const uint32_t *>(a.err) + d.pix_base + i0;
     for (int b = threadIdx.x; b < 3 * kMedBins; b += kMedThreads)
         (&hist[0][0])[b] = 0;
     pdl_wait();
-    uint32_t kept[KEEP ? kMedKeep : 1];
-    if (KEEP) {
+    // (a group that lies past the slice is left out)
+    uint32_t kept[kMedKeep];
 #pragma unroll
-        for (int u = 0; u < kMedKeep; ++u) {
-            const int64_t i = i0 + u * kMedThreads + threadIdx.x;
-            kept[u] = i < i1 ? v[i] : kInfBits;
+    for (int g = 0; g < kMedKeep; g += kMedGroup)
+        if ((uint32_t)g * kMedThreads < len) {
+#pragma unroll
+            for (int u = g; u < g + kMedGroup; ++u) {
+                const uint32_t i = u * kMedThreads + threadIdx.x;
+                kept[u] = i < len ? v[i] : kInfBits;
+            }
         }
-    }
     __syncthreads();
     uint32_t prefix = 0, mask = 0, k = 0, m = 0;
 #pragma unroll
     for (int pass = 0; pass < 3; ++pass) {
         uint32_t *h = hist[pass];
-        if (KEEP) {
+        auto count = [&](uint32_t x) {
+            if (x < kInfBits && (x & mask) == prefix)
+                atomicAdd(&h[(x >> med_shift(pass)) & med_mask(pass)], 1u);
+        };
 #pragma unroll
-            for (int u = 0; u < kMedKeep; ++u)
-                if (kept[u] < kInfBits && (kept[u] & mask) == prefix)
-                    atomicAdd(&h[(kept[u] >> med_shift(pass)) & med_mask(pass)], 1u);
-        } else {
-            for (int64_t base = i0 + threadIdx.x; base < i1; base += kMedUnroll * kMedThreads) {
-                uint32_t x[kMedUnroll];
+        for (int g = 0; g < kMedKeep; g += kMedGroup)
+            if ((uint32_t)g * kMedThreads < len) {
 #pragma unroll
-                for (int u = 0; u < kMedUnroll; ++u)
-                    x[u] = base + u * kMedThreads < i1 ? v[base + u * kMedThreads] : kInfBits;
-#pragma unroll
-                for (int u = 0; u < kMedUnroll; ++u)
-                    if (x[u] < kInfBits && (x[u] & mask) == prefix)
-                        atomicAdd(&h[(x[u] >> med_shift(pass)) & med_mask(pass)], 1u);
+                for (int u = g; u < g + kMedGroup; ++u)
+                    count(kept[u]);
             }
+        for (uint32_t base = kMedKeep * kMedThreads + threadIdx.x; base < len; base += kMedUnroll * kMedThreads) {
+            uint32_t x[kMedUnroll];
+#pragma unroll
+            for (int u = 0; u < kMedUnroll; ++u)
+                x[u] = base + u * kMedThreads < len ? v[base + u * kMedThreads] : kInfBits;
+#pragma unroll
+            for (int u = 0; u < kMedUnroll; ++u)
+                count(x[u]);
         }
         cluster_sync();
         // the cluster's counts of bins 2t and 2t + 1, their exclusive scan,
@@ -206,8 +219,7 @@ void track_loss(const TrackArgs &a, cudaStream_t s)
 
 void track_median(const TrackArgs &a, cudaStream_t s)
 {
-    launch_pdl(a.max_pix <= (int64_t)kMedCluster * kMedKeep * kMedThreads ? k_track_median<true> : k_track_median<false>,
-               a.n_track * kMedCluster, kMedThreads, 0, s, a);
+    launch_pdl(k_track_median, a.n_track * kMedCluster, kMedThreads, 0, s, a);
 }
 
 void track_tiles(const TrackArgs &a, cudaStream_t s) { launch_pdl(k_track_loss, a.n_tiles, 256, 0, s, a); }

@@ -236,3 +236,10 @@ def test_track_median_sizes(gs, ctx, w, h, kind):
         assert med[k] == want
         np.testing.assert_array_equal(inl[o:o + len(d)].astype(bool), (t > 0) & (e <= np.float32(50.0) * want))
         o += len(d)
+
+
+@pytest.mark.parametrize("w,h", [(256, 128), (257, 128), (640, 512), (641, 512), (1200, 680)])
+def test_track_median_kept_pixels(gs, ctx, w, h):
+    # one group of four pixels per thread and the first pixels of the next;
+    # all 40 kept in registers (327,680 pixels), and the first ones beyond
+    test_track_median_sizes(gs, ctx, w, h, "spread")
