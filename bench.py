@@ -52,7 +52,7 @@ BWD_FLOPS_CONTRIB = 64.0
 # current kernel (the fused forward + adjoint that the timed calls run, and
 # the two-kernel adjoint); None while the kernel has changed since the capture
 FB_TRAFFIC_BYTES = 323.629568e6
-BWD_TRAFFIC_BYTES = 185.502976e6
+BWD_TRAFFIC_BYTES = 210.119680e6
 FP32_LANES = 128
 PEAK_FILE = os.path.join(ROOT, "MEASURED_PEAKS.json")
 
@@ -335,18 +335,20 @@ def run_ours(args):
         roof = {"kernel": names[dom], "bound": "hbm", "achieved": None, "peak": hbm, "unit": "GB/s", "frac": None,
                 "traffic": None}
     # HBM-bound steps: algorithmic bytes per launch / CUDA-event time.
-    # Projection: 56 B per Gaussian of each moving submap + 52 B (48 B
-    # record + 4 B count) per visible (keyframe, Gaussian).  Tile lists:
-    # 16 B entry read per visible record, 8 B written at placement and 8 B
-    # read + 8 B written by the per-tile sort per duplicate, 8 B range per tile.
+    # Projection: 56 B read per Gaussian of each moving submap, a 4 B extent
+    # written per (keyframe, Gaussian) and 92 B (48 B record, 32 B auxiliary,
+    # 12 B list entry) per visible one.  Tile lists: the extents and the
+    # entries read, 8 B written at placement and 8 B read + 4 B written by the
+    # per-tile sort per duplicate, 8 B range per tile.
     I8 = torch.tensor(np.stack([np.eye(3, 4)] * 8).reshape(8, 12), dtype=torch.float32, device="cuda")
     vis = sum(int((gs.gs_project(ctx, g, I8, cams, with_aux=False)[2] > 0).sum())
               for g, cams in ((tgt, c["src_cams"]), (src, c["tgt_cams"])))
     tiles = 16 * ((1200 + 15) // 16) * ((680 + 15) // 16)
+    extents = 4.0 * (tgt.n * len(c["src_cams"]) + src.n * len(c["tgt_cams"]))
     hbm_peak = pk.get("hbm_gbs", 6800.0)
     hbm = {}
-    for name, nbytes in (("project", 56.0 * (src.n + tgt.n) + 52.0 * vis),
-                         ("bin", 16.0 * vis + 24.0 * dups + 8.0 * tiles)):
+    for name, nbytes in (("project", 56.0 * (src.n + tgt.n) + extents + 92.0 * vis),
+                         ("bin", extents + 12.0 * vis + 20.0 * dups + 8.0 * tiles)):
         ms = per_launch_ms[names.index(name)]
         gbs = nbytes / (ms / 1000.0) / 1e9
         hbm[name] = {"bytes_per_launch": nbytes, "ms_per_launch": float(ms), "achieved_gbs": gbs,

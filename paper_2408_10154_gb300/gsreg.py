@@ -469,7 +469,7 @@ def _views(views):
     n = len(views)
     arr = (gs_view_t * max(n, 1))()
     if n:
-        # gs_view_t: two pointers, then the camera's 18 words (and 8 bytes to the next)
+        # gs_view_t: two pointers, then the camera's 18 words
         w = np.frombuffer(arr, np.uint8).reshape(n, -1)
         w[:, :16] = np.array([(rgb.data_ptr(), depth.data_ptr()) for _, rgb, depth in views],
                              np.uint64).view(np.uint8).reshape(n, 16)
